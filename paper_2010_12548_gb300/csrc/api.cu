@@ -344,7 +344,6 @@ sdb_status raster_common(const PolyEdges& pe, uint32_t grid_bits, uint32_t k,
     set_error("n = %llu points: at most 2^32 - 1 per call", (unsigned long long)n);
     return SDB_EINVAL;
   }
-  if (tile_bits == 0) tile_bits = 13;
   if (tile_bits > 14) {
     set_error("tile_bits %u outside 1..14 (0 = default 13)", tile_bits);
     return SDB_EINVAL;

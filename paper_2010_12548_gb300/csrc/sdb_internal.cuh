@@ -439,6 +439,8 @@ sdb_status launch_join(const uint32_t* x, const uint32_t* y, const int32_t* attr
 // sort.cu: device-wide primitives
 template <class T>
 sdb_status exclusive_scan(const T* in, T* out, size_t n, T* d_total, cudaStream_t s);
+// out[i] = in[0] + ... + in[i - 1] in 64 bits, i in [0, n] (n + 1 entries)
+sdb_status exclusive_scan_i32(const int32_t* in, int64_t* out, size_t n, cudaStream_t s);
 // keys-only LSD sort of packed covering records (record_pack) on their key
 // bits [first_bit, first_bit + bits); the result is split into keys
 // (*keys_out, one of keys / tmp) and standard values (vals_out)

@@ -43,23 +43,33 @@ __device__ T block_exclusive_scan(T v, T* s_warp, T* total) {
   return r;
 }
 
+// the value of an input element in the sums' type (signed inputs sign-extend)
 template <class T>
-__global__ __launch_bounds__(SCAN_THREADS) void scan_reduce_kernel(const T* in, size_t n, T* sums) {
+__device__ __forceinline__ T scan_value(T v) {
+  return v;
+}
+template <class T>
+__device__ __forceinline__ T scan_value(int32_t v) {
+  return (T)(int64_t)v;
+}
+
+template <class T, class In>
+__global__ __launch_bounds__(SCAN_THREADS) void scan_reduce_kernel(const In* in, size_t n, T* sums) {
   __shared__ T s_warp[SCAN_THREADS / 32 + 1];
   size_t base = (size_t)blockIdx.x * SCAN_TILE;
   T acc = 0;
 #pragma unroll
   for (int i = 0; i < SCAN_ITEMS; ++i) {
     size_t g = base + (size_t)i * SCAN_THREADS + threadIdx.x;
-    if (g < n) acc += in[g];
+    if (g < n) acc += scan_value<T>(in[g]);
   }
   T tot;
   block_exclusive_scan<T>(acc, s_warp, &tot);
   if (threadIdx.x == 0) sums[blockIdx.x] = tot;
 }
 
-template <class T>
-__global__ __launch_bounds__(SCAN_THREADS) void scan_tile_kernel(const T* in, T* out, size_t n,
+template <class T, class In>
+__global__ __launch_bounds__(SCAN_THREADS) void scan_tile_kernel(const In* in, T* out, size_t n,
                                                                  const T* block_off, T* d_total) {
   __shared__ T s_warp[SCAN_THREADS / 32 + 1];
   size_t base = (size_t)blockIdx.x * SCAN_TILE + (size_t)threadIdx.x * SCAN_ITEMS;
@@ -68,7 +78,7 @@ __global__ __launch_bounds__(SCAN_THREADS) void scan_tile_kernel(const T* in, T*
 #pragma unroll
   for (int i = 0; i < SCAN_ITEMS; ++i) {
     size_t g = base + i;
-    v[i] = g < n ? in[g] : T(0);
+    v[i] = g < n ? scan_value<T>(in[g]) : T(0);
     acc += v[i];
   }
   T tot;
@@ -357,15 +367,16 @@ __global__ void compact_flagged_kernel(const uint64_t* in, size_t n, const uint3
 
 }  // namespace
 
-template <class T>
-sdb_status exclusive_scan(const T* in, T* out, size_t n, T* d_total, cudaStream_t s) {
+namespace {
+template <class T, class In>
+sdb_status scan_impl(const In* in, T* out, size_t n, T* d_total, cudaStream_t s) {
   if (n == 0) {
     if (d_total) SDB_TRY_CUDA(cudaMemsetAsync(d_total, 0, sizeof(T), s));
     return SDB_OK;
   }
   size_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
   if (nb == 1) {
-    scan_tile_kernel<T><<<1, SCAN_THREADS, 0, s>>>(in, out, n, nullptr, d_total);
+    scan_tile_kernel<T, In><<<1, SCAN_THREADS, 0, s>>>(in, out, n, nullptr, d_total);
     note_launch();
     SDB_TRY_CUDA(cudaGetLastError());
     return SDB_OK;
@@ -374,14 +385,25 @@ sdb_status exclusive_scan(const T* in, T* out, size_t n, T* d_total, cudaStream_
   T *sums, *soff;
   SDB_TRY(sc.get(&sums, nb));
   SDB_TRY(sc.get(&soff, nb));
-  scan_reduce_kernel<T><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, n, sums);
+  scan_reduce_kernel<T, In><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, n, sums);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
-  SDB_TRY(exclusive_scan<T>(sums, soff, nb, nullptr, s));
-  scan_tile_kernel<T><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, out, n, soff, d_total);
+  SDB_TRY((scan_impl<T, T>(sums, soff, nb, nullptr, s)));
+  scan_tile_kernel<T, In><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, out, n, soff, d_total);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
   return SDB_OK;
+}
+}  // namespace
+
+template <class T>
+sdb_status exclusive_scan(const T* in, T* out, size_t n, T* d_total, cudaStream_t s) {
+  return scan_impl<T, T>(in, out, n, d_total, s);
+}
+
+sdb_status exclusive_scan_i32(const int32_t* in, int64_t* out, size_t n, cudaStream_t s) {
+  uint64_t* o = reinterpret_cast<uint64_t*>(out);
+  return scan_impl<uint64_t, int32_t>(in, o, n, o + n, s);
 }
 
 template sdb_status exclusive_scan<uint32_t>(const uint32_t*, uint32_t*, size_t, uint32_t*, cudaStream_t);
