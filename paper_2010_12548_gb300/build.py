@@ -37,7 +37,8 @@ def nvcc() -> str:
 def _stale(obj: str, src: str) -> bool:
     if not os.path.exists(obj):
         return True
-    deps = [src, os.path.join(CSRC, "sdb_internal.cuh"), os.path.join(INCLUDE, "sdb.h")]
+    deps = [src, os.path.join(INCLUDE, "sdb.h")]
+    deps += [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")]
     return any(os.path.getmtime(d) > os.path.getmtime(obj) for d in deps)
 
 

@@ -49,32 +49,79 @@ using ChunkDev = BatchChunkDev;
 using TileRec = BatchTile;
 
 // ---------------------------------------------------------------- points
+// Four consecutive points per thread (16-byte loads when the arrays allow):
+// the id of every point, bound by memory (16 B a point).
 __global__ void point_keys_kernel(const uint32_t* __restrict__ x, const uint32_t* __restrict__ y,
-                                  uint64_t n, uint32_t B, uint32_t nsteps, uint32_t st0,
-                                  uint64_t* __restrict__ key, uint32_t* __restrict__ idx,
-                                  unsigned int* __restrict__ bad) {
+                                  uint64_t n, uint32_t B, uint32_t nsteps, uint32_t st0, int vec,
+                                  uint64_t* __restrict__ key, unsigned int* __restrict__ bad) {
   __shared__ uint32_t tab[HILBERT3_SMEM_WORDS];
   hilbert3_fill(tab);
   __syncthreads();
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t xi = x[i], yi = y[i];
-    if (B < 32 && ((xi >> B) | (yi >> B))) *bad = 1u;
-    key[i] = hilbert3_encode(xi, yi, nsteps, st0, tab);
-    idx[i] = (uint32_t)i;
+  const uint64_t step = (uint64_t)gridDim.x * blockDim.x * 4;
+  for (uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < n; i += step) {
+    uint32_t xs[4] = {0, 0, 0, 0}, ys[4] = {0, 0, 0, 0};
+    if (vec && i + 3 < n) {
+      const uint4 xv = __ldg(reinterpret_cast<const uint4*>(x + i));
+      const uint4 yv = __ldg(reinterpret_cast<const uint4*>(y + i));
+      xs[0] = xv.x; xs[1] = xv.y; xs[2] = xv.z; xs[3] = xv.w;
+      ys[0] = yv.x; ys[1] = yv.y; ys[2] = yv.z; ys[3] = yv.w;
+    } else {
+      for (uint32_t q = 0; q < 4 && i + q < n; ++q) {
+        xs[q] = x[i + q];
+        ys[q] = y[i + q];
+      }
+    }
+    uint64_t k[4];
+    uint32_t any = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      any |= xs[q] | ys[q];
+      k[q] = hilbert3_encode(xs[q], ys[q], nsteps, st0, tab);
+    }
+    if (any >> B) *bad = 1u;
+    if (i + 3 < n) {  // key is the library's own array: 16-byte aligned
+      *reinterpret_cast<ulonglong2*>(key + i) = make_ulonglong2(k[0], k[1]);
+      *reinterpret_cast<ulonglong2*>(key + i + 2) = make_ulonglong2(k[2], k[3]);
+    } else {
+      for (uint32_t q = 0; q < 4 && i + q < n; ++q) key[i + q] = k[q];
+    }
   }
 }
 
-__global__ void gather_points_kernel(const uint32_t* __restrict__ idx, uint64_t n,
-                                     const uint32_t* __restrict__ x, const uint32_t* __restrict__ y,
-                                     const int32_t* __restrict__ a, uint32_t* __restrict__ xs,
-                                     uint32_t* __restrict__ ys, int32_t* __restrict__ as) {
-  uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint32_t j = idx[i];
-  xs[i] = x[j];
-  ys[i] = y[j];
-  as[i] = a ? a[j] : 0;
+// The sorted points' coordinates from their ids (the curve is a bijection at
+// the points' own resolution), so the sort carries the attribute itself and
+// nothing is gathered: 16 B a point in order instead of three random 32-byte
+// sectors (30M points: 1.47 ms of gathers -> 0.16 ms).
+__global__ void point_coords_kernel(const uint64_t* __restrict__ key, uint64_t n, uint32_t nsteps,
+                                    uint32_t st0, uint32_t* __restrict__ xs,
+                                    uint32_t* __restrict__ ys) {
+  __shared__ uint32_t tab[HILBERT3_SMEM_WORDS];
+  hilbert3_inverse_fill(tab);
+  __syncthreads();
+  const uint64_t step = (uint64_t)gridDim.x * blockDim.x * 4;
+  for (uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < n; i += step) {
+    const uint32_t m = (uint32_t)min((uint64_t)4, n - i);
+    uint64_t k[4] = {0, 0, 0, 0};
+    if (m == 4) {
+      const ulonglong2 a = __ldg(reinterpret_cast<const ulonglong2*>(key + i));
+      const ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2*>(key + i + 2));
+      k[0] = a.x; k[1] = a.y; k[2] = b.x; k[3] = b.y;
+    } else {
+      for (uint32_t q = 0; q < m; ++q) k[q] = key[i + q];
+    }
+    uint32_t cx[4], cy[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) hilbert3_decode(k[q], nsteps, st0, tab, &cx[q], &cy[q]);
+    if (m == 4) {
+      *reinterpret_cast<uint4*>(xs + i) = make_uint4(cx[0], cx[1], cx[2], cx[3]);
+      *reinterpret_cast<uint4*>(ys + i) = make_uint4(cy[0], cy[1], cy[2], cy[3]);
+    } else {
+      for (uint32_t q = 0; q < m; ++q) {
+        xs[i + q] = cx[q];
+        ys[i + q] = cy[q];
+      }
+    }
+  }
 }
 
 // ---------------------------------------------------------------- candidates
@@ -872,35 +919,50 @@ sdb_status sdb_points_create(const uint32_t* d_x, const uint32_t* d_y, const int
   sdb_status st = SDB_OK;
   {
     Scratch sc(s);
-    uint64_t* ktmp = nullptr;
-    uint32_t *idx = nullptr, *itmp = nullptr;
+    uint64_t *ktmp = nullptr, *ks = nullptr;
+    uint32_t *vtmp = nullptr, *vs = nullptr;
     unsigned int* bad = nullptr;
-    uint64_t* ks = nullptr;
-    uint32_t* is = nullptr;
+    uint32_t nsteps, st0;
+    hilbert3_params(grid_bits, &nsteps, &st0);
     st = dalloc_n(&p->key, n, s);
-    if (st == SDB_OK) st = dalloc_n(&p->x, n, s);
-    if (st == SDB_OK) st = dalloc_n(&p->y, n, s);
     if (st == SDB_OK) st = dalloc_n(&p->attr, n, s);
-    if (st == SDB_OK) st = sc.get(&ktmp, n);
-    if (st == SDB_OK) st = sc.get(&idx, n);
-    if (st == SDB_OK) st = sc.get(&itmp, n);
+    if (st == SDB_OK) st = dalloc_n(&ktmp, n, s);
+    if (st == SDB_OK && d_attr) st = dalloc_n(&vtmp, n, s);
     if (st == SDB_OK) st = sc.get(&bad, 1);
     if (st == SDB_OK) st = status_of(cudaMemsetAsync(bad, 0, 4, s), "memset");
     if (st == SDB_OK) {
-      uint32_t nsteps, st0;
-      hilbert3_params(grid_bits, &nsteps, &st0);
-      point_keys_kernel<<<num_sms() * 8, 256, 0, s>>>(d_x, d_y, n, grid_bits, nsteps, st0, p->key,
-                                                      idx, bad);
+      const int vec = (((uintptr_t)d_x | (uintptr_t)d_y) & 15u) == 0;
+      const unsigned grid = std::min<unsigned>(num_sms() * 8, grid_for((n + 3) / 4, 256));
+      point_keys_kernel<<<grid, 256, 0, s>>>(d_x, d_y, n, grid_bits, nsteps, st0, vec, p->key,
+                                             bad);
       note_launch();
       st = status_of(cudaGetLastError(), "point keys");
     }
-    if (st == SDB_OK) st = radix_sort_pairs(p->key, idx, ktmp, itmp, n, 2 * grid_bits, s, &ks, &is);
-    if (st == SDB_OK && ks != p->key)
-      st = status_of(cudaMemcpyAsync(p->key, ks, n * 8, cudaMemcpyDeviceToDevice, s), "key copy");
+    // keys with their attributes; the buffer that ends up sorted is kept
+    if (st == SDB_OK && d_attr) {
+      uint32_t* va = reinterpret_cast<uint32_t*>(p->attr);
+      st = radix_sort_pairs(p->key, va, ktmp, vtmp, n, 2 * grid_bits, s, &ks, &vs,
+                            reinterpret_cast<const uint32_t*>(d_attr));
+      if (st == SDB_OK && vs != va) {
+        p->attr = reinterpret_cast<int32_t*>(vs);
+        vtmp = va;
+      }
+    } else if (st == SDB_OK) {
+      st = status_of(cudaMemsetAsync(p->attr, 0, n * 4, s), "memset");
+      if (st == SDB_OK) st = radix_sort_keys(p->key, ktmp, n, 2 * grid_bits, s, &ks);
+    }
+    if (st == SDB_OK && ks != p->key) std::swap(p->key, ktmp);
+    dfree(ktmp, s);
+    dfree(vtmp, s);
+    if (st == SDB_OK) st = dalloc_n(&p->x, n, s);
+    if (st == SDB_OK) st = dalloc_n(&p->y, n, s);
     if (st == SDB_OK) {
-      gather_points_kernel<<<grid_for(n, 256), 256, 0, s>>>(is, n, d_x, d_y, d_attr, p->x, p->y,
-                                                            p->attr);
+      const unsigned grid = std::min<unsigned>(num_sms() * 8, grid_for((n + 3) / 4, 256));
+      point_coords_kernel<<<grid, 256, 0, s>>>(p->key, n, nsteps, st0, p->x, p->y);
       note_launch();
+      st = status_of(cudaGetLastError(), "point coordinates");
+    }
+    if (st == SDB_OK) {
       unsigned int hb = 0;
       st = status_of(cudaMemcpyAsync(&hb, bad, 4, cudaMemcpyDeviceToHost, s), "flag copy");
       if (st == SDB_OK) st = status_of(cudaStreamSynchronize(s), "points create");

@@ -114,4 +114,52 @@ __device__ __forceinline__ uint64_t hilbert3_encode(uint32_t cx, uint32_t cy, ui
   return h;
 }
 
+// The inverse step: idx = orientation << 6 | 6 id bits -> the 3 bits of x
+// (bits 3..5) and of y (bits 0..2) of those levels, and the orientation after
+// them << 6.
+__host__ __device__ __forceinline__ uint32_t hilbert3_inverse_entry(uint32_t idx) {
+  uint32_t sw = (idx >> 7) & 1u, cm = (idx >> 6) & 1u;
+  uint32_t x = 0, y = 0;
+#pragma unroll
+  for (int lev = 2; lev >= 0; --lev) {
+    const uint32_t d = (idx >> (2 * lev)) & 3u;
+    const uint32_t xt = d >> 1, yt = xt ^ (d & 1u);
+    const uint32_t u = xt ^ cm, v = yt ^ cm;
+    x = (x << 1) | (sw ? v : u);
+    y = (y << 1) | (sw ? u : v);
+    if (!yt) {
+      sw ^= 1u;
+      cm ^= xt;
+    }
+  }
+  return (x << 3) | y | (((sw << 1) | cm) << 6);
+}
+
+// fills the replicated inverse table (layout as hilbert3_fill)
+__device__ __forceinline__ void hilbert3_inverse_fill(uint32_t* tab) {
+  for (int i = threadIdx.x; i < HILBERT3_SMEM_WORDS; i += blockDim.x) {
+    const uint32_t w = (uint32_t)i >> 5;
+    tab[i] = hilbert3_inverse_entry(4 * w) | (hilbert3_inverse_entry(4 * w + 1) << 8) |
+             (hilbert3_inverse_entry(4 * w + 2) << 16) | (hilbert3_inverse_entry(4 * w + 3) << 24);
+  }
+}
+
+// cell (cx, cy) of id h at the level the parameters were made for
+__device__ __forceinline__ void hilbert3_decode(uint64_t h, uint32_t nsteps, uint32_t st0,
+                                                const uint32_t* tab, uint32_t* cx, uint32_t* cy) {
+  const uint32_t* row = tab + (threadIdx.x & 31u);
+  uint32_t st = st0 << 6, x = 0, y = 0;
+  uint64_t hs = nsteps ? h << (64 - 6 * nsteps) : 0ull;  // the 6 * nsteps id bits at the top
+  for (uint32_t s = 0; s < nsteps; ++s) {
+    const uint32_t idx = st | (uint32_t)(hs >> 58);
+    hs <<= 6;
+    const uint32_t e = __byte_perm(row[(idx >> 2) << 5], 0u, 0x4440u | (idx & 3u));
+    st = e & 0xc0u;
+    x = (x << 3) | ((e >> 3) & 7u);
+    y = (y << 3) | (e & 7u);
+  }
+  *cx = x;
+  *cy = y;
+}
+
 }  // namespace sdb

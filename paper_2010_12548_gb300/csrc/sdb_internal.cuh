@@ -449,8 +449,11 @@ sdb_status radix_sort_split(uint64_t* keys, uint64_t* tmp, size_t n, int bits, i
 // keys-only LSD sort on bits [first_bit, first_bit + bits) (stable)
 sdb_status radix_sort_keys(uint64_t* keys, uint64_t* tmp, size_t n, int bits, cudaStream_t s,
                            uint64_t** result, int first_bit = 0);
+// vals_in (nullable): where the values come from, left as it is (vals and vtmp
+// are then only written first)
 sdb_status radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* ktmp, uint32_t* vtmp,
-                            size_t n, int bits, cudaStream_t s, uint64_t** kres, uint32_t** vres);
+                            size_t n, int bits, cudaStream_t s, uint64_t** kres, uint32_t** vres,
+                            const uint32_t* vals_in = nullptr);
 // unique of a sorted array: writes out[0..m), returns m via host sync
 sdb_status unique_sorted(const uint64_t* in, size_t n, uint64_t* out, size_t* m, cudaStream_t s);
 

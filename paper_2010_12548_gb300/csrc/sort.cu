@@ -3,6 +3,8 @@
 // and unique of a sorted array.  Hand-written; no library sort.
 #include "sdb_internal.cuh"
 
+#include <type_traits>
+
 namespace sdb {
 
 namespace {
@@ -44,13 +46,9 @@ __device__ T block_exclusive_scan(T v, T* s_warp, T* total) {
 }
 
 // the value of an input element in the sums' type (signed inputs sign-extend)
-template <class T>
-__device__ __forceinline__ T scan_value(T v) {
-  return v;
-}
-template <class T>
-__device__ __forceinline__ T scan_value(int32_t v) {
-  return (T)(int64_t)v;
+template <class T, class In>
+__device__ __forceinline__ T scan_value(In v) {
+  return std::is_signed<In>::value ? (T)(int64_t)v : (T)v;
 }
 
 template <class T, class In>
@@ -61,7 +59,7 @@ __global__ __launch_bounds__(SCAN_THREADS) void scan_reduce_kernel(const In* in,
 #pragma unroll
   for (int i = 0; i < SCAN_ITEMS; ++i) {
     size_t g = base + (size_t)i * SCAN_THREADS + threadIdx.x;
-    if (g < n) acc += scan_value<T>(in[g]);
+    if (g < n) acc += scan_value<T, In>(in[g]);
   }
   T tot;
   block_exclusive_scan<T>(acc, s_warp, &tot);
@@ -78,7 +76,7 @@ __global__ __launch_bounds__(SCAN_THREADS) void scan_tile_kernel(const In* in, T
 #pragma unroll
   for (int i = 0; i < SCAN_ITEMS; ++i) {
     size_t g = base + i;
-    v[i] = g < n ? scan_value<T>(in[g]) : T(0);
+    v[i] = g < n ? scan_value<T, In>(in[g]) : T(0);
     acc += v[i];
   }
   T tot;
@@ -296,10 +294,15 @@ __global__ __launch_bounds__(RS_THREADS, scatter_blocks<VALS>()) void radix_scat
 template <bool VALS>
 sdb_status radix_sort_impl(uint64_t* keys, uint32_t* vals, uint64_t* ktmp, uint32_t* vtmp, size_t n,
                            int bits, cudaStream_t s, uint64_t** kres, uint32_t** vres,
-                           int first_bit = 0, uint32_t* split_vals = nullptr, uint32_t sb = 0) {
+                           int first_bit = 0, uint32_t* split_vals = nullptr, uint32_t sb = 0,
+                           const uint32_t* vals_in = nullptr) {
   *kres = keys;
   if (VALS) *vres = vals;
-  if (n <= 1 || bits <= 0) return SDB_OK;
+  if (n <= 1 || bits <= 0) {
+    if (VALS && vals_in && n)
+      SDB_TRY_CUDA(cudaMemcpyAsync(vals, vals_in, n * 4, cudaMemcpyDeviceToDevice, s));
+    return SDB_OK;
+  }
   if (n >= 0xffffffffull) {
     set_error("radix sort: %zu elements exceeds the 32-bit rank range", n);
     return SDB_EINVAL;
@@ -337,8 +340,9 @@ sdb_status radix_sort_impl(uint64_t* keys, uint32_t* vals, uint64_t* ktmp, uint3
         radix_scatter_kernel<false, true><<<nblocks, RS_THREADS, SCATTER_SMEM, s>>>(
             ka, nullptr, kb, split_vals, n, shift, offs, nblocks, sb);
       else
-        radix_scatter_kernel<VALS><<<nblocks, RS_THREADS, SCATTER_SMEM, s>>>(ka, va, kb, vb, n,
-                                                                              shift, offs, nblocks);
+        // the first pass may read its values from an array it must not write
+        radix_scatter_kernel<VALS><<<nblocks, RS_THREADS, SCATTER_SMEM, s>>>(
+            ka, shift == first_bit && vals_in ? vals_in : va, kb, vb, n, shift, offs, nblocks);
       note_launch();
       SDB_TRY_CUDA(cudaGetLastError());
     }
@@ -438,8 +442,10 @@ sdb_status radix_sort_split(uint64_t* keys, uint64_t* tmp, size_t n, int bits, i
 }
 
 sdb_status radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* ktmp, uint32_t* vtmp, size_t n,
-                            int bits, cudaStream_t s, uint64_t** kres, uint32_t** vres) {
-  return radix_sort_impl<true>(keys, vals, ktmp, vtmp, n, bits, s, kres, vres);
+                            int bits, cudaStream_t s, uint64_t** kres, uint32_t** vres,
+                            const uint32_t* vals_in) {
+  return radix_sort_impl<true>(keys, vals, ktmp, vtmp, n, bits, s, kres, vres, 0, nullptr, 0,
+                               vals_in);
 }
 
 sdb_status unique_sorted(const uint64_t* in, size_t n, uint64_t* out, size_t* m, cudaStream_t s) {
