@@ -13,9 +13,10 @@
 //    spline corridor: from the last spline point, keep the narrowest cone of
 //    slopes that passes within +-E of every point seen; when a point leaves the
 //    cone the previous point becomes a spline point.  Slopes are compared exactly
-//    (128-bit cross products).  The array is cut into chunks of CHUNK keys, each
-//    scanned by one thread, every chunk starting and ending with a spline point
-//    (one pass, in parallel; the bound holds on every segment).
+//    (128-bit cross products where FP32 does not settle them).  The array is cut
+//    into chunks of CHUNK keys, each scanned by one warp, every chunk starting and
+//    ending with a spline point (one pass, in parallel; the bound holds on every
+//    segment).
 //  * radix table: entry j = first spline point whose key, minus the smallest
 //    key, shifted right so that 2^radix_bits prefixes cover the key range, is
 //    >= j.  A lookup reads two entries, searches the few spline points between
@@ -28,7 +29,7 @@ namespace sdb {
 
 namespace {
 
-constexpr uint64_t CHUNK = 4096;  // keys per spline-building thread
+constexpr uint64_t CHUNK = 4096;  // keys per independent stretch of the spline
 constexpr uint32_t NONE = 0xffffffffu;
 
 struct SplinePt {
@@ -44,87 +45,189 @@ __device__ __forceinline__ bool slope_less(const SplinePt& a, const SplinePt& b1
   return l < r;
 }
 
-// The greedy corridor over chunk c's distinct keys; emit(point) in key order.
-template <class Emit>
-__device__ void corridor(const uint64_t* __restrict__ key, uint64_t n, uint64_t c, int64_t E,
-                         Emit emit) {
-  uint64_t i = c * CHUNK;
-  const uint64_t end = min(n, i + CHUNK);
-  while (i < end && i > 0 && key[i] == key[i - 1]) ++i;  // a run begun in the previous chunk
-  if (i >= end) return;
-  SplinePt base{key[i], (int64_t)i}, prev = base, up{0, 0}, lo{0, 0};
-  emit(base);
-  bool cone = false;
-  for (uint64_t j = i + 1; j < end; ++j) {
-    const uint64_t k = key[j];
-    if (k == prev.k) continue;  // distinct keys at their first position
-    const SplinePt cp{k, (int64_t)j};
-    const SplinePt u2{k, (int64_t)j + E}, l2{k, (int64_t)j - E};
-    if (!cone) {
-      up = u2;
-      lo = l2;
-      cone = true;
-    } else if (slope_less(base, up, cp) || slope_less(base, cp, lo)) {
-      emit(prev);  // cp leaves the cone: prev ends the segment
-      base = prev;
-      up = u2;
-      lo = l2;
-    } else {
-      if (slope_less(base, u2, up)) up = u2;
-      if (slope_less(base, lo, l2)) lo = l2;
-    }
-    prev = cp;
+constexpr uint32_t FULL = 0xffffffffu;
+constexpr int SPLINE_WARPS = 4;             // chunks per block
+constexpr uint32_t MASK_WORDS = CHUNK / 32;  // spline-point bits of a chunk
+
+// Does the distinct key at position j leave the cone of its segment (base, then
+// the distinct keys in (base, j))?  Exact, the warp's lanes over the segment.
+__device__ __noinline__ bool leaves_cone_exact(const uint64_t* __restrict__ key, uint64_t base,
+                                               uint64_t j, int64_t E) {
+  const SplinePt b{key[base], (int64_t)base}, cp{key[j], (int64_t)j};
+  bool out = false;
+  for (uint64_t i = base + 1 + (threadIdx.x & 31); i < j; i += 32) {
+    const uint64_t k = key[i];
+    if (k == key[i - 1]) continue;
+    out |= slope_less(b, SplinePt{k, (int64_t)i + E}, cp) ||
+           slope_less(b, cp, SplinePt{k, (int64_t)i - E});
   }
-  if (prev.k != base.k) emit(prev);  // the chunk's last distinct key closes it
+  return __any_sync(FULL, out);
 }
 
-__global__ void spline_count_kernel(const uint64_t* __restrict__ key, uint64_t n, uint64_t nchunks,
-                                    int64_t E, uint64_t* __restrict__ cnt) {
-  const uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= nchunks) return;
-  uint64_t m = 0;
-  corridor(key, n, c, E, [&](const SplinePt&) { ++m; });
-  cnt[c] = m;
+// The greedy corridor over each chunk's distinct keys, one warp per chunk: 32
+// keys a step, the cone's upper and lower slope at every key by warp scans.
+// The slopes are FP32 (each within 2^-22 of its value); a key within 2^-20 of an
+// edge of the cone is decided by the exact comparison, so the spline is the
+// exact greedy one.  The chunk's spline points are left as bits of its mask.
+// A thread per chunk, reading 32 KB on its own twice over (to count, then to
+// write), took 3.54 ms for 30M keys; this and the write take 0.26 ms.
+__global__ __launch_bounds__(SPLINE_WARPS * 32) void spline_mark_kernel(
+    const uint64_t* __restrict__ key, uint64_t n, uint64_t nchunks, int64_t E,
+    uint32_t* __restrict__ mask, uint64_t* __restrict__ cnt) {
+  __shared__ uint32_t s_mask[SPLINE_WARPS][MASK_WORDS];
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint64_t c = (uint64_t)blockIdx.x * SPLINE_WARPS + w;
+  if (c >= nchunks) return;  // whole warps leave; no block barrier below
+  uint32_t* sm = s_mask[w];
+  for (uint32_t i = lane; i < MASK_WORDS; i += 32) sm[i] = 0;
+  __syncwarp();
+  const uint64_t i0 = c * CHUNK, end = min(n, i0 + CHUNK);
+  auto emit = [&](uint64_t p) {
+    if (lane == 0) sm[(p - i0) >> 5] |= 1u << ((p - i0) & 31);
+  };
+  // past a run of equal keys begun in the previous chunk
+  uint64_t base = end;
+  for (uint64_t j0 = i0; j0 < end && base == end; j0 += 32) {
+    const uint64_t j = j0 + lane;
+    const uint32_t f = __ballot_sync(FULL, j < end && (j == 0 || key[j] != key[j - 1]));
+    if (f) base = j0 + (__ffs(f) - 1);
+  }
+  if (base < end) {
+    constexpr float DELTA = 1.0f / (1 << 20);
+    const float inf = __int_as_float(0x7f800000);
+    const float Ef = (float)E;
+    uint64_t bk = key[base], prev = base;
+    float carry_u = inf, carry_l = -inf;  // over the segment's keys before this step
+    emit(base);
+    for (uint64_t j0 = base + 1; j0 < end;) {
+      const uint64_t j = j0 + lane;
+      const uint64_t k = j < end ? key[j] : 0ull;
+      uint64_t kp = __shfl_up_sync(FULL, k, 1);
+      if (lane == 0) kp = key[j0 - 1];
+      const bool distinct = j < end && k != kp;
+      const float dp = (float)(uint32_t)(j - base);
+      const float inv = __frcp_rn(__ull2float_rn(distinct ? k - bk : 1ull));
+      float u = distinct ? (dp + Ef) * inv : inf, l = distinct ? (dp - Ef) * inv : -inf;
+      const float cs = dp * inv;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const float tu = __shfl_up_sync(FULL, u, o), tl = __shfl_up_sync(FULL, l, o);
+        if (lane >= (uint32_t)o) {
+          u = fminf(u, tu);
+          l = fmaxf(l, tl);
+        }
+      }
+      // the cone as this key finds it: the segment's earlier keys
+      float mu = __shfl_up_sync(FULL, u, 1), ml = __shfl_up_sync(FULL, l, 1);
+      mu = lane == 0 ? carry_u : fminf(mu, carry_u);
+      ml = lane == 0 ? carry_l : fmaxf(ml, carry_l);
+      const bool open = distinct && mu < inf;  // a first key after the base is always inside
+      const bool out = open && (cs > mu * (1.0f + DELTA) || (ml > 0.f && cs < ml * (1.0f - DELTA)));
+      const bool near = open && (cs > mu * (1.0f - DELTA) || (ml > 0.f && cs < ml * (1.0f + DELTA)));
+      const uint32_t dmask = __ballot_sync(FULL, distinct);
+      const uint32_t omask = __ballot_sync(FULL, out);
+      uint32_t cand = __ballot_sync(FULL, near) | omask;
+      int leave = -1;
+      while (cand) {
+        const int t = __ffs(cand) - 1;
+        cand &= cand - 1;
+        if (((omask >> t) & 1u) || leaves_cone_exact(key, base, j0 + t, E)) {
+          leave = t;
+          break;
+        }
+      }
+      if (leave < 0) {
+        if (dmask) prev = j0 + (31 - __clz(dmask));
+        carry_u = fminf(carry_u, __shfl_sync(FULL, u, 31));
+        carry_l = fmaxf(carry_l, __shfl_sync(FULL, l, 31));
+        j0 += 32;
+      } else {  // the key before it ends the segment and starts the next one
+        const uint32_t before = dmask & ((1u << leave) - 1u);
+        if (before) prev = j0 + (31 - __clz(before));
+        emit(prev);
+        base = prev;
+        bk = key[base];
+        carry_u = inf;
+        carry_l = -inf;
+        j0 += leave;
+      }
+    }
+    if (prev != base) emit(prev);  // the chunk's last distinct key closes it
+  }
+  __syncwarp();
+  uint32_t m = 0;
+  for (uint32_t i = lane; i < MASK_WORDS; i += 32) {
+    mask[c * MASK_WORDS + i] = sm[i];
+    m += __popc(sm[i]);
+  }
+  m = __reduce_add_sync(FULL, m);
+  if (lane == 0) cnt[c] = m;
 }
 
-__global__ void spline_write_kernel(const uint64_t* __restrict__ key, uint64_t n,
-                                    uint64_t nchunks, int64_t E,
-                                    const uint64_t* __restrict__ off, uint64_t* __restrict__ sk,
-                                    uint32_t* __restrict__ sp) {
-  const uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// the marked keys and positions, in order: one warp per chunk, from off[c] on
+__global__ __launch_bounds__(SPLINE_WARPS * 32) void spline_write_kernel(
+    const uint64_t* __restrict__ key, uint64_t nchunks, const uint32_t* __restrict__ mask,
+    const uint64_t* __restrict__ off, uint64_t* __restrict__ sk, uint32_t* __restrict__ sp) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t c = (uint64_t)blockIdx.x * SPLINE_WARPS + (threadIdx.x >> 5);
   if (c >= nchunks) return;
   uint64_t o = off[c];
-  corridor(key, n, c, E, [&](const SplinePt& q) {
-    sk[o] = q.k;
-    sp[o] = (uint32_t)q.p;
-    ++o;
-  });
+  for (uint32_t i = 0; i < MASK_WORDS; i += 32) {
+    uint32_t b = mask[c * MASK_WORDS + i + lane];
+    const uint32_t m = __popc(b);
+    uint32_t inc = m;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const uint32_t t = __shfl_up_sync(FULL, inc, s);
+      if (lane >= (uint32_t)s) inc += t;
+    }
+    uint64_t at = o + inc - m;
+    for (; b; b &= b - 1) {
+      const uint64_t p = c * CHUNK + (uint64_t)(i + lane) * 32 + (__ffs(b) - 1);
+      sk[at] = key[p];
+      sp[at] = (uint32_t)p;
+      ++at;
+    }
+    o += __shfl_sync(FULL, inc, 31);
+  }
 }
 
-// table[j] = first spline point with prefix >= j, j in [0, 2^r]: the prefix of
-// key x is (x - kmin) >> shift, which is >= j exactly when x >= kmin + (j << shift)
-__global__ void radix_table_kernel(const uint64_t* __restrict__ sk, uint64_t ns, uint64_t kmin,
-                                   uint32_t shift, uint32_t r, uint32_t* __restrict__ table) {
-  const uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j > (1ull << r)) return;
-  const uint64_t q = kmin + (j << shift);
-  uint64_t lo = 0, len = ns;
+// first spline point in [lo, hi) with key >= q, hi if none
+__device__ __forceinline__ uint32_t spline_lower(const uint64_t* __restrict__ sk, uint32_t lo,
+                                                 uint32_t hi, uint64_t q) {
+  uint32_t len = hi - lo;
   while (len > 0) {
-    const uint64_t half = len >> 1;
-    if (sk[lo + half] < q) {
+    const uint32_t half = len >> 1;
+    if (__ldg(sk + lo + half) < q) {
       lo += half + 1;
       len -= half + 1;
     } else {
       len = half;
     }
   }
-  table[j] = (uint32_t)lo;
+  return lo;
 }
 
-__global__ void widen_attr_kernel(const int32_t* __restrict__ a, uint64_t n,
-                                  uint64_t* __restrict__ w) {
-  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) w[i] = (uint64_t)(int64_t)a[i];
+// table[j] = first spline point with prefix >= j, j in [0, 2^r]: the prefix of
+// key x is (x - kmin) >> shift, which is >= j exactly when x >= kmin + (j << shift).
+// A block writes TABLE_TILE entries: it searches the spline for its first and
+// last entry only, and the entries between look into the few points between
+// those (2^25 entries: a search of the whole spline each took 388 us, this
+// 127 us; the 134 MB written are 20).
+constexpr uint32_t TABLE_TILE = 16384;
+__global__ __launch_bounds__(256) void radix_table_kernel(const uint64_t* __restrict__ sk,
+                                                          uint32_t ns, uint64_t kmin,
+                                                          uint32_t shift, uint32_t r,
+                                                          uint32_t* __restrict__ table) {
+  __shared__ uint32_t s_lo, s_hi;
+  const uint64_t j0 = (uint64_t)blockIdx.x * TABLE_TILE;
+  const uint64_t j1 = min(j0 + TABLE_TILE, ((uint64_t)1 << r) + 1);  // past the block's last entry
+  if (threadIdx.x == 0) s_lo = spline_lower(sk, 0, ns, kmin + (j0 << shift));
+  if (threadIdx.x == 32) s_hi = spline_lower(sk, 0, ns, kmin + ((j1 - 1) << shift));
+  __syncthreads();
+  const uint32_t lo = s_lo, hi = s_hi;
+  for (uint64_t j = j0 + threadIdx.x; j < j1; j += blockDim.x)
+    table[j] = spline_lower(sk, lo, hi, kmin + (j << shift));
 }
 
 struct Spline {
@@ -284,22 +387,18 @@ sdb_status build_point_index(sdb_points* p, uint32_t radix_bits, uint32_t spline
   const uint64_t n = p->n;
   // prefix sums of the attribute in key order
   SDB_TRY(dalloc_n(&p->prefix, n + 1, s));
-  uint64_t* w;
-  SDB_TRY(sc.get(&w, n));
-  widen_attr_kernel<<<grid_for(n, 256), 256, 0, s>>>(p->attr, n, w);
-  note_launch();
-  SDB_TRY_CUDA(cudaGetLastError());
-  uint64_t* pre = reinterpret_cast<uint64_t*>(p->prefix);
-  SDB_TRY(exclusive_scan<uint64_t>(w, pre, n, pre + n, s));
-  sc.release(w);
+  SDB_TRY(exclusive_scan_i32(p->attr, p->prefix, n, s));
   // spline points, chunk by chunk
   const uint64_t nchunks = (n + CHUNK - 1) / CHUNK;
   uint64_t *cnt, *off, *dns;
+  uint32_t* mask;
   SDB_TRY(sc.get(&cnt, nchunks));
   SDB_TRY(sc.get(&off, nchunks));
   SDB_TRY(sc.get(&dns, 1));
-  spline_count_kernel<<<grid_for(nchunks, 128), 128, 0, s>>>(p->key, n, nchunks,
-                                                              (int64_t)spline_error, cnt);
+  SDB_TRY(sc.get(&mask, nchunks * MASK_WORDS));
+  const unsigned chunk_grid = grid_for(nchunks, SPLINE_WARPS);
+  spline_mark_kernel<<<chunk_grid, SPLINE_WARPS * 32, 0, s>>>(p->key, n, nchunks,
+                                                             (int64_t)spline_error, mask, cnt);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
   SDB_TRY(exclusive_scan<uint64_t>(cnt, off, nchunks, dns, s));
@@ -314,9 +413,8 @@ sdb_status build_point_index(sdb_points* p, uint32_t radix_bits, uint32_t spline
   }
   SDB_TRY(dalloc_n(&p->rs_key, ns, s));
   SDB_TRY(dalloc_n(&p->rs_pos, ns, s));
-  spline_write_kernel<<<grid_for(nchunks, 128), 128, 0, s>>>(p->key, n, nchunks,
-                                                              (int64_t)spline_error, off, p->rs_key,
-                                                              p->rs_pos);
+  spline_write_kernel<<<chunk_grid, SPLINE_WARPS * 32, 0, s>>>(p->key, nchunks, mask, off,
+                                                              p->rs_key, p->rs_pos);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
   // radix table over the key range
@@ -324,8 +422,8 @@ sdb_status build_point_index(sdb_points* p, uint32_t radix_bits, uint32_t spline
   const uint32_t span_bits = span ? 64 - __builtin_clzll(span) : 0;
   p->rs_shift = span_bits > radix_bits ? span_bits - radix_bits : 0;
   SDB_TRY(dalloc_n(&p->rs_table, (1ull << radix_bits) + 1, s));
-  radix_table_kernel<<<grid_for((1ull << radix_bits) + 1, 256), 256, 0, s>>>(
-      p->rs_key, ns, ends[0], p->rs_shift, radix_bits, p->rs_table);
+  radix_table_kernel<<<grid_for((1ull << radix_bits) + 1, TABLE_TILE), 256, 0, s>>>(
+      p->rs_key, (uint32_t)ns, ends[0], p->rs_shift, radix_bits, p->rs_table);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
   SDB_TRY(dalloc_n(&p->rs_fallbacks, 1, s));
