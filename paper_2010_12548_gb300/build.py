@@ -19,7 +19,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OUT = os.path.join(HERE, "libsdb.so")
 BUILD = os.path.join(ROOT, "_build")
-SOURCES = ["api.cu", "cover.cu", "sort.cu", "join.cu", "learned.cu", "noalloc.cu", "batch.cu",
+SOURCES = ["api.cu", "cover.cu", "covertiles.cu", "sort.cu", "join.cu", "learned.cu", "noalloc.cu", "batch.cu",
            "pointindex.cu", "raster.cu",
            "server.cu", "table.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

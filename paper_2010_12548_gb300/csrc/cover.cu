@@ -20,10 +20,12 @@
 // (coordinates < 2^30, products < 2^61, int64).  The root parity comes from a
 // rightward ray from (0,0)+.
 //
-// Emitted cells become (lo = h * 4^(F-L), level) records; a sweep over all
+// Where the queries' levels are deep enough the refinement stops five levels above
+// the finest one and the rest is done in bitmaps (covertiles.cu).  Otherwise, and
+// for overlapping polygons, emitted cells become (lo = h * 4^(F-L), level) records; a sweep over all
 // record endpoints (sort, unique, per-interval polygon lists, merge of equal
 // neighbours) gives the canonical ranges.
-#include "sdb_internal.cuh"
+#include "cover_internal.cuh"
 
 #include <algorithm>
 #include <atomic>
@@ -62,22 +64,6 @@ __device__ __forceinline__ void put_record(uint64_t* __restrict__ rk, uint32_t* 
   }
 }
 
-struct Edge {
-  int32_t ax, ay, bx, by;
-};
-
-// A frontier cell of one (query, polygon) pair at level L: cell (cx, cy), its
-// Hilbert id at level L and the curve's orientation (sw << 1 | cm) below it,
-// so a child's id is one more digit; its edge list elist[eoff, eoff + ecnt)
-// and the perturbed parity of its lower-left corner.
-struct __align__(16) Item {
-  uint64_t hid;
-  uint32_t pair, cx, cy, eoff;
-  uint32_t ecnt_par;  // edge count | parity << 31
-  uint32_t orient;
-};
-static_assert(sizeof(Item) == 32, "two 16-byte loads per item");
-
 __device__ __forceinline__ uint64_t qof(uint64_t key, uint32_t qshift) {
   return qshift >= 64 ? 0ull : key >> qshift;
 }
@@ -101,30 +87,33 @@ __device__ __forceinline__ uint32_t pert_ray_cross(const Edge& e, int64_t qx, in
   return (e.by > e.ay) ? (sd > 0) : (sd < 0);
 }
 
-// Offsets for three per-thread counts, with one atomic per counter and block
+// Offsets for N per-thread counts, with one atomic per counter and block
 // (blockDim.x == 256): warp scans, then warp prefixes in shared memory.  Every
 // thread of the block must call it.
-__device__ __forceinline__ void block_alloc3(const uint32_t (&n)[3],
-                                             unsigned long long* __restrict__ ctr,
-                                             unsigned long long (&off)[3]) {
-  __shared__ uint32_t wsum[3][8];
-  __shared__ unsigned long long base[3];
+template <int N>
+__device__ __forceinline__ void block_alloc(const uint32_t (&n)[N],
+                                            unsigned long long* __restrict__ ctr,
+                                            unsigned long long (&off)[N]) {
+  __shared__ uint32_t wsum[N][8];
+  __shared__ unsigned long long base[N];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  uint32_t inc[3] = {n[0], n[1], n[2]};
+  uint32_t inc[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) inc[j] = n[j];
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
+    for (int j = 0; j < N; ++j) {
       const uint32_t t = __shfl_up_sync(FULL, inc[j], o);
       if (lane >= o) inc[j] += t;
     }
   }
   if (lane == 31) {
 #pragma unroll
-    for (int j = 0; j < 3; ++j) wsum[j][w] = inc[j];
+    for (int j = 0; j < N; ++j) wsum[j][w] = inc[j];
   }
   __syncthreads();
-  if (threadIdx.x < 3) {
+  if (threadIdx.x < N) {
     const int j = threadIdx.x;
     uint32_t t = 0;
     for (int k = 0; k < 8; ++k) {
@@ -136,8 +125,16 @@ __device__ __forceinline__ void block_alloc3(const uint32_t (&n)[3],
   }
   __syncthreads();
 #pragma unroll
-  for (int j = 0; j < 3; ++j) off[j] = base[j] + wsum[j][w] + inc[j] - n[j];
+  for (int j = 0; j < N; ++j) off[j] = base[j] + wsum[j][w] + inc[j] - n[j];
 }
+
+// Where a level's boundary children go when they are tiles: cells TILE_DEPTH
+// levels above their query's finest level, with their edge lists
+struct TileOut {
+  Item* items;
+  uint32_t* elist;
+  unsigned long long item_base, edge_base;  // filled by earlier levels
+};
 
 __global__ void build_edges_kernel(const uint32_t* __restrict__ vx, const uint32_t* __restrict__ vy,
                                    const uint32_t* __restrict__ next, uint32_t V,
@@ -317,7 +314,9 @@ __device__ __forceinline__ uint32_t edge_vs_children(const Edge& e, int32_t px, 
 // its first lane writes the records and child items.  Child edge lists keep
 // the parent's edge order (a ballot per child and chunk of G edges); the meet
 // masks of the first 8 chunks are kept in a register for that second pass.
-template <int G, bool NC>
+// TILES: a query's refinement ends TILE_DEPTH levels above its finest level, its
+// boundary children of that level going to the tile list (covertiles.cu).
+template <int G, bool NC, bool TILES>
 __global__ __launch_bounds__(256) void expand_level_kernel(
     const Item* __restrict__ items, uint32_t n_items, const uint32_t* __restrict__ elist,
     const Edge* __restrict__ edges, const uint32_t* __restrict__ pair_query,
@@ -325,7 +324,7 @@ __global__ __launch_bounds__(256) void expand_level_kernel(
     uint32_t bflag, uint32_t B, uint32_t L, Item* __restrict__ next_items,
     uint32_t* __restrict__ next_elist,
     uint64_t* __restrict__ rec_key, uint32_t* __restrict__ rec_val, uint32_t sb,
-    unsigned long long rec_base, unsigned long long* __restrict__ counters) {
+    unsigned long long rec_base, TileOut tiles, unsigned long long* __restrict__ counters) {
   const uint64_t gt = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool active = gt / G < n_items;
   const uint32_t t = (uint32_t)(gt / G);  // item of this lane's group
@@ -394,7 +393,7 @@ __global__ __launch_bounds__(256) void expand_level_kernel(
       uint32_t inside = (par ^ (flip >> c)) & 1u;
       if (!((keep >> c) & 1u)) continue;
       if (cnt[c] > 0) {
-        if (cl == F) {
+        if (!TILES && cl == F) {
           n_rec += (bkeep >> c) & 1u;
         } else {
           ++n_it;
@@ -405,10 +404,28 @@ __global__ __launch_bounds__(256) void expand_level_kernel(
       }
     }
   }
-  // counters: 0 child items, 1 child edge entries, 2 records
-  unsigned long long off[3];
-  block_alloc3({n_it, n_ed, n_rec}, counters, off);
-  unsigned long long io = off[0], eo = off[1], ro = off[2];
+  // counters: 0 child items, 1 child edge entries, 2 records, 3 and 4 tile items
+  // and their edge entries
+  unsigned long long io, eo, ro;
+  if constexpr (TILES) {
+    const bool fin = cl + TILE_DEPTH == F;
+    unsigned long long off[5];
+    block_alloc<5>({fin ? 0u : n_it, fin ? 0u : n_ed, n_rec, fin ? n_it : 0u, fin ? n_ed : 0u},
+                   counters, off);
+    io = fin ? off[3] + tiles.item_base : off[0];
+    eo = fin ? off[4] + tiles.edge_base : off[1];
+    ro = off[2];
+    if (fin) {
+      next_items = tiles.items;
+      next_elist = tiles.elist;
+    }
+  } else {
+    unsigned long long off[3];
+    block_alloc<3>({n_it, n_ed, n_rec}, counters, off);
+    io = off[0];
+    eo = off[1];
+    ro = off[2];
+  }
   if (!active) return;
   const uint32_t leader = lane & ~(uint32_t)(G - 1);
   if (G > 1) {
@@ -433,11 +450,11 @@ __global__ __launch_bounds__(256) void expand_level_kernel(
     const uint64_t chid = (it.hid << 2) | ((xt << 1) | (xt ^ yt));
     const uint32_t corient = yt ? it.orient : (it.orient ^ 2u ^ xt);
     uint32_t inside = (par ^ (flip >> c)) & 1u;
-    if (cnt[c] > 0 && cl == F && !((bkeep >> c) & 1u)) {
+    if (!TILES && cnt[c] > 0 && cl == F && !((bkeep >> c) & 1u)) {
       cnt[c] = 0;  // non-conservative: a boundary cell whose centre lies outside
       continue;
     }
-    bool emit = (cnt[c] > 0) ? (cl == F) : (inside != 0);
+    bool emit = (cnt[c] > 0) ? (!TILES && cl == F) : (inside != 0);
     if (emit) {
       if (gl == 0) {
         put_record(rec_key, rec_val, rec_base + ro++, qbits | (chid << shift),
@@ -863,20 +880,12 @@ __global__ __launch_bounds__(MT) void merge_emit_kernel(MergeCtx c, const uint32
   }
 }
 
-// per query (one thread each): its offset and record count, its sentinel
-// (start 4^F), and the single empty range of a query without records
-struct QueryFix {
-  uint64_t extra;      // entries of earlier queries that are no ranges of groups
-  uint64_t next_head;  // first record of the next query with records (or n)
-  uint32_t prev;       // the last earlier query with records (or NONE)
-  uint32_t head;       // the query's first record (or NONE)
-};
-
 __global__ void merge_finish_kernel(const QueryFix* __restrict__ qf,
                                     const uint64_t* __restrict__ qopen,
                                     const uint32_t* __restrict__ qlist,
                                     const CoverQuery* __restrict__ qs, uint32_t Q,
-                                    uint64_t* __restrict__ start, uint32_t* __restrict__ list_off,
+                                    const uint64_t* __restrict__ coff, uint64_t n_elements,
+                                    uint64_t n_cells, uint64_t* __restrict__ start, uint32_t* __restrict__ list_off,
                                     uint32_t* __restrict__ pay, uint64_t* __restrict__ qoff,
                                     uint64_t* __restrict__ qcells) {
   const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -888,7 +897,8 @@ __global__ void merge_finish_kernel(const QueryFix* __restrict__ qf,
     qoff[q] = qopen[2 * q] + f.extra;
     e = qopen[2 * q + 1] + f.extra;
     L = qlist[2 * q + 1];
-    qcells[q] = f.next_head - f.head;
+    qcells[q] = coff ? (f.next_head < n_elements ? coff[f.next_head] : n_cells) - coff[f.head]
+                     : f.next_head - f.head;
   } else {
     const uint64_t ro = f.prev == NONE ? 0ull : qopen[2 * f.prev + 1];
     L = f.prev == NONE ? 0u : qlist[2 * f.prev + 1];
@@ -1110,21 +1120,8 @@ static sdb_status merge_records(uint64_t* key, uint32_t* val, uint64_t n, const 
   }
   // entries: the groups' ranges, plus per query its sentinel, plus the empty
   // range of a query without records
-  std::vector<QueryFix> hq(Q);
-  uint64_t extra = 0;
-  uint32_t prev = NONE;
-  for (uint32_t q = 0; q < Q; ++q) {
-    hq[q].extra = extra;
-    hq[q].head = hhead[q];
-    hq[q].prev = prev;
-    extra += hhead[q] == NONE ? 2 : 1;
-    if (hhead[q] != NONE) prev = q;
-  }
-  uint64_t next = n;
-  for (uint32_t q = Q; q-- > 0;) {
-    hq[q].next_head = next;
-    if (hhead[q] != NONE) next = hhead[q];
-  }
+  std::vector<QueryFix> hq;
+  const uint64_t extra = query_fixes(hhead, n, &hq);
   const uint64_t E = (tot >> 32) + extra;
   const uint64_t nids = tot & 0xffffffffull;
   if (E >= 0x7fffffffull) {  // entry indices travel in 31 bits of the packed payload
@@ -1136,13 +1133,11 @@ static sdb_status merge_records(uint64_t* key, uint32_t* val, uint64_t n, const 
   SDB_TRY(dalloc_n(&out->pay, E, s));
   SDB_TRY(dalloc_n(&out->list_ids, nids ? nids : 1, s));
   QueryFix* dq;
-  uint64_t *qopen, *qoff, *qcells, *dextra;
+  uint64_t *qopen, *dextra;
   uint32_t* qlist;
   SDB_TRY(sc.get(&dq, Q));
   SDB_TRY(sc.get(&qopen, 2 * (size_t)Q));
   SDB_TRY(sc.get(&qlist, 2 * (size_t)Q));
-  SDB_TRY(sc.get(&qoff, (size_t)Q + 1));
-  SDB_TRY(sc.get(&qcells, Q));
   SDB_TRY(sc.get(&dextra, Q));
   std::vector<uint64_t> hextra(Q);
   for (uint32_t q = 0; q < Q; ++q) hextra[q] = hq[q].extra;
@@ -1156,8 +1151,42 @@ static sdb_status merge_records(uint64_t* key, uint32_t* val, uint64_t n, const 
     note_launch();
     SDB_TRY_CUDA(cudaGetLastError());
   }
-  merge_finish_kernel<<<grid_for(Q, 256), 256, 0, s>>>(dq, qopen, qlist, d_qs, Q, out->start,
-                                                       out->list_off, out->pay, qoff, qcells);
+  out->E = E;
+  out->nids = nids;
+  return finish_queries(dq, qopen, qlist, d_qs, Q, nullptr, n, n, out, s);
+}
+
+uint64_t query_fixes(const std::vector<uint32_t>& head, uint64_t n, std::vector<QueryFix>* out) {
+  const uint32_t Q = (uint32_t)head.size();
+  std::vector<QueryFix>& f = *out;
+  f.resize(Q);
+  uint64_t extra = 0;
+  uint32_t prev = NONE;
+  for (uint32_t q = 0; q < Q; ++q) {
+    f[q].extra = extra;
+    f[q].head = head[q];
+    f[q].prev = prev;
+    extra += head[q] == NONE ? 2 : 1;
+    if (head[q] != NONE) prev = q;
+  }
+  uint64_t next = n;
+  for (uint32_t q = Q; q-- > 0;) {
+    f[q].next_head = next;
+    if (head[q] != NONE) next = head[q];
+  }
+  return extra;
+}
+
+sdb_status finish_queries(const QueryFix* dq, const uint64_t* qopen, const uint32_t* qlist,
+                          const CoverQuery* d_qs, uint32_t Q, const uint64_t* coff,
+                          uint64_t n_elements, uint64_t n_cells, CoverSet* out, cudaStream_t s) {
+  Scratch sc(s);
+  uint64_t *qoff, *qcells;
+  SDB_TRY(sc.get(&qoff, (size_t)Q + 1));
+  SDB_TRY(sc.get(&qcells, Q));
+  merge_finish_kernel<<<grid_for(Q, 256), 256, 0, s>>>(dq, qopen, qlist, d_qs, Q, coff, n_elements,
+                                                       n_cells, out->start, out->list_off,
+                                                       out->pay, qoff, qcells);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
   out->qoff.assign((size_t)Q + 1, 0);
@@ -1167,8 +1196,6 @@ static sdb_status merge_records(uint64_t* key, uint32_t* val, uint64_t n, const 
   SDB_TRY_CUDA(cudaMemcpyAsync(out->qcells.data(), qcells, (size_t)Q * 8, cudaMemcpyDeviceToHost,
                                s));
   SDB_TRY_CUDA(cudaStreamSynchronize(s));
-  out->E = E;
-  out->nids = nids;
   return SDB_OK;
 }
 
@@ -1188,18 +1215,22 @@ static sdb_status launch_expand(uint32_t G, const Item* items, uint32_t n_items,
                          const CoverQuery* qs, uint32_t qshift, uint32_t bflag, bool noncons,
                          uint32_t B, uint32_t L,
                          Item* nitems, uint32_t* nel, uint64_t* rkey, uint32_t* rval, uint32_t sb,
-                         unsigned long long rec_base, unsigned long long* ctr, cudaStream_t s) {
+                         unsigned long long rec_base, const TileOut* tiles,
+                         unsigned long long* ctr, cudaStream_t s) {
   const size_t threads = (size_t)n_items * G;
-#define SDB_EXPAND(g)                                                                          \
-  case g:                                                                                      \
-    if (noncons)                                                                               \
-      expand_level_kernel<g, true><<<grid_for(threads, 256), 256, 0, s>>>(                     \
-          items, n_items, elist, edges, pq, ps, qs, qshift, bflag, B, L, nitems, nel, rkey,     \
-          rval, sb, rec_base, ctr);                                                            \
-    else                                                                                       \
-      expand_level_kernel<g, false><<<grid_for(threads, 256), 256, 0, s>>>(                    \
-          items, n_items, elist, edges, pq, ps, qs, qshift, bflag, B, L, nitems, nel, rkey,     \
-          rval, sb, rec_base, ctr);                                                            \
+  const TileOut to = tiles ? *tiles : TileOut{};
+#define SDB_EXPAND_AS(g, nc, tl)                                                               \
+  expand_level_kernel<g, nc, tl><<<grid_for(threads, 256), 256, 0, s>>>(                       \
+      items, n_items, elist, edges, pq, ps, qs, qshift, bflag, B, L, nitems, nel, rkey, rval,  \
+      sb, rec_base, to, ctr)
+#define SDB_EXPAND(g)                  \
+  case g:                              \
+    if (tiles)                         \
+      SDB_EXPAND_AS(g, false, true);   \
+    else if (noncons)                  \
+      SDB_EXPAND_AS(g, true, false);   \
+    else                               \
+      SDB_EXPAND_AS(g, false, false);  \
     break;
   switch (G) {
     SDB_EXPAND(1)
@@ -1213,6 +1244,7 @@ static sdb_status launch_expand(uint32_t G, const Item* items, uint32_t n_items,
       return SDB_EINVAL;
   }
 #undef SDB_EXPAND
+#undef SDB_EXPAND_AS
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
   return SDB_OK;
@@ -1226,12 +1258,14 @@ static sdb_status launch_expand(uint32_t G, const Item* items, uint32_t n_items,
 // build that needs more still grows.
 struct BuildShape {
   uint32_t B, Q, NP, V, Fmax;
+  bool tiles;
   bool operator==(const BuildShape& o) const {
-    return B == o.B && Q == o.Q && NP == o.NP && V == o.V && Fmax == o.Fmax;
+    return B == o.B && Q == o.Q && NP == o.NP && V == o.V && Fmax == o.Fmax && tiles == o.tiles;
   }
 };
 struct BuildHint {
   uint64_t rec = 1ull << 20, items = 1ull << 12, edges = 1ull << 14;
+  uint64_t tiles = 1ull << 14, tile_edges = 1ull << 15;
 };
 std::mutex g_hint_mu;
 std::vector<std::pair<BuildShape, BuildHint>> g_hints;  // most recent last, at most 16
@@ -1260,9 +1294,96 @@ uint64_t pow2_at_least(uint64_t v) {
   return p;
 }
 
-sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStream_t s,
-                           CoverSet* out) {
+// room for `need` elements in *p, of which the first n are kept (`hint`: the
+// smallest size worth allocating)
+template <class T>
+static sdb_status grow(T** p, uint64_t n, uint64_t need, uint64_t hint, uint64_t* cap,
+                       cudaStream_t s) {
+  if (need <= *cap) return SDB_OK;
+  const uint64_t nc = std::max(pow2_at_least(need), hint);
+  T* q = nullptr;
+  SDB_TRY(dalloc_n(&q, nc, s));
+  if (n) {
+    const cudaError_t e = cudaMemcpyAsync(q, *p, n * sizeof(T), cudaMemcpyDeviceToDevice, s);
+    if (e != cudaSuccess) {
+      dfree(q, s);
+      return cuda_status(e, "growing a buffer", __FILE__, __LINE__);
+    }
+  }
+  dfree(*p, s);
+  *p = q;
+  *cap = nc;
+  return SDB_OK;
+}
+
+// A query's viewport in tiles of its level, and whether the last levels of all
+// queries' refinement go through tile bitmaps: the levels above must be deep
+// enough to spread the polygons over the tiles (a warp takes a tile's polygons
+// one after the other), and the boundary cells are kept by touching only.
+static bool use_tiles(const CoverSpec& spec) {
+  constexpr uint32_t MIN_LEVEL = 8;
+  if (spec.noncons || spec.NP == 0) return false;
+  std::vector<uint32_t> np(spec.Q, 0);
+  for (uint32_t i = 0; i < spec.NP; ++i) ++np[spec.pair_query[i]];
+  for (uint32_t q = 0; q < spec.Q; ++q) {
+    const CoverQuery& Q = spec.q[q];
+    if (Q.F < MIN_LEVEL) return false;
+    const uint32_t sh = spec.B - (Q.F - TILE_DEPTH);
+    const uint64_t nx = ((uint64_t)(Q.x1 - 1) >> sh) - (Q.x0 >> sh) + 1;
+    const uint64_t ny = ((uint64_t)(Q.y1 - 1) >> sh) - (Q.y0 >> sh) + 1;
+    if (np[q] > 64 + 2 * nx * ny) return false;
+  }
+  return true;
+}
+
+// Whether a polygon probably holds a vertex of another one (a few polygons' first
+// vertices against all): overlapping polygons cannot be merged tile by tile, and
+// finding that out from the tiles costs a third of the build.  A guess only.
+static bool overlap_likely(const PolyEdges& pe) {
+  if (pe.P < 2 || pe.V > (1u << 16)) return false;
+  std::vector<uint32_t> bb(4 * (size_t)pe.P);
+  for (uint32_t j = 0; j < pe.P; ++j) {
+    uint32_t x0 = ~0u, y0 = ~0u, x1 = 0, y1 = 0;
+    for (uint32_t v = pe.edge_off[j]; v < pe.edge_off[j + 1]; ++v) {
+      x0 = std::min(x0, pe.x[v]);
+      y0 = std::min(y0, pe.y[v]);
+      x1 = std::max(x1, pe.x[v]);
+      y1 = std::max(y1, pe.y[v]);
+    }
+    bb[4 * j] = x0;
+    bb[4 * j + 1] = y0;
+    bb[4 * j + 2] = x1;
+    bb[4 * j + 3] = y1;
+  }
+  const uint32_t samples = std::min(pe.P, 64u);
+  for (uint32_t k = 0; k < samples; ++k) {
+    const uint32_t i = (uint32_t)((uint64_t)k * pe.P / samples);
+    const int64_t px = pe.x[pe.edge_off[i]], py = pe.y[pe.edge_off[i]];
+    for (uint32_t j = 0; j < pe.P; ++j) {
+      if (j == i || px <= bb[4 * j] || px >= bb[4 * j + 2] || py <= bb[4 * j + 1] ||
+          py >= bb[4 * j + 3])
+        continue;
+      bool in = false, shared = false;
+      for (uint32_t v = pe.edge_off[j]; v < pe.edge_off[j + 1] && !shared; ++v) {
+        const int64_t ax = pe.x[v], ay = pe.y[v], bx = pe.x[pe.next[v]], by = pe.y[pe.next[v]];
+        shared = ax == px && ay == py;  // a tiling's common vertex
+        if ((ay > py) != (by > py)) {
+          const int64_t o = (bx - ax) * (py - ay) - (by - ay) * (px - ax);
+          in ^= by > ay ? o > 0 : o < 0;
+        }
+      }
+      if (in && !shared) return true;
+    }
+  }
+  return false;
+}
+
+// One pass of the builder.  With tiles, *outcome may say that nothing was made
+// and the refinement has to go down to the finest level instead.
+static sdb_status build_pass(const PolyEdges& pe, const CoverSpec& spec, bool tiles,
+                             cudaStream_t s, CoverSet* out, TileOutcome* outcome) {
   TraceScope tr("cover.build", s);
+  *outcome = TileOutcome::made;
   const uint32_t P = pe.P;
   const uint32_t V = pe.V;
   const uint32_t B = spec.B, Q = spec.Q, NP = spec.NP;
@@ -1317,11 +1438,11 @@ sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStrea
   for (uint32_t i = 0; i < NP; ++i) max_slot = spec.pair_slot[i] > max_slot ? spec.pair_slot[i] : max_slot;
   uint32_t sb = (uint32_t)bits_for(max_slot);
   if (sb < 1) sb = 1;
-  if (key_bits + (int)sb + 6 > 64) sb = 0;
-  const BuildShape shape{B, Q, NP, V, Fmax};
+  if (key_bits + (int)sb + 6 > 64 || tiles) sb = 0;
+  const BuildShape shape{B, Q, NP, V, Fmax, tiles};
   const BuildHint hint = hint_for(shape);
   BuildHint seen;
-  seen.rec = seen.items = seen.edges = 0;
+  seen.rec = seen.items = seen.edges = seen.tiles = seen.tile_edges = 0;
   uint64_t rec_cap = hint.rec, n_rec = 0;
   if (rec_cap < 8ull * NP) rec_cap = 8ull * NP;
   uint64_t* rkey = nullptr;
@@ -1340,8 +1461,9 @@ sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStrea
 
   const uint32_t bflag = spec.flags ? VAL_FLAG : 0u;  // boundary records' flag
   unsigned long long* ctr;
-  SDB_TRY(sc.get(&ctr, 3));
-  SDB_TRY_CUDA(cudaMemsetAsync(ctr, 0, 3 * sizeof(unsigned long long), s));
+  constexpr int NCTR = 5;
+  SDB_TRY(sc.get(&ctr, NCTR));
+  SDB_TRY_CUDA(cudaMemsetAsync(ctr, 0, NCTR * sizeof(unsigned long long), s));
   // frontier cells and edge lists, two buffers each (this level's, the next's)
   struct Frontier {
     Item* f[2] = {nullptr, nullptr};
@@ -1376,6 +1498,18 @@ sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStrea
     note_launch();
     SDB_TRY_CUDA(cudaGetLastError());
   }
+  // tiles and their edge lists, filled by the levels where queries end
+  struct Tiles {
+    Item* items = nullptr;
+    uint32_t* elist = nullptr;
+    uint64_t n = 0, ne = 0, cap = 0, ecap = 0;
+    cudaStream_t s;
+    ~Tiles() {
+      dfree(items, s);
+      dfree(elist, s);
+    }
+  } tl;
+  tl.s = s;
   unsigned long long h0[3];
   SDB_TRY(read_u64(ctr, h0, 3, s));
   uint64_t n_items = h0[0], n_edges = 0;
@@ -1386,8 +1520,9 @@ sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStrea
   uint32_t* cur_el = elist;
   tr_up.end();
   TraceScope tr_lv("cover.levels", s);
-  for (uint32_t L = 0; L < Fmax && n_items > 0; ++L) {
-    const bool last = (L + 1 == Fmax);
+  const uint32_t Lend = tiles ? Fmax - TILE_DEPTH : Fmax;  // levels to expand
+  for (uint32_t L = 0; L < Lend && n_items > 0; ++L) {
+    const bool last = (L + 1 == Lend);
     // capacity: every record and every child item comes from one of 4
     // children; every child edge entry from one (edge, child) pair
     if (n_rec + 4 * n_items > rec_cap) {
@@ -1434,7 +1569,17 @@ sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStrea
       nitems = fbuf[1];
       nel = ebuf[1];
     }
-    SDB_TRY_CUDA(cudaMemsetAsync(ctr, 0, 3 * sizeof(unsigned long long), s));
+    TileOut tile_out{};
+    if (tiles) {
+      bool ends = false;  // a query's tiles come from this level
+      for (uint32_t q = 0; q < Q && !ends; ++q) ends = spec.q[q].F == L + 1 + TILE_DEPTH;
+      if (ends) {
+        SDB_TRY(grow(&tl.items, tl.n, tl.n + 4 * n_items, hint.tiles, &tl.cap, s));
+        SDB_TRY(grow(&tl.elist, tl.ne, tl.ne + 4 * n_edges, hint.tile_edges, &tl.ecap, s));
+      }
+      tile_out = TileOut{tl.items, tl.elist, tl.n, tl.ne};
+    }
+    SDB_TRY_CUDA(cudaMemsetAsync(ctr, 0, NCTR * sizeof(unsigned long long), s));
     // lanes per item: about the level's mean edge count, a power of two <= 32
     const uint64_t mean = (n_edges + n_items - 1) / n_items;
     uint32_t G = 1;
@@ -1443,12 +1588,12 @@ sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStrea
     {
       TraceScope tr("cover.expand", s);
       SDB_TRY(launch_expand(G, items, (uint32_t)n_items, cur_el, edges, d_pq, d_ps, d_qs, qshift,
-                            bflag, spec.noncons, B, L, nitems, nel, rkey, rval, sb, n_rec, ctr,
-                            s));
+                            bflag, spec.noncons, B, L, nitems, nel, rkey, rval, sb, n_rec,
+                            tiles ? &tile_out : nullptr, ctr, s));
       SDB_TRY_CUDA(cudaGetLastError());
     }
-    unsigned long long h[3];
-    SDB_TRY(read_u64(ctr, h, 3, s));
+    unsigned long long h[NCTR];
+    SDB_TRY(read_u64(ctr, h, NCTR, s));
     // the next level reads what this one wrote
     std::swap(fbuf[0], fbuf[1]);
     std::swap(fcap[0], fcap[1]);
@@ -1460,6 +1605,13 @@ sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStrea
     n_items = last ? 0 : h[0];
     n_edges = h[1];
     n_rec += h[2];
+    tl.n += h[3];
+    tl.ne += h[4];
+    if (tl.n > 0xffffffffull || tl.ne > 0xffffffffull) {
+      set_error("covering: %llu tiles, %llu edge entries exceed the 32-bit index range",
+                (unsigned long long)tl.n, (unsigned long long)tl.ne);
+      return SDB_ENOMEM;
+    }
     seen.items = std::max<uint64_t>(seen.items, pow2_at_least(4 * n_items));
     seen.edges = std::max<uint64_t>(seen.edges, pow2_at_least(4 * n_edges));
   }
@@ -1467,9 +1619,27 @@ sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStrea
   seen.rec = std::max<uint64_t>(pow2_at_least(n_rec), 1ull << 16);
   seen.items = std::max<uint64_t>(seen.items, 1ull << 12);
   seen.edges = std::max<uint64_t>(seen.edges, 1ull << 14);
+  seen.tiles = std::max<uint64_t>(tl.cap, 1ull << 14);
+  seen.tile_edges = std::max<uint64_t>(tl.ecap, 1ull << 15);
   keep_hint(shape, seen);
+  if (tiles)
+    return cover_tiles(rkey, rval, n_rec, tl.items, tl.n, tl.elist, edges, d_pq, d_ps, d_qs, spec,
+                       qshift, key_bits, s, out, outcome);
   out->ncells = n_rec;
   return merge_records(rkey, rval, n_rec, spec, d_qs, qshift, key_bits, sb, s, out);
+}
+
+sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStream_t s,
+                           CoverSet* out) {
+  TileOutcome outcome = TileOutcome::crowded;
+  if (use_tiles(spec) && !(spec.Q == 1 && overlap_likely(pe)))
+    SDB_TRY(build_pass(pe, spec, true, s, out, &outcome));
+  if (outcome == TileOutcome::made) return SDB_OK;
+  if (outcome == TileOutcome::nested && spec.Q != 1) {
+    set_error("batched coverings need polygons that do not overlap within a query");
+    return SDB_EINVAL;
+  }
+  return build_pass(pe, spec, false, s, out, &outcome);
 }
 
 sdb_status finish_covering(sdb_covering* cov, cudaStream_t s);

@@ -1,0 +1,877 @@
+// Covering tiles: the last TILE_DEPTH levels of the covering's refinement, done
+// as bitmaps instead of cell by cell.
+//
+// The level-synchronous refinement (cover.cu) stops TILE_DEPTH levels above a
+// query's finest level.  What it has produced by then -- interior cells of the
+// coarser levels and boundary cells ("tiles" of 32 x 32 finest cells, each with
+// the polygon's edges that meet it and the parity of its corner) -- is about a
+// fiftieth of the finest covering, and only that is sorted by (query, curve
+// position).  A covering then needs, per tile and polygon, which of the 1024
+// finest cells belong to it:
+//   * a cell that an edge touches does (closed cell, closed edge).  Lane = row of
+//     the tile; the edge clipped to the row's closed strip covers one run of
+//     cells, found exactly: the column at which the edge's line meets a row line is
+//     a quotient of at most 32, estimated in FP32 and settled by its remainder.
+//   * an untouched cell does when its corner is inside: the tile corner's parity
+//     and the crossings from there up the left side and along the row's line,
+//     decided with the refinement's symbolic perturbation (cover.cu).
+// The 32 row words become 32 words in curve order (bit t of the tile = curve
+// position t).  There a quadtree cell of level l is an aligned run of 4^l bits,
+// so the covering's records (maximal untouched cells, and the viewport clip that
+// keeps or drops a record as a whole) and the starts of the canonical ranges
+// (positions where a polygon's bit changes) are shifts and masks of whole words.
+// Ranges are written from the bitmaps directly: no record of a finest cell is
+// ever stored, sorted or merged.
+//
+// One warp per tile.  For the 263-zone sweep (eps 2^12 .. 2^6, 1.2e8 records)
+// this stage takes 2.5 ms (raster 1.26, ranges 0.67, sort and bookkeeping 0.5)
+// where the refinement to the finest level, its sort and its merge took 9.3
+// (2.4, 4.5 and 2.2, and the counters of five more levels).
+#include "cover_internal.cuh"
+
+#include <algorithm>
+#include <string>
+#include <vector>
+
+namespace sdb {
+
+namespace {
+
+constexpr unsigned FULL = 0xffffffffu;
+constexpr uint32_t NONE = 0xffffffffu;
+constexpr int TPB = 256;
+constexpr int WPB = TPB / 32;
+
+// element info: slot (bits 0..25), covers the group's first cell (26), with the
+// boundary flag (27), covers its last cell (28), with the flag (29), tile (30)
+constexpr uint32_t INFO_SLOT = (1u << 26) - 1u;
+constexpr uint32_t INFO_FIRST = 26, INFO_LAST = 28, INFO_TILE = 1u << 30;
+
+// ---------------------------------------------------------------- rasterising
+// floor(f / d) for d > 0 where it lies in [-2, 34], else some value on the same
+// side of that interval; *exact: f is a multiple of d.  rd is about 1 / d: the
+// estimate is within one, the remainder decides.
+__device__ __forceinline__ int column_of(int64_t f, int64_t d, float rd, bool* exact) {
+  const float q = fminf(fmaxf(__ll2float_rn(f) * rd, -2.0f), 34.0f);
+  int t = (int)floorf(q);
+  int64_t r = f - (int64_t)t * d;
+  if (r < 0) {
+    --t;
+    r += d;
+  } else if (r >= d) {
+    ++t;
+    r -= d;
+  }
+  *exact = r == 0;
+  return t;
+}
+
+// Row words of one polygon in one tile (lane = row, bit = column): *touched the
+// cells that an edge meets, *inside the untouched cells in the polygon.  px, py
+// is the tile's corner, sh the finest cells' side (log2), par the parity of the
+// perturbed corner.  All lanes take part.
+//
+// For an edge from a up to b, f(row) = cross(b - a, (px, Y0) - a) over dy side is
+// the column at which the edge's line meets the row's lower line: one exact small
+// quotient per row, whose remainder tells whether a column line is met exactly.
+__device__ __forceinline__ void raster_tile(const Edge* __restrict__ edges,
+                                            const uint32_t* __restrict__ elist, uint32_t ecnt,
+                                            int32_t px, int32_t py, uint32_t sh, uint32_t par,
+                                            uint32_t* touched, uint32_t* inside) {
+  const int lane = threadIdx.x & 31;
+  const int32_t s = 1 << sh;
+  const int32_t Y0 = py + lane * s, Y1 = Y0 + s;  // the row's closed strip
+  uint32_t T = 0, H = 0, V = 0;  // touched; flips along the row; flip of the row's corner
+  for (uint32_t base = 0; base < ecnt; base += 32) {
+    Edge E{0, 0, 0, 0};
+    if (base + lane < ecnt) {
+      E = edges[__ldg(elist + base + lane)];
+      if (E.by < E.ay) E = Edge{E.bx, E.by, E.ax, E.ay};  // upwards
+    }
+    const int m = (int)min(32u, ecnt - base);
+    for (int e = 0; e < m; ++e) {
+      const int32_t ax = __shfl_sync(FULL, E.ax, e), ay = __shfl_sync(FULL, E.ay, e);
+      const int32_t bx = __shfl_sync(FULL, E.bx, e), by = __shfl_sync(FULL, E.by, e);
+      const int32_t dx = bx - ax, dy = by - ay;
+      const int64_t d = (int64_t)dy << sh, step = (int64_t)dx << sh;
+      const int64_t f0 = (int64_t)dx * (py - ay) - (int64_t)dy * (px - ax);
+      const int64_t f = f0 + lane * step;
+      const float rd = dy > 0 ? __frcp_rn(__ll2float_rn(d)) : 0.0f;
+      bool exl, exu, ex32;
+      const int tl = column_of(f, d, rd, &exl);
+      int tu = __shfl_down_sync(FULL, tl, 1);
+      exu = __shfl_down_sync(FULL, (int)exl, 1) != 0;
+      const int t32 = column_of(f0 + 32 * step, d, rd, &ex32);  // the tile's upper line
+      if (lane == 31) {
+        tu = t32;
+        exu = ex32;
+      }
+      // the clipped edge's ends by column: where it leaves the strip, or its own
+      // end inside it (a horizontal edge always has both ends inside)
+      const bool cut_lo = Y0 > ay, cut_hi = Y1 < by;
+      const int t_lo = cut_lo ? tl : (ax - px) >> sh, t_hi = cut_hi ? tu : (bx - px) >> sh;
+      const bool e_lo = cut_lo ? exl : ((ax - px) & (s - 1)) == 0;
+      const bool e_hi = cut_hi ? exu : ((bx - px) & (s - 1)) == 0;
+      // closed cells: one more to the left when the left end is on a column line
+      const int m0 = dx >= 0 ? t_lo - e_lo : t_hi - e_hi, m1 = dx >= 0 ? t_hi : t_lo;
+      if (by >= Y0 && ay <= Y1 && m1 >= 0 && m0 <= 31)
+        T |= (FULL << max(m0, 0)) & (FULL >> (31 - min(m1, 31)));
+      // perturbed side of the row's left corner, and of the tile's
+      const bool tie = dy == 0 && dx > 0;
+      const bool pos = f > 0 || (f == 0 && tie), pos0 = f0 > 0 || (f0 == 0 && tie);
+      if ((ax > px) != (bx > px)) V ^= (uint32_t)(pos != pos0);
+      // the edge crosses the row's line right of that corner: every later corner flips
+      if (ay <= Y0 && by > Y0 && pos && tl < 31) H ^= FULL << (tl + 1);
+    }
+  }
+  *touched = T;
+  *inside = (((par ^ V) & 1u) ? ~H : H) & ~T;
+}
+
+// ---------------------------------------------------------------- curve order
+// The tile's curve by 2 x 2 blocks: lane l holds curve positions 32 l .. 32 l + 31,
+// the blocks 8 l .. 8 l + 7 of the curve over 16 x 16 blocks.  s_blk[i * 32 + l]
+// describes block 8 l + i in the plain orientation -- bits 0..6 the byte offset of
+// its two row words (8 by), bits 8..12 its first column (2 bx), bits 16..21 its
+// own orientation times 16 -- and s_blk[256 + ...] the same with x and y swapped;
+// complementing is an XOR of the fields.  s_perm[orientation * 16 + v] puts a
+// block's four cells v (bit 2 y + x) in curve order.
+constexpr uint32_t BLK_COMPLEMENT = (15u << 3) | (15u << 9) | (1u << 20);
+struct CurveTables {
+  uint32_t blk[512];
+  uint8_t perm[64];
+};
+__device__ __forceinline__ void fill_curve(CurveTables& t) {
+  for (uint32_t k = threadIdx.x; k < 256; k += TPB) {
+    uint32_t sw = 0, cm = 0, x = 0, y = 0;
+    for (int lev = TILE_DEPTH - 2; lev >= 0; --lev) {
+      const uint32_t d = (k >> (2 * lev)) & 3u;
+      const uint32_t xt = d >> 1, yt = xt ^ (d & 1u);
+      const uint32_t u = xt ^ cm, v = yt ^ cm;
+      x = (x << 1) | (sw ? v : u);
+      y = (y << 1) | (sw ? u : v);
+      if (!yt) {
+        sw ^= 1u;
+        cm ^= xt;
+      }
+    }
+    const uint32_t at = (k & 7u) * 32 + (k >> 3), o = (sw << 1) | cm;
+    t.blk[at] = (y << 3) | (x << 9) | (o << 20);
+    t.blk[256 + at] = (x << 3) | (y << 9) | ((o ^ 2u) << 20);
+  }
+  for (uint32_t k = threadIdx.x; k < 64; k += TPB) {
+    const uint32_t sw = k >> 5, cm = (k >> 4) & 1u;
+    uint32_t out = 0;
+    for (uint32_t d = 0; d < 4; ++d) {
+      const uint32_t xt = d >> 1, yt = xt ^ (d & 1u);
+      const uint32_t u = xt ^ cm, v = yt ^ cm;
+      const uint32_t x = sw ? v : u, y = sw ? u : v;
+      out |= ((k >> (2 * y + x)) & 1u) << d;
+    }
+    t.perm[k] = (uint8_t)out;
+  }
+}
+
+// N row words (lane = row) to curve order (lane l: positions 32 l .. 32 l + 31)
+// through shared memory, a 2 x 2 block at a time: one 8-byte read of its two
+// rows, one read of the permutation.  (A bit at a time took 450 instructions for
+// two words; this takes 190.)
+template <int N>
+__device__ __forceinline__ void to_curve(const uint32_t (&rows)[N], uint32_t (&out)[N],
+                                         uint32_t orient, const CurveTables& t,
+                                         uint32_t (*s_rows)[32]) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+#pragma unroll
+  for (int n = 0; n < N; ++n) s_rows[n][lane] = rows[n];
+  __syncwarp();
+  const uint32_t flip = (orient & 1u) ? BLK_COMPLEMENT : 0u;
+  const uint32_t* blk = t.blk + ((orient & 2u) ? 256 : 0) + lane;
+#pragma unroll
+  for (int n = 0; n < N; ++n) out[n] = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t e = blk[i * 32] ^ flip;
+    const uint32_t c = (e >> 8) & 31u;
+    const uint8_t* perm = t.perm + ((e >> 16) & 0x30u);
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+      const uint2 w = *reinterpret_cast<const uint2*>(
+          reinterpret_cast<const unsigned char*>(s_rows[n]) + (e & 0x78u));
+      const uint32_t v = ((w.x >> c) & 3u) | (((w.y >> c) & 3u) << 2);
+      out[n] |= (uint32_t)perm[v] << (4 * i);
+    }
+  }
+}
+
+// per aligned run of 4, 16, 64, 256 bits: all ones if any bit of the run is set
+__device__ __forceinline__ uint32_t any4(uint32_t v) {
+  v |= v >> 1;
+  v |= v >> 2;
+  return (v & 0x11111111u) * 15u;
+}
+__device__ __forceinline__ uint32_t any16(uint32_t v) {
+  return ((v & 0xffffu) ? 0xffffu : 0u) | ((v >> 16) ? 0xffff0000u : 0u);
+}
+__device__ __forceinline__ uint32_t any_lanes(uint32_t v, int lanes) {  // lanes = 2 or 8
+  const uint32_t b = __ballot_sync(FULL, v != 0);
+  const uint32_t g = (threadIdx.x & 31) & ~(uint32_t)(lanes - 1);
+  return ((b >> g) & ((1u << lanes) - 1u)) ? FULL : 0u;
+}
+
+// What a warp needs of one polygon in one tile, in sorted order (32 bytes)
+struct __align__(16) TileRec {
+  int32_t px, py;     // the tile's corner
+  uint32_t eoff, ecnt_par;
+  uint32_t slot;
+  uint32_t geo;       // finest side (log2) | orientation << 8 | clipped << 10
+  uint32_t query;
+  uint32_t bits;      // its bitmap's place (its tile item)
+};
+
+struct TileArgs {
+  const TileRec* rec;      // per element (tiles' only)
+  const uint32_t* elist;
+  const Edge* edges;
+  const CoverQuery* qs;
+  uint32_t qshift, flags;
+  const uint64_t* key;     // sorted keys
+  uint64_t ne;
+  const uint2* heads;      // tile groups: first element, elements
+  const uint32_t* n_heads;
+  uint32_t* bits;          // per item 32 words in curve order: the polygon's cells
+  uint32_t* bbits;         // the same for its boundary cells (flagged coverings)
+  uint32_t* info;          // per element
+  uint32_t* cells;         // per element: records of the group (at its head)
+  uint64_t* inner;         // per element, at tile heads: ranges that start inside
+                           // the tile << 32 | their list entries
+  unsigned int* flag;      // [0] nested, [1] a tile with too many polygons
+  unsigned long long* front;  // boundary cells one level above the finest
+};
+
+// One warp per tile: the bitmaps of its polygons, what they add to the covering.
+// Bound by instruction issue and, a tile being a chain of dependent loads, by the
+// warps in flight: with a 64-bit division per edge, a bit-by-bit curve order and
+// 92 registers (two blocks per SM) it took 3.06 ms for the 263-zone sweep, with
+// small quotients, 2 x 2 blocks and 64 registers 1.26 ms.
+__global__ __launch_bounds__(TPB, 4) void tile_raster_kernel(TileArgs A) {
+  __shared__ CurveTables s_curve;
+  __shared__ __align__(16) uint32_t s_rows[WPB][2][32];
+  fill_curve(s_curve);
+  __syncthreads();
+  if (A.flag[1]) return;  // a crowded tile: the refinement takes over
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t nh = *A.n_heads;
+  for (uint32_t g = blockIdx.x * WPB + w; g < nh; g += gridDim.x * WPB) {
+    const uint2 head = A.heads[g];
+    const uint32_t a = head.x, k = head.y;
+    uint32_t starts = 0, ncell = 0, u[5] = {0, 0, 0, 0, 0}, fr = 0;
+    for (uint32_t i = a; i < a + k; ++i) {
+      const TileRec R = A.rec[i];
+      const uint32_t sh = R.geo & 0xffu, orient = (R.geo >> 8) & 3u;
+      uint32_t rows[2], curve[2];
+      raster_tile(A.edges, A.elist + R.eoff, R.ecnt_par & 0x7fffffffu, R.px, R.py, sh,
+                  R.ecnt_par >> 31, &rows[0], &rows[1]);
+      to_curve<2>(rows, curve, orient, s_curve, s_rows[w]);
+      const uint32_t T = curve[0];
+      uint32_t I = curve[1];
+      // runs that hold a touched cell, level by level
+      const uint32_t t1 = any4(T), t2 = any16(t1), t3 = any_lanes(t2, 2), t4 = any_lanes(t3, 8);
+      // the interior cells by the level of their record (the largest untouched run)
+      uint32_t c0 = I & t1, c1 = I & ~t1 & t2, c2 = I & ~t2 & t3, c3 = I & ~t3 & t4, c4 = I & ~t4;
+      uint32_t tk = T, f1 = t1;
+      if (R.geo >> 10) {
+        // viewport clip: a record stays when its cell holds lattice points of it
+        const CoverQuery Q = A.qs[R.query];
+        const int64_t side = (int64_t)1 << sh, y = R.py + lane * side;
+        uint32_t row[1] = {0}, box[1];
+        if (y < (int64_t)Q.y1 && y + side > (int64_t)Q.y0) {
+          // columns with px + m side < x1 and px + (m + 1) side > x0
+          const int64_t lo = ((int64_t)Q.x0 - R.px) >> sh, hi = ((int64_t)Q.x1 - 1 - R.px) >> sh;
+          if (hi >= 0 && lo <= 31)
+            row[0] = (FULL << (lo < 0 ? 0 : lo)) & (FULL >> (31 - (hi > 31 ? 31 : hi)));
+        }
+        to_curve<1>(row, box, orient, s_curve, s_rows[w]);
+        const uint32_t b1 = any4(box[0]), b2 = any16(b1), b3 = any_lanes(b2, 2),
+                       b4 = any_lanes(b3, 8);
+        tk &= box[0];
+        c0 &= box[0];
+        c1 &= b1;
+        c2 &= b2;
+        c3 &= b3;
+        c4 &= b4;
+        f1 &= b1;
+        I = c0 | c1 | c2 | c3 | c4;
+      }
+      const uint32_t cover = tk | I;
+      A.bits[(uint64_t)R.bits * 32 + lane] = cover;
+      if (A.flags) A.bbits[(uint64_t)R.bits * 32 + lane] = tk;
+      // records in 256ths: a cell of a run of 4^l cells is 1 / 4^l of a record
+      ncell += 256 * (uint32_t)__popc(tk | c0) + 64 * (uint32_t)__popc(c1) +
+               16 * (uint32_t)__popc(c2) + 4 * (uint32_t)__popc(c3) + (uint32_t)__popc(c4);
+      fr += __popc(f1 & 0x11111111u);
+      u[0] |= tk | c0;
+      u[1] |= c1;
+      u[2] |= c2;
+      u[3] |= c3;
+      u[4] |= c4;
+      // positions where this polygon's part of the set changes
+      uint32_t prev = __shfl_up_sync(FULL, cover, 1);
+      starts |= cover ^ ((cover << 1) | (prev >> 31));
+      if (A.flags) {
+        prev = __shfl_up_sync(FULL, tk, 1);
+        starts |= tk ^ ((tk << 1) | (prev >> 31));
+      }
+      const uint32_t last = __shfl_sync(FULL, cover, 31) >> 31;
+      const uint32_t blast = A.flags ? __shfl_sync(FULL, tk, 31) >> 31 : 0u;
+      if (lane == 0)
+        A.info[i] = R.slot | ((cover & 1u) << INFO_FIRST) |
+                    (A.flags ? (tk & 1u) << (INFO_FIRST + 1) : 0u) | (last << INFO_LAST) |
+                    (blast << (INFO_LAST + 1)) | INFO_TILE;
+    }
+    // two polygons' records that share cells must be the same cell
+    const bool clash = k > 1 && ((u[0] & (u[1] | u[2] | u[3] | u[4])) ||
+                                 (u[1] & (u[2] | u[3] | u[4])) || (u[2] & (u[3] | u[4])) ||
+                                 (u[3] & u[4]));
+    if (__any_sync(FULL, clash) && lane == 0) A.flag[0] = 1u;
+    if (lane == 0) starts &= ~1u;  // the tile's first position is the group's head
+    // list entries of the inner starts
+    uint32_t ent = 0;
+    for (uint32_t i = a; i < a + k; ++i)
+      ent += __popc(starts & A.bits[(uint64_t)A.rec[i].bits * 32 + lane]);
+    const uint32_t ns = __reduce_add_sync(FULL, __popc(starts));
+    ent = __reduce_add_sync(FULL, ent);
+    ncell = __reduce_add_sync(FULL, ncell);
+    fr = __reduce_add_sync(FULL, fr);
+    if (lane == 0) {
+      A.inner[a] = ((uint64_t)ns << 32) | ent;
+      A.cells[a] = ncell >> 8;
+      // frontier size, as the refinement would meet it; spread over counters
+      atomicAdd(A.front + (g & 255u), (unsigned long long)fr);
+    }
+  }
+}
+
+// ---------------------------------------------------------------- elements
+// keys of the tile items, appended to the coarse records' keys
+__global__ void tile_keys_kernel(const Item* __restrict__ items, uint64_t n,
+                                 const uint32_t* __restrict__ pair_query, uint32_t qshift,
+                                 uint64_t n_rec, uint64_t* __restrict__ key) {
+  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const Item it = items[i];
+  const uint64_t q = qshift >= 64 ? 0ull : (uint64_t)pair_query[it.pair] << qshift;
+  key[n_rec + i] = q | (it.hid << (2 * TILE_DEPTH));
+}
+
+__global__ void iota_kernel(uint32_t* __restrict__ p, uint64_t n) {
+  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) p[i] = (uint32_t)i;
+}
+
+// The coarse records' info, level and record count, and the tile groups (any
+// order): their polygons' records in sorted order, ascending by slot, written by
+// the thread of the group's first element.
+__global__ void element_kernel(const uint64_t* __restrict__ key, const uint32_t* __restrict__ idx,
+                               const uint32_t* __restrict__ val, uint64_t n_rec, uint64_t ne,
+                               const Item* __restrict__ items,
+                               const uint32_t* __restrict__ pair_query,
+                               const uint32_t* __restrict__ pair_slot,
+                               const CoverQuery* __restrict__ qs, uint32_t B,
+                               uint2* __restrict__ heads, uint32_t* __restrict__ n_heads,
+                               uint32_t* __restrict__ info, uint8_t* __restrict__ level,
+                               uint32_t* __restrict__ cells, TileRec* __restrict__ rec,
+                               unsigned int* __restrict__ flag) {
+  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  uint32_t k = 0;
+  if (i < ne) {
+    const uint32_t el = idx[i];
+    if (el < n_rec) {
+      const uint32_t v = val[el];
+      info[i] = (v & INFO_SLOT) | (1u << INFO_FIRST) | (1u << INFO_LAST);
+      level[i] = (uint8_t)((v >> 26) & 31u);
+      cells[i] = 1;
+    } else {
+      level[i] = (uint8_t)TILE_DEPTH;
+      info[i] = INFO_TILE;
+      const uint64_t q = key[i];
+      const bool head = i == 0 || key[i - 1] != q;
+      if (!head) {
+        cells[i] = 0;  // the head's warp counts for the tile
+      } else if (i + TILE_MAX_GROUP < ne && key[i + TILE_MAX_GROUP] == q) {
+        flag[1] = 1u;
+      } else {
+        for (uint64_t j = i; j < ne && key[j] == q; ++j, ++k) {
+          const uint32_t e = idx[j];
+          if (e < n_rec) {  // another polygon's cell with the tile's start
+            flag[0] = 1u;
+            break;
+          }
+          const uint32_t ti = e - (uint32_t)n_rec;
+          const Item it = items[ti];
+          const uint32_t qi = pair_query[it.pair];
+          const CoverQuery Q = qs[qi];
+          const uint32_t sh = B - Q.F;
+          TileRec R;
+          R.px = (int32_t)(it.cx << (sh + TILE_DEPTH));
+          R.py = (int32_t)(it.cy << (sh + TILE_DEPTH));
+          R.eoff = it.eoff;
+          R.ecnt_par = it.ecnt_par;
+          R.slot = pair_slot[it.pair];
+          const int64_t side = (int64_t)1 << (sh + TILE_DEPTH);
+          const bool clip = R.px < (int64_t)Q.x0 || R.py < (int64_t)Q.y0 ||
+                            R.px + side > (int64_t)Q.x1 || R.py + side > (int64_t)Q.y1;
+          R.geo = sh | (it.orient << 8) | ((uint32_t)clip << 10);
+          R.query = qi;
+          R.bits = ti;
+          uint64_t at = j;  // insertion by slot
+          while (at > i && rec[at - 1].slot > R.slot) {
+            rec[at] = rec[at - 1];
+            --at;
+          }
+          rec[at] = R;
+        }
+      }
+    }
+  }
+  const uint32_t b = __ballot_sync(FULL, k > 0);
+  uint32_t at = 0;
+  if (b && (threadIdx.x & 31) == 0) at = atomicAdd(n_heads, (uint32_t)__popc(b));
+  at = __shfl_sync(FULL, at, 0) + __popc(b & ((1u << (threadIdx.x & 31)) - 1u));
+  if (k > 0) heads[at] = make_uint2((uint32_t)i, k);
+}
+
+// ---------------------------------------------------------------- ranges
+struct GroupArgs {
+  const uint64_t* key;
+  const uint32_t* info;
+  const uint8_t* level;
+  const uint64_t* inner;
+  uint64_t ne, lomask;
+  uint32_t qshift;
+  const CoverQuery* qs;
+};
+
+__device__ __forceinline__ uint32_t gq(const GroupArgs& A, uint64_t key) {
+  return A.qshift >= 64 ? 0u : (uint32_t)(key >> A.qshift);
+}
+// the list entry of element info at the group's first / last cell
+__device__ __forceinline__ uint32_t info_entry(uint32_t v, uint32_t which) {
+  return (v & INFO_SLOT) | (((v >> (which + 1)) & 1u) << 31);
+}
+
+// a group's set at its last cell equals another's at its first cell
+__device__ bool same_ends(const GroupArgs& A, uint64_t pa, uint64_t pe, uint64_t a, uint64_t e) {
+  uint32_t n0 = 0, n1 = 0;
+  for (uint64_t i = pa; i < pe; ++i) n0 += (A.info[i] >> INFO_LAST) & 1u;
+  for (uint64_t i = a; i < e; ++i) n1 += (A.info[i] >> INFO_FIRST) & 1u;
+  if (n0 != n1) return false;
+  for (uint64_t i = a; i < e; ++i) {
+    const uint32_t v = A.info[i];
+    if (!((v >> INFO_FIRST) & 1u)) continue;
+    bool found = false;
+    for (uint64_t j = pa; j < pe && !found; ++j)
+      found = ((A.info[j] >> INFO_LAST) & 1u) &&
+              info_entry(A.info[j], INFO_LAST) == info_entry(v, INFO_FIRST);
+    if (!found) return false;
+  }
+  return true;
+}
+
+// Per element: 0, or at the head of a group the ranges it opens (<< 32) and their
+// list entries; code: bit 0 an empty gap before it, bit 1 itself, bit 2 the empty
+// tail of its query, bit 3 the query's first group, bit 4 its last.  A gap, a
+// group or a tail opens a range when its set differs from what comes before.
+__global__ void group_count_kernel(GroupArgs A, uint64_t* __restrict__ cnt,
+                                   uint8_t* __restrict__ code, uint32_t* __restrict__ qhead,
+                                   unsigned int* __restrict__ flag) {
+  const uint64_t a = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (a >= A.ne || flag[1]) return;  // (a crowded tile: nothing is made)
+  const uint64_t key = A.key[a];
+  if (a > 0 && A.key[a - 1] == key) {
+    cnt[a] = 0;
+    code[a] = 0;
+    return;
+  }
+  const uint32_t lev = A.level[a], q = gq(A, key);
+  const uint64_t lo = key & A.lomask, hi = lo + (1ull << (2 * lev));
+  bool nest = false;
+  uint32_t nfirst = 0, nlast = 0;
+  uint64_t e = a;
+  for (; e < A.ne && A.key[e] == key; ++e) {
+    const uint32_t v = A.info[e];
+    nest |= A.level[e] != lev || ((v ^ A.info[a]) & INFO_TILE);
+    nfirst += (v >> INFO_FIRST) & 1u;
+    nlast += (v >> INFO_LAST) & 1u;
+  }
+  const bool first = a == 0 || gq(A, A.key[a - 1]) != q;
+  const bool last = e == A.ne || gq(A, A.key[e]) != q;
+  bool gap = lo > 0, opens_gap = gap, opens_head = gap ? nfirst != 0 : true;
+  if (!first) {
+    const uint64_t pkey = A.key[a - 1];
+    uint64_t pa = a - 1;
+    bool plast = (A.info[pa] >> INFO_LAST) & 1u;
+    while (pa > 0 && A.key[pa - 1] == pkey) {
+      --pa;
+      plast |= (A.info[pa] >> INFO_LAST) & 1u;
+    }
+    const uint64_t pend = (pkey & A.lomask) + (1ull << (2 * A.level[pa]));
+    nest |= lo < pend;  // the previous cell reaches into this one
+    gap = lo > pend;
+    opens_gap = gap && plast;
+    opens_head = gap ? nfirst != 0 : !same_ends(A, pa, a, a, e);
+  }
+  const bool opens_tail = last && hi < (1ull << (2 * A.qs[q].F)) && nlast != 0;
+  const uint64_t in = (A.info[a] & INFO_TILE) ? A.inner[a] : 0ull;
+  cnt[a] = in + ((uint64_t)(opens_gap + opens_head + opens_tail) << 32) + (opens_head ? nfirst : 0u);
+  code[a] = (uint8_t)(opens_gap | (opens_head << 1) | (opens_tail << 2) | (first << 3) | (last << 4));
+  if (first) qhead[q] = (uint32_t)a;
+  if (nest) flag[0] = 1u;
+}
+
+struct RangeOut {
+  uint64_t* start;
+  uint32_t* list_off;
+  uint32_t* list_ids;
+  uint32_t* pay;
+  uint64_t* qopen;  // per query: ranges before its first group, after its last
+  uint32_t* qlist;  // per query: list entries before its first group, after its last
+};
+
+// inserts v into the ascending list out[0, t) by slot
+__device__ __forceinline__ void insert_entry(uint32_t* out, uint32_t t, uint32_t v) {
+  uint32_t j = t;
+  while (j > 0 && (out[j - 1] & INFO_SLOT) > (v & INFO_SLOT)) {
+    out[j] = out[j - 1];
+    --j;
+  }
+  out[j] = v;
+}
+
+__device__ __forceinline__ uint32_t pay_of(uint32_t n, uint32_t entry, uint64_t e) {
+  return n == 0 ? NONE
+         : n == 1 ? (entry & INFO_SLOT) | ((entry >> 31) << 30)
+                  : 0x80000000u | (uint32_t)e;
+}
+
+// the ranges outside the tiles: gaps, groups' first ranges, tails
+__global__ void group_emit_kernel(GroupArgs A, const uint64_t* __restrict__ off,
+                                  const uint8_t* __restrict__ code,
+                                  const uint64_t* __restrict__ extra, RangeOut o) {
+  const uint64_t a = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (a >= A.ne) return;
+  const uint64_t key = A.key[a];
+  if (a > 0 && A.key[a - 1] == key) return;
+  const uint32_t c = code[a], q = gq(A, key), lev = A.level[a];
+  const uint64_t lo = key & A.lomask, hi = lo + (1ull << (2 * lev));
+  uint64_t ro = off[a] >> 32;
+  uint32_t L = (uint32_t)off[a];
+  if (c & 8u) {
+    o.qopen[2 * q] = ro;
+    o.qlist[2 * q] = L;
+  }
+  uint64_t e = ro + extra[q];
+  if (c & 1u) {
+    uint64_t from = 0;
+    if (!(c & 8u)) {  // the end of the previous group's cell
+      const uint64_t pkey = A.key[a - 1];
+      from = (pkey & A.lomask) + (1ull << (2 * A.level[a - 1]));
+    }
+    o.start[e] = from;
+    o.list_off[e] = L;
+    o.pay[e] = NONE;
+    ++e;
+  }
+  if (c & 2u) {
+    uint32_t n = 0, one = 0;
+    for (uint64_t i = a; i < A.ne && A.key[i] == key; ++i) {
+      const uint32_t v = A.info[i];
+      if (!((v >> INFO_FIRST) & 1u)) continue;
+      one = info_entry(v, INFO_FIRST);
+      insert_entry(o.list_ids + L, n++, one);
+    }
+    o.start[e] = lo;
+    o.list_off[e] = L;
+    o.pay[e] = pay_of(n, one, e);
+    L += n;
+    ++e;
+  }
+  const uint64_t in = (A.info[a] & INFO_TILE) ? A.inner[a] : 0ull;
+  e += in >> 32;
+  L += (uint32_t)in;
+  if (c & 4u) {
+    o.start[e] = hi;
+    o.list_off[e] = L;
+    o.pay[e] = NONE;
+    ++e;
+  }
+  if (c & 16u) {
+    o.qopen[2 * q + 1] = e - extra[q];
+    o.qlist[2 * q + 1] = L;
+  }
+}
+
+// The ranges that start inside a tile: one warp per tile.  The start positions
+// are listed in shared memory first, so that lane i then makes the i-th of 32
+// ranges and the arrays are written side by side (each lane making the ranges of
+// its own 32 positions left most lanes waiting: 1.02 -> 0.67 ms for the sweep).
+__global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64_t* __restrict__ off,
+                                                        const uint8_t* __restrict__ code,
+                                                        const uint64_t* __restrict__ extra,
+                                                        uint64_t lomask, RangeOut o) {
+  constexpr uint32_t STAGE = 4;  // polygons of a tile held in shared memory
+  __shared__ uint32_t s_h[WPB][STAGE][32];
+  __shared__ uint32_t s_slot[WPB][STAGE];
+  __shared__ uint16_t s_pos[WPB][1024];
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t nh = *A.n_heads;
+  for (uint32_t g = blockIdx.x * WPB + w; g < nh; g += gridDim.x * WPB) {
+    const uint2 head = A.heads[g];
+    const uint32_t a = head.x, k = head.y;
+    const uint32_t ns = (uint32_t)(A.inner[a] >> 32);
+    if (ns == 0) continue;
+    const uint64_t key = A.key[a], pre = off[a];
+    const uint32_t c = code[a];
+    uint32_t starts = 0, nfirst = 0;
+    __syncwarp();
+    for (uint32_t j = 0; j < k; ++j) {
+      const TileRec* R = A.rec + a + j;
+      const uint32_t h = A.bits[(uint64_t)R->bits * 32 + lane];
+      uint32_t prev = __shfl_up_sync(FULL, h, 1);
+      starts |= h ^ ((h << 1) | (prev >> 31));
+      if (A.flags) {
+        const uint32_t b = A.bbits[(uint64_t)R->bits * 32 + lane];
+        prev = __shfl_up_sync(FULL, b, 1);
+        starts |= b ^ ((b << 1) | (prev >> 31));
+      }
+      nfirst += __shfl_sync(FULL, h, 0) & 1u;
+      if (j < STAGE) {
+        s_h[w][j][lane] = h;
+        if (lane == 0) s_slot[w][j] = R->slot;
+      }
+    }
+    if (lane == 0) starts &= ~1u;
+    uint32_t at = __popc(starts);
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t t = __shfl_up_sync(FULL, at, d);
+      if (lane >= (uint32_t)d) at += t;
+    }
+    at -= __popc(starts);
+    for (uint32_t m = starts; m; m &= m - 1) s_pos[w][at++] = (uint16_t)(32 * lane + __ffs(m) - 1);
+    __syncwarp();
+    const uint32_t q = A.qshift >= 64 ? 0u : (uint32_t)(key >> A.qshift);
+    uint64_t e0 = (pre >> 32) + extra[q] + (c & 1u) + ((c >> 1) & 1u);
+    uint32_t L0 = (uint32_t)pre + ((c & 2u) ? nfirst : 0u);
+    const uint64_t lo = key & lomask;
+    for (uint32_t i0 = 0; i0 < ns; i0 += 32) {
+      const bool on = i0 + lane < ns;
+      const uint32_t pos = on ? s_pos[w][i0 + lane] : 0u;
+      const uint32_t wi = pos >> 5, bi = pos & 31u;
+      auto has = [&](uint32_t j) {
+        const uint32_t h =
+            j < STAGE ? s_h[w][j][wi] : A.bits[(uint64_t)A.rec[a + j].bits * 32 + wi];
+        return (h >> bi) & 1u;
+      };
+      uint32_t n = 0;
+      if (on)
+        for (uint32_t j = 0; j < k; ++j) n += has(j);
+      uint32_t inc = n;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t t = __shfl_up_sync(FULL, inc, d);
+        if (lane >= (uint32_t)d) inc += t;
+      }
+      if (on) {
+        const uint64_t e = e0 + i0 + lane;
+        const uint32_t L = L0 + inc - n;
+        uint32_t one = 0, t = L;
+        for (uint32_t j = 0; j < k; ++j) {  // the polygons ascend by slot
+          if (!has(j)) continue;
+          one = j < STAGE ? s_slot[w][j] : A.rec[a + j].slot;
+          if (A.flags) one |= ((A.bbits[(uint64_t)A.rec[a + j].bits * 32 + wi] >> bi) & 1u) << 31;
+          o.list_ids[t++] = one;
+        }
+        o.start[e] = lo + pos;
+        o.list_off[e] = L;
+        o.pay[e] = pay_of(n, one, e);
+      }
+      L0 += __shfl_sync(FULL, inc, 31);
+    }
+  }
+}
+
+}  // namespace
+
+sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_rec, const Item* items,
+                       uint64_t n_tile, const uint32_t* elist, const Edge* edges,
+                       const uint32_t* pair_query, const uint32_t* pair_slot,
+                       const CoverQuery* d_qs, const CoverSpec& spec, uint32_t qshift,
+                       int key_bits, cudaStream_t s, CoverSet* out, TileOutcome* outcome) {
+  TraceScope tr("cover.tiles", s);
+  *outcome = TileOutcome::made;
+  Scratch sc(s);
+  const uint32_t Q = spec.Q;
+  const uint64_t ne = n_rec + n_tile;
+  if (ne >= 0xffffffffull) {
+    set_error("covering: %llu cells exceed the 32-bit index range", (unsigned long long)ne);
+    return SDB_ENOMEM;
+  }
+  uint64_t *keys, *ktmp, *sk;
+  uint32_t *ix, *ixtmp, *si;
+  SDB_TRY(sc.get(&keys, ne));
+  SDB_TRY(sc.get(&ktmp, ne));
+  SDB_TRY(sc.get(&ix, ne));
+  SDB_TRY(sc.get(&ixtmp, ne));
+  if (n_rec)
+    SDB_TRY_CUDA(cudaMemcpyAsync(keys, rkey, n_rec * 8, cudaMemcpyDeviceToDevice, s));
+  if (n_tile) {
+    tile_keys_kernel<<<grid_for(n_tile, 256), 256, 0, s>>>(items, n_tile, pair_query, qshift, n_rec,
+                                                          keys);
+    note_launch();
+  }
+  if (ne) {
+    iota_kernel<<<grid_for(ne, 256), 256, 0, s>>>(ix, ne);
+    note_launch();
+  }
+  SDB_TRY_CUDA(cudaGetLastError());
+  {
+    // every element starts on a multiple of a tile: the low key bits are zero
+    TraceScope tr1("cover.sort", s);
+    SDB_TRY(radix_sort_pairs(keys, ix, ktmp, ixtmp, ne, key_bits - 2 * TILE_DEPTH, s, &sk, &si,
+                             nullptr, 2 * TILE_DEPTH));
+  }
+  uint2* heads;
+  TileRec* rec;
+  uint32_t *n_heads, *info, *cells, *bits, *bbits = nullptr, *qhead;
+  uint8_t *level, *code;
+  uint64_t *inner, *cnt, *off, *coff, *tot;
+  unsigned int* dflag;  // nested, crowded
+  unsigned long long* front;
+  SDB_TRY(sc.get(&heads, n_tile));
+  SDB_TRY(sc.get(&n_heads, 1));
+  SDB_TRY(sc.get(&rec, ne));
+  SDB_TRY(sc.get(&info, ne));
+  SDB_TRY(sc.get(&cells, ne));
+  SDB_TRY(sc.get(&level, ne));
+  SDB_TRY(sc.get(&code, ne));
+  SDB_TRY(sc.get(&inner, ne));
+  SDB_TRY(sc.get(&cnt, ne));
+  SDB_TRY(sc.get(&off, ne));
+  SDB_TRY(sc.get(&coff, ne));
+  SDB_TRY(sc.get(&tot, 2));
+  SDB_TRY(sc.get(&qhead, Q));
+  SDB_TRY(sc.get(&dflag, 2));
+  SDB_TRY(sc.get(&front, 256));
+  SDB_TRY(sc.get(&bits, n_tile * 32));
+  if (spec.flags) SDB_TRY(sc.get(&bbits, n_tile * 32));
+  SDB_TRY_CUDA(cudaMemsetAsync(n_heads, 0, 4, s));
+  SDB_TRY_CUDA(cudaMemsetAsync(dflag, 0, 8, s));
+  SDB_TRY_CUDA(cudaMemsetAsync(tot, 0, 16, s));
+  SDB_TRY_CUDA(cudaMemsetAsync(front, 0, 256 * 8, s));
+  SDB_TRY_CUDA(cudaMemsetAsync(qhead, 0xff, (size_t)Q * 4, s));
+  TileArgs ta{};
+  ta.rec = rec;
+  ta.elist = elist;
+  ta.edges = edges;
+  ta.qs = d_qs;
+  ta.qshift = qshift;
+  ta.flags = spec.flags ? 1u : 0u;
+  ta.key = sk;
+  ta.ne = ne;
+  ta.heads = heads;
+  ta.n_heads = n_heads;
+  ta.bits = bits;
+  ta.bbits = bbits;
+  ta.info = info;
+  ta.cells = cells;
+  ta.inner = inner;
+  ta.flag = dflag;
+  ta.front = front;
+  GroupArgs ga{sk, info, level, inner, ne, qshift >= 64 ? ~0ull : ((1ull << qshift) - 1ull),
+               qshift, d_qs};
+  const unsigned tile_grid =
+      (unsigned)std::min<uint64_t>((n_tile + WPB - 1) / WPB, (uint64_t)num_sms() * 32);
+  if (ne) {
+    element_kernel<<<grid_for(ne, 256), 256, 0, s>>>(sk, si, rval, n_rec, ne, items, pair_query,
+                                                    pair_slot, d_qs, spec.B, heads, n_heads, info,
+                                                    level, cells, rec, dflag);
+    note_launch();
+    if (n_tile) {
+      TraceScope tr1("cover.raster", s);
+      tile_raster_kernel<<<tile_grid, TPB, 0, s>>>(ta);
+      note_launch();
+    }
+    group_count_kernel<<<grid_for(ne, 256), 256, 0, s>>>(ga, cnt, code, qhead, dflag);
+    note_launch();
+    SDB_TRY_CUDA(cudaGetLastError());
+    SDB_TRY(exclusive_scan<uint64_t>(cnt, off, ne, tot, s));
+    SDB_TRY(exclusive_scan_u32(cells, coff, ne, tot + 1, s));
+  }
+  uint64_t htot[2] = {0, 0};
+  unsigned int hflag[2] = {0, 0};
+  std::vector<uint32_t> hhead(Q);
+  std::vector<unsigned long long> hfront(256);
+  SDB_TRY_CUDA(cudaMemcpyAsync(htot, tot, 16, cudaMemcpyDeviceToHost, s));
+  SDB_TRY_CUDA(cudaMemcpyAsync(hflag, dflag, 8, cudaMemcpyDeviceToHost, s));
+  SDB_TRY_CUDA(cudaMemcpyAsync(hhead.data(), qhead, (size_t)Q * 4, cudaMemcpyDeviceToHost, s));
+  SDB_TRY_CUDA(cudaMemcpyAsync(hfront.data(), front, 256 * 8, cudaMemcpyDeviceToHost, s));
+  SDB_TRY_CUDA(cudaStreamSynchronize(s));
+  if (hflag[0] || hflag[1]) {
+    *outcome = hflag[1] ? TileOutcome::crowded : TileOutcome::nested;
+    return SDB_OK;
+  }
+  unsigned long long nfront = 0;
+  for (unsigned long long v : hfront) nfront += v;
+  const uint64_t ncells = htot[1];
+  // the limits of the refinement to the finest level
+  if (4 * nfront > 0xffffffffull) {
+    set_error("covering: the last level's frontier is too large (%llu cells)", nfront);
+    return SDB_ENOMEM;
+  }
+  if (ncells >= 0xffffffffull) {
+    set_error("covering: %llu cells exceed the 32-bit index range", (unsigned long long)ncells);
+    return SDB_ENOMEM;
+  }
+  // entries: the groups' ranges, plus per query its sentinel, plus the empty
+  // range of a query without records
+  std::vector<QueryFix> hq;
+  std::vector<uint64_t> hextra(Q);
+  const uint64_t extra = query_fixes(hhead, ne, &hq);
+  for (uint32_t q = 0; q < Q; ++q) hextra[q] = hq[q].extra;
+  const uint64_t E = (htot[0] >> 32) + extra, nids = htot[0] & 0xffffffffull;
+  if (E >= 0x7fffffffull) {  // entry indices travel in 31 bits of the packed payload
+    set_error("covering: %llu ranges exceed the 32-bit index range", (unsigned long long)E);
+    return SDB_ENOMEM;
+  }
+  SDB_TRY(dalloc_n(&out->start, E, s));
+  SDB_TRY(dalloc_n(&out->list_off, E, s));
+  SDB_TRY(dalloc_n(&out->pay, E, s));
+  SDB_TRY(dalloc_n(&out->list_ids, nids ? nids : 1, s));
+  QueryFix* dq;
+  uint64_t *qopen, *dextra;
+  uint32_t* qlist;
+  SDB_TRY(sc.get(&dq, Q));
+  SDB_TRY(sc.get(&qopen, 2 * (size_t)Q));
+  SDB_TRY(sc.get(&qlist, 2 * (size_t)Q));
+  SDB_TRY(sc.get(&dextra, Q));
+  SDB_TRY_CUDA(cudaMemcpyAsync(dq, hq.data(), (size_t)Q * sizeof(QueryFix), cudaMemcpyHostToDevice, s));
+  SDB_TRY_CUDA(cudaMemcpyAsync(dextra, hextra.data(), (size_t)Q * 8, cudaMemcpyHostToDevice, s));
+  if (ne) {
+    TraceScope tr1("cover.emit", s);
+    const RangeOut ro{out->start, out->list_off, out->list_ids, out->pay, qopen, qlist};
+    group_emit_kernel<<<grid_for(ne, 256), 256, 0, s>>>(ga, off, code, dextra, ro);
+    note_launch();
+    if (n_tile) {
+      tile_emit_kernel<<<tile_grid, TPB, 0, s>>>(ta, off, code, dextra, ga.lomask, ro);
+      note_launch();
+    }
+    SDB_TRY_CUDA(cudaGetLastError());
+  }
+  out->E = E;
+  out->nids = nids;
+  out->ncells = ncells;
+  return finish_queries(dq, qopen, qlist, d_qs, Q, coff, ne, ncells, out, s);
+}
+
+}  // namespace sdb

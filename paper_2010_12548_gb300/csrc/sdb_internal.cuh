@@ -439,6 +439,9 @@ sdb_status launch_join(const uint32_t* x, const uint32_t* y, const int32_t* attr
 // sort.cu: device-wide primitives
 template <class T>
 sdb_status exclusive_scan(const T* in, T* out, size_t n, T* d_total, cudaStream_t s);
+// 64-bit sums of 32-bit values, the total in *d_total
+sdb_status exclusive_scan_u32(const uint32_t* in, uint64_t* out, size_t n, uint64_t* d_total,
+                              cudaStream_t s);
 // out[i] = in[0] + ... + in[i - 1] in 64 bits, i in [0, n] (n + 1 entries)
 sdb_status exclusive_scan_i32(const int32_t* in, int64_t* out, size_t n, cudaStream_t s);
 // keys-only LSD sort of packed covering records (record_pack) on their key
@@ -449,11 +452,11 @@ sdb_status radix_sort_split(uint64_t* keys, uint64_t* tmp, size_t n, int bits, i
 // keys-only LSD sort on bits [first_bit, first_bit + bits) (stable)
 sdb_status radix_sort_keys(uint64_t* keys, uint64_t* tmp, size_t n, int bits, cudaStream_t s,
                            uint64_t** result, int first_bit = 0);
-// vals_in (nullable): where the values come from, left as it is (vals and vtmp
+// on key bits [first_bit, first_bit + bits); vals_in (nullable): where the values come from, left as it is (vals and vtmp
 // are then only written first)
 sdb_status radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* ktmp, uint32_t* vtmp,
                             size_t n, int bits, cudaStream_t s, uint64_t** kres, uint32_t** vres,
-                            const uint32_t* vals_in = nullptr);
+                            const uint32_t* vals_in = nullptr, int first_bit = 0);
 // unique of a sorted array: writes out[0..m), returns m via host sync
 sdb_status unique_sorted(const uint64_t* in, size_t n, uint64_t* out, size_t* m, cudaStream_t s);
 

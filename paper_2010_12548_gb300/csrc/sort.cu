@@ -405,6 +405,11 @@ sdb_status exclusive_scan(const T* in, T* out, size_t n, T* d_total, cudaStream_
   return scan_impl<T, T>(in, out, n, d_total, s);
 }
 
+sdb_status exclusive_scan_u32(const uint32_t* in, uint64_t* out, size_t n, uint64_t* d_total,
+                              cudaStream_t s) {
+  return scan_impl<uint64_t, uint32_t>(in, out, n, d_total, s);
+}
+
 sdb_status exclusive_scan_i32(const int32_t* in, int64_t* out, size_t n, cudaStream_t s) {
   uint64_t* o = reinterpret_cast<uint64_t*>(out);
   return scan_impl<uint64_t, int32_t>(in, o, n, o + n, s);
@@ -443,9 +448,9 @@ sdb_status radix_sort_split(uint64_t* keys, uint64_t* tmp, size_t n, int bits, i
 
 sdb_status radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* ktmp, uint32_t* vtmp, size_t n,
                             int bits, cudaStream_t s, uint64_t** kres, uint32_t** vres,
-                            const uint32_t* vals_in) {
-  return radix_sort_impl<true>(keys, vals, ktmp, vtmp, n, bits, s, kres, vres, 0, nullptr, 0,
-                               vals_in);
+                            const uint32_t* vals_in, int first_bit) {
+  return radix_sort_impl<true>(keys, vals, ktmp, vtmp, n, bits, s, kres, vres, first_bit, nullptr,
+                               0, vals_in);
 }
 
 sdb_status unique_sorted(const uint64_t* in, size_t n, uint64_t* out, size_t* m, cudaStream_t s) {
