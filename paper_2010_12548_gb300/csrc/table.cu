@@ -34,23 +34,12 @@ namespace sdb {
 
 namespace {
 
-// last r in [0, R] with start[r] <= h (start[0] = 0 <= h)
-__device__ __forceinline__ uint32_t last_le(const uint64_t* __restrict__ start, uint64_t R,
-                                            uint64_t h) {
-  uint64_t lo = 0, len = R + 1;
-  while (len > 1) {
-    const uint64_t half = len >> 1;
-    if (__ldg(start + lo + half) <= h) lo += half;
-    len -= half;
-  }
-  return (uint32_t)lo;
-}
-
-// the row-major position of the cell of level L0 whose curve id is b: the
-// digits from the top (plain orientation there) give the transformed quadrant
-// (xt, yt) = (d >> 1, (d >> 1) ^ (d & 1)), undone by the orientation (sw, cm);
-// yt = 0 transposes, and also complements when xt = 1
-__device__ __forceinline__ uint64_t bucket_cell(uint64_t b, uint32_t L0) {
+// the row-major position of the cell of level L0 whose curve id is b, and the
+// curve's orientation (sw << 1 | cm) below it: the digits from the top (plain
+// orientation there) give the transformed quadrant (xt, yt) = (d >> 1, (d >> 1) ^
+// (d & 1)), undone by the orientation (sw, cm); yt = 0 transposes, and also
+// complements when xt = 1
+__device__ __forceinline__ uint64_t bucket_cell(uint64_t b, uint32_t L0, uint32_t* orient) {
   uint32_t sw = 0, cm = 0, cx = 0, cy = 0;
   for (int lev = (int)L0 - 1; lev >= 0; --lev) {
     const uint32_t d = (uint32_t)(b >> (2 * lev)) & 3u;
@@ -63,6 +52,7 @@ __device__ __forceinline__ uint64_t bucket_cell(uint64_t b, uint32_t L0) {
       cm ^= xt;
     }
   }
+  *orient = (sw << 1) | cm;
   return ((uint64_t)cy << L0) | cx;
 }
 
@@ -136,18 +126,21 @@ __global__ __launch_bounds__(1024) void tile_prefix_kernel(uint32_t* __restrict_
   }
 }
 
-// per bucket (curve order): r0 = max-scan of the marks; a bucket inside one
-// range stores that range's payload at its cell's row-major position, a
-// bucket that meets several ranges is flagged
+// per bucket (curve order): r0 = max-scan of the marks, left in mark; a bucket
+// inside one range stores that range's payload at its cell's row-major position, a
+// bucket that meets several ranges is flagged (bit 31 of mark: ranges stay below
+// 2^30) and counted per tile
+constexpr uint32_t MARK_MIXED = 0x80000000u;
 __global__ __launch_bounds__(TB) void table_fill_kernel(
-    const uint32_t* __restrict__ mark, const uint32_t* __restrict__ tpre, uint64_t nb,
+    uint32_t* __restrict__ mark, const uint32_t* __restrict__ tpre, uint64_t nb,
     const uint64_t* __restrict__ start, const uint32_t* __restrict__ pay, uint32_t shift,
-    uint32_t L0, uint32_t* __restrict__ tab, uint32_t* __restrict__ mixed) {
+    uint32_t L0, uint32_t* __restrict__ tab, uint32_t* __restrict__ tcount) {
   __shared__ uint32_t s[TB / 32];
   __shared__ uint32_t carry;
   const uint64_t b0 = (uint64_t)blockIdx.x * TT;
   if (threadIdx.x == 0) carry = tpre[blockIdx.x];
   __syncthreads();
+  uint32_t count = 0;
   for (uint32_t base = 0; base < TT && b0 + base < nb; base += TB) {
     const uint64_t b = b0 + base + threadIdx.x;
     const uint32_t v = b < nb ? mark[b] : 0u;
@@ -158,33 +151,58 @@ __global__ __launch_bounds__(TB) void table_fill_kernel(
     for (uint32_t w = 0; w < (threadIdx.x >> 5); ++w) wpre = max(wpre, s[w]);
     const uint32_t c = carry;
     const uint32_t r0 = max(c, max(wpre, inc));
+    bool mix = false;
     if (b < nb) {
       const uint64_t lo = b << shift, hi = lo + ((1ull << shift) - 1);
       // the bucket meets several ranges iff the next range starts inside it
-      const bool mix = start[r0 + 1] <= hi;
-      mixed[b] = mix ? 1u : 0u;
-      if (!mix) tab[bucket_cell(b, L0)] = pay[r0];
+      mix = start[r0 + 1] <= hi;
+      mark[b] = r0 | (mix ? MARK_MIXED : 0u);
+      uint32_t orient;
+      if (!mix) tab[bucket_cell(b, L0, &orient)] = pay[r0];
     }
-    __syncthreads();
+    count += __syncthreads_count(mix);
     if (threadIdx.x == TB - 1) carry = r0;
     __syncthreads();
   }
+  if (threadIdx.x == 0) tcount[blockIdx.x] = count;
 }
 
-__global__ void table_mixed_kernel(const uint64_t* __restrict__ start, uint64_t R,
-                                   uint32_t shift, uint32_t L0, uint64_t nb,
-                                   const uint32_t* __restrict__ mixed,
-                                   const uint32_t* __restrict__ rank, uint32_t* __restrict__ tab,
-                                   uint2* __restrict__ win, uint32_t* __restrict__ mpos) {
-  for (uint64_t b = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; b < nb;
-       b += (uint64_t)gridDim.x * blockDim.x) {
-    if (!mixed[b]) continue;
-    const uint64_t lo = b << shift, hi = lo + ((1ull << shift) - 1);
-    const uint32_t m = rank[b];
-    const uint64_t pos = bucket_cell(b, L0);
-    tab[pos] = TAB_MIXED | m;
-    win[m] = make_uint2(last_le(start, R, lo), last_le(start, R, hi));
-    mpos[m] = (uint32_t)pos;
+// The mixed buckets, ranked in curve order from their tiles' offsets: table entry,
+// window and the cell's place, orientation (bits 26, 27) and curve id.  The last
+// range of a window is the next bucket's first one, or the one before it when that
+// starts with the next bucket.
+__global__ __launch_bounds__(TB) void table_mixed_kernel(
+    const uint64_t* __restrict__ start, uint64_t R, uint32_t shift, uint32_t L0, uint64_t nb,
+    const uint32_t* __restrict__ mark, const uint32_t* __restrict__ toff,
+    uint32_t* __restrict__ tab, uint2* __restrict__ win, uint32_t* __restrict__ mpos,
+    uint32_t* __restrict__ mid) {
+  __shared__ uint32_t s[TB / 32];
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint64_t b0 = (uint64_t)blockIdx.x * TT;
+  uint32_t rank = toff[blockIdx.x];
+  for (uint32_t base = 0; base < TT && b0 + base < nb; base += TB) {
+    const uint64_t b = b0 + base + threadIdx.x;
+    const uint32_t v = b < nb ? mark[b] : 0u;
+    const bool mix = (v & MARK_MIXED) != 0;
+    const uint32_t bal = __ballot_sync(0xffffffffu, mix);
+    if (lane == 0) s[w] = __popc(bal);
+    __syncthreads();
+    uint32_t m = rank + __popc(bal & ((1u << lane) - 1u));
+    for (uint32_t i = 0; i < TB / 32; ++i) {
+      if (i < w) m += s[i];
+      rank += s[i];
+    }
+    if (mix) {
+      uint32_t orient;
+      const uint32_t pos = (uint32_t)bucket_cell(b, L0, &orient);
+      const uint32_t next = b + 1 < nb ? mark[b + 1] & ~MARK_MIXED : (uint32_t)R;
+      const uint32_t last = next - (start[next] == (b + 1) << shift ? 1u : 0u);
+      tab[pos] = TAB_MIXED | m;
+      win[m] = make_uint2(v & ~MARK_MIXED, last);
+      mpos[m] = pos | (orient << 26);
+      mid[m] = (uint32_t)b;
+    }
+    __syncthreads();
   }
 }
 
@@ -200,42 +218,85 @@ __device__ __forceinline__ uint32_t last_le_in(const uint64_t* __restrict__ star
   return lo;
 }
 
-// The second level.  Mixed bucket m (row-major cell pos = mpos[m] of level L0)
-// splits into S x S sub-cells of level L1 = L0 + s2 (S = 2^s2), stored
-// row-major within the bucket at sub[m * S^2 + (sy << s2 | sx)].  A sub-cell is
-// again a quadtree cell, so its finest ids are one contiguous block
-// [hs << 2 (F - L1), (hs + 1) << 2 (F - L1)), hs its curve id at level L1; the
-// ranges holding the block's first and last id lie in the bucket's window.
-// Pass 1 (write = false) flags the sub-cells that meet several ranges and
-// stores the payload of the others; pass 2 writes TAB_MIXED | m2 and the
-// window of the m2-th flagged sub-cell.
-__global__ void table_sub_kernel(const uint64_t* __restrict__ start, const uint32_t* __restrict__ pay,
-                                 const uint2* __restrict__ win, const uint32_t* __restrict__ mpos,
-                                 uint64_t M, uint32_t L0, uint32_t s2, uint32_t F,
-                                 uint32_t* __restrict__ sub, uint32_t* __restrict__ flag,
-                                 const uint32_t* __restrict__ rank2, uint2* __restrict__ win2,
-                                 bool write) {
-  const uint64_t per = 1ull << (2 * s2);
-  const uint32_t L1 = L0 + s2, sh = 2 * (F - L1);
-  for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < M * per;
-       t += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t m = t >> (2 * s2);
-    const uint32_t j = (uint32_t)(t & (per - 1));
-    if (write && !flag[t]) continue;
-    const uint32_t pos = mpos[m];
-    const uint32_t cx = pos & ((1u << L0) - 1u), cy = pos >> L0;
-    const uint32_t sx = j & ((1u << s2) - 1u), sy = j >> s2;
-    const uint64_t hs = hilbert_id((cx << s2) | sx, (cy << s2) | sy, L1);
-    const uint64_t lo = hs << sh, hi = lo + ((1ull << sh) - 1);
+// The second level.  Mixed bucket m (row-major cell of level L0) splits into
+// S x S sub-cells of level L1 = L0 + s2 (S = 2^s2), stored row-major within the
+// bucket at sub[m * S^2 + (sy << s2 | sx)].  A sub-cell is again a quadtree cell:
+// the j-th along the curve holds the finest ids [lo, lo + 4^(F - L1)), lo = the
+// bucket's first id + (j << 2 (F - L1)).  One warp per bucket takes its sub-cells in
+// curve order, so one search of the bucket's window per sub-cell gives its first
+// range and, from the next one's, its last.  A sub-cell inside one range stores its
+// payload; the others store TAB_MIXED | their rank in the bucket, their windows go
+// to cand (S^2 places a bucket) and their number to mcount; a second pass adds the
+// buckets' offsets.  (A thread per sub-cell, encoding its id and searching for both
+// ends, in two full passes and a scan over all sub-cells: 0.65 ms for the four
+// coverings of the 263-zone sweep; this 0.25.)
+constexpr uint32_t SUB_MAX = 3;
+__global__ __launch_bounds__(256) void table_sub_kernel(
+    const uint64_t* __restrict__ start, const uint32_t* __restrict__ pay,
+    const uint2* __restrict__ win, const uint32_t* __restrict__ mpos,
+    const uint32_t* __restrict__ mid, uint32_t M, uint32_t shift, uint32_t s2,
+    uint32_t* __restrict__ sub, uint2* __restrict__ cand, uint32_t* __restrict__ mcount) {
+  // place of the j-th sub-cell along the curve, by orientation
+  __shared__ uint8_t s_place[4 << (2 * SUB_MAX)];
+  const uint32_t per = 1u << (2 * s2);
+  for (uint32_t i = threadIdx.x; i < 4 * per; i += blockDim.x) {
+    const uint32_t o = i >> (2 * s2), j = i & (per - 1);
+    uint32_t sw = o >> 1, cm = o & 1u, x = 0, y = 0;
+    for (int lev = (int)s2 - 1; lev >= 0; --lev) {
+      const uint32_t d = (j >> (2 * lev)) & 3u;
+      const uint32_t xt = d >> 1, yt = xt ^ (d & 1u);
+      const uint32_t u = xt ^ cm, v = yt ^ cm;
+      x = (x << 1) | (sw ? v : u);
+      y = (y << 1) | (sw ? u : v);
+      if (!yt) {
+        sw ^= 1u;
+        cm ^= xt;
+      }
+    }
+    s_place[i] = (uint8_t)((y << s2) | x);
+  }
+  __syncthreads();
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t sh2 = shift - 2 * s2;
+  for (uint32_t m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; m < M;
+       m += (gridDim.x * blockDim.x) >> 5) {
     const uint2 w = win[m];
-    const uint32_t r0 = last_le_in(start, w.x, w.y, lo), r1 = last_le_in(start, r0, w.y, hi);
-    if (!write) {
-      flag[t] = r0 != r1 ? 1u : 0u;
-      if (r0 == r1) sub[t] = pay[r0];
-    } else {
-      const uint32_t m2 = rank2[t];
-      sub[t] = TAB_MIXED | m2;
-      win2[m2] = make_uint2(r0, r1);
+    const uint32_t o = mpos[m] >> 26;
+    const uint64_t lo = (uint64_t)mid[m] << shift;
+    uint32_t n = 0;
+    for (uint32_t j0 = 0; j0 < per; j0 += 32) {
+      const uint32_t j = j0 + lane;
+      // first range of sub-cell j (the bucket's own at j = 0)
+      const uint32_t r0 =
+          j < per ? last_le_in(start, w.x, w.y, lo + ((uint64_t)j << sh2)) : w.y;
+      uint32_t rn = __shfl_down_sync(0xffffffffu, r0, 1);
+      if (lane == 31 && j + 1 < per) rn = last_le_in(start, r0, w.y, lo + ((uint64_t)(j + 1) << sh2));
+      uint32_t r1 = w.y;
+      if (j + 1 < per) r1 = rn - (start[rn] == lo + ((uint64_t)(j + 1) << sh2) ? 1u : 0u);
+      const bool on = j < per, mix = on && r0 != r1;
+      const uint32_t bal = __ballot_sync(0xffffffffu, mix);
+      const uint32_t rank = n + __popc(bal & ((1u << lane) - 1u));
+      if (on) sub[(uint64_t)m * per + s_place[o * per + j]] = mix ? TAB_MIXED | rank : pay[r0];
+      if (mix) cand[(uint64_t)m * per + rank] = make_uint2(r0, r1);
+      n += __popc(bal);
+    }
+    if (lane == 0) mcount[m] = n;
+  }
+}
+
+__global__ __launch_bounds__(256) void table_sub_rank_kernel(
+    const uint32_t* __restrict__ moff, const uint32_t* __restrict__ mcount, uint32_t M,
+    uint32_t s2, const uint2* __restrict__ cand, uint32_t* __restrict__ sub,
+    uint2* __restrict__ win2) {
+  const uint32_t lane = threadIdx.x & 31, per = 1u << (2 * s2);
+  for (uint32_t m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; m < M;
+       m += (gridDim.x * blockDim.x) >> 5) {
+    const uint32_t off = moff[m], n = mcount[m];
+    const uint64_t base = (uint64_t)m * per;
+    for (uint32_t i = lane; i < n; i += 32) win2[off + i] = cand[base + i];
+    for (uint32_t j = lane; j < per; j += 32) {
+      const uint32_t e = sub[base + j];
+      if (e >= TAB_MIXED && e != 0xFFFFFFFFu) sub[base + j] = e + off;
     }
   }
 }
@@ -277,7 +338,11 @@ __global__ void table_top_kernel(const uint32_t* __restrict__ tab, uint32_t L0, 
 __global__ void top_count_kernel(const uint32_t* __restrict__ word, uint32_t nt,
                                  uint32_t* __restrict__ count) {
   const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < nt && word[c] < TOP_WORD_ASK) atomicAdd(&count[word[c]], 1u);
+  const uint32_t v = c < nt ? word[c] : TOP_WORD_ASK;
+  // neighbouring cells mostly hold the same polygon: one atomic per polygon and warp
+  const uint32_t peers = __match_any_sync(0xffffffffu, v);
+  if (v < TOP_WORD_ASK && (threadIdx.x & 31) == __ffs(peers) - 1)
+    atomicAdd(&count[v], (uint32_t)__popc(peers));
 }
 
 // the byte of each cell: its payload's palette index (map), or TOP_NONE / TOP_ASK
@@ -320,13 +385,13 @@ sdb_status build_cell_table(sdb_covering* cov, uint32_t table_bits, cudaStream_t
   cov->sub_bits = 0;
   cov->sub_mixed = 0;
   Scratch sc(s);
-  uint32_t *mixed, *rank, *dtot, *mark, *tpre;
+  uint32_t *dtot, *mark, *tpre, *tcount, *toff;
   const uint64_t nt = (nb + TT - 1) / TT;
   SDB_TRY(dalloc_n(&cov->tab, nb, s));
-  SDB_TRY(sc.get(&mixed, nb));
-  SDB_TRY(sc.get(&rank, nb));
   SDB_TRY(sc.get(&mark, nb));
   SDB_TRY(sc.get(&tpre, nt));
+  SDB_TRY(sc.get(&tcount, nt));
+  SDB_TRY(sc.get(&toff, nt));
   SDB_TRY(sc.get(&dtot, 1));
   SDB_TRY_CUDA(cudaMemsetAsync(mark, 0, nb * 4, s));
   table_marks_kernel<<<grid_for(cov->R, 256), 256, 0, s>>>(cov->start, cov->R, shift, nb, mark);
@@ -339,11 +404,10 @@ sdb_status build_cell_table(sdb_covering* cov, uint32_t table_bits, cudaStream_t
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
   table_fill_kernel<<<(unsigned)nt, TB, 0, s>>>(mark, tpre, nb, cov->start, cov->pay, shift, T / 2,
-                                                cov->tab, mixed);
+                                                cov->tab, tcount);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
-  const unsigned grid = grid_for(nb, 256);
-  SDB_TRY(exclusive_scan<uint32_t>(mixed, rank, nb, dtot, s));
+  SDB_TRY(exclusive_scan<uint32_t>(tcount, toff, nt, dtot, s));
   uint32_t M = 0;
   SDB_TRY_CUDA(cudaMemcpyAsync(&M, dtot, 4, cudaMemcpyDeviceToHost, s));
   SDB_TRY_CUDA(cudaStreamSynchronize(s));
@@ -354,33 +418,35 @@ sdb_status build_cell_table(sdb_covering* cov, uint32_t table_bits, cudaStream_t
   while (s2 > 0 && (uint64_t)M << (2 * s2) >= (uint64_t)TAB_MIXED_MAX) --s2;
   uint64_t M2 = 0;
   if (M > 0) {
-    uint32_t* mpos;
+    uint32_t *mpos, *mid;
     SDB_TRY(sc.get(&mpos, M));
+    SDB_TRY(sc.get(&mid, M));
     SDB_TRY(dalloc_n(&cov->win, M, s));
-    table_mixed_kernel<<<grid, 256, 0, s>>>(cov->start, cov->R, shift, L0, nb, mixed, rank,
-                                            cov->tab, cov->win, mpos);
+    table_mixed_kernel<<<(unsigned)nt, TB, 0, s>>>(cov->start, cov->R, shift, L0, nb, mark, toff,
+                                                   cov->tab, cov->win, mpos, mid);
     note_launch();
     SDB_TRY_CUDA(cudaGetLastError());
     if (s2 > 0) {
-      const uint64_t ns = M << (2 * s2);
-      uint32_t *flag2, *rank2;
+      const uint64_t ns = (uint64_t)M << (2 * s2);
+      uint32_t *mcount, *moff;
+      uint2* cand;
       SDB_TRY(dalloc_n(&cov->sub, ns, s));
-      SDB_TRY(sc.get(&flag2, ns));
-      SDB_TRY(sc.get(&rank2, ns));
-      const unsigned g2 = grid_for(ns, 256);
-      table_sub_kernel<<<g2, 256, 0, s>>>(cov->start, cov->pay, cov->win, mpos, M, L0, s2,
-                                          cov->F, cov->sub, flag2, nullptr, nullptr, false);
+      SDB_TRY(sc.get(&cand, ns));
+      SDB_TRY(sc.get(&mcount, M));
+      SDB_TRY(sc.get(&moff, M));
+      const unsigned g2 = std::min<unsigned>(grid_for((size_t)M * 32, 256), num_sms() * 32);
+      table_sub_kernel<<<g2, 256, 0, s>>>(cov->start, cov->pay, cov->win, mpos, mid, M, shift, s2,
+                                          cov->sub, cand, mcount);
       note_launch();
       SDB_TRY_CUDA(cudaGetLastError());
-      SDB_TRY(exclusive_scan<uint32_t>(flag2, rank2, ns, dtot, s));
+      SDB_TRY(exclusive_scan<uint32_t>(mcount, moff, M, dtot, s));
       uint32_t m2 = 0;
       SDB_TRY_CUDA(cudaMemcpyAsync(&m2, dtot, 4, cudaMemcpyDeviceToHost, s));
       SDB_TRY_CUDA(cudaStreamSynchronize(s));
       M2 = m2;
       if (M2 > 0) {
         SDB_TRY(dalloc_n(&cov->win2, M2, s));
-        table_sub_kernel<<<g2, 256, 0, s>>>(cov->start, cov->pay, cov->win, mpos, M, L0, s2,
-                                            cov->F, cov->sub, flag2, rank2, cov->win2, true);
+        table_sub_rank_kernel<<<g2, 256, 0, s>>>(moff, mcount, M, s2, cand, cov->sub, cov->win2);
         note_launch();
         SDB_TRY_CUDA(cudaGetLastError());
       }
