@@ -356,7 +356,6 @@ struct BatchCore {
   BatchTile* tiles = nullptr;
   uint64_t ntiles = 0;
   std::vector<uint64_t> qtile;  // host, Q + 1: tiles of query q
-  unsigned long long* heads = nullptr;  // Q + 1 work counters
   void release(cudaStream_t s);
 };
 // viewport, level and output slot of one query (sbase/R/chunk left to the caller)
