@@ -788,7 +788,10 @@ sdb_status batch_core_run(BatchCore* c, int mode, uint64_t* count, int64_t* sum,
 // Coverings of queries [q0, q0 + nq) of a pair list, built in chunks that are
 // halved and retried when they overflow the builder's 32-bit ranges or memory.
 // Appends CoverSets to *sets and fills sbase/R/chunk of hq.
-sdb_status build_query_coverings(const PolyEdges& pe, uint32_t B,
+// Only the polygons that some pair of a chunk names go to the builder (and the
+// device): a batch of views meets a few hundred of the 40,000 tracts, and uploading
+// all of their 900k vertices per batch took as long as building the coverings.
+sdb_status build_query_coverings(const PolySet& polys, uint32_t B,
                                  const std::vector<CoverQuery>& cq,
                                  const std::vector<uint32_t>& pp, const std::vector<uint32_t>& pq,
                                  const std::vector<uint32_t>& ps, std::vector<BatchQueryDev>& hq,
@@ -802,7 +805,7 @@ sdb_status build_query_coverings(const PolyEdges& pe, uint32_t B,
     pfirst[q] = i;
   }
   uint32_t chunk_q = 512;
-  std::vector<uint32_t> pq_local;
+  std::vector<uint32_t> pq_local, pp_local, cx, cy, local(polys.P, NONE);
   for (uint32_t q0 = 0; q0 < Q;) {
     // queries of a chunk share 64-bit keys: query bits above 2 * (finest level)
     uint32_t nq = std::min(chunk_q, Q - q0);
@@ -816,12 +819,34 @@ sdb_status build_query_coverings(const PolyEdges& pe, uint32_t B,
     const uint64_t pa = pfirst[q0], pb = pfirst[q0 + nq];
     pq_local.assign(pq.begin() + pa, pq.begin() + pb);
     for (auto& v : pq_local) v -= q0;
+    PolyEdges pe;
+    pe.edge_off.push_back(0);
+    pp_local.resize(pb - pa);
+    cx.clear();
+    cy.clear();
+    for (uint64_t i = pa; i < pb; ++i) {
+      const uint32_t j = pp[i], v0 = polys.off[j], v1 = polys.off[j + 1];
+      if (local[j] == NONE) {
+        local[j] = pe.P++;
+        const uint32_t at = (uint32_t)cx.size();
+        cx.insert(cx.end(), polys.x + v0, polys.x + v1);
+        cy.insert(cy.end(), polys.y + v0, polys.y + v1);
+        for (uint32_t v = v0; v < v1; ++v)
+          pe.next.push_back(at + (polys.next ? polys.next[v] - v0 : v + 1 < v1 ? v + 1 - v0 : 0));
+        pe.edge_off.push_back((uint32_t)cx.size());
+      }
+      pp_local[i - pa] = local[j];
+    }
+    for (uint64_t i = pa; i < pb; ++i) local[pp[i]] = NONE;
+    pe.V = (uint32_t)cx.size();
+    pe.x = cx.data();
+    pe.y = cy.data();
     CoverSpec spec;
     spec.B = B;
     spec.Q = nq;
     spec.q = cq.data() + q0;
     spec.NP = (uint32_t)(pb - pa);
-    spec.pair_poly = pp.data() + pa;
+    spec.pair_poly = pp_local.data();
     spec.pair_query = pq_local.data();
     spec.pair_slot = ps.data() + pa;
     CoverSet set;
@@ -882,15 +907,18 @@ sdb_status polygon_bboxes(const sdb_polygons* polys, uint32_t B, std::vector<uin
       return SDB_EINVAL;
     }
     uint32_t mnx = ~0u, mny = ~0u, mxx = 0, mxy = 0;
-    for (uint32_t v = polys->ring_off[j]; v < polys->ring_off[j + 1]; ++v) {
-      if (polys->x[v] >= G || polys->y[v] >= G) {
-        set_error("vertex %u outside the grid", v);
-        return SDB_EINVAL;
-      }
+    const uint32_t v0 = polys->ring_off[j], v1 = polys->ring_off[j + 1];
+    for (uint32_t v = v0; v < v1; ++v) {
       mnx = std::min(mnx, polys->x[v]);
       mxx = std::max(mxx, polys->x[v]);
       mny = std::min(mny, polys->y[v]);
       mxy = std::max(mxy, polys->y[v]);
+    }
+    if (mxx >= G || mxy >= G) {
+      uint32_t v = v0;
+      while (polys->x[v] < G && polys->y[v] < G) ++v;
+      set_error("vertex %u outside the grid", v);
+      return SDB_EINVAL;
     }
     (*bb)[4 * j] = mnx;
     (*bb)[4 * j + 1] = mny;
@@ -1067,7 +1095,7 @@ sdb_status sdb_batch_create(const sdb_points* pts, const sdb_polygons* polys,
   b->core.pts = pts;
   b->core.Q = n_queries;
   b->core.out_len = out_off;
-  sdb_status st = build_query_coverings(poly_edges(polys), B, cq, pp, pq, ps, hq, &b->cs, 0, s,
+  sdb_status st = build_query_coverings(PolySet{P, polys->ring_off, polys->x, polys->y, nullptr}, B, cq, pp, pq, ps, hq, &b->cs, 0, s,
                                         &b->n_ranges, &b->n_cells, &b->max_ranges);
   if (st == SDB_OK) {
     b->core.hq = hq;

@@ -88,10 +88,12 @@ __device__ __forceinline__ uint32_t pert_ray_cross(const Edge& e, int64_t qx, in
 }
 
 // Offsets for N per-thread counts, with one atomic per counter and block
-// (blockDim.x == 256): warp scans, then warp prefixes in shared memory.  Every
-// thread of the block must call it.
+// (blockDim.x == 256): warp scans, then warp prefixes in shared memory.  The first
+// two counters are the next level's (its cells and edge entries), the others the
+// build's.  Every thread of the block must call it.
 template <int N>
 __device__ __forceinline__ void block_alloc(const uint32_t (&n)[N],
+                                            unsigned long long* __restrict__ next,
                                             unsigned long long* __restrict__ ctr,
                                             unsigned long long (&off)[N]) {
   __shared__ uint32_t wsum[N][8];
@@ -121,7 +123,7 @@ __device__ __forceinline__ void block_alloc(const uint32_t (&n)[N],
       wsum[j][k] = t;
       t += v;
     }
-    base[j] = t ? atomicAdd(&ctr[j], (unsigned long long)t) : 0ull;
+    base[j] = t ? atomicAdd(j < 2 ? next + j : ctr + (j - 2), (unsigned long long)t) : 0ull;
   }
   __syncthreads();
 #pragma unroll
@@ -133,7 +135,6 @@ __device__ __forceinline__ void block_alloc(const uint32_t (&n)[N],
 struct TileOut {
   Item* items;
   uint32_t* elist;
-  unsigned long long item_base, edge_base;  // filled by earlier levels
 };
 
 __global__ void build_edges_kernel(const uint32_t* __restrict__ vx, const uint32_t* __restrict__ vy,
@@ -209,7 +210,8 @@ __global__ void root_items_kernel(const uint32_t* __restrict__ edge_off,
                                   const CoverQuery* __restrict__ qs, uint32_t NP, uint32_t qshift,
                                   uint32_t bflag, bool noncons, uint32_t B, Item* __restrict__ items,
                                   uint64_t* __restrict__ rec_key, uint32_t* __restrict__ rec_val,
-                                  uint32_t sb, unsigned long long* __restrict__ counters) {
+                                  uint32_t sb, unsigned long long* __restrict__ next_counters,
+                                  unsigned long long* __restrict__ counters) {
   uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
   if (p >= NP) return;
@@ -229,7 +231,7 @@ __global__ void root_items_kernel(const uint32_t* __restrict__ edge_off,
       if (!keep) return;
     }
     if (lane == 0) {
-      unsigned long long r = atomicAdd(&counters[2], 1ull);
+      unsigned long long r = atomicAdd(&counters[0], 1ull);
       // the whole grid as one boundary cell
       put_record(rec_key, rec_val, r, qshift >= 64 ? 0ull : ((uint64_t)qi << qshift),
                  pair_slot[p] | bflag, sb);
@@ -241,7 +243,7 @@ __global__ void root_items_kernel(const uint32_t* __restrict__ edge_off,
   for (uint32_t v = a + lane; v < b; v += 32) par ^= pert_ray_cross(edges[v], 0, 0);
   par = __popc(__ballot_sync(FULL, par)) & 1u;
   if (lane == 0) {
-    unsigned long long i = atomicAdd(&counters[0], 1ull);
+    unsigned long long i = atomicAdd(&next_counters[0], 1ull);
     items[i] = Item{0ull, p, 0, 0, a, (b - a) | (par << 31), 0u};
   }
 }
@@ -318,15 +320,19 @@ __device__ __forceinline__ uint32_t edge_vs_children(const Edge& e, int32_t px, 
 // boundary children of that level going to the tile list (covertiles.cu).
 template <int G, bool NC, bool TILES>
 __global__ __launch_bounds__(256) void expand_level_kernel(
-    const Item* __restrict__ items, uint32_t n_items, const uint32_t* __restrict__ elist,
+    const Item* __restrict__ items, const unsigned long long* __restrict__ n_items,
+    const uint32_t* __restrict__ elist,
     const Edge* __restrict__ edges, const uint32_t* __restrict__ pair_query,
     const uint32_t* __restrict__ pair_slot, const CoverQuery* __restrict__ qs, uint32_t qshift,
     uint32_t bflag, uint32_t B, uint32_t L, Item* __restrict__ next_items,
     uint32_t* __restrict__ next_elist,
     uint64_t* __restrict__ rec_key, uint32_t* __restrict__ rec_val, uint32_t sb,
-    unsigned long long rec_base, TileOut tiles, unsigned long long* __restrict__ counters) {
+    TileOut tiles, unsigned long long* __restrict__ next_counters,
+    unsigned long long* __restrict__ counters) {
   const uint64_t gt = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool active = gt / G < n_items;
+  // the level's size as the level before left it (the grid covers a bound of it)
+  const bool active = gt / G < *n_items;
+  if ((uint64_t)blockIdx.x * blockDim.x / G >= *n_items) return;  // whole blocks
   const uint32_t t = (uint32_t)(gt / G);  // item of this lane's group
   const uint32_t gl = (uint32_t)(gt % G); // lane within the group
   const uint32_t lane = threadIdx.x & 31;
@@ -404,16 +410,15 @@ __global__ __launch_bounds__(256) void expand_level_kernel(
       }
     }
   }
-  // counters: 0 child items, 1 child edge entries, 2 records, 3 and 4 tile items
-  // and their edge entries
+  // child items and their edge entries; records; tile items and their edge entries
   unsigned long long io, eo, ro;
   if constexpr (TILES) {
     const bool fin = cl + TILE_DEPTH == F;
     unsigned long long off[5];
     block_alloc<5>({fin ? 0u : n_it, fin ? 0u : n_ed, n_rec, fin ? n_it : 0u, fin ? n_ed : 0u},
-                   counters, off);
-    io = fin ? off[3] + tiles.item_base : off[0];
-    eo = fin ? off[4] + tiles.edge_base : off[1];
+                   next_counters, counters, off);
+    io = fin ? off[3] : off[0];
+    eo = fin ? off[4] : off[1];
     ro = off[2];
     if (fin) {
       next_items = tiles.items;
@@ -421,7 +426,7 @@ __global__ __launch_bounds__(256) void expand_level_kernel(
     }
   } else {
     unsigned long long off[3];
-    block_alloc<3>({n_it, n_ed, n_rec}, counters, off);
+    block_alloc<3>({n_it, n_ed, n_rec}, next_counters, counters, off);
     io = off[0];
     eo = off[1];
     ro = off[2];
@@ -457,7 +462,7 @@ __global__ __launch_bounds__(256) void expand_level_kernel(
     bool emit = (cnt[c] > 0) ? (!TILES && cl == F) : (inside != 0);
     if (emit) {
       if (gl == 0) {
-        put_record(rec_key, rec_val, rec_base + ro++, qbits | (chid << shift),
+        put_record(rec_key, rec_val, ro++, qbits | (chid << shift),
                    slot | ((F - cl) << 26) | (cnt[c] > 0 ? bflag : 0u), sb);
       }
       cnt[c] = 0;  // a finest boundary cell needs no edge list
@@ -1210,19 +1215,20 @@ void CoverSet::release(cudaStream_t s) {
   pay = nullptr;
 }
 
-static sdb_status launch_expand(uint32_t G, const Item* items, uint32_t n_items, const uint32_t* elist,
+static sdb_status launch_expand(uint32_t G, const Item* items, uint64_t most,
+                         const unsigned long long* n_items, const uint32_t* elist,
                          const Edge* edges, const uint32_t* pq, const uint32_t* ps,
                          const CoverQuery* qs, uint32_t qshift, uint32_t bflag, bool noncons,
                          uint32_t B, uint32_t L,
                          Item* nitems, uint32_t* nel, uint64_t* rkey, uint32_t* rval, uint32_t sb,
-                         unsigned long long rec_base, const TileOut* tiles,
+                         const TileOut* tiles, unsigned long long* next_ctr,
                          unsigned long long* ctr, cudaStream_t s) {
-  const size_t threads = (size_t)n_items * G;
+  const size_t threads = (size_t)most * G;
   const TileOut to = tiles ? *tiles : TileOut{};
 #define SDB_EXPAND_AS(g, nc, tl)                                                               \
   expand_level_kernel<g, nc, tl><<<grid_for(threads, 256), 256, 0, s>>>(                       \
       items, n_items, elist, edges, pq, ps, qs, qshift, bflag, B, L, nitems, nel, rkey, rval,  \
-      sb, rec_base, to, ctr)
+      sb, to, next_ctr, ctr)
 #define SDB_EXPAND(g)                  \
   case g:                              \
     if (tiles)                         \
@@ -1419,9 +1425,11 @@ static sdb_status build_pass(const PolyEdges& pe, const CoverSpec& spec, bool ti
   SDB_TRY(sc.get(&d_ps, NP));
   SDB_TRY(sc.get(&d_qs, Q));
   SDB_TRY_CUDA(cudaMemcpyAsync(d_off, pe.edge_off.data(), (P + 1) * 4ull, cudaMemcpyHostToDevice, s));
-  SDB_TRY_CUDA(cudaMemcpyAsync(d_x, pe.x, V * 4ull, cudaMemcpyHostToDevice, s));
-  SDB_TRY_CUDA(cudaMemcpyAsync(d_y, pe.y, V * 4ull, cudaMemcpyHostToDevice, s));
-  SDB_TRY_CUDA(cudaMemcpyAsync(d_vp, pe.next.data(), V * 4ull, cudaMemcpyHostToDevice, s));
+  if (V) {
+    SDB_TRY_CUDA(cudaMemcpyAsync(d_x, pe.x, V * 4ull, cudaMemcpyHostToDevice, s));
+    SDB_TRY_CUDA(cudaMemcpyAsync(d_y, pe.y, V * 4ull, cudaMemcpyHostToDevice, s));
+    SDB_TRY_CUDA(cudaMemcpyAsync(d_vp, pe.next.data(), V * 4ull, cudaMemcpyHostToDevice, s));
+  }
   if (NP) {
     SDB_TRY_CUDA(cudaMemcpyAsync(d_pp, spec.pair_poly, NP * 4ull, cudaMemcpyHostToDevice, s));
     SDB_TRY_CUDA(cudaMemcpyAsync(d_pq, spec.pair_query, NP * 4ull, cudaMemcpyHostToDevice, s));
@@ -1461,9 +1469,14 @@ static sdb_status build_pass(const PolyEdges& pe, const CoverSpec& spec, bool ti
 
   const uint32_t bflag = spec.flags ? VAL_FLAG : 0u;  // boundary records' flag
   unsigned long long* ctr;
-  constexpr int NCTR = 5;
-  SDB_TRY(sc.get(&ctr, NCTR));
-  SDB_TRY_CUDA(cudaMemsetAsync(ctr, 0, NCTR * sizeof(unsigned long long), s));
+  // counters: records, tiles, tile edge entries, then per level its cells and
+  // edge entries (level 0: the roots)
+  constexpr uint32_t NG = 3;
+  const uint32_t nctr = NG + 2 * (Fmax + 1);
+  std::vector<unsigned long long> h(nctr, 0);
+  SDB_TRY(sc.get(&ctr, nctr));
+  SDB_TRY_CUDA(cudaMemsetAsync(ctr, 0, nctr * sizeof(unsigned long long), s));
+  auto level_ctr = [&](uint32_t L) { return ctr + NG + 2 * L; };
   // frontier cells and edge lists, two buffers each (this level's, the next's)
   struct Frontier {
     Item* f[2] = {nullptr, nullptr};
@@ -1494,7 +1507,7 @@ static sdb_status build_pass(const PolyEdges& pe, const CoverSpec& spec, bool ti
   if (NP) {
     root_items_kernel<<<grid_for((size_t)NP * 32, 256), 256, 0, s>>>(
         d_off, edges, d_pp, d_pq, d_ps, d_qs, NP, qshift, bflag, spec.noncons, B, items, rkey, rval,
-        sb, ctr);
+        sb, level_ctr(0), ctr);
     note_launch();
     SDB_TRY_CUDA(cudaGetLastError());
   }
@@ -1510,110 +1523,126 @@ static sdb_status build_pass(const PolyEdges& pe, const CoverSpec& spec, bool ti
     }
   } tl;
   tl.s = s;
-  unsigned long long h0[3];
-  SDB_TRY(read_u64(ctr, h0, 3, s));
-  uint64_t n_items = h0[0], n_edges = 0;
-  n_rec = h0[2];
-  for (uint32_t i = 0; i < NP; ++i)
-    if (spec.q[spec.pair_query[i]].F > 0)
-      n_edges += pe.edge_off[spec.pair_poly[i] + 1] - pe.edge_off[spec.pair_poly[i]];
+  // the roots by query (one per pair, or a record where the finest level is 0)
+  uint64_t n_items = 0, n_edges = 0;
+  for (uint32_t i = 0; i < NP; ++i) {
+    if (spec.q[spec.pair_query[i]].F == 0) continue;
+    ++n_items;
+    n_edges += pe.edge_off[spec.pair_poly[i] + 1] - pe.edge_off[spec.pair_poly[i]];
+  }
+  n_rec = NP - n_items;  // at most
+  bool counted = false;  // n_rec is the device's count
   uint32_t* cur_el = elist;
   tr_up.end();
   TraceScope tr_lv("cover.levels", s);
   const uint32_t Lend = tiles ? Fmax - TILE_DEPTH : Fmax;  // levels to expand
-  for (uint32_t L = 0; L < Lend && n_items > 0; ++L) {
-    const bool last = (L + 1 == Lend);
-    // capacity: every record and every child item comes from one of 4
-    // children; every child edge entry from one (edge, child) pair
-    if (n_rec + 4 * n_items > rec_cap) {
-      uint64_t nc = rec_cap;
-      while (nc < n_rec + 4 * n_items) nc *= 2;
-      uint64_t* k2 = nullptr;
-      uint32_t* v2 = nullptr;
-      SDB_TRY(dalloc_n(&k2, nc, s));
-      SDB_TRY_CUDA(cudaMemcpyAsync(k2, rkey, n_rec * 8, cudaMemcpyDeviceToDevice, s));
-      dfree(rkey, s);
-      rkey = k2;
-      if (!sb) {
-        SDB_TRY(dalloc_n(&v2, nc, s));
-        SDB_TRY_CUDA(cudaMemcpyAsync(v2, rval, n_rec * 4, cudaMemcpyDeviceToDevice, s));
-        dfree(rval, s);
-        rval = v2;
-      }
-      rec_cap = nc;
-    }
-    if (4 * n_items > 0xffffffffull || 4 * n_edges > 0xffffffffull) {
-      set_error("covering: level %u frontier too large (%llu cells, %llu edge entries)", L,
-                (unsigned long long)n_items, (unsigned long long)n_edges);
-      return SDB_ENOMEM;
-    }
-    Item* nitems = nullptr;
-    uint32_t* nel = nullptr;
-    if (!last) {
-      // the other buffer of each pair, grown (contents are dead) when short
-      sdb_status st = SDB_OK;
-      if (fcap[1] < 4 * n_items) {
-        dfree(fbuf[1], s);
-        fbuf[1] = nullptr;
-        fcap[1] = pow2_at_least(4 * n_items);
-        st = dalloc_n(&fbuf[1], fcap[1], s);
-      }
-      if (st == SDB_OK && ecap[1] < 4 * n_edges) {
-        if (fr.own_e[1]) dfree(ebuf[1], s);
-        ebuf[1] = nullptr;
-        fr.own_e[1] = true;
-        ecap[1] = pow2_at_least(4 * n_edges);
-        st = dalloc_n(&ebuf[1], ecap[1], s);
-      }
-      if (st != SDB_OK) return st;
-      nitems = fbuf[1];
-      nel = ebuf[1];
-    }
-    TileOut tile_out{};
-    if (tiles) {
-      bool ends = false;  // a query's tiles come from this level
-      for (uint32_t q = 0; q < Q && !ends; ++q) ends = spec.q[q].F == L + 1 + TILE_DEPTH;
-      if (ends) {
-        SDB_TRY(grow(&tl.items, tl.n, tl.n + 4 * n_items, hint.tiles, &tl.cap, s));
-        SDB_TRY(grow(&tl.elist, tl.ne, tl.ne + 4 * n_edges, hint.tile_edges, &tl.ecap, s));
-      }
-      tile_out = TileOut{tl.items, tl.elist, tl.n, tl.ne};
-    }
-    SDB_TRY_CUDA(cudaMemsetAsync(ctr, 0, NCTR * sizeof(unsigned long long), s));
+  // A level's size is known on the device when the level before has run.  The host
+  // waits for it only every few levels: a cell has at most 4 children and an edge
+  // list entry at most 4 copies, so while that bound is small the buffers are made
+  // for it and the next levels are launched over it.
+  constexpr uint64_t CHAIN_ITEMS = 1ull << 17, CHAIN_EDGES = 1ull << 22;
+  for (uint32_t L = 0; L < Lend && n_items > 0;) {
+    uint64_t bi = n_items, be = n_edges;  // bounds of the level in hand
     // lanes per item: about the level's mean edge count, a power of two <= 32
     const uint64_t mean = (n_edges + n_items - 1) / n_items;
     uint32_t G = 1;
     if (mean >= 4)
       while (G < 32 && G < mean) G <<= 1;
-    {
-      TraceScope tr("cover.expand", s);
-      SDB_TRY(launch_expand(G, items, (uint32_t)n_items, cur_el, edges, d_pq, d_ps, d_qs, qshift,
-                            bflag, spec.noncons, B, L, nitems, nel, rkey, rval, sb, n_rec,
-                            tiles ? &tile_out : nullptr, ctr, s));
-      SDB_TRY_CUDA(cudaGetLastError());
-    }
-    unsigned long long h[NCTR];
-    SDB_TRY(read_u64(ctr, h, NCTR, s));
-    // the next level reads what this one wrote
-    std::swap(fbuf[0], fbuf[1]);
-    std::swap(fcap[0], fcap[1]);
-    std::swap(ebuf[0], ebuf[1]);
-    std::swap(ecap[0], ecap[1]);
-    std::swap(fr.own_e[0], fr.own_e[1]);
-    items = fbuf[0];
-    cur_el = ebuf[0];
-    n_items = last ? 0 : h[0];
-    n_edges = h[1];
-    n_rec += h[2];
-    tl.n += h[3];
-    tl.ne += h[4];
+    const uint32_t L0 = L;
+    do {
+      const bool last = (L + 1 == Lend);
+      // capacity: every record and every child item comes from one of 4
+      // children; every child edge entry from one (edge, child) pair
+      if (n_rec + 4 * bi > rec_cap) {
+        const uint64_t keep = n_rec;
+        uint64_t nc = rec_cap;
+        while (nc < n_rec + 4 * bi) nc *= 2;
+        uint64_t cap = rec_cap;
+        SDB_TRY(grow(&rkey, keep < rec_cap ? keep : rec_cap, nc, 1, &cap, s));
+        if (!sb) {
+          cap = rec_cap;
+          SDB_TRY(grow(&rval, keep < rec_cap ? keep : rec_cap, nc, 1, &cap, s));
+        }
+        rec_cap = nc;
+      }
+      if (4 * bi > 0xffffffffull || 4 * be > 0xffffffffull) {
+        set_error("covering: level %u frontier too large (%llu cells, %llu edge entries)", L,
+                  (unsigned long long)bi, (unsigned long long)be);
+        return SDB_ENOMEM;
+      }
+      Item* nitems = nullptr;
+      uint32_t* nel = nullptr;
+      if (!last) {
+        // the other buffer of each pair, grown (contents are dead) when short
+        sdb_status st = SDB_OK;
+        if (fcap[1] < 4 * bi) {
+          dfree(fbuf[1], s);
+          fbuf[1] = nullptr;
+          fcap[1] = pow2_at_least(4 * bi);
+          st = dalloc_n(&fbuf[1], fcap[1], s);
+        }
+        if (st == SDB_OK && ecap[1] < 4 * be) {
+          if (fr.own_e[1]) dfree(ebuf[1], s);
+          ebuf[1] = nullptr;
+          fr.own_e[1] = true;
+          ecap[1] = pow2_at_least(4 * be);
+          st = dalloc_n(&ebuf[1], ecap[1], s);
+        }
+        if (st != SDB_OK) return st;
+        nitems = fbuf[1];
+        nel = ebuf[1];
+      }
+      TileOut tile_out{};
+      if (tiles) {
+        bool ends = false;  // a query's tiles come from this level
+        for (uint32_t q = 0; q < Q && !ends; ++q) ends = spec.q[q].F == L + 1 + TILE_DEPTH;
+        if (ends) {
+          SDB_TRY(grow(&tl.items, tl.n, tl.n + 4 * bi, hint.tiles, &tl.cap, s));
+          SDB_TRY(grow(&tl.elist, tl.ne, tl.ne + 4 * be, hint.tile_edges, &tl.ecap, s));
+          tl.n += 4 * bi;  // at most, until the counters are read
+          tl.ne += 4 * be;
+        }
+        tile_out = TileOut{tl.items, tl.elist};
+      }
+      {
+        TraceScope tr("cover.expand", s);
+        SDB_TRY(launch_expand(G, items, bi, level_ctr(L), cur_el, edges, d_pq, d_ps, d_qs, qshift,
+                              bflag, spec.noncons, B, L, nitems, nel, rkey, rval, sb,
+                              tiles ? &tile_out : nullptr, level_ctr(L + 1), ctr, s));
+      }
+      n_rec += 4 * bi;
+      // the next level reads what this one writes
+      std::swap(fbuf[0], fbuf[1]);
+      std::swap(fcap[0], fcap[1]);
+      std::swap(ebuf[0], ebuf[1]);
+      std::swap(ecap[0], ecap[1]);
+      std::swap(fr.own_e[0], fr.own_e[1]);
+      items = fbuf[0];
+      cur_el = ebuf[0];
+      bi *= 4;
+      be *= 4;
+      ++L;
+    } while (L < Lend && bi <= CHAIN_ITEMS && be <= CHAIN_EDGES);
+    SDB_TRY(read_u64(ctr, h.data(), (int)nctr, s));
+    counted = true;
+    n_rec = h[0];
+    tl.n = h[1];
+    tl.ne = h[2];
     if (tl.n > 0xffffffffull || tl.ne > 0xffffffffull) {
       set_error("covering: %llu tiles, %llu edge entries exceed the 32-bit index range",
                 (unsigned long long)tl.n, (unsigned long long)tl.ne);
       return SDB_ENOMEM;
     }
-    seen.items = std::max<uint64_t>(seen.items, pow2_at_least(4 * n_items));
-    seen.edges = std::max<uint64_t>(seen.edges, pow2_at_least(4 * n_edges));
+    for (uint32_t l = L0 + 1; l <= L && l < Lend; ++l) {
+      seen.items = std::max<uint64_t>(seen.items, pow2_at_least(4 * h[NG + 2 * l]));
+      seen.edges = std::max<uint64_t>(seen.edges, pow2_at_least(4 * h[NG + 2 * l + 1]));
+    }
+    n_items = L < Lend ? h[NG + 2 * L] : 0;
+    n_edges = h[NG + 2 * L + 1];
+  }
+  if (!counted && NP) {  // only records of whole grids
+    SDB_TRY(read_u64(ctr, h.data(), 1, s));
+    n_rec = h[0];
   }
   tr_lv.end();
   seen.rec = std::max<uint64_t>(pow2_at_least(n_rec), 1ull << 16);
@@ -1642,7 +1671,7 @@ sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStrea
   return build_pass(pe, spec, false, s, out, &outcome);
 }
 
-sdb_status finish_covering(sdb_covering* cov, cudaStream_t s);
+sdb_status finish_covering(sdb_covering* cov, cudaStream_t s, bool wait = true);
 
 sdb_status build_covering_device(const PolyEdges& pe, uint32_t B, uint32_t k, uint32_t options,
                                  cudaStream_t s, sdb_covering* cov) {
@@ -1684,7 +1713,7 @@ sdb_status build_covering_device(const PolyEdges& pe, uint32_t B, uint32_t k, ui
 }
 
 // the binary search's shared-memory sample of the starts, and the size
-sdb_status finish_covering(sdb_covering* cov, cudaStream_t s) {
+sdb_status finish_covering(sdb_covering* cov, cudaStream_t s, bool wait) {
   const uint32_t SAMPLE_MAX = 2048;
   const uint64_t keys = cov->R + 1;
   uint32_t stride = (uint32_t)((keys + SAMPLE_MAX - 1) / SAMPLE_MAX);
@@ -1697,7 +1726,7 @@ sdb_status finish_covering(sdb_covering* cov, cudaStream_t s) {
   cov->sample_n = ns;
   cov->sample_stride = stride;
   cov->bytes = (size_t)keys * 16 + (size_t)cov->nids * 4 + (size_t)ns * 8;
-  SDB_TRY_CUDA(cudaStreamSynchronize(s));
+  if (wait) SDB_TRY_CUDA(cudaStreamSynchronize(s));
   return SDB_OK;
 }
 
@@ -1790,7 +1819,7 @@ sdb_status build_coverings_multi(const PolyEdges& pe, uint32_t B, const uint32_t
     rebase_pay_kernel<<<grid_for(e, 256), 256, 0, s>>>(cs.pay + a, e, (uint32_t)a, c->pay);
     note_launch();
     rc = ck(cudaGetLastError());
-    if (rc == SDB_OK) rc = finish_covering(c, s);
+    if (rc == SDB_OK) rc = finish_covering(c, s, i + 1 == nq);  // one wait for all
   }
   cs.release(s);
   return rc;

@@ -243,6 +243,14 @@ struct PolyEdges {
   std::vector<uint32_t> edge_off;
   std::vector<uint32_t> next;
 };
+// Polygons as their caller holds them; next == nullptr: one ring per polygon.
+struct PolySet {
+  uint32_t P;
+  const uint32_t* off;  // P + 1
+  const uint32_t* x;
+  const uint32_t* y;
+  const uint32_t* next;
+};
 PolyEdges poly_edges(const sdb_polygons* p);
 PolyEdges poly_edges(const sdb_multipolygons* p);
 sdb_status validate_polygons(const sdb_polygons* polys, uint32_t grid_bits);
@@ -372,7 +380,7 @@ sdb_status batch_core_index(BatchCore* c, uint32_t min_ranges, uint32_t ranges_p
 sdb_status batch_core_run(BatchCore* c, int mode, uint64_t* count, int64_t* sum, cudaStream_t s);
 // coverings for queries cq (pairs in query order), chunked; fills sbase/R/chunk
 // of hq with chunk indices starting at chunk_base
-sdb_status build_query_coverings(const PolyEdges& pe, uint32_t B,
+sdb_status build_query_coverings(const PolySet& polys, uint32_t B,
                                  const std::vector<CoverQuery>& cq,
                                  const std::vector<uint32_t>& pp, const std::vector<uint32_t>& pq,
                                  const std::vector<uint32_t>& ps, std::vector<BatchQueryDev>& hq,

@@ -212,7 +212,8 @@ sdb_status process(sdb_server* S, std::vector<std::shared_ptr<Ticket>>& batch, c
     }
     std::vector<CoverSet> sets;
     uint64_t nr = 0, nc = 0, mr = 0;
-    rc = sdb::build_query_coverings(S->pe, S->B, cq, pp, pq, ps, mq, &sets,
+    const sdb::PolySet ps_all{S->pe.P, S->pe.edge_off.data(), S->pe.x, S->pe.y, S->pe.next.data()};
+    rc = sdb::build_query_coverings(ps_all, S->B, cq, pp, pq, ps, mq, &sets,
                                     (uint32_t)chunks.size(), s, &nr, &nc, &mr);
     for (auto& set : sets) {
       auto c = std::make_shared<Chunk>();
