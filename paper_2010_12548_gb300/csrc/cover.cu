@@ -890,12 +890,13 @@ __global__ void merge_finish_kernel(const QueryFix* __restrict__ qf,
                                     const uint32_t* __restrict__ qlist,
                                     const CoverQuery* __restrict__ qs, uint32_t Q,
                                     const uint64_t* __restrict__ coff, uint64_t n_elements,
-                                    uint64_t n_cells, uint64_t* __restrict__ start, uint32_t* __restrict__ list_off,
-                                    uint32_t* __restrict__ pay, uint64_t* __restrict__ qoff,
+                                    uint64_t n_cells, const QueryOut* __restrict__ out,
+                                    uint64_t* __restrict__ qoff,
                                     uint64_t* __restrict__ qcells) {
   const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= Q) return;
   const QueryFix f = qf[q];
+  const QueryOut O = out[q];
   uint64_t e;
   uint32_t L;
   if (f.head != NONE) {
@@ -909,15 +910,15 @@ __global__ void merge_finish_kernel(const QueryFix* __restrict__ qf,
     L = f.prev == NONE ? 0u : qlist[2 * f.prev + 1];
     e = ro + f.extra;
     qoff[q] = e;
-    start[e] = 0;
-    list_off[e] = L;
-    pay[e] = NONE;
+    O.start[e] = 0;
+    O.list_off[e] = L - O.l0;
+    O.pay[e] = NONE;
     ++e;
     qcells[q] = 0;
   }
-  start[e] = 1ull << (2 * qs[q].F);
-  list_off[e] = L;
-  pay[e] = NONE;
+  O.start[e] = 1ull << (2 * qs[q].F);
+  O.list_off[e] = L - O.l0;
+  O.pay[e] = NONE;
   if (q == Q - 1) qoff[Q] = e + 1;
 }
 
@@ -1158,7 +1159,12 @@ static sdb_status merge_records(uint64_t* key, uint32_t* val, uint64_t n, const 
   }
   out->E = E;
   out->nids = nids;
-  return finish_queries(dq, qopen, qlist, d_qs, Q, nullptr, n, n, out, s);
+  QueryOut* dout;
+  SDB_TRY(sc.get(&dout, Q));
+  const std::vector<QueryOut> hout(Q, QueryOut{out->start, out->list_off, out->list_ids, out->pay, 0, 0});
+  SDB_TRY_CUDA(cudaMemcpyAsync(dout, hout.data(), (size_t)Q * sizeof(QueryOut),
+                               cudaMemcpyHostToDevice, s));
+  return finish_queries(dq, qopen, qlist, d_qs, Q, nullptr, n, n, dout, out, s);
 }
 
 uint64_t query_fixes(const std::vector<uint32_t>& head, uint64_t n, std::vector<QueryFix>* out) {
@@ -1184,14 +1190,14 @@ uint64_t query_fixes(const std::vector<uint32_t>& head, uint64_t n, std::vector<
 
 sdb_status finish_queries(const QueryFix* dq, const uint64_t* qopen, const uint32_t* qlist,
                           const CoverQuery* d_qs, uint32_t Q, const uint64_t* coff,
-                          uint64_t n_elements, uint64_t n_cells, CoverSet* out, cudaStream_t s) {
+                          uint64_t n_elements, uint64_t n_cells, const QueryOut* d_out,
+                          CoverSet* out, cudaStream_t s) {
   Scratch sc(s);
   uint64_t *qoff, *qcells;
   SDB_TRY(sc.get(&qoff, (size_t)Q + 1));
   SDB_TRY(sc.get(&qcells, Q));
   merge_finish_kernel<<<grid_for(Q, 256), 256, 0, s>>>(dq, qopen, qlist, d_qs, Q, coff, n_elements,
-                                                       n_cells, out->start, out->list_off,
-                                                       out->pay, qoff, qcells);
+                                                       n_cells, d_out, qoff, qcells);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
   out->qoff.assign((size_t)Q + 1, 0);
@@ -1205,6 +1211,13 @@ sdb_status finish_queries(const QueryFix* dq, const uint64_t* qopen, const uint3
 }
 
 void CoverSet::release(cudaStream_t s) {
+  for (CoverSlice& c : slices) {
+    dfree(c.start, s);
+    dfree(c.list_off, s);
+    dfree(c.list_ids, s);
+    dfree(c.pay, s);
+  }
+  slices.clear();
   dfree(start, s);
   dfree(list_off, s);
   dfree(list_ids, s);
@@ -1770,6 +1783,7 @@ sdb_status build_coverings_multi(const PolyEdges& pe, uint32_t B, const uint32_t
   spec.pair_slot = ps.data();
   spec.flags = (options & SDB_COVER_BOUNDARY_FLAGS) != 0;
   spec.noncons = (options & SDB_COVER_NONCONSERVATIVE) != 0;
+  spec.split = true;
   CoverSet cs;
   sdb_status st = nq > 1 ? build_coverings(pe, spec, s, &cs) : SDB_EINVAL;
   if (st != SDB_OK) {
@@ -1782,6 +1796,29 @@ sdb_status build_coverings_multi(const PolyEdges& pe, uint32_t B, const uint32_t
       SDB_TRY(build_covering_device(pe, B, ks[i], options, s, covs[i]));
     }
     return SDB_OK;
+  }
+  if (!cs.slices.empty()) {  // written where they belong
+    sdb_status rc = SDB_OK;
+    for (uint32_t i = 0; i < nq && rc == SDB_OK; ++i) {
+      sdb_covering* c = covs[i];
+      CoverSlice& sl = cs.slices[i];
+      c->B = B;
+      c->k = ks[i];
+      c->F = B - ks[i];
+      c->P = P;
+      c->flagged = spec.flags;
+      c->R = sl.E - 1;
+      c->nids = sl.nids;
+      c->ncells = cs.qcells[i];
+      c->start = sl.start;
+      c->list_off = sl.list_off;
+      c->list_ids = sl.list_ids;
+      c->pay = sl.pay;
+      sl = CoverSlice{};
+      rc = finish_covering(c, s, i + 1 == nq);  // one wait for all
+    }
+    cs.release(s);
+    return rc;
   }
   // each query's slice [qoff[i], qoff[i+1]) (its last entry the sentinel)
   std::vector<uint32_t> lo(nq + 1, 0);

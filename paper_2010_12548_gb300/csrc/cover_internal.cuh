@@ -34,6 +34,17 @@ struct QueryFix {
   uint32_t prev;       // the last earlier query with records (or NONE)
   uint32_t head;       // the query's first record (or NONE)
 };
+// Where a query's ranges go: arrays indexed by the entry's number over all queries
+// (a query with arrays of its own holds them moved back by e0 entries and l0 list
+// entries), and what is taken off the numbers stored in them.
+struct QueryOut {
+  uint64_t* start;
+  uint32_t* list_off;
+  uint32_t* list_ids;
+  uint32_t* pay;
+  uint64_t e0;
+  uint32_t l0;
+};
 // the queries' fixes from their first records (of n, 0xffffffff: none); returns
 // the entries that are no ranges of groups
 uint64_t query_fixes(const std::vector<uint32_t>& head, uint64_t n, std::vector<QueryFix>* out);
@@ -42,7 +53,8 @@ uint64_t query_fixes(const std::vector<uint32_t>& head, uint64_t n, std::vector<
 // every element is one record.
 sdb_status finish_queries(const QueryFix* dq, const uint64_t* qopen, const uint32_t* qlist,
                           const CoverQuery* d_qs, uint32_t Q, const uint64_t* coff,
-                          uint64_t n_elements, uint64_t n_cells, CoverSet* out, cudaStream_t s);
+                          uint64_t n_elements, uint64_t n_cells, const QueryOut* d_out,
+                          CoverSet* out, cudaStream_t s);
 
 enum class TileOutcome { made, nested, crowded };
 // The covering set from the n_rec coarse records (rkey, rval) and the n_tile

@@ -530,10 +530,7 @@ __global__ void group_count_kernel(GroupArgs A, uint64_t* __restrict__ cnt,
 }
 
 struct RangeOut {
-  uint64_t* start;
-  uint32_t* list_off;
-  uint32_t* list_ids;
-  uint32_t* pay;
+  const QueryOut* q;
   uint64_t* qopen;  // per query: ranges before its first group, after its last
   uint32_t* qlist;  // per query: list entries before its first group, after its last
 };
@@ -546,6 +543,13 @@ __device__ __forceinline__ void insert_entry(uint32_t* out, uint32_t t, uint32_t
     --j;
   }
   out[j] = v;
+}
+
+// the ranges and list entries before each query's first group (~0: no records)
+__global__ void query_offsets_kernel(const uint32_t* __restrict__ qhead, uint32_t Q,
+                                     const uint64_t* __restrict__ off, uint64_t* __restrict__ qoff) {
+  const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < Q) qoff[q] = qhead[q] == NONE ? ~0ull : off[qhead[q]];
 }
 
 __device__ __forceinline__ uint32_t pay_of(uint32_t n, uint32_t entry, uint64_t e) {
@@ -571,15 +575,16 @@ __global__ void group_emit_kernel(GroupArgs A, const uint64_t* __restrict__ off,
     o.qlist[2 * q] = L;
   }
   uint64_t e = ro + extra[q];
+  const QueryOut O = o.q[q];
   if (c & 1u) {
     uint64_t from = 0;
     if (!(c & 8u)) {  // the end of the previous group's cell
       const uint64_t pkey = A.key[a - 1];
       from = (pkey & A.lomask) + (1ull << (2 * A.level[a - 1]));
     }
-    o.start[e] = from;
-    o.list_off[e] = L;
-    o.pay[e] = NONE;
+    O.start[e] = from;
+    O.list_off[e] = L - O.l0;
+    O.pay[e] = NONE;
     ++e;
   }
   if (c & 2u) {
@@ -588,11 +593,11 @@ __global__ void group_emit_kernel(GroupArgs A, const uint64_t* __restrict__ off,
       const uint32_t v = A.info[i];
       if (!((v >> INFO_FIRST) & 1u)) continue;
       one = info_entry(v, INFO_FIRST);
-      insert_entry(o.list_ids + L, n++, one);
+      insert_entry(O.list_ids + L, n++, one);
     }
-    o.start[e] = lo;
-    o.list_off[e] = L;
-    o.pay[e] = pay_of(n, one, e);
+    O.start[e] = lo;
+    O.list_off[e] = L - O.l0;
+    O.pay[e] = pay_of(n, one, e - O.e0);
     L += n;
     ++e;
   }
@@ -600,9 +605,9 @@ __global__ void group_emit_kernel(GroupArgs A, const uint64_t* __restrict__ off,
   e += in >> 32;
   L += (uint32_t)in;
   if (c & 4u) {
-    o.start[e] = hi;
-    o.list_off[e] = L;
-    o.pay[e] = NONE;
+    O.start[e] = hi;
+    O.list_off[e] = L - O.l0;
+    O.pay[e] = NONE;
     ++e;
   }
   if (c & 16u) {
@@ -664,6 +669,7 @@ __global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64
     uint64_t e0 = (pre >> 32) + extra[q] + (c & 1u) + ((c >> 1) & 1u);
     uint32_t L0 = (uint32_t)pre + ((c & 2u) ? nfirst : 0u);
     const uint64_t lo = key & lomask;
+    const QueryOut O = o.q[q];
     for (uint32_t i0 = 0; i0 < ns; i0 += 32) {
       const bool on = i0 + lane < ns;
       const uint32_t pos = on ? s_pos[w][i0 + lane] : 0u;
@@ -690,11 +696,11 @@ __global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64
           if (!has(j)) continue;
           one = j < STAGE ? s_slot[w][j] : A.rec[a + j].slot;
           if (A.flags) one |= ((A.bbits[(uint64_t)A.rec[a + j].bits * 32 + wi] >> bi) & 1u) << 31;
-          o.list_ids[t++] = one;
+          O.list_ids[t++] = one;
         }
-        o.start[e] = lo + pos;
-        o.list_off[e] = L;
-        o.pay[e] = pay_of(n, one, e);
+        O.start[e] = lo + pos;
+        O.list_off[e] = L - O.l0;
+        O.pay[e] = pay_of(n, one, e - O.e0);
       }
       L0 += __shfl_sync(FULL, inc, 31);
     }
@@ -808,6 +814,16 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
     SDB_TRY(exclusive_scan<uint64_t>(cnt, off, ne, tot, s));
     SDB_TRY(exclusive_scan_u32(cells, coff, ne, tot + 1, s));
   }
+  uint64_t* dqoff;
+  SDB_TRY(sc.get(&dqoff, Q));
+  if (ne) {
+    query_offsets_kernel<<<grid_for(Q, 256), 256, 0, s>>>(qhead, Q, off, dqoff);
+    note_launch();
+    SDB_TRY_CUDA(cudaGetLastError());
+  }
+  std::vector<uint64_t> hqoff(Q, ~0ull);
+  if (ne && spec.split)
+    SDB_TRY_CUDA(cudaMemcpyAsync(hqoff.data(), dqoff, (size_t)Q * 8, cudaMemcpyDeviceToHost, s));
   uint64_t htot[2] = {0, 0};
   unsigned int hflag[2] = {0, 0};
   std::vector<uint32_t> hhead(Q);
@@ -844,10 +860,36 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
     set_error("covering: %llu ranges exceed the 32-bit index range", (unsigned long long)E);
     return SDB_ENOMEM;
   }
-  SDB_TRY(dalloc_n(&out->start, E, s));
-  SDB_TRY(dalloc_n(&out->list_off, E, s));
-  SDB_TRY(dalloc_n(&out->pay, E, s));
-  SDB_TRY(dalloc_n(&out->list_ids, nids ? nids : 1, s));
+  std::vector<QueryOut> hout(Q);
+  if (spec.split) {
+    out->slices.assign(Q, CoverSlice{});
+    uint64_t next = htot[0];
+    for (uint32_t q = Q; q-- > 0;) {  // a query ends where the next one with records begins
+      CoverSlice& c = out->slices[q];
+      const bool any = hqoff[q] != ~0ull;
+      const uint64_t at = any ? hqoff[q] : next;
+      c.E = (any ? (next >> 32) - (at >> 32) : 1) + 1;
+      c.nids = any ? (next & 0xffffffffull) - (at & 0xffffffffull) : 0;
+      SDB_TRY(dalloc_n(&c.start, c.E, s));
+      SDB_TRY(dalloc_n(&c.list_off, c.E, s));
+      SDB_TRY(dalloc_n(&c.pay, c.E, s));
+      SDB_TRY(dalloc_n(&c.list_ids, c.nids ? c.nids : 1, s));
+      const uint64_t e0 = (at >> 32) + hextra[q];
+      const uint32_t l0 = (uint32_t)at;
+      hout[q] = QueryOut{c.start - e0, c.list_off - e0, c.list_ids - l0, c.pay - e0, e0, l0};
+      next = at;
+    }
+  } else {
+    SDB_TRY(dalloc_n(&out->start, E, s));
+    SDB_TRY(dalloc_n(&out->list_off, E, s));
+    SDB_TRY(dalloc_n(&out->pay, E, s));
+    SDB_TRY(dalloc_n(&out->list_ids, nids ? nids : 1, s));
+    hout.assign(Q, QueryOut{out->start, out->list_off, out->list_ids, out->pay, 0, 0});
+  }
+  QueryOut* dout;
+  SDB_TRY(sc.get(&dout, Q));
+  SDB_TRY_CUDA(cudaMemcpyAsync(dout, hout.data(), (size_t)Q * sizeof(QueryOut),
+                               cudaMemcpyHostToDevice, s));
   QueryFix* dq;
   uint64_t *qopen, *dextra;
   uint32_t* qlist;
@@ -859,7 +901,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   SDB_TRY_CUDA(cudaMemcpyAsync(dextra, hextra.data(), (size_t)Q * 8, cudaMemcpyHostToDevice, s));
   if (ne) {
     TraceScope tr1("cover.emit", s);
-    const RangeOut ro{out->start, out->list_off, out->list_ids, out->pay, qopen, qlist};
+    const RangeOut ro{dout, qopen, qlist};
     group_emit_kernel<<<grid_for(ne, 256), 256, 0, s>>>(ga, off, code, dextra, ro);
     note_launch();
     if (n_tile) {
@@ -871,7 +913,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   out->E = E;
   out->nids = nids;
   out->ncells = ncells;
-  return finish_queries(dq, qopen, qlist, d_qs, Q, coff, ne, ncells, out, s);
+  return finish_queries(dq, qopen, qlist, d_qs, Q, coff, ne, ncells, dout, out, s);
 }
 
 }  // namespace sdb

@@ -292,12 +292,23 @@ struct CoverSpec {
   const uint32_t* pair_slot = nullptr;
   bool flags = false;    // boundary flags on list entries (result range, Sec. 6)
   bool noncons = false;  // finest boundary cells kept only when their centre is inside
+  bool split = false;    // arrays of its own for every query, where the builder can
 };
 // Result, device arrays from the library pool.  Query q's ranges are entries
 // [qoff[q], qoff[q+1] - 1) of start/list_off/pay; entry qoff[q+1] - 1 is a
 // sentinel with start 4^F and an empty list, so list_off[i+1] - list_off[i] is
 // the length of range i's list for every range.
+// (With spec.split and slices filled, every query has arrays of its own there, its
+// list references counting from its own first entry, and the arrays here are null.)
+struct CoverSlice {
+  uint64_t* start = nullptr;
+  uint32_t* list_off = nullptr;
+  uint32_t* list_ids = nullptr;
+  uint32_t* pay = nullptr;
+  uint64_t E = 0, nids = 0;
+};
 struct CoverSet {
+  std::vector<CoverSlice> slices;
   uint64_t* start = nullptr;     // E
   uint32_t* list_off = nullptr;  // E
   uint32_t* list_ids = nullptr;  // nids (slot ids)
