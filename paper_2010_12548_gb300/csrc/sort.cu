@@ -71,22 +71,55 @@ __global__ __launch_bounds__(SCAN_THREADS) void scan_tile_kernel(const In* in, T
                                                                  const T* block_off, T* d_total) {
   __shared__ T s_warp[SCAN_THREADS / 32 + 1];
   size_t base = (size_t)blockIdx.x * SCAN_TILE + (size_t)threadIdx.x * SCAN_ITEMS;
+  // a thread's eight elements are one aligned stretch: 16-byte reads and writes
+  // where the arrays allow (8-byte prefixes written one by one touched every
+  // 32-byte sector four times: 30M of them 133 us, this 72)
+  const bool whole = base + SCAN_ITEMS <= n &&
+                     ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0;
   T v[SCAN_ITEMS];
   T acc = 0;
+  if (whole) {
+    constexpr int PER = 16 / sizeof(In);
 #pragma unroll
-  for (int i = 0; i < SCAN_ITEMS; ++i) {
-    size_t g = base + i;
-    v[i] = g < n ? scan_value<T, In>(in[g]) : T(0);
-    acc += v[i];
+    for (int i = 0; i < SCAN_ITEMS; i += PER) {
+      alignas(16) In x[PER];
+      *reinterpret_cast<uint4*>(x) = *reinterpret_cast<const uint4*>(in + base + i);
+#pragma unroll
+      for (int j = 0; j < PER; ++j) v[i + j] = scan_value<T, In>(x[j]);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) {
+      size_t g = base + i;
+      v[i] = g < n ? scan_value<T, In>(in[g]) : T(0);
+    }
   }
+#pragma unroll
+  for (int i = 0; i < SCAN_ITEMS; ++i) acc += v[i];
   T tot;
   T pre = block_exclusive_scan<T>(acc, s_warp, &tot);
   T off = (block_off ? block_off[blockIdx.x] : T(0)) + pre;
 #pragma unroll
   for (int i = 0; i < SCAN_ITEMS; ++i) {
-    size_t g = base + i;
-    if (g < n) out[g] = off;
-    off += v[i];
+    const T t = v[i];
+    v[i] = off;
+    off += t;
+  }
+  if (whole) {
+    constexpr int PER = 16 / sizeof(T);
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; i += PER) {
+      alignas(16) T x[PER];
+#pragma unroll
+      for (int j = 0; j < PER; ++j) x[j] = v[i + j];
+      *reinterpret_cast<uint4*>(out + base + i) = *reinterpret_cast<const uint4*>(x);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) {
+      size_t g = base + i;
+      if (g < n) out[g] = v[i];
+    }
   }
   if (d_total && blockIdx.x == gridDim.x - 1 && threadIdx.x == SCAN_THREADS - 1) {
     *d_total = off;  // last thread holds the grand total after its items
