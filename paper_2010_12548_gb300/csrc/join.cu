@@ -34,6 +34,9 @@
 #include "hilbert.cuh"
 #include "sdb_internal.cuh"
 
+#include <algorithm>
+#include <mutex>
+
 namespace sdb {
 
 namespace {
@@ -511,6 +514,88 @@ __host__ __device__ inline size_t top_bytes(const JoinArgs& A) {
   return ((size_t)1 << (2 * A.top_lev)) + 4 * TOP_PALETTE;
 }
 
+// ------------------------------------------------ clearing the outputs
+// All of a join's outputs in one launch (a memset per array took 1.3 us each), and
+// the join kernel after it starts while this one runs: it fills its shared memory
+// and waits for the cleared outputs only then (grid_wait).  This launch itself
+// waits for everything before it on the stream, so the join's inputs are complete
+// when either starts.
+constexpr uint32_t ZERO_MAX = 16;
+struct ZeroArgs {
+  unsigned long long* p[ZERO_MAX];
+  uint32_t n[ZERO_MAX];
+  uint32_t m = 0;
+  void add(void* q, uint64_t words) {
+    p[m] = reinterpret_cast<unsigned long long*>(q);
+    n[m++] = (uint32_t)words;
+  }
+};
+__global__ void zero_kernel(ZeroArgs z) {
+  cudaTriggerProgrammaticLaunchCompletion();
+  const uint32_t a = blockIdx.y;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < z.n[a]; i += gridDim.x * blockDim.x)
+    z.p[a][i] = 0ull;
+}
+// until the launch before this one (zero_kernel, if the launch says so) is complete
+__device__ __forceinline__ void grid_wait() { cudaGridDependencySynchronize(); }
+
+sdb_status launch_zero(const ZeroArgs& z, cudaStream_t s) {
+  uint32_t most = 1;
+  for (uint32_t i = 0; i < z.m; ++i) most = std::max(most, z.n[i]);
+  if (z.m == 0) return SDB_OK;
+  zero_kernel<<<dim3(std::min(grid_for(most, 256), 64u), z.m), 256, 0, s>>>(z);
+  note_launch();
+  SDB_TRY_CUDA(cudaGetLastError());
+  return SDB_OK;
+}
+
+// launches kern after a zero_kernel (early: overlapping it) or by itself
+template <class Args>
+sdb_status launch_after(void (*kern)(Args), unsigned blocks, int threads, size_t smem,
+                        cudaStream_t s, bool early, const Args& args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = early ? 1 : 0;
+  SDB_TRY_CUDA(cudaLaunchKernelEx(&cfg, kern, args));
+  note_launch();
+  SDB_TRY_CUDA(cudaGetLastError());
+  return SDB_OK;
+}
+
+// resident blocks per SM of one kernel by its shared memory, asked once for the
+// sizes in use (the question costs as much as a launch)
+struct OccupancyCache {
+  std::mutex m;
+  struct Entry {
+    int dev = -1, per_sm = 0;
+    size_t smem = 0;
+  } e[8];
+  int next = 0;
+  sdb_status get(const void* kern, int threads, size_t smem, int* per_sm) {
+    int dev = 0;
+    SDB_TRY_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(m);
+    for (const Entry& x : e)
+      if (x.dev == dev && x.smem == smem) {
+        *per_sm = x.per_sm;
+        return SDB_OK;
+      }
+    SDB_TRY(occupancy(kern, threads, smem, per_sm));
+    e[next].dev = dev;
+    e[next].smem = smem;
+    e[next].per_sm = *per_sm;
+    next = (next + 1) & 7;
+    return SDB_OK;
+  }
+};
+
 template <int LOOKUP, bool SMEM, bool SUM, bool RANGE, bool TOP = false>
 __global__ __launch_bounds__(TOP ? TOP_THREADS : THREADS, TOP ? TOP_BLOCKS : 4) void join_kernel(JoinArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -547,6 +632,7 @@ __global__ __launch_bounds__(TOP ? TOP_THREADS : THREADS, TOP ? TOP_BLOCKS : 4) 
     for (uint32_t i = threadIdx.x; i < TOP_PALETTE; i += TPB) s_pal[i] = __ldg(A.top_pal + i);
   }
   if (SMEM) acc_zero<SUM, RANGE>(acc, A.P);
+  grid_wait();
   __syncthreads();
 
   const uint32_t lane = threadIdx.x & 31;
@@ -678,7 +764,7 @@ __global__ __launch_bounds__(TOP ? TOP_THREADS : THREADS, TOP ? TOP_BLOCKS : 4) 
 }
 
 template <int LOOKUP, bool SMEM, bool SUM, bool RANGE, bool TOP = false>
-sdb_status launch_t(const JoinArgs& A, cudaStream_t s) {
+sdb_status launch_t(const JoinArgs& A, cudaStream_t s, bool early) {
   constexpr int TPB = TOP ? TOP_THREADS : THREADS;
   size_t smem = hilbert_bytes(LOOKUP) + stage_bytes(LOOKUP, A, TPB);
   if (SMEM) smem += acc_bytes(A.P, SUM, RANGE);
@@ -688,7 +774,8 @@ sdb_status launch_t(const JoinArgs& A, cudaStream_t s) {
   if (smem > 48 * 1024)
     SDB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
-  SDB_TRY(occupancy(reinterpret_cast<const void*>(kern), TPB, smem, &per_sm));
+  static OccupancyCache cache;
+  SDB_TRY(cache.get(reinterpret_cast<const void*>(kern), TPB, smem, &per_sm));
   // ask for no more shared memory than the resident blocks use (plus the 1 KB
   // the system reserves per block): the rest of the SM's unified memory stays
   // L1 cache, whose lines hold the lookups' gathers in flight
@@ -698,10 +785,7 @@ sdb_status launch_t(const JoinArgs& A, cudaStream_t s) {
   const uint64_t need = (A.n + 4 * TPB - 1) / (4 * TPB);  // tiles
   if (blocks > need) blocks = need > 0 ? need : 1;
   TraceScope tr("join", s);
-  kern<<<(unsigned)blocks, TPB, smem, s>>>(A);
-  note_launch();
-  SDB_TRY_CUDA(cudaGetLastError());
-  return SDB_OK;
+  return launch_after(kern, (unsigned)blocks, TPB, smem, s, early, A);
 }
 
 
@@ -734,6 +818,7 @@ __global__ __launch_bounds__(THREADS, 4) void join_multi_kernel(MultiArgs M) {
 #pragma unroll
     for (int e = 0; e < MULTI; ++e)
       if (e < (int)M.E) acc_zero<SUM, false>(acc[e], (uint32_t)P);
+  grid_wait();
   __syncthreads();
 
   const uint32_t gmask = ~((1u << A0.B) - 1u);
@@ -807,7 +892,7 @@ __global__ __launch_bounds__(THREADS, 4) void join_multi_kernel(MultiArgs M) {
 }
 
 template <int LOOKUP, bool SMEM, bool SUM>
-sdb_status launch_multi_t(const MultiArgs& M, cudaStream_t s) {
+sdb_status launch_multi_t(const MultiArgs& M, cudaStream_t s, bool early) {
   size_t smem = HILBERT3_SMEM_BYTES;
   if (SMEM) smem += (size_t)M.E * acc_bytes(M.c[0].P, SUM, false);
   smem = (smem + 15) & ~(size_t)15;
@@ -820,10 +905,7 @@ sdb_status launch_multi_t(const MultiArgs& M, cudaStream_t s) {
   uint64_t blocks = (uint64_t)num_sms() * per_sm;
   const uint64_t need = (M.c[0].n + 4 * THREADS - 1) / (4 * THREADS);
   if (blocks > need) blocks = need > 0 ? need : 1;
-  kern<<<(unsigned)blocks, THREADS, smem, s>>>(M);
-  note_launch();
-  SDB_TRY_CUDA(cudaGetLastError());
-  return SDB_OK;
+  return launch_after(kern, (unsigned)blocks, THREADS, smem, s, early, M);
 }
 
 // ------------------------------------------------ an eps sweep through the tables
@@ -926,6 +1008,7 @@ __global__ __launch_bounds__(TOP_THREADS, TOP_BLOCKS) void sweep_kernel(
   }
   if (SMEM)
     for (uint32_t e = 0; e < E; ++e) acc_zero<SUM, false>(acc_at<SUM, false>(accb + e * ab, P), (uint32_t)P);
+  grid_wait();
   __syncthreads();
 
   const uint32_t lane = threadIdx.x & 31;
@@ -1035,7 +1118,7 @@ __global__ __launch_bounds__(TOP_THREADS, TOP_BLOCKS) void sweep_kernel(
 }
 
 template <int LOOKUP, bool SMEM, bool SUM>
-sdb_status launch_sweep_t(const SweepArgs& S, cudaStream_t s) {
+sdb_status launch_sweep_t(const SweepArgs& S, cudaStream_t s, bool early) {
   size_t smem = sweep_top_off(SMEM ? S.c[0].P : 0, SUM);
   if (S.top) smem += ((size_t)1 << (2 * S.top_lev)) + 4 * TOP_PALETTE;
   smem = (smem + 15) & ~(size_t)15;
@@ -1043,56 +1126,59 @@ sdb_status launch_sweep_t(const SweepArgs& S, cudaStream_t s) {
   if (smem > 48 * 1024)
     SDB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
-  SDB_TRY(occupancy(reinterpret_cast<const void*>(kern), TOP_THREADS, smem, &per_sm));
+  static OccupancyCache cache;
+  SDB_TRY(cache.get(reinterpret_cast<const void*>(kern), TOP_THREADS, smem, &per_sm));
   SDB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                     carveout_pct((size_t)per_sm * (smem + sizeof(SweepArgs::c) + 1024))));
   uint64_t blocks = (uint64_t)num_sms() * per_sm;
   const uint64_t need = (S.c[0].n + 4 * TOP_THREADS - 1) / (4 * TOP_THREADS);
   if (blocks > need) blocks = need > 0 ? need : 1;
   TraceScope tr("join", s);
-  kern<<<(unsigned)blocks, TOP_THREADS, smem, s>>>(S);
-  note_launch();
-  SDB_TRY_CUDA(cudaGetLastError());
-  return SDB_OK;
+  return launch_after(kern, (unsigned)blocks, TOP_THREADS, smem, s, early, S);
 }
 
 template <bool RANGE>
-sdb_status launch_pick(const JoinArgs& A, int lookup, bool has_sum, cudaStream_t s) {
+sdb_status launch_pick(const JoinArgs& A, int lookup, bool has_sum, cudaStream_t s, bool early) {
   const bool smem = A.P <= (RANGE ? SMEM_POLYS_RANGE : SMEM_POLYS);
   if (lookup == SDB_LOOKUP_BINARY) {
     if (smem)
-      return has_sum ? launch_t<0, true, true, RANGE>(A, s) : launch_t<0, true, false, RANGE>(A, s);
-    return has_sum ? launch_t<0, false, true, RANGE>(A, s) : launch_t<0, false, false, RANGE>(A, s);
+      return has_sum ? launch_t<0, true, true, RANGE>(A, s, early) : launch_t<0, true, false, RANGE>(A, s, early);
+    return has_sum ? launch_t<0, false, true, RANGE>(A, s, early) : launch_t<0, false, false, RANGE>(A, s, early);
   }
-  if constexpr (!RANGE) {  // the table lookups with the top level in shared memory
-    if (A.top && lookup == SDB_LOOKUP_TABLE) {
+  // The table lookups with the top level in shared memory.  The range join's
+  // accumulators (32 bytes a polygon) leave room for two blocks per SM up to about
+  // 640 polygons; above that its 64 warps without the level are better.
+  const bool top =
+      A.top && (!RANGE || !smem || acc_bytes(A.P, has_sum, RANGE) <= (size_t)20 * 1024);
+  {
+    if (top && lookup == SDB_LOOKUP_TABLE) {
       if (smem)
-        return has_sum ? launch_t<3, true, true, false, true>(A, s)
-                       : launch_t<3, true, false, false, true>(A, s);
-      return has_sum ? launch_t<3, false, true, false, true>(A, s)
-                     : launch_t<3, false, false, false, true>(A, s);
+        return has_sum ? launch_t<3, true, true, RANGE, true>(A, s, early)
+                       : launch_t<3, true, false, RANGE, true>(A, s, early);
+      return has_sum ? launch_t<3, false, true, RANGE, true>(A, s, early)
+                     : launch_t<3, false, false, RANGE, true>(A, s, early);
     }
-    if (A.top && lookup == SDB_LOOKUP_TABLE_LEARNED) {
+    if (top && lookup == SDB_LOOKUP_TABLE_LEARNED) {
       if (smem)
-        return has_sum ? launch_t<4, true, true, false, true>(A, s)
-                       : launch_t<4, true, false, false, true>(A, s);
-      return has_sum ? launch_t<4, false, true, false, true>(A, s)
-                     : launch_t<4, false, false, false, true>(A, s);
+        return has_sum ? launch_t<4, true, true, RANGE, true>(A, s, early)
+                       : launch_t<4, true, false, RANGE, true>(A, s, early);
+      return has_sum ? launch_t<4, false, true, RANGE, true>(A, s, early)
+                     : launch_t<4, false, false, RANGE, true>(A, s, early);
     }
   }
   if (lookup == SDB_LOOKUP_TABLE) {
     if (smem)
-      return has_sum ? launch_t<3, true, true, RANGE>(A, s) : launch_t<3, true, false, RANGE>(A, s);
-    return has_sum ? launch_t<3, false, true, RANGE>(A, s) : launch_t<3, false, false, RANGE>(A, s);
+      return has_sum ? launch_t<3, true, true, RANGE>(A, s, early) : launch_t<3, true, false, RANGE>(A, s, early);
+    return has_sum ? launch_t<3, false, true, RANGE>(A, s, early) : launch_t<3, false, false, RANGE>(A, s, early);
   }
   if (lookup == SDB_LOOKUP_TABLE_LEARNED) {
     if (smem)
-      return has_sum ? launch_t<4, true, true, RANGE>(A, s) : launch_t<4, true, false, RANGE>(A, s);
-    return has_sum ? launch_t<4, false, true, RANGE>(A, s) : launch_t<4, false, false, RANGE>(A, s);
+      return has_sum ? launch_t<4, true, true, RANGE>(A, s, early) : launch_t<4, true, false, RANGE>(A, s, early);
+    return has_sum ? launch_t<4, false, true, RANGE>(A, s, early) : launch_t<4, false, false, RANGE>(A, s, early);
   }
   if (smem)
-    return has_sum ? launch_t<1, true, true, RANGE>(A, s) : launch_t<1, true, false, RANGE>(A, s);
-  return has_sum ? launch_t<1, false, true, RANGE>(A, s) : launch_t<1, false, false, RANGE>(A, s);
+    return has_sum ? launch_t<1, true, true, RANGE>(A, s, early) : launch_t<1, true, false, RANGE>(A, s, early);
+  return has_sum ? launch_t<1, false, true, RANGE>(A, s, early) : launch_t<1, false, false, RANGE>(A, s, early);
 }
 
 }  // namespace
@@ -1102,13 +1188,14 @@ sdb_status launch_join(const uint32_t* x, const uint32_t* y, const int32_t* attr
                        cudaStream_t s, bool zero, uint64_t* bcount, int64_t* bsum,
                        uint64_t* babs) {
   if (zero) {
-    SDB_TRY_CUDA(cudaMemsetAsync(count, 0, (size_t)cov->P * 8, s));
-    if (sum) SDB_TRY_CUDA(cudaMemsetAsync(sum, 0, (size_t)cov->P * 8, s));
-    if (bcount) SDB_TRY_CUDA(cudaMemsetAsync(bcount, 0, (size_t)cov->P * 8, s));
-    if (bsum) SDB_TRY_CUDA(cudaMemsetAsync(bsum, 0, (size_t)cov->P * 8, s));
-    if (babs) SDB_TRY_CUDA(cudaMemsetAsync(babs, 0, (size_t)cov->P * 8, s));
-    if (lookup == SDB_LOOKUP_LEARNED || lookup == SDB_LOOKUP_TABLE_LEARNED)
-      SDB_TRY_CUDA(cudaMemsetAsync(cov->fallbacks, 0, sizeof(unsigned long long), s));
+    ZeroArgs z;
+    z.add(count, cov->P);
+    if (sum) z.add(sum, cov->P);
+    if (bcount) z.add(bcount, cov->P);
+    if (bsum) z.add(bsum, cov->P);
+    if (babs) z.add(babs, cov->P);
+    if (lookup == SDB_LOOKUP_LEARNED || lookup == SDB_LOOKUP_TABLE_LEARNED) z.add(cov->fallbacks, 1);
+    SDB_TRY(launch_zero(z, s));
   }
   if (n == 0) return SDB_OK;
   JoinArgs A{};
@@ -1154,7 +1241,8 @@ sdb_status launch_join(const uint32_t* x, const uint32_t* y, const int32_t* attr
   A.bsum = reinterpret_cast<unsigned long long*>(bsum);
   A.babs = reinterpret_cast<unsigned long long*>(babs);
   const bool has_sum = sum != nullptr;
-  return bcount ? launch_pick<true>(A, lookup, has_sum, s) : launch_pick<false>(A, lookup, has_sum, s);
+  return bcount ? launch_pick<true>(A, lookup, has_sum, s, zero)
+                : launch_pick<false>(A, lookup, has_sum, s, zero);
 }
 
 namespace {
@@ -1250,20 +1338,23 @@ sdb_status launch_join_multi(const uint32_t* x, const uint32_t* y, const int32_t
       if (covs[e0 + e]->F > covs[e0 + finest]->F) finest = e;
     MultiArgs M{};
     M.E = m;
+    ZeroArgs z;
     for (uint32_t e = 0; e < m; ++e) {
       const sdb_covering* c = covs[e0 + e];
       if (zero) {
-        SDB_TRY_CUDA(cudaMemsetAsync(count + (size_t)(e0 + e) * P, 0, (size_t)P * 8, s));
-        if (sum) SDB_TRY_CUDA(cudaMemsetAsync(sum + (size_t)(e0 + e) * P, 0, (size_t)P * 8, s));
-        if (lookup == SDB_LOOKUP_LEARNED || lookup == SDB_LOOKUP_TABLE_LEARNED)
-          SDB_TRY_CUDA(cudaMemsetAsync(c->fallbacks, 0, sizeof(unsigned long long), s));
+        z.add(count + (size_t)(e0 + e) * P, P);
+        if (sum) z.add(sum + (size_t)(e0 + e) * P, P);
+        if (lookup == SDB_LOOKUP_LEARNED || lookup == SDB_LOOKUP_TABLE_LEARNED) z.add(c->fallbacks, 1);
       }
       M.c[e] = join_args(x, y, attr, n, c, count + (size_t)(e0 + e) * P,
                          sum ? sum + (size_t)(e0 + e) * P : nullptr);
       M.shift[e] = 2 * (covs[e0 + finest]->F - c->F);
     }
     if (lookup == SDB_LOOKUP_TABLE || lookup == SDB_LOOKUP_TABLE_LEARNED) {
-      if (n == 0) continue;
+      if (n == 0) {
+        SDB_TRY(launch_zero(z, s));
+        continue;
+      }
       SweepArgs S{};
       S.E = m;
       for (uint32_t e = 0; e < m; ++e) S.c[e] = M.c[e];
@@ -1290,17 +1381,18 @@ sdb_status launch_join_multi(const uint32_t* x, const uint32_t* y, const int32_t
         S.top_lev = Lt;
         S.top_xy = covs[e0]->B - Lt;
       }
+      SDB_TRY(launch_zero(z, s));  // right before the sweep, which starts beside it
       const bool smem = (uint64_t)MULTI * P <= SMEM_POLYS;
       const bool has_sum = sum != nullptr;
       sdb_status st;
       if (lookup == SDB_LOOKUP_TABLE)
-        st = smem ? (has_sum ? launch_sweep_t<3, true, true>(S, s) : launch_sweep_t<3, true, false>(S, s))
-                  : (has_sum ? launch_sweep_t<3, false, true>(S, s)
-                             : launch_sweep_t<3, false, false>(S, s));
+        st = smem ? (has_sum ? launch_sweep_t<3, true, true>(S, s, zero) : launch_sweep_t<3, true, false>(S, s, zero))
+                  : (has_sum ? launch_sweep_t<3, false, true>(S, s, zero)
+                             : launch_sweep_t<3, false, false>(S, s, zero));
       else
-        st = smem ? (has_sum ? launch_sweep_t<4, true, true>(S, s) : launch_sweep_t<4, true, false>(S, s))
-                  : (has_sum ? launch_sweep_t<4, false, true>(S, s)
-                             : launch_sweep_t<4, false, false>(S, s));
+        st = smem ? (has_sum ? launch_sweep_t<4, true, true>(S, s, zero) : launch_sweep_t<4, true, false>(S, s, zero))
+                  : (has_sum ? launch_sweep_t<4, false, true>(S, s, zero)
+                             : launch_sweep_t<4, false, false>(S, s, zero));
       SDB_TRY(st);
       continue;
     }
@@ -1309,16 +1401,17 @@ sdb_status launch_join_multi(const uint32_t* x, const uint32_t* y, const int32_t
     M.c[0].k = Af.k;
     M.c[0].nsteps = Af.nsteps;
     M.c[0].st0 = Af.st0;
+    SDB_TRY(launch_zero(z, s));
     if (n == 0) continue;
     const bool smem = (uint64_t)m * P <= SMEM_POLYS;
     const bool has_sum = sum != nullptr;
     sdb_status st;
     if (lookup == SDB_LOOKUP_BINARY)
-      st = smem ? (has_sum ? launch_multi_t<0, true, true>(M, s) : launch_multi_t<0, true, false>(M, s))
-                : (has_sum ? launch_multi_t<0, false, true>(M, s) : launch_multi_t<0, false, false>(M, s));
+      st = smem ? (has_sum ? launch_multi_t<0, true, true>(M, s, zero) : launch_multi_t<0, true, false>(M, s, zero))
+                : (has_sum ? launch_multi_t<0, false, true>(M, s, zero) : launch_multi_t<0, false, false>(M, s, zero));
     else
-      st = smem ? (has_sum ? launch_multi_t<1, true, true>(M, s) : launch_multi_t<1, true, false>(M, s))
-                : (has_sum ? launch_multi_t<1, false, true>(M, s) : launch_multi_t<1, false, false>(M, s));
+      st = smem ? (has_sum ? launch_multi_t<1, true, true>(M, s, zero) : launch_multi_t<1, true, false>(M, s, zero))
+                : (has_sum ? launch_multi_t<1, false, true>(M, s, zero) : launch_multi_t<1, false, false>(M, s, zero));
     SDB_TRY(st);
   }
   return SDB_OK;
