@@ -1355,12 +1355,13 @@ static bool use_tiles(const CoverSpec& spec) {
   return true;
 }
 
-// Whether a polygon probably holds a vertex of another one (a few polygons' first
-// vertices against all): overlapping polygons cannot be merged tile by tile, and
-// finding that out from the tiles costs a third of the build.  A guess only.
-static bool overlap_likely(const PolyEdges& pe) {
-  if (pe.P < 2 || pe.V > (1u << 16)) return false;
-  std::vector<uint32_t> bb(4 * (size_t)pe.P);
+// Whether more than MAX_OVERLAP polygons probably lie over one another (some
+// polygons' first vertices against the boxes of all): finding that out from the
+// tiles costs a third of the build.  A guess only.
+static bool overlap_deep(const PolyEdges& pe) {
+  if (pe.P <= MAX_OVERLAP || pe.V > (1u << 16)) return false;
+  std::vector<uint32_t> over(64, 0);
+  const uint32_t samples = std::min<uint32_t>(pe.P, 64);
   for (uint32_t j = 0; j < pe.P; ++j) {
     uint32_t x0 = ~0u, y0 = ~0u, x1 = 0, y1 = 0;
     for (uint32_t v = pe.edge_off[j]; v < pe.edge_off[j + 1]; ++v) {
@@ -1369,31 +1370,13 @@ static bool overlap_likely(const PolyEdges& pe) {
       x1 = std::max(x1, pe.x[v]);
       y1 = std::max(y1, pe.y[v]);
     }
-    bb[4 * j] = x0;
-    bb[4 * j + 1] = y0;
-    bb[4 * j + 2] = x1;
-    bb[4 * j + 3] = y1;
-  }
-  const uint32_t samples = std::min(pe.P, 64u);
-  for (uint32_t k = 0; k < samples; ++k) {
-    const uint32_t i = (uint32_t)((uint64_t)k * pe.P / samples);
-    const int64_t px = pe.x[pe.edge_off[i]], py = pe.y[pe.edge_off[i]];
-    for (uint32_t j = 0; j < pe.P; ++j) {
-      if (j == i || px <= bb[4 * j] || px >= bb[4 * j + 2] || py <= bb[4 * j + 1] ||
-          py >= bb[4 * j + 3])
-        continue;
-      bool in = false, shared = false;
-      for (uint32_t v = pe.edge_off[j]; v < pe.edge_off[j + 1] && !shared; ++v) {
-        const int64_t ax = pe.x[v], ay = pe.y[v], bx = pe.x[pe.next[v]], by = pe.y[pe.next[v]];
-        shared = ax == px && ay == py;  // a tiling's common vertex
-        if ((ay > py) != (by > py)) {
-          const int64_t o = (bx - ax) * (py - ay) - (by - ay) * (px - ax);
-          in ^= by > ay ? o > 0 : o < 0;
-        }
-      }
-      if (in && !shared) return true;
+    for (uint32_t k = 0; k < samples; ++k) {
+      const uint32_t v = pe.edge_off[(uint64_t)k * pe.P / samples];
+      over[k] += pe.x[v] > x0 && pe.x[v] < x1 && pe.y[v] > y0 && pe.y[v] < y1;
     }
   }
+  for (uint32_t n : over)
+    if (n > MAX_OVERLAP) return true;
   return false;
 }
 
@@ -1674,7 +1657,7 @@ static sdb_status build_pass(const PolyEdges& pe, const CoverSpec& spec, bool ti
 sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStream_t s,
                            CoverSet* out) {
   TileOutcome outcome = TileOutcome::crowded;
-  if (use_tiles(spec) && !(spec.Q == 1 && overlap_likely(pe)))
+  if (use_tiles(spec) && !(spec.Q == 1 && overlap_deep(pe)))
     SDB_TRY(build_pass(pe, spec, true, s, out, &outcome));
   if (outcome == TileOutcome::made) return SDB_OK;
   if (outcome == TileOutcome::nested && spec.Q != 1) {

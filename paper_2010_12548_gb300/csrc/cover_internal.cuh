@@ -25,6 +25,9 @@ static_assert(sizeof(Item) == 32, "two 16-byte loads per item");
 constexpr uint32_t TILE_DEPTH = 5;
 // polygons of one tile that a warp takes one after the other
 constexpr uint32_t TILE_MAX_GROUP = 512;
+// polygons over one another, above the tiles, that one thread sorts and compares (its
+// work grows with their square; at 512 it still beats the refinement, covertiles.cu)
+constexpr uint32_t MAX_OVERLAP = 512;
 
 // per query (one thread each): its offset and record count, its sentinel
 // (start 4^F), and the single empty range of a query without records
@@ -58,9 +61,9 @@ sdb_status finish_queries(const QueryFix* dq, const uint64_t* qopen, const uint3
 
 enum class TileOutcome { made, nested, crowded };
 // The covering set from the n_rec coarse records (rkey, rval) and the n_tile
-// tile items with their edge lists (covertiles.cu).  nested: cells of
-// different polygons overlap at different levels; crowded: a tile meets too many
-// polygons; then nothing is made.
+// tile items with their edge lists (covertiles.cu).  nested: cells of different
+// polygons of one of several queries overlap at different levels; crowded: a tile
+// meets too many polygons, or too many lie over one another; then nothing is made.
 sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_rec, const Item* items,
                        uint64_t n_tile, const uint32_t* elist, const Edge* edges,
                        const uint32_t* pair_query, const uint32_t* pair_slot,

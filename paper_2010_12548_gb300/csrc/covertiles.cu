@@ -24,7 +24,7 @@
 // ever stored, sorted or merged.
 //
 // One warp per tile.  For the 263-zone sweep (eps 2^12 .. 2^6, 1.2e8 records)
-// this stage takes 2.5 ms (raster 1.26, ranges 0.67, sort and bookkeeping 0.5)
+// this stage takes 2.4 ms (raster 1.26, ranges 0.61, sort and bookkeeping 0.5)
 // where the refinement to the finest level, its sort and its merge took 9.3
 // (2.4, 4.5 and 2.2, and the counters of five more levels).
 #include "cover_internal.cuh"
@@ -245,7 +245,8 @@ struct TileArgs {
   uint32_t* cells;         // per element: records of the group (at its head)
   uint64_t* inner;         // per element, at tile heads: ranges that start inside
                            // the tile << 32 | their list entries
-  unsigned int* flag;      // [0] nested, [1] a tile with too many polygons
+  unsigned int* flag;      // [0] nested cells, [1] a tile with too many polygons,
+                           // [2] polygons that overlap inside a tile
   unsigned long long* front;  // boundary cells one level above the finest
 };
 
@@ -333,7 +334,7 @@ __global__ __launch_bounds__(TPB, 4) void tile_raster_kernel(TileArgs A) {
     const bool clash = k > 1 && ((u[0] & (u[1] | u[2] | u[3] | u[4])) ||
                                  (u[1] & (u[2] | u[3] | u[4])) || (u[2] & (u[3] | u[4])) ||
                                  (u[3] & u[4]));
-    if (__any_sync(FULL, clash) && lane == 0) A.flag[0] = 1u;
+    if (__any_sync(FULL, clash) && lane == 0) A.flag[2] = 1u;
     if (lane == 0) starts &= ~1u;  // the tile's first position is the group's head
     // list entries of the inner starts
     uint32_t ent = 0;
@@ -394,20 +395,18 @@ __global__ void element_kernel(const uint64_t* __restrict__ key, const uint32_t*
     } else {
       level[i] = (uint8_t)TILE_DEPTH;
       info[i] = INFO_TILE;
+      // (the sort is stable: a key's coarse cells come before its tiles)
       const uint64_t q = key[i];
-      const bool head = i == 0 || key[i - 1] != q;
+      const bool lead = i == 0 || key[i - 1] != q;
+      const bool head = lead || idx[i - 1] < n_rec;
+      if (!lead && head) flag[0] = 1u;  // another polygon's cell with the tile's start
       if (!head) {
         cells[i] = 0;  // the head's warp counts for the tile
       } else if (i + TILE_MAX_GROUP < ne && key[i + TILE_MAX_GROUP] == q) {
         flag[1] = 1u;
       } else {
         for (uint64_t j = i; j < ne && key[j] == q; ++j, ++k) {
-          const uint32_t e = idx[j];
-          if (e < n_rec) {  // another polygon's cell with the tile's start
-            flag[0] = 1u;
-            break;
-          }
-          const uint32_t ti = e - (uint32_t)n_rec;
+          const uint32_t ti = idx[j] - (uint32_t)n_rec;
           const Item it = items[ti];
           const uint32_t qi = pair_query[it.pair];
           const CoverQuery Q = qs[qi];
@@ -450,7 +449,18 @@ struct GroupArgs {
   uint64_t ne, lomask;
   uint32_t qshift;
   const CoverQuery* qs;
+  // elementary intervals of nested cells (see nested_groups) instead of cells: their
+  // ends; inner then holds for every head
+  const uint64_t* end;
 };
+
+// the first id after element i, whose key is at lo
+__device__ __forceinline__ uint64_t end_of(const GroupArgs& A, uint64_t i, uint64_t lo) {
+  return A.end ? A.end[i] : lo + (1ull << (2 * A.level[i]));
+}
+__device__ __forceinline__ uint64_t inner_of(const GroupArgs& A, uint64_t i) {
+  return A.end || (A.info[i] & INFO_TILE) ? A.inner[i] : 0ull;
+}
 
 __device__ __forceinline__ uint32_t gq(const GroupArgs& A, uint64_t key) {
   return A.qshift >= 64 ? 0u : (uint32_t)(key >> A.qshift);
@@ -484,7 +494,8 @@ __device__ bool same_ends(const GroupArgs& A, uint64_t pa, uint64_t pe, uint64_t
 // group or a tail opens a range when its set differs from what comes before.
 __global__ void group_count_kernel(GroupArgs A, uint64_t* __restrict__ cnt,
                                    uint8_t* __restrict__ code, uint32_t* __restrict__ qhead,
-                                   unsigned int* __restrict__ flag) {
+                                   unsigned int* __restrict__ flag,
+                                   unsigned long long* __restrict__ entries) {
   const uint64_t a = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= A.ne || flag[1]) return;  // (a crowded tile: nothing is made)
   const uint64_t key = A.key[a];
@@ -493,14 +504,14 @@ __global__ void group_count_kernel(GroupArgs A, uint64_t* __restrict__ cnt,
     code[a] = 0;
     return;
   }
-  const uint32_t lev = A.level[a], q = gq(A, key);
-  const uint64_t lo = key & A.lomask, hi = lo + (1ull << (2 * lev));
+  const uint32_t q = gq(A, key);
+  const uint64_t lo = key & A.lomask, hi = end_of(A, a, lo);
   bool nest = false;
   uint32_t nfirst = 0, nlast = 0;
   uint64_t e = a;
   for (; e < A.ne && A.key[e] == key; ++e) {
     const uint32_t v = A.info[e];
-    nest |= A.level[e] != lev || ((v ^ A.info[a]) & INFO_TILE);
+    if (!A.end) nest |= A.level[e] != A.level[a] || ((v ^ A.info[a]) & INFO_TILE);
     nfirst += (v >> INFO_FIRST) & 1u;
     nlast += (v >> INFO_LAST) & 1u;
   }
@@ -515,15 +526,17 @@ __global__ void group_count_kernel(GroupArgs A, uint64_t* __restrict__ cnt,
       --pa;
       plast |= (A.info[pa] >> INFO_LAST) & 1u;
     }
-    const uint64_t pend = (pkey & A.lomask) + (1ull << (2 * A.level[pa]));
+    const uint64_t pend = end_of(A, pa, pkey & A.lomask);
     nest |= lo < pend;  // the previous cell reaches into this one
     gap = lo > pend;
     opens_gap = gap && plast;
     opens_head = gap ? nfirst != 0 : !same_ends(A, pa, a, a, e);
   }
   const bool opens_tail = last && hi < (1ull << (2 * A.qs[q].F)) && nlast != 0;
-  const uint64_t in = (A.info[a] & INFO_TILE) ? A.inner[a] : 0ull;
+  const uint64_t in = inner_of(A, a);
   cnt[a] = in + ((uint64_t)(opens_gap + opens_head + opens_tail) << 32) + (opens_head ? nfirst : 0u);
+  if (entries)  // nested cells: more list entries than raster cells are possible
+    atomicAdd(entries, (unsigned long long)((uint32_t)in) + (opens_head ? nfirst : 0u));
   code[a] = (uint8_t)(opens_gap | (opens_head << 1) | (opens_tail << 2) | (first << 3) | (last << 4));
   if (first) qhead[q] = (uint32_t)a;
   if (nest) flag[0] = 1u;
@@ -566,8 +579,8 @@ __global__ void group_emit_kernel(GroupArgs A, const uint64_t* __restrict__ off,
   if (a >= A.ne) return;
   const uint64_t key = A.key[a];
   if (a > 0 && A.key[a - 1] == key) return;
-  const uint32_t c = code[a], q = gq(A, key), lev = A.level[a];
-  const uint64_t lo = key & A.lomask, hi = lo + (1ull << (2 * lev));
+  const uint32_t c = code[a], q = gq(A, key);
+  const uint64_t lo = key & A.lomask, hi = end_of(A, a, lo);
   uint64_t ro = off[a] >> 32;
   uint32_t L = (uint32_t)off[a];
   if (c & 8u) {
@@ -580,7 +593,7 @@ __global__ void group_emit_kernel(GroupArgs A, const uint64_t* __restrict__ off,
     uint64_t from = 0;
     if (!(c & 8u)) {  // the end of the previous group's cell
       const uint64_t pkey = A.key[a - 1];
-      from = (pkey & A.lomask) + (1ull << (2 * A.level[a - 1]));
+      from = end_of(A, a - 1, pkey & A.lomask);
     }
     O.start[e] = from;
     O.list_off[e] = L - O.l0;
@@ -601,7 +614,7 @@ __global__ void group_emit_kernel(GroupArgs A, const uint64_t* __restrict__ off,
     L += n;
     ++e;
   }
-  const uint64_t in = (A.info[a] & INFO_TILE) ? A.inner[a] : 0ull;
+  const uint64_t in = inner_of(A, a);
   e += in >> 32;
   L += (uint32_t)in;
   if (c & 4u) {
@@ -622,12 +635,20 @@ __global__ void group_emit_kernel(GroupArgs A, const uint64_t* __restrict__ off,
 // a warp takes up to 32 tiles in a row, its lanes read what belongs to one tile each
 // at once, and a tile's polygon records are read while the tile before is written.
 // (263-zone sweep: 1.02 ms with each lane making the ranges of its own positions,
-// 0.67 with the list, 0.61 with the reads ahead; 0.79 before them with a sweep.s
+// 0.67 with the list, 0.61 with the reads ahead; 0.79 before them with a sweep's
 // own arrays per covering.)
+// BASE: polygons whose coarser cells hold the whole tile come on top (base: per tile
+// its group's first element, of which the base polygons are the first ones).
+struct TileBase {
+  const uint2* at;       // per tile head: its group's first element, base polygons
+  const uint32_t* info;  // the groups' elements
+};
+template <bool BASE>
 __global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64_t* __restrict__ off,
                                                         const uint8_t* __restrict__ code,
                                                         const uint64_t* __restrict__ extra,
-                                                        uint64_t lomask, RangeOut o) {
+                                                        uint64_t lomask, TileBase base,
+                                                        RangeOut o) {
   constexpr uint32_t STAGE = 4;  // polygons of a tile held in registers and shared memory
   __shared__ uint32_t s_h[WPB][STAGE][32];
   __shared__ uint16_t s_pos[WPB][1024];
@@ -640,12 +661,14 @@ __global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64
    uint2 my_head = make_uint2(0, 0);
    uint64_t my_key = 0, my_pre = 0;
    uint32_t my_ns = 0, my_c = 0;
+   uint2 my_base = make_uint2(0, 0);
    if (lane < in_run) {
      my_head = A.heads[g0 + lane];
+     my_base = BASE ? base.at[my_head.x] : make_uint2(my_head.x, 0);
      my_ns = (uint32_t)(A.inner[my_head.x] >> 32);
      my_key = A.key[my_head.x];
-     my_pre = off[my_head.x];
-     my_c = code[my_head.x];
+     my_pre = off[my_base.x];
+     my_c = code[my_base.x];
    }
    uint32_t nb = 0, nslot = 0;  // lane j: polygon j's bitmap and slot, of the next tile
    auto fetch = [&](uint32_t i) {
@@ -701,7 +724,9 @@ __global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64
     __syncwarp();
     const uint32_t q = A.qshift >= 64 ? 0u : (uint32_t)(key >> A.qshift);
     uint64_t e0 = (pre >> 32) + extra[q] + (c & 1u) + ((c >> 1) & 1u);
-    uint32_t L0 = (uint32_t)pre + ((c & 2u) ? nfirst : 0u);
+    const uint32_t b0 = BASE ? __shfl_sync(FULL, my_base.x, i) : 0u;
+    const uint32_t nb0 = BASE ? __shfl_sync(FULL, my_base.y, i) : 0u;
+    uint32_t L0 = (uint32_t)pre + ((c & 2u) ? nfirst + nb0 : 0u);
     const uint64_t lo = key & lomask;
     const QueryOut O = o.q[q];
     uint32_t slots[STAGE];
@@ -722,6 +747,7 @@ __global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64
       };
       if (on)
         for (uint32_t j = STAGE; j < k; ++j) n += more(j);
+      if (BASE && on) n += nb0;
       uint32_t inc = n;
 #pragma unroll
       for (int d = 1; d < 32; d <<= 1) {
@@ -732,7 +758,17 @@ __global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64
         const uint64_t e = e0 + i0 + lane;
         const uint32_t L = L0 + inc - n;
         uint32_t one = 0, t = L;
+        uint32_t bi0 = 0;  // base polygons written (they ascend too)
+        auto put_base = [&](uint32_t below) {
+          for (; (int)bi0 < (int)nb0; ++bi0) {
+            const uint32_t v = base.info[b0 + bi0] & INFO_SLOT;
+            if (v >= below) break;
+            one = v;
+            O.list_ids[t++] = v;
+          }
+        };
         auto put = [&](uint32_t j, uint32_t slot) {  // the polygons ascend by slot
+          put_base(slot);
           one = slot;
           if (A.flags) one |= ((A.bbits[(uint64_t)A.rec[a + j].bits * 32 + wi] >> bi) & 1u) << 31;
           O.list_ids[t++] = one;
@@ -742,6 +778,7 @@ __global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64
           if ((set >> j) & 1u) put(j, slots[j]);
         for (uint32_t j = STAGE; j < k; ++j)
           if (more(j)) put(j, A.rec[a + j].slot);
+        put_base(~0u);
         O.start[e] = lo + pos;
         O.list_off[e] = L - O.l0;
         O.pay[e] = pay_of(n, one, e - O.e0);
@@ -750,6 +787,227 @@ __global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64
     }
    }
   }
+}
+
+// ---------------------------------------------------------------- nested cells
+// One query whose polygons overlap: a coarser cell of one polygon may hold cells and
+// tiles of others.  The elements' ends cut the ids into elementary intervals, each a
+// tile or free of them; a coarser cell counts for every interval it spans.  The
+// intervals' polygons (in slot order), then their tiles', become the elements of
+// groups like the ones above, an interval each.  Only the few coarse cells are
+// sorted and paired, where the refinement to the finest level does so with every
+// cell: 64 stars with holes at eps 64, uploaded, covered, indexed and joined, 1600 us
+// -> 1069 us.  A group's set is compared and ordered by one thread; polygons laid over
+// one another, eps 64 and 16, refinement -> here: 2 of them 0.87 -> 0.60 and 1.06
+// -> 0.71 ms, 64: 1.70 -> 0.92 and 4.12 -> 1.32, 512: 29.6 -> 10.8 and 268 -> 26.
+// With more than MAX_OVERLAP over one another the refinement takes over.
+
+__global__ void ends_kernel(const uint64_t* __restrict__ key, const uint8_t* __restrict__ level,
+                            uint64_t ne, uint64_t top, uint64_t* __restrict__ bp) {
+  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < ne) {
+    bp[2 * i] = key[i];
+    bp[2 * i + 1] = key[i] + (1ull << (2 * level[i]));
+  } else if (i == ne) {
+    bp[2 * ne] = 0;
+    bp[2 * ne + 1] = top;
+  }
+}
+
+__device__ __forceinline__ uint32_t place_of(const uint64_t* __restrict__ b, uint32_t m, uint64_t v) {
+  uint32_t lo = 0;
+  for (uint32_t len = m; len > 0;) {
+    const uint32_t half = len >> 1;
+    if (b[lo + half] < v) {
+      lo += half + 1;
+      len -= half + 1;
+    } else {
+      len = half;
+    }
+  }
+  return lo;
+}
+
+// per element its first interval and how many it spans (a tile: none, its own)
+__global__ void element_spans_kernel(const uint64_t* __restrict__ key,
+                                     const uint8_t* __restrict__ level,
+                                     const uint32_t* __restrict__ info, uint64_t ne,
+                                     const uint64_t* __restrict__ b, uint32_t m,
+                                     uint32_t* __restrict__ first, uint32_t* __restrict__ span) {
+  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= ne) return;
+  const uint32_t k = place_of(b, m, key[i]);
+  first[i] = k;
+  span[i] = (info[i] & INFO_TILE) ? 0u : place_of(b, m, key[i] + (1ull << (2 * level[i]))) - k;
+}
+
+// pair i of (interval, slot): of the element e with poff[e] <= i < poff[e + 1]
+__global__ void span_pairs_kernel(const uint64_t* __restrict__ poff, uint64_t ne,
+                                  const uint32_t* __restrict__ first,
+                                  const uint32_t* __restrict__ info, uint64_t T, uint32_t pbits,
+                                  uint64_t* __restrict__ pairs) {
+  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= T) return;
+  uint64_t e = 0;
+  for (uint64_t len = ne; len > 1;) {
+    const uint64_t half = len >> 1;
+    if (poff[e + half] <= i) e += half;
+    len -= half;
+  }
+  pairs[i] = ((uint64_t)(first[e] + (uint32_t)(i - poff[e])) << pbits) | (info[e] & INFO_SLOT);
+}
+
+__global__ void pair_lengths_kernel(const uint64_t* __restrict__ pairs, uint64_t T, uint32_t pbits,
+                                    uint32_t* __restrict__ len, uint32_t* __restrict__ count,
+                                    unsigned int* __restrict__ flag) {
+  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= T) return;
+  const uint32_t k = (uint32_t)(pairs[i] >> pbits);
+  if (atomicAdd(&len[k], 1u) == MAX_OVERLAP) flag[1] = 1u;
+  atomicAdd(&count[k], 1u);
+}
+__global__ void tile_lengths_kernel(const uint2* __restrict__ heads,
+                                    const uint32_t* __restrict__ n_heads,
+                                    const uint32_t* __restrict__ first,
+                                    uint32_t* __restrict__ count) {
+  const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g < *n_heads) atomicAdd(&count[first[heads[g].x]], heads[g].y);
+}
+
+struct NestedOut {
+  uint64_t* key;
+  uint64_t* end;
+  uint32_t* info;
+  uint64_t* inner;
+  uint2* base;  // per tile head (by its old element): group's first element, base polygons
+};
+__global__ void base_elements_kernel(const uint64_t* __restrict__ pairs, uint64_t T, uint32_t pbits,
+                                     const uint64_t* __restrict__ b,
+                                     const uint32_t* __restrict__ eoff,
+                                     const uint32_t* __restrict__ poff, NestedOut o) {
+  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= T) return;
+  const uint32_t k = (uint32_t)(pairs[i] >> pbits);
+  const uint32_t at = eoff[k] + (uint32_t)(i - poff[k]);
+  o.key[at] = b[k];
+  o.end[at] = b[k + 1];
+  o.info[at] = (uint32_t)(pairs[i] & ((1ull << pbits) - 1)) | (1u << INFO_FIRST) | (1u << INFO_LAST);
+}
+__global__ void tile_elements_kernel(const uint2* __restrict__ heads,
+                                     const uint32_t* __restrict__ n_heads,
+                                     const uint32_t* __restrict__ first,
+                                     const uint32_t* __restrict__ info,
+                                     const uint64_t* __restrict__ inner,
+                                     const uint64_t* __restrict__ b,
+                                     const uint32_t* __restrict__ len,
+                                     const uint32_t* __restrict__ eoff, NestedOut o) {
+  const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= *n_heads) return;
+  const uint2 h = heads[g];
+  const uint32_t k = first[h.x], e = eoff[k], n = len[k];
+  for (uint32_t j = 0; j < h.y; ++j) {
+    o.key[e + n + j] = b[k];
+    o.end[e + n + j] = b[k + 1];
+    o.info[e + n + j] = info[h.x + j];
+  }
+  // every range that starts inside the tile lists the base polygons too
+  const uint64_t in = inner[h.x];
+  o.inner[e] = in + (uint64_t)n * (uint32_t)(in >> 32);
+  o.base[h.x] = make_uint2(e, n);
+}
+
+// the groups of nested cells: *ga, their number of elements *ne2, and the tiles'
+// base polygons, all from sc
+sdb_status nested_groups(const TileArgs& ta, const uint8_t* level, uint64_t n_tile, uint32_t F,
+                         uint32_t slots, Scratch& sc, cudaStream_t s, GroupArgs* ga, TileBase* tb) {
+  const uint64_t ne = ta.ne, nbp = 2 * ne + 2, top = 1ull << (2 * F);
+  uint64_t *bp, *bptmp, *bps, *b, *poff, *dT;
+  uint32_t *first, *span;
+  SDB_TRY(sc.get(&bp, nbp));
+  SDB_TRY(sc.get(&bptmp, nbp));
+  SDB_TRY(sc.get(&b, nbp));
+  SDB_TRY(sc.get(&first, ne));
+  SDB_TRY(sc.get(&span, ne));
+  SDB_TRY(sc.get(&poff, ne));
+  SDB_TRY(sc.get(&dT, 1));
+  ends_kernel<<<grid_for(ne + 1, 256), 256, 0, s>>>(ta.key, level, ne, top, bp);
+  note_launch();
+  SDB_TRY_CUDA(cudaGetLastError());
+  SDB_TRY(radix_sort_keys(bp, bptmp, nbp, 2 * (int)(F - TILE_DEPTH) + 1, s, &bps, 2 * TILE_DEPTH));
+  size_t m = 0;
+  SDB_TRY(unique_sorted(bps, nbp, b, &m, s));
+  if (m < 2 || m > 0xfffffff0ull) {
+    set_error("covering: %zu breakpoints out of range", m);
+    return SDB_EINVAL;
+  }
+  const uint32_t nint = (uint32_t)m - 1;
+  element_spans_kernel<<<grid_for(ne, 256), 256, 0, s>>>(ta.key, level, ta.info, ne, b, (uint32_t)m,
+                                                        first, span);
+  note_launch();
+  SDB_TRY_CUDA(cudaGetLastError());
+  SDB_TRY(exclusive_scan_u32(span, poff, ne, dT, s));
+  uint64_t T = 0;
+  SDB_TRY_CUDA(cudaMemcpyAsync(&T, dT, 8, cudaMemcpyDeviceToHost, s));
+  SDB_TRY_CUDA(cudaStreamSynchronize(s));
+  if (T + n_tile >= 0xffffffffull) {
+    set_error("covering: %llu (interval, polygon) pairs exceed the 32-bit list range",
+              (unsigned long long)T);
+    return SDB_ENOMEM;
+  }
+  uint32_t pbits = 1, ibits = 1;
+  while (pbits < 32 && (slots - 1) >> pbits) ++pbits;
+  while (ibits < 32 && nint >> ibits) ++ibits;
+  const uint64_t ne2 = T + n_tile;
+  uint64_t *pairs, *ptmp, *ps;
+  uint32_t *len, *count, *eoff, *loff;
+  NestedOut no{};
+  SDB_TRY(sc.get(&pairs, T));
+  SDB_TRY(sc.get(&ptmp, T));
+  SDB_TRY(sc.get(&len, nint));
+  SDB_TRY(sc.get(&count, nint));
+  SDB_TRY(sc.get(&eoff, nint));
+  SDB_TRY(sc.get(&loff, nint));
+  SDB_TRY(sc.get(&no.key, ne2));
+  SDB_TRY(sc.get(&no.end, ne2));
+  SDB_TRY(sc.get(&no.info, ne2));
+  SDB_TRY(sc.get(&no.inner, ne2));
+  SDB_TRY(sc.get(&no.base, ne));
+  SDB_TRY_CUDA(cudaMemsetAsync(len, 0, (size_t)nint * 4, s));
+  SDB_TRY_CUDA(cudaMemsetAsync(count, 0, (size_t)nint * 4, s));
+  SDB_TRY_CUDA(cudaMemsetAsync(no.inner, 0, (size_t)ne2 * 8, s));
+  ps = pairs;
+  if (T) {
+    span_pairs_kernel<<<grid_for(T, 256), 256, 0, s>>>(poff, ne, first, ta.info, T, pbits, pairs);
+    note_launch();
+    SDB_TRY_CUDA(cudaGetLastError());
+    SDB_TRY(radix_sort_keys(pairs, ptmp, T, (int)(pbits + ibits), s, &ps));
+    pair_lengths_kernel<<<grid_for(T, 256), 256, 0, s>>>(ps, T, pbits, len, count, ta.flag);
+    note_launch();
+  }
+  if (n_tile) {
+    tile_lengths_kernel<<<grid_for(n_tile, 256), 256, 0, s>>>(ta.heads, ta.n_heads, first, count);
+    note_launch();
+  }
+  SDB_TRY_CUDA(cudaGetLastError());
+  SDB_TRY(exclusive_scan<uint32_t>(len, loff, nint, nullptr, s));
+  SDB_TRY(exclusive_scan<uint32_t>(count, eoff, nint, nullptr, s));
+  if (T) {
+    base_elements_kernel<<<grid_for(T, 256), 256, 0, s>>>(ps, T, pbits, b, eoff, loff, no);
+    note_launch();
+  }
+  if (n_tile) {
+    tile_elements_kernel<<<grid_for(n_tile, 256), 256, 0, s>>>(ta.heads, ta.n_heads, first, ta.info,
+                                                              ta.inner, b, len, eoff, no);
+    note_launch();
+  }
+  SDB_TRY_CUDA(cudaGetLastError());
+  ga->key = no.key;
+  ga->info = no.info;
+  ga->inner = no.inner;
+  ga->end = no.end;
+  ga->ne = ne2;
+  *tb = TileBase{no.base, no.info};
+  return SDB_OK;
 }
 
 }  // namespace
@@ -797,7 +1055,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   uint32_t *n_heads, *info, *cells, *bits, *bbits = nullptr, *qhead;
   uint8_t *level, *code;
   uint64_t *inner, *cnt, *off, *coff, *tot;
-  unsigned int* dflag;  // nested, crowded
+  unsigned int* dflag;  // nested, crowded, overlapping inside tiles
   unsigned long long* front;
   SDB_TRY(sc.get(&heads, n_tile));
   SDB_TRY(sc.get(&n_heads, 1));
@@ -812,12 +1070,12 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   SDB_TRY(sc.get(&coff, ne));
   SDB_TRY(sc.get(&tot, 2));
   SDB_TRY(sc.get(&qhead, Q));
-  SDB_TRY(sc.get(&dflag, 2));
+  SDB_TRY(sc.get(&dflag, 3));
   SDB_TRY(sc.get(&front, 256));
   SDB_TRY(sc.get(&bits, n_tile * 32));
   if (spec.flags) SDB_TRY(sc.get(&bbits, n_tile * 32));
   SDB_TRY_CUDA(cudaMemsetAsync(n_heads, 0, 4, s));
-  SDB_TRY_CUDA(cudaMemsetAsync(dflag, 0, 8, s));
+  SDB_TRY_CUDA(cudaMemsetAsync(dflag, 0, 12, s));
   SDB_TRY_CUDA(cudaMemsetAsync(tot, 0, 16, s));
   SDB_TRY_CUDA(cudaMemsetAsync(front, 0, 256 * 8, s));
   SDB_TRY_CUDA(cudaMemsetAsync(qhead, 0xff, (size_t)Q * 4, s));
@@ -840,7 +1098,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   ta.flag = dflag;
   ta.front = front;
   GroupArgs ga{sk, info, level, inner, ne, qshift >= 64 ? ~0ull : ((1ull << qshift) - 1ull),
-               qshift, d_qs};
+               qshift, d_qs, nullptr};
   const unsigned tile_grid =
       (unsigned)std::min<uint64_t>((n_tile + WPB - 1) / WPB, (uint64_t)num_sms() * 32);
   if (ne) {
@@ -853,7 +1111,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
       tile_raster_kernel<<<tile_grid, TPB, 0, s>>>(ta);
       note_launch();
     }
-    group_count_kernel<<<grid_for(ne, 256), 256, 0, s>>>(ga, cnt, code, qhead, dflag);
+    group_count_kernel<<<grid_for(ne, 256), 256, 0, s>>>(ga, cnt, code, qhead, dflag, nullptr);
     note_launch();
     SDB_TRY_CUDA(cudaGetLastError());
     SDB_TRY(exclusive_scan<uint64_t>(cnt, off, ne, tot, s));
@@ -870,15 +1128,15 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   if (ne && spec.split)
     SDB_TRY_CUDA(cudaMemcpyAsync(hqoff.data(), dqoff, (size_t)Q * 8, cudaMemcpyDeviceToHost, s));
   uint64_t htot[2] = {0, 0};
-  unsigned int hflag[2] = {0, 0};
+  unsigned int hflag[3] = {0, 0, 0};
   std::vector<uint32_t> hhead(Q);
   std::vector<unsigned long long> hfront(256);
   SDB_TRY_CUDA(cudaMemcpyAsync(htot, tot, 16, cudaMemcpyDeviceToHost, s));
-  SDB_TRY_CUDA(cudaMemcpyAsync(hflag, dflag, 8, cudaMemcpyDeviceToHost, s));
+  SDB_TRY_CUDA(cudaMemcpyAsync(hflag, dflag, 12, cudaMemcpyDeviceToHost, s));
   SDB_TRY_CUDA(cudaMemcpyAsync(hhead.data(), qhead, (size_t)Q * 4, cudaMemcpyDeviceToHost, s));
   SDB_TRY_CUDA(cudaMemcpyAsync(hfront.data(), front, 256 * 8, cudaMemcpyDeviceToHost, s));
   SDB_TRY_CUDA(cudaStreamSynchronize(s));
-  if (hflag[0] || hflag[1]) {
+  if (hflag[1] || (Q > 1 && (hflag[0] || hflag[2]))) {
     *outcome = hflag[1] ? TileOutcome::crowded : TileOutcome::nested;
     return SDB_OK;
   }
@@ -893,6 +1151,37 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   if (ncells >= 0xffffffffull) {
     set_error("covering: %llu cells exceed the 32-bit index range", (unsigned long long)ncells);
     return SDB_ENOMEM;
+  }
+  TileBase tb{};
+  const bool nested = hflag[0] != 0;  // one query
+  if (nested) {
+    uint32_t slots = 1;
+    for (uint32_t i = 0; i < spec.NP; ++i) slots = std::max(slots, spec.pair_slot[i] + 1);
+    unsigned long long* dent;
+    SDB_TRY(sc.get(&dent, 1));
+    SDB_TRY_CUDA(cudaMemsetAsync(dent, 0, 8, s));
+    SDB_TRY(nested_groups(ta, level, n_tile, spec.q[0].F, slots, sc, s, &ga, &tb));
+    SDB_TRY(sc.get(&cnt, ga.ne));
+    SDB_TRY(sc.get(&off, ga.ne));
+    SDB_TRY(sc.get(&code, ga.ne));
+    group_count_kernel<<<grid_for(ga.ne, 256), 256, 0, s>>>(ga, cnt, code, qhead, dflag, dent);
+    note_launch();
+    SDB_TRY_CUDA(cudaGetLastError());
+    SDB_TRY(exclusive_scan<uint64_t>(cnt, off, ga.ne, tot, s));
+    unsigned long long hent = 0;
+    SDB_TRY_CUDA(cudaMemcpyAsync(htot, tot, 8, cudaMemcpyDeviceToHost, s));
+    SDB_TRY_CUDA(cudaMemcpyAsync(&hent, dent, 8, cudaMemcpyDeviceToHost, s));
+    SDB_TRY_CUDA(cudaMemcpyAsync(hflag, dflag, 12, cudaMemcpyDeviceToHost, s));
+    SDB_TRY_CUDA(cudaStreamSynchronize(s));
+    if (hflag[1]) {
+      *outcome = TileOutcome::crowded;
+      return SDB_OK;
+    }
+    if (hent >= 0xffffffffull) {
+      set_error("covering: %llu list entries exceed the 32-bit list range", hent);
+      return SDB_ENOMEM;
+    }
+    hhead[0] = 0;
   }
   // entries: the groups' ranges, plus per query its sentinel, plus the empty
   // range of a query without records
@@ -947,10 +1236,13 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   if (ne) {
     TraceScope tr1("cover.emit", s);
     const RangeOut ro{dout, qopen, qlist};
-    group_emit_kernel<<<grid_for(ne, 256), 256, 0, s>>>(ga, off, code, dextra, ro);
+    group_emit_kernel<<<grid_for(ga.ne, 256), 256, 0, s>>>(ga, off, code, dextra, ro);
     note_launch();
     if (n_tile) {
-      tile_emit_kernel<<<tile_grid, TPB, 0, s>>>(ta, off, code, dextra, ga.lomask, ro);
+      if (nested)
+        tile_emit_kernel<true><<<tile_grid, TPB, 0, s>>>(ta, off, code, dextra, ga.lomask, tb, ro);
+      else
+        tile_emit_kernel<false><<<tile_grid, TPB, 0, s>>>(ta, off, code, dextra, ga.lomask, tb, ro);
       note_launch();
     }
     SDB_TRY_CUDA(cudaGetLastError());

@@ -2,7 +2,7 @@
 covering (ranges, lists, raster cells) where the refinement ends in tiles -- at
 the shallowest levels that do and at unit cells, with boundary flags, with gaps
 between polygons, many polygons in one tile (staged, beyond the stage, and too
-many) and polygons that overlap inside tiles only."""
+many) and polygons that overlap, inside tiles only and over coarser cells."""
 import math
 
 import numpy as np
@@ -73,6 +73,29 @@ def test_overlap_inside_tiles_only(cuda, sdblib, orc):
         rings.append([(x0, y0), (x0 + 3 * s + 40, y0), (x0 + 3 * s + 40, y0 + 300), (x0, y0 + 300)])
     for flags in (0, 1):
         check(sdblib, orc, polygons(rings, B), B, F, flags)
+
+
+@pytest.mark.parametrize("flags", [0, 1])
+@pytest.mark.parametrize("layers", [2, 9, 90, 512, 520])
+def test_nested_cells(cuda, sdblib, orc, layers, flags):
+    """Polygons over one another: coarse cells of some hold coarse cells and tiles
+    of others, up to and beyond the polygons that a thread orders (slots both
+    ascending and descending with size), with tiles shared and apart."""
+    B, F = 13, 10
+    sizes = [400 + 3400 * j // layers for j in range(layers)]
+    for order in (sizes, sizes[::-1]):
+        rings = [[(4000 - r, 3900 - r), (4011 + r, 3907 - r // 2), (4000 + r, 4100 + r // 2),
+                  (3990 - r // 3, 4000 + r)] for r in order]
+        check(sdblib, orc, polygons(rings, B), B, F, flags)
+
+
+@pytest.mark.parametrize("F", [8, 11])
+def test_nested_stars(cuda, sdblib, orc, F):
+    """Stars with holes anywhere on the grid."""
+    B = 13
+    S = W.holed_stars(np.random.default_rng(F), 12, B, radius=(2 ** 8, 2 ** 10))
+    for flags in (0, 1):
+        check(sdblib, orc, S, B, F, flags)
 
 
 def test_records_and_viewport_clip(cuda, sdblib, orc):
