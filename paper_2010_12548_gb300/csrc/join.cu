@@ -912,13 +912,31 @@ sdb_status launch_multi_t(const MultiArgs& M, cudaStream_t s, bool early) {
 // One pass over the points for up to MULTI coverings of the same polygons with
 // cell tables (an eps sweep): each point is read once; a combined top level in
 // shared memory -- a top cell whose payload is the same single polygon in
-// every covering -- answers it for all coverings at once; otherwise each
-// covering's table and second level answer it in turn.  Points in mixed cells
-// of any covering wait in one per-warp queue (the covering's number in the top
-// two bits of the queued cell index) and are searched 32 at a time, so the
-// kernel holds one copy of the window search per queue drain, not one per
-// covering and point (an unrolled form spent two thirds of its cycles waiting
-// for instructions).
+// every covering -- answers it for all coverings at once, into one common
+// accumulator set that the flush adds to every covering.  Other points are queued
+// per warp and, 32 at a time, go through each covering's table and second level in
+// turn.  Points in mixed cells of any covering wait in a second per-warp queue (the
+// covering's number in the top two bits of the queued cell index) and are searched
+// 32 at a time, so the kernel holds one copy of the table code and one of the
+// window search (an unrolled form spent two thirds of its cycles waiting for
+// instructions).
+//
+// Points that the combined top level does not answer are one in six on the benchmark's
+// coverings, spread over almost every warp: from the queue the table code runs once
+// per 32 such points instead of once per 32 points, with all coverings' reads in
+// flight together.  Each such read holds a line of L1 until it is there, so one
+// block of 1024 threads, whose shared memory leaves L1 92 KB, is far better than two of
+// 512, which leave it 28 KB: four coverings (eps 2^12 .. 2^6) of 263 zones over 30M
+// points, 1024 x 1: 210 us; 512 x 2: 334 us; two 768-thread blocks without the queue
+// and the common set: 348 us.  One block also has room for the accumulators of more
+// polygons; three coverings over 10M points, that form -> this one: 700 polygons
+// (which it added in global memory) 978 -> 180 us, 1500: 1179 -> 440, without sums
+// 2500: 496 -> 270; beyond, in global memory, 6000 with sums: 784 -> 688.
+struct AskQueue {
+  uint32_t x[QCAP], y[QCAP];
+  int32_t a[QCAP];
+};
+
 struct SweepArgs {
   JoinArgs c[MULTI];       // per covering: its table, lookup and outputs
   uint32_t E;
@@ -956,15 +974,28 @@ __global__ void sweep_top_kernel(TopSet t, uint32_t nt, uint8_t* __restrict__ ou
 constexpr uint32_t SWEEP_E_SHIFT = 30;
 static_assert(MULTI <= 4 && TAB_MIXED_MAX < (1u << SWEEP_E_SHIFT), "covering bits");
 
+constexpr int SWEEP_THREADS = 1024;
+constexpr int SWEEP_WARPS = SWEEP_THREADS / 32;
+constexpr uint32_t SWEEP_FLUSH_TILES = 15;
+static_assert((uint64_t)(SWEEP_FLUSH_TILES * SWEEP_THREADS * 4 + SWEEP_WARPS * 2 * (QCAP - 1)) *
+                      65535u < (1ull << 32),
+              "low-half counter could wrap");
+static_assert((uint64_t)(SWEEP_FLUSH_TILES * SWEEP_THREADS * 4 + SWEEP_WARPS * 2 * (QCAP - 1)) *
+                      32768u < (1ull << 31),
+              "high-half counter could wrap");
+
 // shared-memory layout of the sweep: the compact cell-id table, the per-warp
-// queues, MULTI accumulator sets, then (with a combined top level) its bytes
-// and palette
+// queues of mixed-cell points and of points for the tables, MULTI accumulator sets
+// and the common one, then (with a combined top level) its bytes and palette
 __host__ __device__ constexpr size_t sweep_queue_off() { return HILBERT3_COMPACT_BYTES; }
+__host__ __device__ constexpr size_t sweep_ask_off() {
+  return sweep_queue_off() + (size_t)SWEEP_WARPS * QCAP * sizeof(QEnt);
+}
 __host__ __device__ constexpr size_t sweep_acc_off() {
-  return sweep_queue_off() + (size_t)(TOP_THREADS / 32) * QCAP * sizeof(QEnt);
+  return sweep_ask_off() + (size_t)SWEEP_WARPS * sizeof(AskQueue);
 }
 __host__ __device__ constexpr size_t sweep_top_off(size_t P, bool SUM) {
-  return (sweep_acc_off() + MULTI * acc_bytes(P, SUM, false) + 15) & ~(size_t)15;
+  return (sweep_acc_off() + (MULTI + 1) * acc_bytes(P, SUM, false) + 15) & ~(size_t)15;
 }
 
 template <int LOOKUP, bool SMEM, bool SUM>
@@ -977,19 +1008,50 @@ __device__ __forceinline__ void sweep_resolve(QEnt Q, const uint32_t* s_tab,
                                           s_args[e]);
 }
 
+// every covering's accumulators and the common ones into the outputs, cleared
+template <bool SUM>
+__device__ void sweep_flush(unsigned char* accb, size_t ab, uint32_t P, uint32_t E,
+                            const JoinArgs* s_args) {
+  const Acc com = acc_at<SUM, false>(accb + MULTI * ab, P);
+  for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) {
+    const uint32_t cc = com.cnt[i];
+    long long ct = 0;
+    com.cnt[i] = 0;
+    if (SUM) {
+      ct = (long long)com.hi[i] * 65536 + (long long)com.lo[i];
+      com.lo[i] = 0;
+      com.hi[i] = 0;
+    }
+    for (uint32_t e = 0; e < E; ++e) {
+      const Acc acc = acc_at<SUM, false>(accb + e * ab, P);
+      const unsigned long long c = (unsigned long long)cc + acc.cnt[i];
+      if (!c) continue;
+      atomicAdd(&s_args[e].count[i], c);
+      acc.cnt[i] = 0;
+      if (SUM) {
+        const long long tot = ct + (long long)acc.hi[i] * 65536 + (long long)acc.lo[i];
+        atomicAdd(&s_args[e].sum[i], (unsigned long long)tot);
+        acc.lo[i] = 0;
+        acc.hi[i] = 0;
+      }
+    }
+  }
+}
+
 template <int LOOKUP, bool SMEM, bool SUM>
-__global__ __launch_bounds__(TOP_THREADS, TOP_BLOCKS) void sweep_kernel(
+__global__ __launch_bounds__(SWEEP_THREADS, 1) void sweep_kernel(
     const __grid_constant__ SweepArgs S) {
   extern __shared__ __align__(16) unsigned char smem[];
   // the coverings' arguments, read with a covering index known only at run time
   __shared__ JoinArgs s_args[MULTI];
-  constexpr int TPB = TOP_THREADS;
+  constexpr int TPB = SWEEP_THREADS;
   const JoinArgs& A0 = S.c[0];
   const uint32_t E = S.E;
   const size_t P = SMEM ? A0.P : 0;
   const size_t ab = acc_bytes(P, SUM, false);
   uint32_t* s_tab = reinterpret_cast<uint32_t*>(smem);
   QEnt* s_q = reinterpret_cast<QEnt*>(smem + sweep_queue_off()) + (threadIdx.x >> 5) * QCAP;
+  AskQueue* s_ask = reinterpret_cast<AskQueue*>(smem + sweep_ask_off()) + (threadIdx.x >> 5);
   unsigned char* accb = smem + sweep_acc_off();
   uint8_t* s_top = smem + sweep_top_off(P, SUM);
   uint32_t* s_pal = reinterpret_cast<uint32_t*>(s_top + ((size_t)1 << (2 * S.top_lev)));
@@ -998,7 +1060,7 @@ __global__ __launch_bounds__(TOP_THREADS, TOP_BLOCKS) void sweep_kernel(
     static_assert(sizeof(JoinArgs) % 4 == 0, "word copy");
     const uint32_t* src = reinterpret_cast<const uint32_t*>(S.c);
     uint32_t* dst = reinterpret_cast<uint32_t*>(s_args);
-    for (uint32_t i = threadIdx.x; i < E * (sizeof(JoinArgs) / 4); i += TPB) dst[i] = src[i];
+    for (uint32_t i = threadIdx.x; i < MULTI * (sizeof(JoinArgs) / 4); i += TPB) dst[i] = src[i];
   }
   if (S.top) {
     const uint4* src = reinterpret_cast<const uint4*>(S.top);
@@ -1007,14 +1069,63 @@ __global__ __launch_bounds__(TOP_THREADS, TOP_BLOCKS) void sweep_kernel(
     for (uint32_t i = threadIdx.x; i < TOP_PALETTE; i += TPB) s_pal[i] = __ldg(S.pal + i);
   }
   if (SMEM)
-    for (uint32_t e = 0; e < E; ++e) acc_zero<SUM, false>(acc_at<SUM, false>(accb + e * ab, P), (uint32_t)P);
+    for (uint32_t e = 0; e <= MULTI; ++e) acc_zero<SUM, false>(acc_at<SUM, false>(accb + e * ab, P), (uint32_t)P);
   grid_wait();
   __syncthreads();
+  const Acc common = acc_at<SUM, false>(accb + MULTI * ab, P);
 
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
-  uint32_t qn = 0;  // entries in this warp's queue (warp-uniform)
+  uint32_t qn = 0, an = 0;  // entries in this warp's queues (warp-uniform)
   const uint32_t gmask = ~((1u << A0.B) - 1u);
+
+  // A batch of queued points through every covering's tables: the coverings' entries
+  // are read side by side, then their second levels, then the payloads are added and
+  // the mixed cells queued (as many coverings' as fit before a window search is due).
+  auto ask_all = [&](bool on, uint32_t x, uint32_t y, int32_t a) {
+    uint32_t en[MULTI];
+#pragma unroll
+    for (int e = 0; e < MULTI; ++e) {
+      const JoinArgs& A = s_args[e];
+      en[e] = on && e < (int)E ? __ldg(A.tab + (((y >> A.txy) << A.tlev) | (x >> A.txy))) : NONE;
+    }
+#pragma unroll
+    for (int e = 0; e < MULTI; ++e) {
+      const JoinArgs& A = s_args[e];
+      if (en[e] >= TAB_MIXED && en[e] != NONE && A.sub) {
+        const uint32_t smask = (1u << A.s2) - 1u;
+        en[e] = __ldg(A.sub + (((uint64_t)(en[e] & ~TAB_MIXED) << (2 * A.s2)) |
+                               (((y >> A.txy2) & smask) << A.s2) | ((x >> A.txy2) & smask)));
+      }
+    }
+    uint32_t pend = 0;  // coverings whose mixed cells wait for room in the queue
+#pragma unroll
+    for (int e = 0; e < MULTI; ++e) {
+      const bool mix = en[e] >= TAB_MIXED && en[e] != NONE;
+      if (!mix) add_pay<SMEM, SUM, false>(en[e], a, acc_at<SUM, false>(accb + e * ab, P), s_args[e]);
+      if (__any_sync(FULL, mix)) pend |= 1u << e;
+    }
+    while (pend) {
+#pragma unroll
+      for (int e = 0; e < MULTI; ++e) {
+        const bool mix = en[e] >= TAB_MIXED && en[e] != NONE;
+        const uint32_t bal = __ballot_sync(FULL, mix);
+        if (!((pend >> e) & 1u) || qn + __popc(bal) > QCAP) continue;
+        pend &= ~(1u << e);
+        if (mix)
+          s_q[qn + __popc(bal & lt)] = QEnt{x, y, (en[e] & ~TAB_MIXED) | ((uint32_t)e << SWEEP_E_SHIFT), a};
+        qn += __popc(bal);
+      }
+      if (qn >= 32) {  // a full warp of held-back points: search their windows
+        __syncwarp();
+        qn -= 32;
+        const QEnt Q = s_q[qn + lane];
+        __syncwarp();
+        sweep_resolve<LOOKUP, SMEM, SUM>(Q, s_tab, accb, ab, P, s_args);
+      }
+    }
+  };
+
   const uint64_t per_tile = (uint64_t)TPB * 4;
   const uint64_t ntiles = (A0.n + per_tile - 1) / per_tile;
   uint32_t since_flush = 0;
@@ -1043,13 +1154,9 @@ __global__ __launch_bounds__(TOP_THREADS, TOP_BLOCKS) void sweep_kernel(
         as[q] = (SUM && ok[q]) ? A0.attr[e0 + q] : 0;
       }
     }
-    if (!SUM) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) as[q] = 0;
-    }
-    // the combined top level: a payload shared by every covering, NONE, or ask
+    // the combined top level: a payload shared by every covering, none, or ask
     bool ask[4];
-    uint32_t pc[4];
+    uint32_t bal[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const bool in = ok[q] && !((xs[q] | ys[q]) & gmask);
@@ -1057,84 +1164,85 @@ __global__ __launch_bounds__(TOP_THREADS, TOP_BLOCKS) void sweep_kernel(
                             : (S.top ? s_top[((ys[q] >> S.top_xy) << S.top_lev) | (xs[q] >> S.top_xy)]
                                      : TOP_ASK);
       ask[q] = v == TOP_ASK;
-      pc[q] = v < TOP_NONE ? s_pal[v] : NONE;
-    }
-    // covering by covering (a loop the compiler keeps rolled): the table
-    // entries of the points the top level did not answer, all four gathers in
-    // flight, then the second level; mixed cells go to the queue
-#pragma unroll 1
-    for (uint32_t e = 0; e < E; ++e) {
-      const JoinArgs& A = s_args[e];
-      const Acc acc = acc_at<SUM, false>(accb + e * ab, P);
-      uint32_t en[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        en[q] = ask[q] ? __ldg(A.tab + (((ys[q] >> A.txy) << A.tlev) | (xs[q] >> A.txy))) : pc[q];
-      if (A.sub) {
-        const uint32_t smask = (1u << A.s2) - 1u;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (ask[q] && en[q] >= TAB_MIXED && en[q] != NONE)
-            en[q] = __ldg(A.sub + (((uint64_t)(en[q] & ~TAB_MIXED) << (2 * A.s2)) |
-                                   (((ys[q] >> A.txy2) & smask) << A.s2) |
-                                   ((xs[q] >> A.txy2) & smask)));
+      bal[q] = __ballot_sync(FULL, ask[q]);
+      if (v < TOP_NONE) {
+        const uint32_t p = s_pal[v];
+        if (SMEM) {
+          add_one<true, SUM, false>(p, as[q], 0u, common, A0);
+        } else {
+          for (uint32_t e = 0; e < E; ++e) add_one<false, SUM, false>(p, as[q], 0u, common, s_args[e]);
+        }
       }
+    }
+    uint32_t pend = 15u;
+    do {  // as many of the four as fit before a batch is due
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const bool mix = ask[q] && en[q] >= TAB_MIXED && en[q] != NONE;
-        const uint32_t bal = __ballot_sync(FULL, mix);
-        if (mix) {
-          QEnt& Q = s_q[qn + __popc(bal & lt)];
-          Q.x = xs[q];
-          Q.y = ys[q];
-          Q.m = (en[q] & ~TAB_MIXED) | (e << SWEEP_E_SHIFT);
-          Q.a = as[q];
-        } else {
-          add_pay<SMEM, SUM, false>(en[q], as[q], acc, A);
+        if (!((pend >> q) & 1u) || an + __popc(bal[q]) > QCAP) continue;
+        pend &= ~(1u << q);
+        if (ask[q]) {
+          const uint32_t at = an + __popc(bal[q] & lt);
+          s_ask->x[at] = xs[q];
+          s_ask->y[at] = ys[q];
+          if (SUM) s_ask->a[at] = as[q];
         }
-        qn += __popc(bal);
-        if (qn >= 32) {  // a full warp of held-back points: search their windows
-          __syncwarp();
-          qn -= 32;
-          const QEnt Q = s_q[qn + lane];
-          __syncwarp();
-          sweep_resolve<LOOKUP, SMEM, SUM>(Q, s_tab, accb, ab, P, s_args);
-        }
+        an += __popc(bal[q]);
       }
-    }
-    if (SMEM && ++since_flush == TOP_FLUSH_TILES) {
+      if (an >= 32) {
+        __syncwarp();
+        an -= 32;
+        const uint32_t x = s_ask->x[an + lane], y = s_ask->y[an + lane];
+        const int32_t a = SUM ? s_ask->a[an + lane] : 0;
+        __syncwarp();
+        ask_all(true, x, y, a);
+      }
+    } while (pend || an >= 32);
+    if (SMEM && ++since_flush == SWEEP_FLUSH_TILES) {
       since_flush = 0;
       __syncthreads();
-      for (uint32_t e = 0; e < E; ++e) flush_acc<SUM, false>(acc_at<SUM, false>(accb + e * ab, P), s_args[e]);
+      sweep_flush<SUM>(accb, ab, (uint32_t)P, E, s_args);
       __syncthreads();
     }
   }
-  __syncwarp();  // the rest of the queue
+  __syncwarp();  // the rest of the queues
+  {
+    const bool on = lane < an;
+    const uint32_t x = on ? s_ask->x[lane] : 0u, y = on ? s_ask->y[lane] : 0u;
+    const int32_t a = SUM && on ? s_ask->a[lane] : 0;
+    ask_all(on, x, y, a);
+  }
+  __syncwarp();
   if (lane < qn) sweep_resolve<LOOKUP, SMEM, SUM>(s_q[lane], s_tab, accb, ab, P, s_args);
   if (SMEM) {
     __syncthreads();
-    for (uint32_t e = 0; e < E; ++e) flush_acc<SUM, false>(acc_at<SUM, false>(accb + e * ab, P), s_args[e]);
+    sweep_flush<SUM>(accb, ab, (uint32_t)P, E, s_args);
   }
 }
 
+size_t sweep_smem(const SweepArgs& S, size_t P, bool SUM) {
+  size_t smem = sweep_top_off(P, SUM);
+  if (S.top) smem += ((size_t)1 << (2 * S.top_lev)) + 4 * TOP_PALETTE;
+  return (smem + 15) & ~(size_t)15;
+}
+// accumulators in shared memory as long as one block holds them
+constexpr size_t SWEEP_SMEM_MAX = 220 * 1024;
+
 template <int LOOKUP, bool SMEM, bool SUM>
 sdb_status launch_sweep_t(const SweepArgs& S, cudaStream_t s, bool early) {
-  size_t smem = sweep_top_off(SMEM ? S.c[0].P : 0, SUM);
-  if (S.top) smem += ((size_t)1 << (2 * S.top_lev)) + 4 * TOP_PALETTE;
-  smem = (smem + 15) & ~(size_t)15;
+  const size_t smem = sweep_smem(S, SMEM ? S.c[0].P : 0, SUM);
   auto kern = sweep_kernel<LOOKUP, SMEM, SUM>;
   if (smem > 48 * 1024)
     SDB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   static OccupancyCache cache;
-  SDB_TRY(cache.get(reinterpret_cast<const void*>(kern), TOP_THREADS, smem, &per_sm));
+  SDB_TRY(cache.get(reinterpret_cast<const void*>(kern), SWEEP_THREADS, smem, &per_sm));
   SDB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                     carveout_pct((size_t)per_sm * (smem + sizeof(SweepArgs::c) + 1024))));
   uint64_t blocks = (uint64_t)num_sms() * per_sm;
-  const uint64_t need = (S.c[0].n + 4 * TOP_THREADS - 1) / (4 * TOP_THREADS);
+  const uint64_t need = (S.c[0].n + 4 * SWEEP_THREADS - 1) / (4 * SWEEP_THREADS);
   if (blocks > need) blocks = need > 0 ? need : 1;
   TraceScope tr("join", s);
-  return launch_after(kern, (unsigned)blocks, TOP_THREADS, smem, s, early, S);
+  return launch_after(kern, (unsigned)blocks, SWEEP_THREADS, smem, s, early, S);
 }
 
 template <bool RANGE>
@@ -1382,8 +1490,8 @@ sdb_status launch_join_multi(const uint32_t* x, const uint32_t* y, const int32_t
         S.top_xy = covs[e0]->B - Lt;
       }
       SDB_TRY(launch_zero(z, s));  // right before the sweep, which starts beside it
-      const bool smem = (uint64_t)MULTI * P <= SMEM_POLYS;
       const bool has_sum = sum != nullptr;
+      const bool smem = sweep_smem(S, P, has_sum) <= SWEEP_SMEM_MAX;
       sdb_status st;
       if (lookup == SDB_LOOKUP_TABLE)
         st = smem ? (has_sum ? launch_sweep_t<3, true, true>(S, s, zero) : launch_sweep_t<3, true, false>(S, s, zero))
