@@ -57,9 +57,6 @@ TABLE_BITS = 22  # its first level, the cell table: 2^22 buckets (16 MB), fewer 
 # profiles/join_kernel_table_learned_eps64_zones263_mobility20M.txt
 JOIN_FINEST_TRAFFIC = {"table_learned": {"eps": 64, "leaf_bits": 16, "root_bits": 0,
                                          "bytes_per_point": 13.934}}
-# DRAM bytes of one launch of radix_scatter_kernel (a keys-only pass) in the
-# sweep's record sort: profiles/radix_scatter_kernel_sweep_zones263.txt
-SCATTER_TRAFFIC = {"records": 117_378_603, "passes": 5, "bytes": 1.8926e9}
 
 
 def leaf_bits_for(n_ranges: int) -> int:
@@ -577,23 +574,6 @@ def main():
                        "avg_launch_ms": join_ms[-1], "algorithmic_bytes_per_point": per_pt,
                        "algorithmic_bytes_per_launch": per_pt * N,
                        "profile": "profiles/join_kernel_table_learned_eps64_zones263_mobility20M.txt"}
-    # the record sort's scatter inside the full step (one launch per pass over
-    # all records): 8 B read + 8 B written per record and pass, 8 + 12 B in the
-    # last pass (keys and values apart)
-    recs = sum(i.n_cells for i in infos)
-    sc_n, sc_ms = trace.get("sort.scatter", (0, 0.0))
-    if sc_n:
-        passes = sc_n / fs_reps
-        sc_bytes = recs * (16 * (passes - 1) + 20) / passes
-        sc_avg = sc_ms / sc_n
-        ach = sc_bytes / (sc_avg / 1e3) / 1e9
-        T = SCATTER_TRAFFIC
-        res["roofline_radix_scatter"] = {
-            "kernel": "radix_scatter_kernel (%d records)" % recs, "bound": "hbm",
-            "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
-            "peak_kind": peak_kind, "avg_launch_ms": sc_avg, "launches_per_step": passes,
-            "traffic": T["bytes"] if T and T["records"] == recs and T["passes"] == passes
-            else None, "algorithmic_bytes_per_launch": sc_bytes}
     for c in covs:
         c.free()
     covs = []
