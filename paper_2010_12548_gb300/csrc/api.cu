@@ -3,6 +3,7 @@
 // host-buffer join that streams point chunks through the device.
 #include "sdb_internal.cuh"
 
+#include <algorithm>
 #include <atomic>
 #include <cstring>
 #include <mutex>
@@ -707,6 +708,8 @@ sdb_status sdb_join_aggregate_host(const uint32_t* h_x, const uint32_t* h_y, con
   if (lookup == SDB_LOOKUP_LEARNED || lookup == SDB_LOOKUP_TABLE_LEARNED)
     for (uint32_t c = 0; c < n_covs; ++c)
       SDB_TRY_CUDA(cudaMemsetAsync(covs[c]->fallbacks, 0, sizeof(unsigned long long), s));
+  // Coverings of a sweep are joined in one pass over the chunk where that is faster
+  // (20M points, four eps: 1400 -> 1280 us, of which the copies take 1150).
   // points per chunk: the joins of the last chunk are not hidden by a copy,
   // but smaller chunks issue more launches per call, and a host whose API calls
   // are slow then falls behind the copies (2^22: 6.00 ms on some hosts, 7.81 on
@@ -744,9 +747,15 @@ sdb_status sdb_join_aggregate_host(const uint32_t* h_x, const uint32_t* h_y, con
       st = cuda_status(e, "chunk copy", __FILE__, __LINE__);
       break;
     }
-    for (uint32_t k = 0; k < n_covs && st == SDB_OK; ++k)
-      st = launch_join(dx[b], dy[b], da[b], m, covs[k], lookup, d_cnt + (size_t)k * P,
-                       d_sum ? d_sum + (size_t)k * P : nullptr, s, false);
+    for (uint32_t k = 0; k < n_covs && st == SDB_OK;) {
+      uint32_t g = std::min(n_covs - k, 4u);  // coverings joined in one pass
+      if (!sweep_pays(covs + k, g, lookup, m)) g = 1;
+      uint64_t* cnt = d_cnt + (size_t)k * P;
+      int64_t* sum = d_sum ? d_sum + (size_t)k * P : nullptr;
+      st = g > 1 ? launch_join_multi(dx[b], dy[b], da[b], m, covs + k, g, lookup, cnt, sum, s, false)
+                 : launch_join(dx[b], dy[b], da[b], m, covs[k], lookup, cnt, sum, s, false);
+      k += g;
+    }
     if (st == SDB_OK && cudaEventRecord(done[b], s) != cudaSuccess)
       st = cuda_status(cudaGetLastError(), "event record", __FILE__, __LINE__);
   }

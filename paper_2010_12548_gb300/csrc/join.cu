@@ -1224,8 +1224,12 @@ size_t sweep_smem(const SweepArgs& S, size_t P, bool SUM) {
   if (S.top) smem += ((size_t)1 << (2 * S.top_lev)) + 4 * TOP_PALETTE;
   return (smem + 15) & ~(size_t)15;
 }
-// accumulators in shared memory as long as one block holds them
+// accumulators in shared memory as long as one block holds them (about 1690 polygons
+// with sums, 5080 without)
 constexpr size_t SWEEP_SMEM_MAX = 220 * 1024;
+// polygons up to which the pass is taken in place of separate joins (see sweep_pays):
+// the sets of more leave L1 too little for the tables' reads
+constexpr uint32_t SWEEP_PAYS_POLYS = 512;
 
 template <int LOOKUP, bool SMEM, bool SUM>
 sdb_status launch_sweep_t(const SweepArgs& S, cudaStream_t s, bool early) {
@@ -1434,6 +1438,16 @@ JoinArgs join_args(const uint32_t* x, const uint32_t* y, const int32_t* attr, ui
   return A;
 }
 }  // namespace
+
+bool sweep_pays(const sdb_covering* const* covs, uint32_t E, int lookup, uint64_t n) {
+  if (lookup != SDB_LOOKUP_TABLE && lookup != SDB_LOOKUP_TABLE_LEARNED) return false;
+  if (E < 2 || E > MULTI || n < (1u << 16) || covs[0]->P > SWEEP_PAYS_POLYS) return false;
+  for (uint32_t e = 0; e < E; ++e)
+    if (!covs[e]->top || covs[e]->top_level != covs[0]->top_level || covs[e]->P != covs[0]->P ||
+        covs[e]->B != covs[0]->B)
+      return false;
+  return true;
+}
 
 sdb_status launch_join_multi(const uint32_t* x, const uint32_t* y, const int32_t* attr,
                              uint64_t n, const sdb_covering* const* covs, uint32_t E, int lookup,

@@ -447,6 +447,11 @@ sdb_status check_lookup(const sdb_covering* cov, int lookup);
 sdb_status launch_join_multi(const uint32_t* x, const uint32_t* y, const int32_t* attr,
                              uint64_t n, const sdb_covering* const* covs, uint32_t E, int lookup,
                              uint64_t* count, int64_t* sum, cudaStream_t s, bool zero);
+// whether that pass beats one join per covering for n points: through cell tables
+// with a combined top level, few polygons.  Joins -> pass, us: 263 zones, four
+// coverings, 1e5 points 66 -> 28, 1.7e7 265 -> 137; two, 27 -> 24 and 134 -> 106.
+// 1500 polygons, three coverings: 1e5 66 -> 63, but 1.7e7 507 -> 642.
+bool sweep_pays(const sdb_covering* const* covs, uint32_t E, int lookup, uint64_t n);
 // bcount / bsum / babs (nullable; the covering must be flagged): result-range
 // partials of Sec. 6 (boundary count, boundary attribute sum, sum of magnitudes)
 sdb_status launch_join(const uint32_t* x, const uint32_t* y, const int32_t* attr, uint64_t n,

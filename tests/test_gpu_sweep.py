@@ -48,3 +48,31 @@ def test_sweep_equals_separate_joins(cuda, sdblib, P, bits):
                 assert torch.equal(cnt, one_c[4 - E:]), (at, m, E)
     for c in covs:
         c.free()
+
+
+@pytest.mark.parametrize("n", [65_535, 65_537, 2 ** 24 + 65_000])
+def test_host_join_of_several_coverings(cuda, sdblib, n):
+    """Host-buffer joins of one to five coverings, some sharing a pass and some not
+    (one without a top level, a chunk too small for a pass), equal device joins."""
+    torch = cuda
+    B = 18
+    T = W.voronoi_tiling(np.random.default_rng(7), 90, B, nverts=(4, 16))
+    covs = sdblib.build_coverings(T, B, [1024, 256, 64, 16])
+    covs.append(sdblib.build_covering(T, B, 32))
+    for i, c in enumerate(covs):
+        sdblib.covering_build_table(c, 10 if i == 4 else 18)
+    rng = np.random.default_rng(n)
+    x, y = (rng.integers(0, 2 ** B + 99, n, dtype=np.uint32) for _ in range(2))
+    a = rng.integers(-2 ** 31, 2 ** 31, n).astype(np.int32)
+    dx, dy, da = (torch.from_numpy(v.view(np.int32)).cuda() for v in (x, y, a))
+    want_c = torch.zeros((5, T.n), dtype=torch.int64, device="cuda")
+    want_s = torch.zeros_like(want_c)
+    for e, c in enumerate(covs):
+        sdblib.join_aggregate(dx, dy, da, c, sdblib.LOOKUP_TABLE, want_c[e], want_s[e])
+    want_c, want_s = want_c.cpu().numpy(), want_s.cpu().numpy()
+    for pick in ([0], [1, 2], [3, 1, 0], [0, 1, 2, 3], [0, 1, 2, 3, 3], [4, 2], [0, 1, 2, 3, 4]):
+        cnt, sm = sdblib.join_aggregate_host(x, y, a, [covs[i] for i in pick], sdblib.LOOKUP_TABLE)
+        assert np.array_equal(np.asarray(cnt).astype(np.int64), want_c[pick]), pick
+        assert np.array_equal(np.asarray(sm), want_s[pick]), pick
+    for c in covs:
+        c.free()
