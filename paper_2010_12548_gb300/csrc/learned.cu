@@ -110,6 +110,61 @@ __global__ void leaf_below_kernel(const uint64_t* __restrict__ start, uint64_t R
   for (uint32_t l = from; l <= lam; ++l) below[l] = (uint32_t)i;
 }
 
+__device__ __forceinline__ float to_float(uint32_t v) { return __uint2float_rn(v); }
+__device__ __forceinline__ float to_float(uint64_t v) { return __ull2float_rn(v); }
+__device__ __forceinline__ void to_floor(float v, int32_t* o) { *o = __float2int_rd(v); }
+__device__ __forceinline__ void to_floor(float v, int64_t* o) { *o = __float2ll_rd(v); }
+
+// The line and window of the leaf [b0, b1) over the ranges [first, first + n).  Bound
+// by the conversions between integers and FP32: a leaf narrower than 2^32 ids holds
+// fewer ranges than that, and 32-bit integers give the same floats and the same clamped
+// positions as 64-bit ones (U unsigned, S signed) in 207 instead of 614 us for the
+// 263-zone sweep's 27M ranges.  (Four loads in flight per lane changed nothing: 623.)
+template <class U, class S>
+__device__ __forceinline__ void fit_leaf(const uint64_t* __restrict__ start, uint64_t first,
+                                         uint64_t n, uint64_t b0, uint64_t b1, LeafRec* lr,
+                                         long long* lo, long long* hi) {
+  const U nn = (U)n;
+  const uint64_t* __restrict__ s = start + first;
+  // pass 1: means; pass 2: centred moments (FP32: the fit only shapes the
+  // windows, which come from the lookup's own arithmetic in pass 3)
+  float sx = 0.f, sy = 0.f;
+  for (U i = threadIdx.x & 31; i < nn; i += 32) {
+    sx += to_float((U)((s[i] > b0 ? s[i] : b0) - b0));
+    sy += to_float(i);
+  }
+  const float inv_n = 1.0f / to_float(nn);
+  const float mx = warp_sum(sx) * inv_n, my = warp_sum(sy) * inv_n;
+  float sxx = 0.f, sxy = 0.f;
+  for (U i = threadIdx.x & 31; i < nn; i += 32) {
+    const float dx = to_float((U)((s[i] > b0 ? s[i] : b0) - b0)) - mx, dy = to_float(i) - my;
+    sxx = fmaf(dx, dx, sxx);
+    sxy = fmaf(dx, dy, sxy);
+  }
+  sxx = warp_sum(sxx);
+  sxy = warp_sum(sxy);
+  const float slope = (sxx > 0.f && sxy > 0.f) ? sxy / sxx : 0.f;
+  lr->a = slope;
+  lr->b = my - slope * mx;
+  // pass 3: error window with the lookup's own FP32 arithmetic (leaf_predict,
+  // positions counted from the leaf's first)
+  auto predict = [&](U x) {
+    S p;
+    to_floor(__fmaf_rn(lr->a, to_float(x), lr->b), &p);
+    p = p < 0 ? 0 : p;
+    return p > (S)(nn - 1) ? (S)(nn - 1) : p;
+  };
+  S ehi = 0, elo = 0;
+  for (U i = threadIdx.x & 31; i < nn; i += 32) {
+    const uint64_t lo_h = s[i] > b0 ? s[i] : b0, hi_h = (s[i + 1] < b1 ? s[i + 1] : b1) - 1;
+    const S up = (S)i - predict((U)(lo_h - b0)), dn = predict((U)(hi_h - b0)) - (S)i;
+    ehi = up > ehi ? up : ehi;
+    elo = dn > elo ? dn : elo;
+  }
+  *hi = warp_max(ehi);
+  *lo = warp_max(elo);
+}
+
 // one warp per leaf: centred least squares (FP32), error window
 __global__ void leaf_fit_kernel(const uint64_t* __restrict__ start, uint64_t R,
                                 const uint64_t* __restrict__ base,
@@ -139,41 +194,11 @@ __global__ void leaf_fit_kernel(const uint64_t* __restrict__ start, uint64_t R,
   lr.first = (uint32_t)first;
   lr.last = (uint32_t)last;
   const uint64_t n = last - first + 1;
-  // pass 1: means; pass 2: centred moments (FP32: the fit only shapes the
-  // windows, which come from the lookup's own arithmetic in pass 3)
-  float sx = 0.f, sy = 0.f;
-  for (uint64_t i = first + lane; i <= last; i += 32) {
-    const uint64_t s = start[i] > b0 ? start[i] : b0;
-    sx += __ull2float_rn(s - b0);
-    sy += (float)(i - first);
-  }
-  const float inv_n = 1.0f / (float)n;
-  const float mx = warp_sum(sx) * inv_n, my = warp_sum(sy) * inv_n;
-  float sxx = 0.f, sxy = 0.f;
-  for (uint64_t i = first + lane; i <= last; i += 32) {
-    const uint64_t s = start[i] > b0 ? start[i] : b0;
-    const float dx = __ull2float_rn(s - b0) - mx, dy = (float)(i - first) - my;
-    sxx = fmaf(dx, dx, sxx);
-    sxy = fmaf(dx, dy, sxy);
-  }
-  sxx = warp_sum(sxx);
-  sxy = warp_sum(sxy);
-  const float slope = (sxx > 0.f && sxy > 0.f) ? sxy / sxx : 0.f;
-  lr.a = slope;
-  lr.b = my - slope * mx;
-  // pass 3: error window with the lookup's own FP32 arithmetic
   long long ehi = 0, elo = 0;
-  for (uint64_t i = first + lane; i <= last; i += 32) {
-    uint64_t lo_h = start[i] > b0 ? start[i] : b0;
-    uint64_t hi_h = (start[i + 1] < b1 ? start[i + 1] : b1) - 1;
-    long long plo = (long long)leaf_predict(lr, lo_h);
-    long long phi = (long long)leaf_predict(lr, hi_h);
-    long long up = (long long)i - plo, dn = phi - (long long)i;
-    ehi = up > ehi ? up : ehi;
-    elo = dn > elo ? dn : elo;
-  }
-  ehi = warp_max(ehi);
-  elo = warp_max(elo);
+  if (b1 - b0 <= 0xffffffffull)
+    fit_leaf<uint32_t, int32_t>(start, first, n, b0, b1, &lr, &elo, &ehi);
+  else
+    fit_leaf<uint64_t, int64_t>(start, first, n, b0, b1, &lr, &elo, &ehi);
   const long long CAP = 1ll << 30;
   lr.errhi = (int32_t)(ehi > CAP ? CAP : ehi);
   lr.errlo = (int32_t)(elo > CAP ? CAP : elo);
