@@ -356,9 +356,11 @@ sdb_status sdb_join_aggregate_host_noalloc(const uint32_t *h_x, const uint32_t *
  * scanline rasterisation), and the masked pixels' aggregates are summed per
  * polygon.  No covering and no precomputation; the result equals
  * sdb_join_aggregate with a covering of the same polygons and eps.  The canvas
- * of 4^F pixels is processed in tiles of 2^tile_bits x 2^tile_bits pixels
- * (0 = 2^13), as many at a time as fit in 8 GiB (16 bytes per pixel), so the
- * cost grows with the canvas: quadratically as eps shrinks.
+ * of 4^F pixels is processed in tiles of 2^tile_bits x 2^tile_bits pixels, as
+ * many at a time as fit in 8 GiB (16 bytes per pixel), so the cost grows with
+ * the canvas: quadratically as eps shrinks.  tile_bits = 0 leaves the choice to
+ * the library: tiles of 2^13, or, where the canvas is much larger than the point
+ * set, the points sorted by pixel in its place (the same limits apply).
  * polys: host arrays as for sdb_build_covering; d_x, d_y, d_attr: n device
  * points (d_attr and d_sum may be NULL); d_count, d_sum: P device entries,
  * zeroed by the call.  Synchronises cuda_stream.
@@ -488,11 +490,10 @@ sdb_status sdb_batch_query_ranges(const sdb_batch *b, uint32_t *h_ranges);
 
 /* Run all queries into d_count / d_sum (out_len device entries each, zeroed by
  * the call; d_sum may be NULL).  mode SDB_BATCH_PERSISTENT: one persistent
- * launch whose blocks pull (query, point tile) work items from a device
- * counter; SDB_BATCH_PER_QUERY: one launch per query; SDB_BATCH_GRAPH: the
- * persistent launch captured once into a CUDA graph (per output pointers) and
- * replayed -- needs a created stream, not the legacy default stream.  All modes
- * give identical results.  Asynchronous. */
+ * launch whose warps stride over the queries' point tiles; SDB_BATCH_PER_QUERY:
+ * one launch per query; SDB_BATCH_GRAPH: the persistent launch captured once into
+ * a CUDA graph (per output pointers) and replayed -- needs a created stream, not
+ * the legacy default stream.  All modes give identical results.  Asynchronous. */
 sdb_status sdb_batch_run(sdb_batch *b, int mode, uint64_t *d_count, int64_t *d_sum,
                          void *cuda_stream);
 
