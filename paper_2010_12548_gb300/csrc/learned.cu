@@ -99,15 +99,29 @@ __device__ __forceinline__ long long warp_max(long long v) {
 
 // below[l] = #{i < R : start_i < base_l} for l in [0, L].  Range i's start
 // goes to leaf lam_i; the leaves lam_{i-1} < l <= lam_i have exactly i starts
-// below their base (lam_{-1} = -1, and start_R = 4^F stands for leaf L).
+// below their base (lam_{-1} = -1, and start_R = 4^F stands for leaf L).  A thread's
+// work is one chain of dependent reads: BELOW_ITEMS starts per thread, all read first
+// (263-zone sweep, 27M ranges: 122 us with one, 101 with four).
+constexpr int BELOW_ITEMS = 4;
 __global__ void leaf_below_kernel(const uint64_t* __restrict__ start, uint64_t R,
                                   const float* __restrict__ knot, uint32_t wshift, float inv_w,
                                   uint32_t L, uint32_t* __restrict__ below) {
-  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i > R) return;
-  const uint32_t lam = i < R ? root_leaf(knot, wshift, inv_w, L, start[i]) : L;
-  const uint32_t from = i == 0 ? 0u : root_leaf(knot, wshift, inv_w, L, start[i - 1]) + 1u;
-  for (uint32_t l = from; l <= lam; ++l) below[l] = (uint32_t)i;
+  const uint64_t i0 = (uint64_t)blockIdx.x * BELOW_ITEMS * blockDim.x + threadIdx.x;
+  uint64_t at[BELOW_ITEMS], before[BELOW_ITEMS];
+#pragma unroll
+  for (int j = 0; j < BELOW_ITEMS; ++j) {
+    const uint64_t i = i0 + j * blockDim.x;
+    at[j] = i <= R ? start[i] : 0ull;
+    before[j] = i > 0 && i <= R ? start[i - 1] : 0ull;
+  }
+#pragma unroll
+  for (int j = 0; j < BELOW_ITEMS; ++j) {
+    const uint64_t i = i0 + j * blockDim.x;
+    if (i > R) return;
+    const uint32_t lam = i < R ? root_leaf(knot, wshift, inv_w, L, at[j]) : L;
+    const uint32_t from = i == 0 ? 0u : root_leaf(knot, wshift, inv_w, L, before[j]) + 1u;
+    for (uint32_t l = from; l <= lam; ++l) below[l] = (uint32_t)i;
+  }
 }
 
 __device__ __forceinline__ float to_float(uint32_t v) { return __uint2float_rn(v); }
@@ -250,7 +264,7 @@ sdb_status build_learned_index(sdb_covering* cov, uint32_t leaf_bits, uint32_t r
                                                                  base);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
-  leaf_below_kernel<<<grid_for((size_t)R + 1, 256), 256, 0, s>>>(cov->start, R, cov->knots, wshift,
+  leaf_below_kernel<<<grid_for((size_t)R + 1, 256 * BELOW_ITEMS), 256, 0, s>>>(cov->start, R, cov->knots, wshift,
                                                                    inv_w, L, below);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());

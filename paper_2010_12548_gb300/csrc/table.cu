@@ -58,15 +58,28 @@ __device__ __forceinline__ uint64_t bucket_cell(uint64_t b, uint32_t L0, uint32_
 
 // mark[b] = the last range r with first bucket fb(r) = b, where fb(r) is the
 // first bucket whose first id is >= start[r] (ranges are sorted: r is the last
-// one when fb(r + 1) differs, so each mark has one writer)
+// one when fb(r + 1) differs, so each mark has one writer).  MARK_ITEMS ranges per
+// thread, all read first: 27M ranges take 92 us with one, 55 with four.
+constexpr int MARK_ITEMS = 4;
 __global__ void table_marks_kernel(const uint64_t* __restrict__ start, uint64_t R, uint32_t shift,
                                    uint64_t nb, uint32_t* __restrict__ mark) {
-  const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= R) return;
+  const uint64_t r0 = (uint64_t)blockIdx.x * MARK_ITEMS * blockDim.x + threadIdx.x;
   const uint64_t round = (1ull << shift) - 1;
-  const uint64_t b = (start[r] + round) >> shift;
-  const uint64_t bn = r + 1 < R ? (start[r + 1] + round) >> shift : nb;
-  if (b < nb && bn != b) mark[b] = (uint32_t)r;
+  uint64_t at[MARK_ITEMS], next[MARK_ITEMS];
+#pragma unroll
+  for (int j = 0; j < MARK_ITEMS; ++j) {
+    const uint64_t r = r0 + j * blockDim.x;
+    at[j] = r < R ? start[r] : 0ull;
+    next[j] = r + 1 < R ? start[r + 1] : 0ull;
+  }
+#pragma unroll
+  for (int j = 0; j < MARK_ITEMS; ++j) {
+    const uint64_t r = r0 + j * blockDim.x;
+    if (r >= R) return;
+    const uint64_t b = (at[j] + round) >> shift;
+    const uint64_t bn = r + 1 < R ? (next[j] + round) >> shift : nb;
+    if (b < nb && bn != b) mark[b] = (uint32_t)r;
+  }
 }
 
 // r0(b) = max(mark[0..b]): the range holding bucket b's first id.  A tile of
@@ -394,7 +407,7 @@ sdb_status build_cell_table(sdb_covering* cov, uint32_t table_bits, cudaStream_t
   SDB_TRY(sc.get(&toff, nt));
   SDB_TRY(sc.get(&dtot, 1));
   SDB_TRY_CUDA(cudaMemsetAsync(mark, 0, nb * 4, s));
-  table_marks_kernel<<<grid_for(cov->R, 256), 256, 0, s>>>(cov->start, cov->R, shift, nb, mark);
+  table_marks_kernel<<<grid_for(cov->R, 256 * MARK_ITEMS), 256, 0, s>>>(cov->start, cov->R, shift, nb, mark);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
   tile_max_kernel<<<(unsigned)nt, TB, 0, s>>>(mark, nb, tpre);
