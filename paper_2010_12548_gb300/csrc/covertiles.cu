@@ -41,6 +41,7 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr uint32_t NONE = 0xffffffffu;
 constexpr int TPB = 256;
 constexpr int WPB = TPB / 32;
+constexpr uint32_t SPREAD = 256;  // counters that a sum over all blocks is spread over
 
 // element info: slot (bits 0..25), covers the group's first cell (26), with the
 // boundary flag (27), covers its last cell (28), with the flag (29), tile (30)
@@ -348,7 +349,7 @@ __global__ __launch_bounds__(TPB, 4) void tile_raster_kernel(TileArgs A) {
       A.inner[a] = ((uint64_t)ns << 32) | ent;
       A.cells[a] = ncell >> 8;
       // frontier size, as the refinement would meet it; spread over counters
-      atomicAdd(A.front + (g & 255u), (unsigned long long)fr);
+      atomicAdd(A.front + (g & (SPREAD - 1)), (unsigned long long)fr);
     }
   }
 }
@@ -488,21 +489,23 @@ __device__ bool same_ends(const GroupArgs& A, uint64_t pa, uint64_t pe, uint64_t
   return true;
 }
 
+// Sums over the groups, apart from the packed words (ranges << 32 | list entries) that
+// the scan adds up: those carry once there are 2^32 list entries, more than there are
+// cells where polygons overlap.  SPREAD counters of ranges, then as many of entries.
+struct GroupTotals {
+  uint64_t ranges = 0, entries = 0;
+};
+
 // Per element: 0, or at the head of a group the ranges it opens (<< 32) and their
 // list entries; code: bit 0 an empty gap before it, bit 1 itself, bit 2 the empty
 // tail of its query, bit 3 the query's first group, bit 4 its last.  A gap, a
 // group or a tail opens a range when its set differs from what comes before.
-__global__ void group_count_kernel(GroupArgs A, uint64_t* __restrict__ cnt,
-                                   uint8_t* __restrict__ code, uint32_t* __restrict__ qhead,
-                                   unsigned int* __restrict__ flag,
-                                   unsigned long long* __restrict__ entries) {
-  const uint64_t a = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= A.ne || flag[1]) return;  // (a crowded tile: nothing is made)
+__device__ uint64_t count_group(const GroupArgs& A, uint64_t a, uint8_t* __restrict__ code,
+                                uint32_t* __restrict__ qhead, unsigned int* __restrict__ flag) {
   const uint64_t key = A.key[a];
   if (a > 0 && A.key[a - 1] == key) {
-    cnt[a] = 0;
     code[a] = 0;
-    return;
+    return 0;
   }
   const uint32_t q = gq(A, key);
   const uint64_t lo = key & A.lomask, hi = end_of(A, a, lo);
@@ -533,13 +536,36 @@ __global__ void group_count_kernel(GroupArgs A, uint64_t* __restrict__ cnt,
     opens_head = gap ? nfirst != 0 : !same_ends(A, pa, a, a, e);
   }
   const bool opens_tail = last && hi < (1ull << (2 * A.qs[q].F)) && nlast != 0;
-  const uint64_t in = inner_of(A, a);
-  cnt[a] = in + ((uint64_t)(opens_gap + opens_head + opens_tail) << 32) + (opens_head ? nfirst : 0u);
-  if (entries)  // nested cells: more list entries than raster cells are possible
-    atomicAdd(entries, (unsigned long long)((uint32_t)in) + (opens_head ? nfirst : 0u));
   code[a] = (uint8_t)(opens_gap | (opens_head << 1) | (opens_tail << 2) | (first << 3) | (last << 4));
   if (first) qhead[q] = (uint32_t)a;
   if (nest) flag[0] = 1u;
+  // one group's entries fit: a tile's 1024 positions times TILE_MAX_GROUP + MAX_OVERLAP
+  return inner_of(A, a) + ((uint64_t)(opens_gap + opens_head + opens_tail) << 32) +
+         (opens_head ? nfirst : 0u);
+}
+
+__global__ __launch_bounds__(256) void group_count_kernel(GroupArgs A, uint64_t* __restrict__ cnt,
+                                                          uint8_t* __restrict__ code,
+                                                          uint32_t* __restrict__ qhead,
+                                                          unsigned int* __restrict__ flag,
+                                                          unsigned long long* __restrict__ sums) {
+  __shared__ uint32_t s_sum[2][8];
+  if (flag[1]) return;  // (a crowded tile: nothing is made)
+  const uint64_t a = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  uint64_t c = 0;
+  if (a < A.ne) cnt[a] = c = count_group(A, a, code, qhead, flag);
+  const uint32_t r = __reduce_add_sync(FULL, (uint32_t)(c >> 32));
+  const uint32_t l = __reduce_add_sync(FULL, (uint32_t)c);
+  if ((threadIdx.x & 31) == 0) {
+    s_sum[0][threadIdx.x >> 5] = r;
+    s_sum[1][threadIdx.x >> 5] = l;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    unsigned long long t = 0;
+    for (int w = 0; w < 8; ++w) t += s_sum[threadIdx.x][w];
+    if (t) atomicAdd(sums + threadIdx.x * SPREAD + (blockIdx.x & (SPREAD - 1)), t);
+  }
 }
 
 struct RangeOut {
@@ -1010,6 +1036,21 @@ sdb_status nested_groups(const TileArgs& ta, const uint8_t* level, uint64_t n_ti
   return SDB_OK;
 }
 
+GroupTotals group_totals(const unsigned long long* sums) {
+  GroupTotals t;
+  for (uint32_t i = 0; i < SPREAD; ++i) {
+    t.ranges += sums[i];
+    t.entries += sums[SPREAD + i];
+  }
+  return t;
+}
+
+// list offsets are 32-bit numbers (a test builds this file with a smaller limit)
+#ifndef SDB_LIST_LIMIT
+#define SDB_LIST_LIMIT 0xffffffffull
+#endif
+constexpr uint64_t LIST_LIMIT = SDB_LIST_LIMIT;
+
 }  // namespace
 
 sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_rec, const Item* items,
@@ -1056,7 +1097,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   uint8_t *level, *code;
   uint64_t *inner, *cnt, *off, *coff, *tot;
   unsigned int* dflag;  // nested, crowded, overlapping inside tiles
-  unsigned long long* front;
+  unsigned long long *front, *sums;  // the last level's frontier, GroupTotals
   SDB_TRY(sc.get(&heads, n_tile));
   SDB_TRY(sc.get(&n_heads, 1));
   SDB_TRY(sc.get(&rec, ne));
@@ -1071,13 +1112,14 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   SDB_TRY(sc.get(&tot, 2));
   SDB_TRY(sc.get(&qhead, Q));
   SDB_TRY(sc.get(&dflag, 3));
-  SDB_TRY(sc.get(&front, 256));
+  SDB_TRY(sc.get(&front, 3 * SPREAD));
+  sums = front + SPREAD;
   SDB_TRY(sc.get(&bits, n_tile * 32));
   if (spec.flags) SDB_TRY(sc.get(&bbits, n_tile * 32));
   SDB_TRY_CUDA(cudaMemsetAsync(n_heads, 0, 4, s));
   SDB_TRY_CUDA(cudaMemsetAsync(dflag, 0, 12, s));
   SDB_TRY_CUDA(cudaMemsetAsync(tot, 0, 16, s));
-  SDB_TRY_CUDA(cudaMemsetAsync(front, 0, 256 * 8, s));
+  SDB_TRY_CUDA(cudaMemsetAsync(front, 0, 3 * SPREAD * 8, s));
   SDB_TRY_CUDA(cudaMemsetAsync(qhead, 0xff, (size_t)Q * 4, s));
   TileArgs ta{};
   ta.rec = rec;
@@ -1111,7 +1153,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
       tile_raster_kernel<<<tile_grid, TPB, 0, s>>>(ta);
       note_launch();
     }
-    group_count_kernel<<<grid_for(ne, 256), 256, 0, s>>>(ga, cnt, code, qhead, dflag, nullptr);
+    group_count_kernel<<<grid_for(ne, 256), 256, 0, s>>>(ga, cnt, code, qhead, dflag, sums);
     note_launch();
     SDB_TRY_CUDA(cudaGetLastError());
     SDB_TRY(exclusive_scan<uint64_t>(cnt, off, ne, tot, s));
@@ -1130,18 +1172,19 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   uint64_t htot[2] = {0, 0};
   unsigned int hflag[3] = {0, 0, 0};
   std::vector<uint32_t> hhead(Q);
-  std::vector<unsigned long long> hfront(256);
+  std::vector<unsigned long long> hsums(3 * SPREAD);
   SDB_TRY_CUDA(cudaMemcpyAsync(htot, tot, 16, cudaMemcpyDeviceToHost, s));
   SDB_TRY_CUDA(cudaMemcpyAsync(hflag, dflag, 12, cudaMemcpyDeviceToHost, s));
   SDB_TRY_CUDA(cudaMemcpyAsync(hhead.data(), qhead, (size_t)Q * 4, cudaMemcpyDeviceToHost, s));
-  SDB_TRY_CUDA(cudaMemcpyAsync(hfront.data(), front, 256 * 8, cudaMemcpyDeviceToHost, s));
+  SDB_TRY_CUDA(cudaMemcpyAsync(hsums.data(), front, 3 * SPREAD * 8, cudaMemcpyDeviceToHost, s));
   SDB_TRY_CUDA(cudaStreamSynchronize(s));
   if (hflag[1] || (Q > 1 && (hflag[0] || hflag[2]))) {
     *outcome = hflag[1] ? TileOutcome::crowded : TileOutcome::nested;
     return SDB_OK;
   }
   unsigned long long nfront = 0;
-  for (unsigned long long v : hfront) nfront += v;
+  for (uint32_t i = 0; i < SPREAD; ++i) nfront += hsums[i];
+  GroupTotals total = group_totals(hsums.data() + SPREAD);
   const uint64_t ncells = htot[1];
   // the limits of the refinement to the finest level
   if (4 * nfront > 0xffffffffull) {
@@ -1157,31 +1200,30 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   if (nested) {
     uint32_t slots = 1;
     for (uint32_t i = 0; i < spec.NP; ++i) slots = std::max(slots, spec.pair_slot[i] + 1);
-    unsigned long long* dent;
-    SDB_TRY(sc.get(&dent, 1));
-    SDB_TRY_CUDA(cudaMemsetAsync(dent, 0, 8, s));
+    SDB_TRY_CUDA(cudaMemsetAsync(sums, 0, 2 * SPREAD * 8, s));
     SDB_TRY(nested_groups(ta, level, n_tile, spec.q[0].F, slots, sc, s, &ga, &tb));
     SDB_TRY(sc.get(&cnt, ga.ne));
     SDB_TRY(sc.get(&off, ga.ne));
     SDB_TRY(sc.get(&code, ga.ne));
-    group_count_kernel<<<grid_for(ga.ne, 256), 256, 0, s>>>(ga, cnt, code, qhead, dflag, dent);
+    group_count_kernel<<<grid_for(ga.ne, 256), 256, 0, s>>>(ga, cnt, code, qhead, dflag, sums);
     note_launch();
     SDB_TRY_CUDA(cudaGetLastError());
     SDB_TRY(exclusive_scan<uint64_t>(cnt, off, ga.ne, tot, s));
-    unsigned long long hent = 0;
     SDB_TRY_CUDA(cudaMemcpyAsync(htot, tot, 8, cudaMemcpyDeviceToHost, s));
-    SDB_TRY_CUDA(cudaMemcpyAsync(&hent, dent, 8, cudaMemcpyDeviceToHost, s));
+    SDB_TRY_CUDA(cudaMemcpyAsync(hsums.data(), sums, 2 * SPREAD * 8, cudaMemcpyDeviceToHost, s));
     SDB_TRY_CUDA(cudaMemcpyAsync(hflag, dflag, 12, cudaMemcpyDeviceToHost, s));
     SDB_TRY_CUDA(cudaStreamSynchronize(s));
     if (hflag[1]) {
       *outcome = TileOutcome::crowded;
       return SDB_OK;
     }
-    if (hent >= 0xffffffffull) {
-      set_error("covering: %llu list entries exceed the 32-bit list range", hent);
-      return SDB_ENOMEM;
-    }
+    total = group_totals(hsums.data());
     hhead[0] = 0;
+  }
+  if (total.entries >= LIST_LIMIT) {
+    set_error("covering: %llu list entries exceed the 32-bit list range",
+              (unsigned long long)total.entries);
+    return SDB_ENOMEM;
   }
   // entries: the groups' ranges, plus per query its sentinel, plus the empty
   // range of a query without records
@@ -1189,7 +1231,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   std::vector<uint64_t> hextra(Q);
   const uint64_t extra = query_fixes(hhead, ne, &hq);
   for (uint32_t q = 0; q < Q; ++q) hextra[q] = hq[q].extra;
-  const uint64_t E = (htot[0] >> 32) + extra, nids = htot[0] & 0xffffffffull;
+  const uint64_t E = total.ranges + extra, nids = total.entries;
   if (E >= 0x7fffffffull) {  // entry indices travel in 31 bits of the packed payload
     set_error("covering: %llu ranges exceed the 32-bit index range", (unsigned long long)E);
     return SDB_ENOMEM;
