@@ -1654,13 +1654,24 @@ static sdb_status build_pass(const PolyEdges& pe, const CoverSpec& spec, bool ti
   return merge_records(rkey, rval, n_rec, spec, d_qs, qshift, key_bits, sb, s, out);
 }
 
+// whether some query's viewport is less than the grid
+static bool clipped(const CoverSpec& spec) {
+  const uint32_t G = 1u << spec.B;
+  return std::any_of(spec.q, spec.q + spec.Q, [G](const CoverQuery& q) {
+    return q.x0 > 0 || q.y0 > 0 || q.x1 < G || q.y1 < G;
+  });
+}
+
 sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStream_t s,
                            CoverSet* out) {
   TileOutcome outcome = TileOutcome::crowded;
   if (use_tiles(spec) && !(spec.Q == 1 && overlap_deep(pe)))
     SDB_TRY(build_pass(pe, spec, true, s, out, &outcome));
   if (outcome == TileOutcome::made) return SDB_OK;
-  if (outcome == TileOutcome::nested && spec.Q != 1) {
+  // A tile is kept when its cell holds points of the viewport, and then counts as a
+  // whole: polygons that overlap only outside a viewport, in a tile at its edge, look
+  // nested.  The refinement drops cells one by one and decides.
+  if (outcome == TileOutcome::nested && spec.Q != 1 && !clipped(spec)) {
     set_error("batched coverings need polygons that do not overlap within a query");
     return SDB_EINVAL;
   }
