@@ -230,6 +230,19 @@ struct __align__(16) TileRec {
   uint32_t bits;      // its bitmap's place (its tile item)
 };
 
+// The tile groups: first element and elements, in any order.  Those of more than CROWD
+// polygons come last (from the array's end backwards): blocks raster them, not warps.
+constexpr uint32_t CROWD = 8;
+struct TileHeads {
+  uint2* at;
+  uint32_t* n;  // the groups of up to CROWD polygons, and the larger ones
+  uint32_t cap;
+  __device__ uint32_t all() const { return n[0] + n[1]; }
+  __device__ uint2 operator[](uint32_t g) const {
+    return g < n[0] ? at[g] : at[cap - 1 - (g - n[0])];
+  }
+};
+
 struct TileArgs {
   const TileRec* rec;      // per element (tiles' only)
   const uint32_t* elist;
@@ -238,8 +251,7 @@ struct TileArgs {
   uint32_t qshift, flags;
   const uint64_t* key;     // sorted keys
   uint64_t ne;
-  const uint2* heads;      // tile groups: first element, elements
-  const uint32_t* n_heads;
+  TileHeads heads;
   uint32_t* bits;          // per item 32 words in curve order: the polygon's cells
   uint32_t* bbits;         // the same for its boundary cells (flagged coverings)
   uint32_t* info;          // per element
@@ -250,6 +262,87 @@ struct TileArgs {
                            // [2] polygons that overlap inside a tile
   unsigned long long* front;  // boundary cells one level above the finest
 };
+
+// What a tile's polygons add up to, per lane
+struct TileSum {
+  uint32_t starts = 0;  // positions where the set of polygons changes
+  uint32_t cells = 0;   // records, in 256ths
+  uint32_t front = 0;   // boundary cells one level above the finest
+  uint32_t u[5] = {0, 0, 0, 0, 0};  // cells by the level of their record
+};
+
+// element i's polygon: its bitmaps, its info, what it adds to the tile
+__device__ __forceinline__ void raster_element(const TileArgs& A, uint32_t i, uint32_t lane,
+                                               const CurveTables& s_curve,
+                                               uint32_t (*s_rows)[32], TileSum& S) {
+  const TileRec R = A.rec[i];
+  const uint32_t sh = R.geo & 0xffu, orient = (R.geo >> 8) & 3u;
+  uint32_t rows[2], curve[2];
+  raster_tile(A.edges, A.elist + R.eoff, R.ecnt_par & 0x7fffffffu, R.px, R.py, sh,
+              R.ecnt_par >> 31, &rows[0], &rows[1]);
+  to_curve<2>(rows, curve, orient, s_curve, s_rows);
+  const uint32_t T = curve[0];
+  uint32_t I = curve[1];
+  // runs that hold a touched cell, level by level
+  const uint32_t t1 = any4(T), t2 = any16(t1), t3 = any_lanes(t2, 2), t4 = any_lanes(t3, 8);
+  // the interior cells by the level of their record (the largest untouched run)
+  uint32_t c0 = I & t1, c1 = I & ~t1 & t2, c2 = I & ~t2 & t3, c3 = I & ~t3 & t4, c4 = I & ~t4;
+  uint32_t tk = T, f1 = t1;
+  if (R.geo >> 10) {
+    // viewport clip: a record stays when its cell holds lattice points of it
+    const CoverQuery Q = A.qs[R.query];
+    const int64_t side = (int64_t)1 << sh, y = R.py + lane * side;
+    uint32_t row[1] = {0}, box[1];
+    if (y < (int64_t)Q.y1 && y + side > (int64_t)Q.y0) {
+      // columns with px + m side < x1 and px + (m + 1) side > x0
+      const int64_t lo = ((int64_t)Q.x0 - R.px) >> sh, hi = ((int64_t)Q.x1 - 1 - R.px) >> sh;
+      if (hi >= 0 && lo <= 31)
+        row[0] = (FULL << (lo < 0 ? 0 : lo)) & (FULL >> (31 - (hi > 31 ? 31 : hi)));
+    }
+    to_curve<1>(row, box, orient, s_curve, s_rows);
+    const uint32_t b1 = any4(box[0]), b2 = any16(b1), b3 = any_lanes(b2, 2),
+                   b4 = any_lanes(b3, 8);
+    tk &= box[0];
+    c0 &= box[0];
+    c1 &= b1;
+    c2 &= b2;
+    c3 &= b3;
+    c4 &= b4;
+    f1 &= b1;
+    I = c0 | c1 | c2 | c3 | c4;
+  }
+  const uint32_t cover = tk | I;
+  A.bits[(uint64_t)R.bits * 32 + lane] = cover;
+  if (A.flags) A.bbits[(uint64_t)R.bits * 32 + lane] = tk;
+  // records in 256ths: a cell of a run of 4^l cells is 1 / 4^l of a record
+  S.cells += 256 * (uint32_t)__popc(tk | c0) + 64 * (uint32_t)__popc(c1) +
+             16 * (uint32_t)__popc(c2) + 4 * (uint32_t)__popc(c3) + (uint32_t)__popc(c4);
+  S.front += __popc(f1 & 0x11111111u);
+  S.u[0] |= tk | c0;
+  S.u[1] |= c1;
+  S.u[2] |= c2;
+  S.u[3] |= c3;
+  S.u[4] |= c4;
+  // positions where this polygon's part of the set changes
+  uint32_t prev = __shfl_up_sync(FULL, cover, 1);
+  S.starts |= cover ^ ((cover << 1) | (prev >> 31));
+  if (A.flags) {
+    prev = __shfl_up_sync(FULL, tk, 1);
+    S.starts |= tk ^ ((tk << 1) | (prev >> 31));
+  }
+  const uint32_t last = __shfl_sync(FULL, cover, 31) >> 31;
+  const uint32_t blast = A.flags ? __shfl_sync(FULL, tk, 31) >> 31 : 0u;
+  if (lane == 0)
+    A.info[i] = R.slot | ((cover & 1u) << INFO_FIRST) |
+                (A.flags ? (tk & 1u) << (INFO_FIRST + 1) : 0u) | (last << INFO_LAST) |
+                (blast << (INFO_LAST + 1)) | INFO_TILE;
+}
+
+// two polygons' records that share cells must be the same cell
+__device__ __forceinline__ bool records_clash(const uint32_t (&u)[5]) {
+  return (u[0] & (u[1] | u[2] | u[3] | u[4])) || (u[1] & (u[2] | u[3] | u[4])) ||
+         (u[2] & (u[3] | u[4])) || (u[3] & u[4]);
+}
 
 // One warp per tile: the bitmaps of its polygons, what they add to the covering.
 // Bound by instruction issue and, a tile being a chain of dependent loads, by the
@@ -263,93 +356,80 @@ __global__ __launch_bounds__(TPB, 4) void tile_raster_kernel(TileArgs A) {
   __syncthreads();
   if (A.flag[1]) return;  // a crowded tile: the refinement takes over
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const uint32_t nh = *A.n_heads;
+  const uint32_t nh = A.heads.n[0];
   for (uint32_t g = blockIdx.x * WPB + w; g < nh; g += gridDim.x * WPB) {
-    const uint2 head = A.heads[g];
+    const uint2 head = A.heads.at[g];
     const uint32_t a = head.x, k = head.y;
-    uint32_t starts = 0, ncell = 0, u[5] = {0, 0, 0, 0, 0}, fr = 0;
-    for (uint32_t i = a; i < a + k; ++i) {
-      const TileRec R = A.rec[i];
-      const uint32_t sh = R.geo & 0xffu, orient = (R.geo >> 8) & 3u;
-      uint32_t rows[2], curve[2];
-      raster_tile(A.edges, A.elist + R.eoff, R.ecnt_par & 0x7fffffffu, R.px, R.py, sh,
-                  R.ecnt_par >> 31, &rows[0], &rows[1]);
-      to_curve<2>(rows, curve, orient, s_curve, s_rows[w]);
-      const uint32_t T = curve[0];
-      uint32_t I = curve[1];
-      // runs that hold a touched cell, level by level
-      const uint32_t t1 = any4(T), t2 = any16(t1), t3 = any_lanes(t2, 2), t4 = any_lanes(t3, 8);
-      // the interior cells by the level of their record (the largest untouched run)
-      uint32_t c0 = I & t1, c1 = I & ~t1 & t2, c2 = I & ~t2 & t3, c3 = I & ~t3 & t4, c4 = I & ~t4;
-      uint32_t tk = T, f1 = t1;
-      if (R.geo >> 10) {
-        // viewport clip: a record stays when its cell holds lattice points of it
-        const CoverQuery Q = A.qs[R.query];
-        const int64_t side = (int64_t)1 << sh, y = R.py + lane * side;
-        uint32_t row[1] = {0}, box[1];
-        if (y < (int64_t)Q.y1 && y + side > (int64_t)Q.y0) {
-          // columns with px + m side < x1 and px + (m + 1) side > x0
-          const int64_t lo = ((int64_t)Q.x0 - R.px) >> sh, hi = ((int64_t)Q.x1 - 1 - R.px) >> sh;
-          if (hi >= 0 && lo <= 31)
-            row[0] = (FULL << (lo < 0 ? 0 : lo)) & (FULL >> (31 - (hi > 31 ? 31 : hi)));
-        }
-        to_curve<1>(row, box, orient, s_curve, s_rows[w]);
-        const uint32_t b1 = any4(box[0]), b2 = any16(b1), b3 = any_lanes(b2, 2),
-                       b4 = any_lanes(b3, 8);
-        tk &= box[0];
-        c0 &= box[0];
-        c1 &= b1;
-        c2 &= b2;
-        c3 &= b3;
-        c4 &= b4;
-        f1 &= b1;
-        I = c0 | c1 | c2 | c3 | c4;
-      }
-      const uint32_t cover = tk | I;
-      A.bits[(uint64_t)R.bits * 32 + lane] = cover;
-      if (A.flags) A.bbits[(uint64_t)R.bits * 32 + lane] = tk;
-      // records in 256ths: a cell of a run of 4^l cells is 1 / 4^l of a record
-      ncell += 256 * (uint32_t)__popc(tk | c0) + 64 * (uint32_t)__popc(c1) +
-               16 * (uint32_t)__popc(c2) + 4 * (uint32_t)__popc(c3) + (uint32_t)__popc(c4);
-      fr += __popc(f1 & 0x11111111u);
-      u[0] |= tk | c0;
-      u[1] |= c1;
-      u[2] |= c2;
-      u[3] |= c3;
-      u[4] |= c4;
-      // positions where this polygon's part of the set changes
-      uint32_t prev = __shfl_up_sync(FULL, cover, 1);
-      starts |= cover ^ ((cover << 1) | (prev >> 31));
-      if (A.flags) {
-        prev = __shfl_up_sync(FULL, tk, 1);
-        starts |= tk ^ ((tk << 1) | (prev >> 31));
-      }
-      const uint32_t last = __shfl_sync(FULL, cover, 31) >> 31;
-      const uint32_t blast = A.flags ? __shfl_sync(FULL, tk, 31) >> 31 : 0u;
-      if (lane == 0)
-        A.info[i] = R.slot | ((cover & 1u) << INFO_FIRST) |
-                    (A.flags ? (tk & 1u) << (INFO_FIRST + 1) : 0u) | (last << INFO_LAST) |
-                    (blast << (INFO_LAST + 1)) | INFO_TILE;
-    }
-    // two polygons' records that share cells must be the same cell
-    const bool clash = k > 1 && ((u[0] & (u[1] | u[2] | u[3] | u[4])) ||
-                                 (u[1] & (u[2] | u[3] | u[4])) || (u[2] & (u[3] | u[4])) ||
-                                 (u[3] & u[4]));
+    TileSum S;
+    for (uint32_t i = a; i < a + k; ++i) raster_element(A, i, lane, s_curve, s_rows[w], S);
+    const bool clash = k > 1 && records_clash(S.u);
     if (__any_sync(FULL, clash) && lane == 0) A.flag[2] = 1u;
-    if (lane == 0) starts &= ~1u;  // the tile's first position is the group's head
+    if (lane == 0) S.starts &= ~1u;  // the tile's first position is the group's head
     // list entries of the inner starts
     uint32_t ent = 0;
     for (uint32_t i = a; i < a + k; ++i)
-      ent += __popc(starts & A.bits[(uint64_t)A.rec[i].bits * 32 + lane]);
-    const uint32_t ns = __reduce_add_sync(FULL, __popc(starts));
+      ent += __popc(S.starts & A.bits[(uint64_t)A.rec[i].bits * 32 + lane]);
+    const uint32_t ns = __reduce_add_sync(FULL, __popc(S.starts));
     ent = __reduce_add_sync(FULL, ent);
-    ncell = __reduce_add_sync(FULL, ncell);
-    fr = __reduce_add_sync(FULL, fr);
+    const uint32_t ncell = __reduce_add_sync(FULL, S.cells);
+    const uint32_t fr = __reduce_add_sync(FULL, S.front);
     if (lane == 0) {
       A.inner[a] = ((uint64_t)ns << 32) | ent;
       A.cells[a] = ncell >> 8;
       // frontier size, as the refinement would meet it; spread over counters
       atomicAdd(A.front + (g & (SPREAD - 1)), (unsigned long long)fr);
+    }
+  }
+}
+
+// The same by one block per tile, its warps sharing the tile's polygons: a warp takes
+// 2.3 us per polygon.
+__global__ __launch_bounds__(TPB) void crowd_raster_kernel(TileArgs A) {
+  __shared__ CurveTables s_curve;
+  __shared__ __align__(16) uint32_t s_rows[WPB][2][32];
+  __shared__ uint32_t s_or[6][32];  // starts, u
+  __shared__ uint32_t s_sum[3];     // cells, front, entries
+  const uint32_t nh = A.heads.n[1];
+  if (blockIdx.x >= nh || A.flag[1]) return;
+  fill_curve(s_curve);
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (uint32_t g = blockIdx.x; g < nh; g += gridDim.x) {
+    const uint2 head = A.heads[A.heads.n[0] + g];
+    const uint32_t a = head.x, k = head.y;
+    __syncthreads();
+    if (threadIdx.x < 6 * 32) s_or[threadIdx.x >> 5][lane] = 0;
+    if (threadIdx.x < 3) s_sum[threadIdx.x] = 0;
+    __syncthreads();
+    TileSum S;
+    for (uint32_t i = a + w; i < a + k; i += WPB) raster_element(A, i, lane, s_curve, s_rows[w], S);
+    atomicOr(&s_or[0][lane], S.starts);
+#pragma unroll
+    for (int l = 0; l < 5; ++l) atomicOr(&s_or[1 + l][lane], S.u[l]);
+    const uint32_t ncell = __reduce_add_sync(FULL, S.cells);
+    const uint32_t fr = __reduce_add_sync(FULL, S.front);
+    if (lane == 0) {
+      atomicAdd(&s_sum[0], ncell);
+      atomicAdd(&s_sum[1], fr);
+    }
+    __syncthreads();
+    uint32_t starts = s_or[0][lane], ent = 0;
+    if (lane == 0) starts &= ~1u;
+    for (uint32_t i = a + w; i < a + k; i += WPB)
+      ent += __popc(starts & A.bits[(uint64_t)A.rec[i].bits * 32 + lane]);
+    ent = __reduce_add_sync(FULL, ent);
+    if (lane == 0) atomicAdd(&s_sum[2], ent);
+    __syncthreads();
+    if (w == 0) {
+      uint32_t u[5];
+#pragma unroll
+      for (int l = 0; l < 5; ++l) u[l] = s_or[1 + l][lane];
+      const uint32_t ns = __reduce_add_sync(FULL, __popc(starts));
+      if (__any_sync(FULL, records_clash(u)) && lane == 0) A.flag[2] = 1u;
+      if (lane == 0) {
+        A.inner[a] = ((uint64_t)ns << 32) | s_sum[2];
+        A.cells[a] = s_sum[0] >> 8;
+        atomicAdd(A.front + (g & (SPREAD - 1)), (unsigned long long)s_sum[1]);
+      }
     }
   }
 }
@@ -371,21 +451,21 @@ __global__ void iota_kernel(uint32_t* __restrict__ p, uint64_t n) {
   if (i < n) p[i] = (uint32_t)i;
 }
 
-// The coarse records' info, level and record count, and the tile groups (any
-// order): their polygons' records in sorted order, ascending by slot, written by
-// the thread of the group's first element.
+// The coarse records' info, level and record count, and the tile groups with their
+// polygons' records ascending by slot: a tile's element finds its group around it and
+// its place among the group's slots.  (One thread inserting a group's records by slot
+// took 0.3 ms at 64 polygons, 13 at 500.)
 __global__ void element_kernel(const uint64_t* __restrict__ key, const uint32_t* __restrict__ idx,
                                const uint32_t* __restrict__ val, uint64_t n_rec, uint64_t ne,
                                const Item* __restrict__ items,
                                const uint32_t* __restrict__ pair_query,
                                const uint32_t* __restrict__ pair_slot,
-                               const CoverQuery* __restrict__ qs, uint32_t B,
-                               uint2* __restrict__ heads, uint32_t* __restrict__ n_heads,
+                               const CoverQuery* __restrict__ qs, uint32_t B, TileHeads heads,
                                uint32_t* __restrict__ info, uint8_t* __restrict__ level,
                                uint32_t* __restrict__ cells, TileRec* __restrict__ rec,
                                unsigned int* __restrict__ flag) {
   const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  uint32_t k = 0;
+  uint32_t k = 0;  // polygons of the group that this element heads
   if (i < ne) {
     const uint32_t el = idx[i];
     if (el < n_rec) {
@@ -398,47 +478,55 @@ __global__ void element_kernel(const uint64_t* __restrict__ key, const uint32_t*
       info[i] = INFO_TILE;
       // (the sort is stable: a key's coarse cells come before its tiles)
       const uint64_t q = key[i];
-      const bool lead = i == 0 || key[i - 1] != q;
-      const bool head = lead || idx[i - 1] < n_rec;
-      if (!lead && head) flag[0] = 1u;  // another polygon's cell with the tile's start
-      if (!head) {
-        cells[i] = 0;  // the head's warp counts for the tile
-      } else if (i + TILE_MAX_GROUP < ne && key[i + TILE_MAX_GROUP] == q) {
+      uint64_t a = i, e = i + 1;
+      while (a > 0 && i - a < TILE_MAX_GROUP && key[a - 1] == q && idx[a - 1] >= n_rec) --a;
+      while (e < ne && e - a <= TILE_MAX_GROUP && key[e] == q) ++e;
+      const bool head = a == i;
+      if (!head) cells[i] = 0;  // the head's warp counts for the tile
+      if (head && i > 0 && key[i - 1] == q) flag[0] = 1u;  // another polygon's cell with the tile's start
+      if (e - a > TILE_MAX_GROUP) {
         flag[1] = 1u;
       } else {
-        for (uint64_t j = i; j < ne && key[j] == q; ++j, ++k) {
-          const uint32_t ti = idx[j] - (uint32_t)n_rec;
-          const Item it = items[ti];
-          const uint32_t qi = pair_query[it.pair];
-          const CoverQuery Q = qs[qi];
-          const uint32_t sh = B - Q.F;
-          TileRec R;
-          R.px = (int32_t)(it.cx << (sh + TILE_DEPTH));
-          R.py = (int32_t)(it.cy << (sh + TILE_DEPTH));
-          R.eoff = it.eoff;
-          R.ecnt_par = it.ecnt_par;
-          R.slot = pair_slot[it.pair];
-          const int64_t side = (int64_t)1 << (sh + TILE_DEPTH);
-          const bool clip = R.px < (int64_t)Q.x0 || R.py < (int64_t)Q.y0 ||
-                            R.px + side > (int64_t)Q.x1 || R.py + side > (int64_t)Q.y1;
-          R.geo = sh | (it.orient << 8) | ((uint32_t)clip << 10);
-          R.query = qi;
-          R.bits = ti;
-          uint64_t at = j;  // insertion by slot
-          while (at > i && rec[at - 1].slot > R.slot) {
-            rec[at] = rec[at - 1];
-            --at;
+        const uint32_t ti = el - (uint32_t)n_rec;
+        const Item it = items[ti];
+        const uint32_t qi = pair_query[it.pair];
+        const CoverQuery Q = qs[qi];
+        const uint32_t sh = B - Q.F;
+        TileRec R;
+        R.px = (int32_t)(it.cx << (sh + TILE_DEPTH));
+        R.py = (int32_t)(it.cy << (sh + TILE_DEPTH));
+        R.eoff = it.eoff;
+        R.ecnt_par = it.ecnt_par;
+        R.slot = pair_slot[it.pair];
+        const int64_t side = (int64_t)1 << (sh + TILE_DEPTH);
+        const bool clip = R.px < (int64_t)Q.x0 || R.py < (int64_t)Q.y0 ||
+                          R.px + side > (int64_t)Q.x1 || R.py + side > (int64_t)Q.y1;
+        R.geo = sh | (it.orient << 8) | ((uint32_t)clip << 10);
+        R.query = qi;
+        R.bits = ti;
+        uint64_t at = a;
+        if (e - a > 1)
+#pragma unroll 4
+          for (uint64_t j = a; j < e; ++j) {
+            const uint32_t o = pair_slot[items[idx[j] - (uint32_t)n_rec].pair];
+            at += o < R.slot || (o == R.slot && j < i);
           }
-          rec[at] = R;
-        }
+        rec[at] = R;
+        if (head) k = (uint32_t)(e - a);
       }
     }
   }
-  const uint32_t b = __ballot_sync(FULL, k > 0);
-  uint32_t at = 0;
-  if (b && (threadIdx.x & 31) == 0) at = atomicAdd(n_heads, (uint32_t)__popc(b));
-  at = __shfl_sync(FULL, at, 0) + __popc(b & ((1u << (threadIdx.x & 31)) - 1u));
-  if (k > 0) heads[at] = make_uint2((uint32_t)i, k);
+  const uint32_t lane = threadIdx.x & 31;
+#pragma unroll
+  for (int large = 0; large < 2; ++large) {
+    const bool mine = k > 0 && (k > CROWD) == (large != 0);
+    const uint32_t b = __ballot_sync(FULL, mine);
+    if (!b) continue;
+    uint32_t at = 0;
+    if (lane == 0) at = atomicAdd(heads.n + large, (uint32_t)__popc(b));
+    at = __shfl_sync(FULL, at, 0) + __popc(b & ((1u << lane) - 1u));
+    if (mine) heads.at[large ? heads.cap - 1 - at : at] = make_uint2((uint32_t)i, k);
+  }
 }
 
 // ---------------------------------------------------------------- ranges
@@ -471,8 +559,44 @@ __device__ __forceinline__ uint32_t info_entry(uint32_t v, uint32_t which) {
   return (v & INFO_SLOT) | (((v >> (which + 1)) & 1u) << 31);
 }
 
+// A group's entries at its first or last cell, as one ascending list: its elements are
+// an ascending run of cells and one of tiles (either may be empty).
+struct EndWalk {
+  const uint32_t* info;
+  uint64_t c, ce, t, te;  // what is left of the runs
+  uint32_t which, seen = 0;
+  bool ordered = true;
+  __device__ EndWalk(const GroupArgs& A, uint64_t a, uint64_t e, uint32_t w)
+      : info(A.info), c(a), te(e), which(w) {
+    for (ce = a; ce < e && !(info[ce] & INFO_TILE);) ++ce;
+    t = ce;
+  }
+  __device__ uint32_t next() {  // NONE: at the end
+    while (c < ce && !((info[c] >> which) & 1u)) ++c;
+    while (t < te && !((info[t] >> which) & 1u)) ++t;
+    if (c == ce && t == te) return NONE;
+    const bool cell = t == te || (c < ce && (info[c] & INFO_SLOT) < (info[t] & INFO_SLOT));
+    const uint32_t v = info[cell ? c++ : t++];
+    ordered &= (v & INFO_SLOT) >= seen;
+    seen = v & INFO_SLOT;
+    return info_entry(v, which);
+  }
+};
+
 // a group's set at its last cell equals another's at its first cell
 __device__ bool same_ends(const GroupArgs& A, uint64_t pa, uint64_t pe, uint64_t a, uint64_t e) {
+  if (pe - pa > 8 && e - a > 8) {  // side by side: 500 polygons against 500 one by one take 10 ms
+    EndWalk x(A, pa, pe, INFO_LAST), y(A, a, e, INFO_FIRST);
+    bool same = true;
+    for (uint32_t u = 0, v = 0; u != NONE || v != NONE;) {
+      u = x.next();
+      v = y.next();
+      same &= u == v;
+      if (!same && !(x.ordered && y.ordered)) break;
+    }
+    if (same || (x.ordered && y.ordered)) return same;
+    // coarser cells of one place are in no order
+  }
   uint32_t n0 = 0, n1 = 0;
   for (uint64_t i = pa; i < pe; ++i) n0 += (A.info[i] >> INFO_LAST) & 1u;
   for (uint64_t i = a; i < e; ++i) n1 += (A.info[i] >> INFO_FIRST) & 1u;
@@ -574,12 +698,16 @@ struct RangeOut {
   uint32_t* qlist;  // per query: list entries before its first group, after its last
 };
 
-// inserts v into the ascending list out[0, t) by slot
-__device__ __forceinline__ void insert_entry(uint32_t* out, uint32_t t, uint32_t v) {
+// inserts v into the list out[0, t) by slot, which ascends up to *last, its last entry
+__device__ __forceinline__ void insert_entry(uint32_t* out, uint32_t t, uint32_t v, uint32_t* last) {
   uint32_t j = t;
-  while (j > 0 && (out[j - 1] & INFO_SLOT) > (v & INFO_SLOT)) {
-    out[j] = out[j - 1];
-    --j;
+  if (t > 0 && (*last & INFO_SLOT) > (v & INFO_SLOT)) {
+    while (j > 0 && (out[j - 1] & INFO_SLOT) > (v & INFO_SLOT)) {
+      out[j] = out[j - 1];
+      --j;
+    }
+  } else {
+    *last = v;
   }
   out[j] = v;
 }
@@ -627,12 +755,12 @@ __global__ void group_emit_kernel(GroupArgs A, const uint64_t* __restrict__ off,
     ++e;
   }
   if (c & 2u) {
-    uint32_t n = 0, one = 0;
+    uint32_t n = 0, one = 0, top = 0;
     for (uint64_t i = a; i < A.ne && A.key[i] == key; ++i) {
       const uint32_t v = A.info[i];
       if (!((v >> INFO_FIRST) & 1u)) continue;
       one = info_entry(v, INFO_FIRST);
-      insert_entry(O.list_ids + L, n++, one);
+      insert_entry(O.list_ids + L, n++, one, &top);
     }
     O.start[e] = lo;
     O.list_off[e] = L - O.l0;
@@ -679,7 +807,7 @@ __global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64
   __shared__ uint32_t s_h[WPB][STAGE][32];
   __shared__ uint16_t s_pos[WPB][1024];
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const uint32_t nh = *A.n_heads;
+  const uint32_t nh = A.heads.n[0];
   // tiles in a row per warp: 32, fewer when there are not enough for all warps
   const uint32_t run = min(32u, max(1u, nh / (gridDim.x * WPB)));
   for (uint32_t g0 = (blockIdx.x * WPB + w) * run; g0 < nh; g0 += gridDim.x * WPB * run) {
@@ -689,7 +817,7 @@ __global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64
    uint32_t my_ns = 0, my_c = 0;
    uint2 my_base = make_uint2(0, 0);
    if (lane < in_run) {
-     my_head = A.heads[g0 + lane];
+     my_head = A.heads.at[g0 + lane];
      my_base = BASE ? base.at[my_head.x] : make_uint2(my_head.x, 0);
      my_ns = (uint32_t)(A.inner[my_head.x] >> 32);
      my_key = A.key[my_head.x];
@@ -815,6 +943,131 @@ __global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64
   }
 }
 
+// The same by one block per tile of more than CROWD polygons, its warps sharing first
+// the polygons, then the ranges, 32 at a time against 32 polygons with several reads in
+// flight.  (512 polygons over one another, 32 x 32 tiles of them: the build 15.5 ms with
+// a warp per tile and one thread ordering its polygons, 6.5 ms; 500 small polygons in one
+// tile 16 -> 0.8 ms.)
+template <bool BASE>
+__global__ __launch_bounds__(TPB) void crowd_emit_kernel(TileArgs A, const uint64_t* __restrict__ off,
+                                                         const uint8_t* __restrict__ code,
+                                                         const uint64_t* __restrict__ extra,
+                                                         uint64_t lomask, TileBase base,
+                                                         RangeOut o) {
+  __shared__ uint32_t s_starts[32], s_first;
+  __shared__ uint16_t s_pos[1024];
+  __shared__ uint32_t s_list[1024];  // the ranges' list entries, then what is before them
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t nh = A.heads.n[1];
+  for (uint32_t g = blockIdx.x; g < nh; g += gridDim.x) {
+    const uint2 head = A.heads[A.heads.n[0] + g];
+    const uint32_t a = head.x, k = head.y;
+    const uint32_t ns = (uint32_t)(A.inner[a] >> 32);
+    if (ns == 0) continue;  // the whole block
+    const uint2 hb = BASE ? base.at[a] : make_uint2(a, 0);
+    const uint32_t nb0 = hb.y;  // base polygons
+    const uint64_t key = A.key[a], pre = off[hb.x], lo = key & lomask;
+    const uint32_t c = code[hb.x];
+    const uint32_t q = A.qshift >= 64 ? 0u : (uint32_t)(key >> A.qshift);
+    const QueryOut O = o.q[q];
+    __syncthreads();
+    if (threadIdx.x < 32) s_starts[lane] = 0;
+    if (threadIdx.x == 0) s_first = 0;
+    __syncthreads();
+    uint32_t starts = 0, first = 0;
+    auto changes = [&](uint32_t v) {
+      const uint32_t prev = __shfl_up_sync(FULL, v, 1);
+      starts |= v ^ ((v << 1) | (prev >> 31));
+    };
+    for (uint32_t i = a + w; i < a + k; i += WPB) {
+      const uint64_t at = (uint64_t)A.rec[i].bits * 32 + lane;
+      const uint32_t v = A.bits[at];
+      first += v & 1u;  // (lane 0's is the tile's first position)
+      changes(v);
+      if (A.flags) changes(A.bbits[at]);
+    }
+    atomicOr(&s_starts[lane], starts);
+    if (lane == 0) atomicAdd(&s_first, first);
+    __syncthreads();
+    if (w == 0) {
+      starts = lane == 0 ? s_starts[0] & ~1u : s_starts[lane];
+      uint32_t at = __popc(starts);
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t t = __shfl_up_sync(FULL, at, d);
+        if (lane >= (uint32_t)d) at += t;
+      }
+      at -= __popc(starts);
+      for (uint32_t m = starts; m; m &= m - 1) s_pos[at++] = (uint16_t)(32 * lane + __ffs(m) - 1);
+    }
+    __syncthreads();
+    // bit j: polygon j0 + j holds the position (all lanes take part)
+    auto members = [&](uint32_t j0, uint32_t pos, bool on) {
+      const uint32_t m = min(32u, k - j0), id = lane < m ? A.rec[a + j0 + lane].bits : 0u;
+      uint32_t v = 0;
+#pragma unroll 8
+      for (uint32_t j = 0; j < m; ++j)
+        v |= ((A.bits[(uint64_t)__shfl_sync(FULL, id, j) * 32 + (pos >> 5)] >> (pos & 31u)) & 1u) << j;
+      return on ? v : 0u;
+    };
+    for (uint32_t i0 = w * 32; i0 < ns; i0 += TPB) {
+      const bool on = i0 + lane < ns;
+      const uint32_t pos = on ? s_pos[i0 + lane] : 0u;
+      uint32_t n = nb0;
+      for (uint32_t j0 = 0; j0 < k; j0 += 32) n += __popc(members(j0, pos, on));
+      if (on) s_list[i0 + lane] = n;
+    }
+    __syncthreads();
+    if (w == 0) {
+      uint32_t sum = 0;
+      for (uint32_t i0 = 0; i0 < ns; i0 += 32) {
+        const uint32_t n = i0 + lane < ns ? s_list[i0 + lane] : 0u;
+        uint32_t inc = n;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const uint32_t t = __shfl_up_sync(FULL, inc, d);
+          if (lane >= (uint32_t)d) inc += t;
+        }
+        if (i0 + lane < ns) s_list[i0 + lane] = sum + inc - n;
+        sum += __shfl_sync(FULL, inc, 31);
+      }
+    }
+    __syncthreads();
+    const uint64_t e0 = (pre >> 32) + extra[q] + (c & 1u) + ((c >> 1) & 1u);
+    const uint32_t L0 = (uint32_t)pre + ((c & 2u) ? s_first + nb0 : 0u);
+    for (uint32_t i0 = w * 32; i0 < ns; i0 += TPB) {
+      const bool on = i0 + lane < ns;
+      const uint32_t pos = on ? s_pos[i0 + lane] : 0u;
+      const uint32_t L = on ? L0 + s_list[i0 + lane] : 0u;
+      uint32_t one = 0, t = L, b = 0;  // b: base polygons written (they ascend too)
+      auto put_base = [&](uint32_t below) {
+        for (; b < nb0; ++b) {
+          const uint32_t v = base.info[hb.x + b] & INFO_SLOT;
+          if (v >= below) break;
+          O.list_ids[t++] = one = v;
+        }
+      };
+      for (uint32_t j0 = 0; j0 < k; j0 += 32)
+        for (uint32_t m = members(j0, pos, on); m; m &= m - 1) {
+          const TileRec& R = A.rec[a + j0 + __ffs(m) - 1];
+          const uint32_t slot = R.slot;
+          if (BASE) put_base(slot);
+          one = slot;
+          if (A.flags)
+            one |= ((A.bbits[(uint64_t)R.bits * 32 + (pos >> 5)] >> (pos & 31u)) & 1u) << 31;
+          O.list_ids[t++] = one;
+        }
+      if (on) {
+        if (BASE) put_base(~0u);
+        const uint64_t e = e0 + i0 + lane;
+        O.start[e] = lo + pos;
+        O.list_off[e] = L - O.l0;
+        O.pay[e] = pay_of(t - L, one, e - O.e0);
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------- nested cells
 // One query whose polygons overlap: a coarser cell of one polygon may hold cells and
 // tiles of others.  The elements' ends cut the ids into elementary intervals, each a
@@ -825,7 +1078,8 @@ __global__ __launch_bounds__(TPB) void tile_emit_kernel(TileArgs A, const uint64
 // cell: 64 stars with holes at eps 64, uploaded, covered, indexed and joined, 1600 us
 // -> 1069 us.  A group's set is compared and ordered by one thread; polygons laid over
 // one another, eps 64 and 16, refinement -> here: 2 of them 0.87 -> 0.60 and 1.06
-// -> 0.71 ms, 64: 1.70 -> 0.92 and 4.12 -> 1.32, 512: 29.6 -> 10.8 and 268 -> 26.
+// -> 0.71 ms, 64: 1.70 -> 0.92 and 4.12 -> 1.32, 512: 29.6 -> 10.8 and 268 -> 26 (before
+// blocks shared the tiles of many polygons; 511 on a 2^13 grid now 11.7 -> 4.0 and 139 -> 6.5).
 // With more than MAX_OVERLAP over one another the refinement takes over.
 
 __global__ void ends_kernel(const uint64_t* __restrict__ key, const uint8_t* __restrict__ level,
@@ -892,12 +1146,10 @@ __global__ void pair_lengths_kernel(const uint64_t* __restrict__ pairs, uint64_t
   if (atomicAdd(&len[k], 1u) == MAX_OVERLAP) flag[1] = 1u;
   atomicAdd(&count[k], 1u);
 }
-__global__ void tile_lengths_kernel(const uint2* __restrict__ heads,
-                                    const uint32_t* __restrict__ n_heads,
-                                    const uint32_t* __restrict__ first,
+__global__ void tile_lengths_kernel(TileHeads heads, const uint32_t* __restrict__ first,
                                     uint32_t* __restrict__ count) {
   const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g < *n_heads) atomicAdd(&count[first[heads[g].x]], heads[g].y);
+  if (g < heads.all()) atomicAdd(&count[first[heads[g].x]], heads[g].y);
 }
 
 struct NestedOut {
@@ -919,16 +1171,14 @@ __global__ void base_elements_kernel(const uint64_t* __restrict__ pairs, uint64_
   o.end[at] = b[k + 1];
   o.info[at] = (uint32_t)(pairs[i] & ((1ull << pbits) - 1)) | (1u << INFO_FIRST) | (1u << INFO_LAST);
 }
-__global__ void tile_elements_kernel(const uint2* __restrict__ heads,
-                                     const uint32_t* __restrict__ n_heads,
-                                     const uint32_t* __restrict__ first,
+__global__ void tile_elements_kernel(TileHeads heads, const uint32_t* __restrict__ first,
                                      const uint32_t* __restrict__ info,
                                      const uint64_t* __restrict__ inner,
                                      const uint64_t* __restrict__ b,
                                      const uint32_t* __restrict__ len,
                                      const uint32_t* __restrict__ eoff, NestedOut o) {
   const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= *n_heads) return;
+  if (g >= heads.all()) return;
   const uint2 h = heads[g];
   const uint32_t k = first[h.x], e = eoff[k], n = len[k];
   for (uint32_t j = 0; j < h.y; ++j) {
@@ -1011,7 +1261,7 @@ sdb_status nested_groups(const TileArgs& ta, const uint8_t* level, uint64_t n_ti
     note_launch();
   }
   if (n_tile) {
-    tile_lengths_kernel<<<grid_for(n_tile, 256), 256, 0, s>>>(ta.heads, ta.n_heads, first, count);
+    tile_lengths_kernel<<<grid_for(n_tile, 256), 256, 0, s>>>(ta.heads, first, count);
     note_launch();
   }
   SDB_TRY_CUDA(cudaGetLastError());
@@ -1022,8 +1272,8 @@ sdb_status nested_groups(const TileArgs& ta, const uint8_t* level, uint64_t n_ti
     note_launch();
   }
   if (n_tile) {
-    tile_elements_kernel<<<grid_for(n_tile, 256), 256, 0, s>>>(ta.heads, ta.n_heads, first, ta.info,
-                                                              ta.inner, b, len, eoff, no);
+    tile_elements_kernel<<<grid_for(n_tile, 256), 256, 0, s>>>(ta.heads, first, ta.info, ta.inner, b, len,
+                                                              eoff, no);
     note_launch();
   }
   SDB_TRY_CUDA(cudaGetLastError());
@@ -1099,7 +1349,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   unsigned int* dflag;  // nested, crowded, overlapping inside tiles
   unsigned long long *front, *sums;  // the last level's frontier, GroupTotals
   SDB_TRY(sc.get(&heads, n_tile));
-  SDB_TRY(sc.get(&n_heads, 1));
+  SDB_TRY(sc.get(&n_heads, 2));
   SDB_TRY(sc.get(&rec, ne));
   SDB_TRY(sc.get(&info, ne));
   SDB_TRY(sc.get(&cells, ne));
@@ -1116,7 +1366,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   sums = front + SPREAD;
   SDB_TRY(sc.get(&bits, n_tile * 32));
   if (spec.flags) SDB_TRY(sc.get(&bbits, n_tile * 32));
-  SDB_TRY_CUDA(cudaMemsetAsync(n_heads, 0, 4, s));
+  SDB_TRY_CUDA(cudaMemsetAsync(n_heads, 0, 8, s));
   SDB_TRY_CUDA(cudaMemsetAsync(dflag, 0, 12, s));
   SDB_TRY_CUDA(cudaMemsetAsync(tot, 0, 16, s));
   SDB_TRY_CUDA(cudaMemsetAsync(front, 0, 3 * SPREAD * 8, s));
@@ -1130,8 +1380,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   ta.flags = spec.flags ? 1u : 0u;
   ta.key = sk;
   ta.ne = ne;
-  ta.heads = heads;
-  ta.n_heads = n_heads;
+  ta.heads = TileHeads{heads, n_heads, (uint32_t)n_tile};
   ta.bits = bits;
   ta.bbits = bbits;
   ta.info = info;
@@ -1143,15 +1392,21 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
                qshift, d_qs, nullptr};
   const unsigned tile_grid =
       (unsigned)std::min<uint64_t>((n_tile + WPB - 1) / WPB, (uint64_t)num_sms() * 32);
+  const unsigned crowd_grid =
+      (unsigned)std::min<uint64_t>((n_tile + CROWD) / (CROWD + 1), (uint64_t)num_sms() * 4);
   if (ne) {
     element_kernel<<<grid_for(ne, 256), 256, 0, s>>>(sk, si, rval, n_rec, ne, items, pair_query,
-                                                    pair_slot, d_qs, spec.B, heads, n_heads, info,
+                                                    pair_slot, d_qs, spec.B, ta.heads, info,
                                                     level, cells, rec, dflag);
     note_launch();
     if (n_tile) {
       TraceScope tr1("cover.raster", s);
       tile_raster_kernel<<<tile_grid, TPB, 0, s>>>(ta);
       note_launch();
+      if (n_tile > CROWD) {
+        crowd_raster_kernel<<<crowd_grid, TPB, 0, s>>>(ta);
+        note_launch();
+      }
     }
     group_count_kernel<<<grid_for(ne, 256), 256, 0, s>>>(ga, cnt, code, qhead, dflag, sums);
     note_launch();
@@ -1286,6 +1541,13 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
       else
         tile_emit_kernel<false><<<tile_grid, TPB, 0, s>>>(ta, off, code, dextra, ga.lomask, tb, ro);
       note_launch();
+      if (n_tile > CROWD) {
+        if (nested)
+          crowd_emit_kernel<true><<<crowd_grid, TPB, 0, s>>>(ta, off, code, dextra, ga.lomask, tb, ro);
+        else
+          crowd_emit_kernel<false><<<crowd_grid, TPB, 0, s>>>(ta, off, code, dextra, ga.lomask, tb, ro);
+        note_launch();
+      }
     }
     SDB_TRY_CUDA(cudaGetLastError());
   }
