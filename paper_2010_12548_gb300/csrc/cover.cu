@@ -1335,11 +1335,77 @@ static sdb_status grow(T** p, uint64_t n, uint64_t need, uint64_t hint, uint64_t
   return SDB_OK;
 }
 
+// Whether more than MAX_OVERLAP polygons probably lie over one another (some
+// polygons' first vertices against the boxes of some others): finding that out from the
+// tiles costs a third of the build.  A guess only, of bounded cost: 16 points, about
+// 1024 boxes (64 points and all boxes took 250 us for 2000 polygons, as long as the
+// build's kernels).
+static bool overlap_deep(const PolyEdges& pe) {
+  if (pe.P <= MAX_OVERLAP || pe.V > (1u << 16)) return false;
+  constexpr uint32_t POINTS = 16;
+  uint32_t px[POINTS], py[POINTS], over[POINTS] = {};
+  for (uint32_t k = 0; k < POINTS; ++k) {
+    const uint32_t v = pe.edge_off[(uint64_t)k * pe.P / POINTS];
+    px[k] = pe.x[v];
+    py[k] = pe.y[v];
+  }
+  const uint32_t step = std::max(1u, pe.P / 1024);
+  for (uint32_t j = 0; j < pe.P; j += step) {
+    uint32_t x0 = ~0u, y0 = ~0u, x1 = 0, y1 = 0;
+    for (uint32_t v = pe.edge_off[j]; v < pe.edge_off[j + 1]; ++v) {
+      x0 = std::min(x0, pe.x[v]);
+      y0 = std::min(y0, pe.y[v]);
+      x1 = std::max(x1, pe.x[v]);
+      y1 = std::max(y1, pe.y[v]);
+    }
+    for (uint32_t k = 0; k < POINTS; ++k)
+      over[k] += (px[k] > x0) & (px[k] < x1) & (py[k] > y0) & (py[k] < y1);
+  }
+  return *std::max_element(over, over + POINTS) * step > MAX_OVERLAP;
+}
+
+// Whether some tile probably meets so many small polygons that the refinement, whose
+// finest cells hold few of them, is faster or the tiles are refused: first vertices
+// counted by tile, of about 4096 polygons at most (40 us).  500 small polygons in one tile:
+// tiles 780 us, refinement 410; 256: 560 and 390 (540 before there were tiles); 128 of
+// them, tiles 440.  More than TILE_MAX_GROUP: both passes, 800 us.
+static bool tiles_crowded(const PolyEdges& pe, const CoverSpec& spec,
+                          const std::vector<uint32_t>& np) {
+  constexpr uint32_t MANY = 256, SAMPLES = 4096, SEEN = 16;
+  uint64_t pairs = 0;
+  for (uint32_t n : np)
+    if (n > MANY) pairs += n;
+  if (pairs == 0) return false;
+  const uint32_t step = (uint32_t)((pairs + SAMPLES - 1) / SAMPLES);
+  struct Count {
+    uint32_t tag, n;  // a tile by 32 bits of its hash
+  };
+  constexpr uint32_t BITS = 13;  // at most half full
+  std::vector<Count> table(1u << BITS, Count{0, 0});
+  uint32_t skip = 0;
+  for (uint32_t i = 0; i < spec.NP; ++i) {
+    const uint32_t q = spec.pair_query[i];
+    if (np[q] <= MANY || skip++ % step) continue;
+    const CoverQuery& Q = spec.q[q];
+    const uint32_t v = pe.edge_off[spec.pair_poly[i]], x = pe.x[v], y = pe.y[v];
+    if (x < Q.x0 || x >= Q.x1 || y < Q.y0 || y >= Q.y1) continue;
+    const uint32_t sh = spec.B - (Q.F - TILE_DEPTH);  // a tile's side: tiles below 2^25 a side
+    const uint64_t key = ((uint64_t)(x >> sh) << 25 | (y >> sh)) ^ ((uint64_t)q << 50);
+    const uint64_t hash = key * 0x9E3779B97F4A7C15ull;
+    const uint32_t tag = (uint32_t)(hash >> 16);
+    uint32_t at = (uint32_t)(hash >> (64 - BITS));
+    while (table[at].n && table[at].tag != tag) at = (at + 1) & ((1u << BITS) - 1);
+    table[at].tag = tag;
+    if (++table[at].n >= SEEN && (uint64_t)table[at].n * step > MANY) return true;
+  }
+  return false;
+}
+
 // A query's viewport in tiles of its level, and whether the last levels of all
 // queries' refinement go through tile bitmaps: the levels above must be deep
 // enough to spread the polygons over the tiles (a warp takes a tile's polygons
 // one after the other), and the boundary cells are kept by touching only.
-static bool use_tiles(const CoverSpec& spec) {
+static bool use_tiles(const PolyEdges& pe, const CoverSpec& spec) {
   constexpr uint32_t MIN_LEVEL = 8;
   if (spec.noncons || spec.NP == 0) return false;
   std::vector<uint32_t> np(spec.Q, 0);
@@ -1352,32 +1418,7 @@ static bool use_tiles(const CoverSpec& spec) {
     const uint64_t ny = ((uint64_t)(Q.y1 - 1) >> sh) - (Q.y0 >> sh) + 1;
     if (np[q] > 64 + 2 * nx * ny) return false;
   }
-  return true;
-}
-
-// Whether more than MAX_OVERLAP polygons probably lie over one another (some
-// polygons' first vertices against the boxes of all): finding that out from the
-// tiles costs a third of the build.  A guess only.
-static bool overlap_deep(const PolyEdges& pe) {
-  if (pe.P <= MAX_OVERLAP || pe.V > (1u << 16)) return false;
-  std::vector<uint32_t> over(64, 0);
-  const uint32_t samples = std::min<uint32_t>(pe.P, 64);
-  for (uint32_t j = 0; j < pe.P; ++j) {
-    uint32_t x0 = ~0u, y0 = ~0u, x1 = 0, y1 = 0;
-    for (uint32_t v = pe.edge_off[j]; v < pe.edge_off[j + 1]; ++v) {
-      x0 = std::min(x0, pe.x[v]);
-      y0 = std::min(y0, pe.y[v]);
-      x1 = std::max(x1, pe.x[v]);
-      y1 = std::max(y1, pe.y[v]);
-    }
-    for (uint32_t k = 0; k < samples; ++k) {
-      const uint32_t v = pe.edge_off[(uint64_t)k * pe.P / samples];
-      over[k] += pe.x[v] > x0 && pe.x[v] < x1 && pe.y[v] > y0 && pe.y[v] < y1;
-    }
-  }
-  for (uint32_t n : over)
-    if (n > MAX_OVERLAP) return true;
-  return false;
+  return !tiles_crowded(pe, spec, np) && !(spec.Q == 1 && overlap_deep(pe));
 }
 
 // One pass of the builder.  With tiles, *outcome may say that nothing was made
@@ -1665,7 +1706,7 @@ static bool clipped(const CoverSpec& spec) {
 sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStream_t s,
                            CoverSet* out) {
   TileOutcome outcome = TileOutcome::crowded;
-  if (use_tiles(spec) && !(spec.Q == 1 && overlap_deep(pe)))
+  if (use_tiles(pe, spec))
     SDB_TRY(build_pass(pe, spec, true, s, out, &outcome));
   if (outcome == TileOutcome::made) return SDB_OK;
   // A tile is kept when its cell holds points of the viewport, and then counts as a

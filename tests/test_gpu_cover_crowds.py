@@ -1,6 +1,7 @@
 """Many polygons in one tile of a covering: at the edges of what warps and blocks take,
 in tiles side by side (the set at a border unchanged), over a coarser cell and at one
-place, entry for entry the oracle's covering; and in a time of the order of a few."""
+place, entry for entry the oracle's covering; and in a time of the order of a few.
+Crowds of small polygons are left to the refinement at once."""
 import time
 
 import numpy as np
@@ -76,3 +77,14 @@ def test_a_crowd_takes_no_longer(cuda, sdblib):
         return min(t)
     few = best(4)
     assert best(500) < 3 * few
+
+
+@pytest.mark.parametrize("n", [257, 1000])
+def test_crowds_of_small_polygons_are_built_once(cuda, sdblib, n):
+    """Launches of the build, against those of the rule that knows no tiles."""
+    P, launched = polygons(squares(n)), []
+    for flags in (0, sdblib.COVER_NONCONSERVATIVE):
+        before = sdblib.launch_count()
+        sdblib.build_covering(P, BITS, EPS, flags=flags).free()
+        launched.append(sdblib.launch_count() - before)
+    assert launched[0] <= launched[1] + 3
