@@ -195,17 +195,21 @@ __global__ __launch_bounds__(CAND_THREADS) void candidates_kernel(
   }
 }
 
+// tiles of at most T points per query, and (n_all) tiles of at most `asked` points in all
 __global__ void tile_count_kernel(const uint32_t* __restrict__ cand,
                                   const uint32_t* __restrict__ ncand, uint32_t Q, uint32_t T,
-                                  uint64_t* __restrict__ ntile) {
+                                  uint32_t asked, uint64_t* __restrict__ ntile,
+                                  unsigned long long* __restrict__ n_all) {
   uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= Q) return;
-  uint64_t t = 0;
+  uint64_t t = 0, all = 0;
   for (uint32_t i = 0; i < ncand[q]; ++i) {
     const uint32_t a = cand[(size_t)q * MAXC * 2 + 2 * i], b = cand[(size_t)q * MAXC * 2 + 2 * i + 1];
     t += ((uint64_t)b - a + T - 1) / T;
+    all += ((uint64_t)b - a + asked - 1) / asked;
   }
   ntile[q] = t;
+  atomicAdd(n_all, (unsigned long long)all);
 }
 
 __global__ void tile_fill_kernel(const uint32_t* __restrict__ cand,
@@ -619,22 +623,32 @@ sdb_status batch_query_dev(uint32_t B, const sdb_query& Qu, uint64_t out_off, Ba
   return SDB_OK;
 }
 
+// The kernel's grid takes every tile for as many units as the largest may have, so tiles
+// longer than PIECE are cut: a tile of "everything" would be 2^26 units for each of a
+// batch's thousands of short ranges, and the units past a range's end add up to seconds.
+constexpr uint32_t PIECE = 16384;
 sdb_status batch_core_tiles(BatchCore* c, uint32_t T, cudaStream_t s) {
   Scratch sc(s);
   uint64_t *nt, *toff, *dtot;
   SDB_TRY(sc.get(&nt, c->Q));
-  SDB_TRY(sc.get(&toff, (size_t)c->Q + 1));
-  SDB_TRY(sc.get(&dtot, 1));
-  tile_count_kernel<<<grid_for(c->Q, 128), 128, 0, s>>>(c->cand, c->ncand, c->Q, T, nt);
-  note_launch();
-  SDB_TRY_CUDA(cudaGetLastError());
-  SDB_TRY(exclusive_scan<uint64_t>(nt, toff, c->Q, dtot, s));
-  SDB_TRY_CUDA(cudaMemcpyAsync(toff + c->Q, dtot, 8, cudaMemcpyDeviceToDevice, s));
-  c->qtile.assign((size_t)c->Q + 1, 0);
-  SDB_TRY_CUDA(cudaMemcpyAsync(c->qtile.data(), toff, ((size_t)c->Q + 1) * 8,
-                               cudaMemcpyDeviceToHost, s));
-  SDB_TRY_CUDA(cudaStreamSynchronize(s));
-  const uint64_t total = c->qtile[c->Q];
+  SDB_TRY(sc.get(&toff, (size_t)c->Q + 2));
+  SDB_TRY(sc.get(&dtot, 2));
+  std::vector<uint64_t> off((size_t)c->Q + 2, 0);
+  uint32_t piece = std::min(T, PIECE);
+  for (;;) {
+    SDB_TRY_CUDA(cudaMemsetAsync(dtot, 0, 16, s));
+    tile_count_kernel<<<grid_for(c->Q, 128), 128, 0, s>>>(
+        c->cand, c->ncand, c->Q, piece, T, nt, reinterpret_cast<unsigned long long*>(dtot + 1));
+    note_launch();
+    SDB_TRY_CUDA(cudaGetLastError());
+    SDB_TRY(exclusive_scan<uint64_t>(nt, toff, c->Q, dtot, s));
+    SDB_TRY_CUDA(cudaMemcpyAsync(toff + c->Q, dtot, 16, cudaMemcpyDeviceToDevice, s));
+    SDB_TRY_CUDA(cudaMemcpyAsync(off.data(), toff, off.size() * 8, cudaMemcpyDeviceToHost, s));
+    SDB_TRY_CUDA(cudaStreamSynchronize(s));
+    if (off[c->Q] < 0xffffffffull || piece == T) break;
+    piece = piece > T / 2 ? T : 2 * piece;  // larger pieces when there are too many
+  }
+  const uint64_t total = off[c->Q];
   if (total >= 0xffffffffull) {
     set_error("batch: %llu tiles exceed the 32-bit range", (unsigned long long)total);
     return SDB_EINVAL;
@@ -642,12 +656,16 @@ sdb_status batch_core_tiles(BatchCore* c, uint32_t T, cudaStream_t s) {
   if (c->tiles) dfree(c->tiles, s);
   c->tiles = nullptr;
   SDB_TRY(dalloc_n(&c->tiles, total, s));
-  tile_fill_kernel<<<grid_for(c->Q, 128), 128, 0, s>>>(c->cand, c->ncand, c->Q, T, toff, c->tiles);
+  tile_fill_kernel<<<grid_for(c->Q, 128), 128, 0, s>>>(c->cand, c->ncand, c->Q, piece, toff,
+                                                       c->tiles);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
   SDB_TRY_CUDA(cudaStreamSynchronize(s));
-  c->ntiles = total;
+  c->ntiles = off[(size_t)c->Q + 1];
+  off.pop_back();
+  c->qtile = std::move(off);
   c->tile = T;
+  c->piece = piece;
   return SDB_OK;
 }
 
@@ -778,11 +796,11 @@ sdb_status batch_core_run(BatchCore* c, int mode, uint64_t* count, int64_t* sum,
   if (mode == SDB_BATCH_PER_QUERY) {
     for (uint32_t q = 0; q < c->Q; ++q)
       if (c->qtile[q + 1] > c->qtile[q])
-        SDB_TRY(launch_batch(A, c->tile, c->ppt, sum != nullptr, (uint32_t)c->qtile[q],
+        SDB_TRY(launch_batch(A, c->piece, c->ppt, sum != nullptr, (uint32_t)c->qtile[q],
                              (uint32_t)c->qtile[q + 1], s));
     return SDB_OK;
   }
-  return launch_batch(A, c->tile, c->ppt, sum != nullptr, 0, (uint32_t)c->ntiles, s);
+  return launch_batch(A, c->piece, c->ppt, sum != nullptr, 0, (uint32_t)c->qtile[c->Q], s);
 }
 
 // Coverings of queries [q0, q0 + nq) of a pair list, built in chunks that are

@@ -371,10 +371,11 @@ struct BatchCore {
   BatchChunkDev* dchunks = nullptr;
   uint32_t* cand = nullptr;   // per query up to 81 candidate point index ranges
   uint32_t* ncand = nullptr;
-  uint32_t tile = 4096, ppt = 2;
+  uint32_t tile = 4096, ppt = 2;  // as set
+  uint32_t piece = 4096;          // points of an entry of tiles at most
   BatchTile* tiles = nullptr;
-  uint64_t ntiles = 0;
-  std::vector<uint64_t> qtile;  // host, Q + 1: tiles of query q
+  uint64_t ntiles = 0;            // tiles of the size set
+  std::vector<uint64_t> qtile;  // host, Q + 1: entries of tiles of query q
   void release(cudaStream_t s);
 };
 // viewport, level and output slot of one query (sbase/R/chunk left to the caller)
