@@ -341,11 +341,12 @@ __global__ __launch_bounds__(THREADS) void batch_kernel(BatchArgs A, uint32_t ti
     const TileRec tr = A.tiles[tile_lo + u / units_per_tile];
     const uint64_t b64 = tr.begin + (u % units_per_tile) * UNIT;
     if (b64 >= tr.end) continue;
-    const uint32_t b = (uint32_t)b64, e = tr.end - b > UNIT ? b + UNIT : tr.end;
+    // (counted from b: b + UNIT may pass 2^32)
+    const uint32_t b = (uint32_t)b64, m = min(tr.end - b, UNIT);
     // the unit's points (past its end: its last point again)
     uint64_t key[G];
 #pragma unroll
-    for (int g = 0; g < G; ++g) key[g] = __ldg(A.key + min(b + g * 32 + lane, e - 1));
+    for (int g = 0; g < G; ++g) key[g] = __ldg(A.key + b + min(g * 32 + lane, m - 1));
     const QueryDev& Q = A.q[tr.q];
     const ChunkDev C = A.chunks[Q.chunk];
     const uint64_t sbase = Q.sbase;
@@ -363,7 +364,7 @@ __global__ __launch_bounds__(THREADS) void batch_kernel(BatchArgs A, uint32_t ti
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       const uint32_t i = b + g * 32 + lane;
-      ok[g] = i < e;
+      ok[g] = g * 32 + lane < m;
       av[g] = (SUM && ok[g]) ? __ldg(A.attr + i) : 0;
       if (!inside && ok[g]) {
         const uint32_t x = __ldg(A.x + i), y = __ldg(A.y + i);
