@@ -562,14 +562,18 @@ sdb_status launch_batch_t(const BatchArgs& A, uint32_t tile, uint32_t lo, uint32
   return SDB_OK;
 }
 
-// the tuning's points per thread, doubled: a unit's two end lookups are shared by
-// twice the points
-sdb_status launch_batch(const BatchArgs& A, uint32_t tile, uint32_t ppt, bool sum, uint32_t lo,
-                        uint32_t hi, cudaStream_t s) {
-  if (ppt == 1) return sum ? launch_batch_t<2, true>(A, tile, lo, hi, s)
-                           : launch_batch_t<2, false>(A, tile, lo, hi, s);
-  if (ppt == 2) return sum ? launch_batch_t<4, true>(A, tile, lo, hi, s)
-                           : launch_batch_t<4, false>(A, tile, lo, hi, s);
+// Points of a lane per unit: the tuning's points per thread, doubled (a unit's two end
+// lookups are shared by twice the points), and fewer while the batch's points are not
+// enough units for 8 warps per SM (64 views of 2000 points each, 4 points per thread:
+// 68 us with units of 256 points, 37 with 128, 29 with 64; 12M points: 149, 145, 213).
+sdb_status launch_batch(const BatchArgs& A, uint32_t tile, uint32_t ppt, uint64_t points, bool sum,
+                        uint32_t lo, uint32_t hi, cudaStream_t s) {
+  uint32_t g = 2 * ppt;
+  while (g > 2 && points < (uint64_t)32 * g * 8 * num_sms()) g /= 2;
+  if (g == 2) return sum ? launch_batch_t<2, true>(A, tile, lo, hi, s)
+                         : launch_batch_t<2, false>(A, tile, lo, hi, s);
+  if (g == 4) return sum ? launch_batch_t<4, true>(A, tile, lo, hi, s)
+                         : launch_batch_t<4, false>(A, tile, lo, hi, s);
   return sum ? launch_batch_t<8, true>(A, tile, lo, hi, s)
              : launch_batch_t<8, false>(A, tile, lo, hi, s);
 }
@@ -797,11 +801,13 @@ sdb_status batch_core_run(BatchCore* c, int mode, uint64_t* count, int64_t* sum,
   if (mode == SDB_BATCH_PER_QUERY) {
     for (uint32_t q = 0; q < c->Q; ++q)
       if (c->qtile[q + 1] > c->qtile[q])
-        SDB_TRY(launch_batch(A, c->piece, c->ppt, sum != nullptr, (uint32_t)c->qtile[q],
-                             (uint32_t)c->qtile[q + 1], s));
+        SDB_TRY(launch_batch(A, c->piece, c->ppt,
+                             std::min(c->candidates, (c->qtile[q + 1] - c->qtile[q]) * c->piece),
+                             sum != nullptr, (uint32_t)c->qtile[q], (uint32_t)c->qtile[q + 1], s));
     return SDB_OK;
   }
-  return launch_batch(A, c->piece, c->ppt, sum != nullptr, 0, (uint32_t)c->qtile[c->Q], s);
+  return launch_batch(A, c->piece, c->ppt, c->candidates, sum != nullptr, 0,
+                      (uint32_t)c->qtile[c->Q], s);
 }
 
 // Coverings of queries [q0, q0 + nq) of a pair list, built in chunks that are
