@@ -195,21 +195,24 @@ __global__ __launch_bounds__(CAND_THREADS) void candidates_kernel(
   }
 }
 
-// tiles of at most T points per query, and (n_all) tiles of at most `asked` points in all
+// tiles of at most T points per query; over all queries, tiles of at most `asked` points
+// (all[0]) and the points of the longest range (all[1])
 __global__ void tile_count_kernel(const uint32_t* __restrict__ cand,
                                   const uint32_t* __restrict__ ncand, uint32_t Q, uint32_t T,
                                   uint32_t asked, uint64_t* __restrict__ ntile,
-                                  unsigned long long* __restrict__ n_all) {
+                                  unsigned long long* __restrict__ all) {
   uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= Q) return;
-  uint64_t t = 0, all = 0;
+  uint64_t t = 0, ta = 0, most = 0;
   for (uint32_t i = 0; i < ncand[q]; ++i) {
     const uint32_t a = cand[(size_t)q * MAXC * 2 + 2 * i], b = cand[(size_t)q * MAXC * 2 + 2 * i + 1];
     t += ((uint64_t)b - a + T - 1) / T;
-    all += ((uint64_t)b - a + asked - 1) / asked;
+    ta += ((uint64_t)b - a + asked - 1) / asked;
+    most = max(most, (uint64_t)(b - a));
   }
   ntile[q] = t;
-  atomicAdd(n_all, (unsigned long long)all);
+  atomicAdd(all, (unsigned long long)ta);
+  atomicMax(all + 1, (unsigned long long)most);
 }
 
 __global__ void tile_fill_kernel(const uint32_t* __restrict__ cand,
@@ -564,8 +567,8 @@ sdb_status launch_batch_t(const BatchArgs& A, uint32_t tile, uint32_t lo, uint32
 
 // Points of a lane per unit: the tuning's points per thread, doubled (a unit's two end
 // lookups are shared by twice the points), and fewer while the batch's points are not
-// enough units for 8 warps per SM (64 views of 2000 points each, 4 points per thread:
-// 68 us with units of 256 points, 37 with 128, 29 with 64; 12M points: 149, 145, 213).
+// enough units for 8 warps per SM (units of 256, 128 and 64 points, one view of 49,000: 21,
+// 17 and 15 us; 64 views of 12M: 138, 140 and 214).
 sdb_status launch_batch(const BatchArgs& A, uint32_t tile, uint32_t ppt, uint64_t points, bool sum,
                         uint32_t lo, uint32_t hi, cudaStream_t s) {
   uint32_t g = 2 * ppt;
@@ -628,26 +631,29 @@ sdb_status batch_query_dev(uint32_t B, const sdb_query& Qu, uint64_t out_off, Ba
   return SDB_OK;
 }
 
-// The kernel's grid takes every tile for as many units as the largest may have, so tiles
-// longer than PIECE are cut: a tile of "everything" would be 2^26 units for each of a
-// batch's thousands of short ranges, and the units past a range's end add up to seconds.
-constexpr uint32_t PIECE = 16384;
+// The kernel's grid takes every tile for as many units as the largest may have, and most
+// ranges of a view are short, so the kernel's tiles are pieces of at most PIECE points
+// whatever size is set: with the units past the ranges' ends of 4096-point tiles, 512 views
+// over 50M points took 245 us instead of 186, and with those of 16384-point tiles, 64 small
+// views took 65 instead of 31.  A tile of "everything" would be 2^26 units for each of a batch's thousands of ranges,
+// seconds of them.
+constexpr uint32_t PIECE = 1024;
 sdb_status batch_core_tiles(BatchCore* c, uint32_t T, cudaStream_t s) {
   Scratch sc(s);
   uint64_t *nt, *toff, *dtot;
   SDB_TRY(sc.get(&nt, c->Q));
-  SDB_TRY(sc.get(&toff, (size_t)c->Q + 2));
-  SDB_TRY(sc.get(&dtot, 2));
-  std::vector<uint64_t> off((size_t)c->Q + 2, 0);
+  SDB_TRY(sc.get(&toff, (size_t)c->Q + 3));
+  SDB_TRY(sc.get(&dtot, 3));
+  std::vector<uint64_t> off((size_t)c->Q + 3, 0);  // offsets, total, tiles asked for, longest
   uint32_t piece = std::min(T, PIECE);
   for (;;) {
-    SDB_TRY_CUDA(cudaMemsetAsync(dtot, 0, 16, s));
+    SDB_TRY_CUDA(cudaMemsetAsync(dtot, 0, 24, s));
     tile_count_kernel<<<grid_for(c->Q, 128), 128, 0, s>>>(
         c->cand, c->ncand, c->Q, piece, T, nt, reinterpret_cast<unsigned long long*>(dtot + 1));
     note_launch();
     SDB_TRY_CUDA(cudaGetLastError());
     SDB_TRY(exclusive_scan<uint64_t>(nt, toff, c->Q, dtot, s));
-    SDB_TRY_CUDA(cudaMemcpyAsync(toff + c->Q, dtot, 16, cudaMemcpyDeviceToDevice, s));
+    SDB_TRY_CUDA(cudaMemcpyAsync(toff + c->Q, dtot, 24, cudaMemcpyDeviceToDevice, s));
     SDB_TRY_CUDA(cudaMemcpyAsync(off.data(), toff, off.size() * 8, cudaMemcpyDeviceToHost, s));
     SDB_TRY_CUDA(cudaStreamSynchronize(s));
     if (off[c->Q] < 0xffffffffull || piece == T) break;
@@ -667,10 +673,10 @@ sdb_status batch_core_tiles(BatchCore* c, uint32_t T, cudaStream_t s) {
   SDB_TRY_CUDA(cudaGetLastError());
   SDB_TRY_CUDA(cudaStreamSynchronize(s));
   c->ntiles = off[(size_t)c->Q + 1];
-  off.pop_back();
+  c->piece = (uint32_t)std::min<uint64_t>(piece, std::max<uint64_t>(off[(size_t)c->Q + 2], 1));
+  off.resize((size_t)c->Q + 1);
   c->qtile = std::move(off);
   c->tile = T;
-  c->piece = piece;
   return SDB_OK;
 }
 
