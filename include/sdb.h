@@ -358,9 +358,11 @@ sdb_status sdb_join_aggregate_host_noalloc(const uint32_t *h_x, const uint32_t *
  * sdb_join_aggregate with a covering of the same polygons and eps.  The canvas
  * of 4^F pixels is processed in tiles of 2^tile_bits x 2^tile_bits pixels, as
  * many at a time as fit in 8 GiB (16 bytes per pixel), so the cost grows with
- * the canvas: quadratically as eps shrinks.  tile_bits = 0 leaves the choice to
- * the library: tiles of 2^13, or, where the canvas is much larger than the point
- * set, the points sorted by pixel in its place (the same limits apply).
+ * the canvas: quadratically as eps shrinks; with several tiles the points are
+ * sorted by tile, 24 bytes a point.  tile_bits = 0 leaves the choice to the
+ * library: one tile of up to 2^13 pixels a side, or, where that is too small for
+ * the canvas or the canvas has more than 2 n + 2^23 pixels, no canvas but the
+ * points sorted by pixel, in 24 bytes a point (the same limits apply).
  * polys: host arrays as for sdb_build_covering; d_x, d_y, d_attr: n device
  * points (d_attr and d_sum may be NULL); d_count, d_sum: P device entries,
  * zeroed by the call.  Synchronises cuda_stream.

@@ -504,12 +504,14 @@ sdb_status raster_join(const PolyEdges& pe, uint32_t B, uint32_t k, const uint32
               F, t);
     return SDB_EINVAL;
   }
-  // The canvas costs 8.5 ps a pixel (cleared, prefix-summed) and, cut into
-  // tiles, a sort of the points by tile; sorting the points by pixel costs
-  // 35 - 50 ps a point and touches no empty pixel.  263 zones, 20M points:
-  // 4^15 pixels 1.66 ms sorted against 11.4 ms, 4^13 1.51 against 1.97, 4^12
-  // 1.4 against 1.04; 1M points: 4^12 0.43 against 0.46; 100M points: 4^14 5.6
-  // against 10.7, 4^13 even.
+  // The canvas costs 8.5 ps a pixel (cleared, prefix-summed) and, cut into tiles, a sort
+  // of the points by tile and a gather, 84 - 97 ps a point; sorting the points by pixel
+  // costs 83 ps a point at 20M and 47 - 56 from 100M on, and touches no empty pixel.  So
+  // a canvas of several tiles is never made, whatever the number of points (263 zones,
+  // 4^15 and 4^14 pixels, ms sorted against canvas: 20M points 1.66 and 11.4 at 4^15; 100M
+  // 5.6 and 10.7 at 4^14; 10^9, the most that was measured, 48 and 122, 47 and 99), and
+  // one tile only where the points are few beside its pixels (20M: 4^13 1.51 against
+  // 1.97, 4^12 1.4 against 1.04; 1M: 4^12 0.43 against 0.46; 100M: 4^13 even).
   const bool sorted = pick && n < 0xffffffffull &&
                       (F > t || (1ull << (2 * F)) > 2 * n + (1ull << 23));
   const uint64_t tps = 1ull << (F - t);  // tiles per side
@@ -588,8 +590,8 @@ sdb_status raster_join(const PolyEdges& pe, uint32_t B, uint32_t k, const uint32
     SDB_TRY_CUDA(cudaMemsetAsync(outside, 0, 4, s));
     uint64_t *key, *ktmp, *ks;
     uint32_t *val = nullptr, *vtmp = nullptr, *vs = nullptr;
-    SDB_TRY(sc.get(&key, n));
-    SDB_TRY(sc.get(&ktmp, n));
+    SDB_TRY(sc.get(&key, n + 1));
+    SDB_TRY(sc.get(&ktmp, n + 1));
     if (sum) {
       SDB_TRY(sc.get(&val, n));
       SDB_TRY(sc.get(&vtmp, n));
@@ -601,9 +603,10 @@ sdb_status raster_join(const PolyEdges& pe, uint32_t B, uint32_t k, const uint32
       SDB_TRY_CUDA(cudaGetLastError());
     }
     if (sum) {
-      int64_t* prefix;
       SDB_TRY(radix_sort_pairs(key, val, ktmp, vtmp, n, 2 * (int)F, s, &ks, &vs));
-      SDB_TRY(sc.get(&prefix, n + 1));
+      // the prefix sums go where the sort's other keys were: 24 bytes a point in all, as
+      // much as the sort by tile takes
+      int64_t* prefix = reinterpret_cast<int64_t*>(ks == key ? ktmp : key);
       SDB_TRY(exclusive_scan_i32(reinterpret_cast<const int32_t*>(vs), prefix, n, s));
       S.prefix = prefix;
     } else {
