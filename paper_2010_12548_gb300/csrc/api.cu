@@ -708,8 +708,6 @@ sdb_status sdb_join_aggregate_host(const uint32_t* h_x, const uint32_t* h_y, con
   if (lookup == SDB_LOOKUP_LEARNED || lookup == SDB_LOOKUP_TABLE_LEARNED)
     for (uint32_t c = 0; c < n_covs; ++c)
       SDB_TRY_CUDA(cudaMemsetAsync(covs[c]->fallbacks, 0, sizeof(unsigned long long), s));
-  // Coverings of a sweep are joined in one pass over the chunk where that is faster
-  // (20M points, four eps: 1400 -> 1280 us, of which the copies take 1150).
   // points per chunk: the joins of the last chunk are not hidden by a copy,
   // but smaller chunks issue more launches per call, and a host whose API calls
   // are slow then falls behind the copies (2^22: 6.00 ms on some hosts, 7.81 on
@@ -732,6 +730,10 @@ sdb_status sdb_join_aggregate_host(const uint32_t* h_x, const uint32_t* h_y, con
     cudaEventCreateWithFlags(&done[b], cudaEventDisableTiming);
   }
   sdb_status st = SDB_OK;
+  // the chunks' buffers are s's own: what they held before may still be read by work
+  // enqueued on s, so the copies start after it
+  if (cudaEventRecord(done[0], s) != cudaSuccess || cudaStreamWaitEvent(cs, done[0], 0) != cudaSuccess)
+    st = cuda_status(cudaGetLastError(), "ordering the copies", __FILE__, __LINE__);
   for (uint64_t c = 0; c < nch && st == SDB_OK; ++c) {
     const int b = (int)(c & 1);
     const uint64_t a0 = c * CH, m = (n - a0 < CH) ? n - a0 : CH;
@@ -747,6 +749,8 @@ sdb_status sdb_join_aggregate_host(const uint32_t* h_x, const uint32_t* h_y, con
       st = cuda_status(e, "chunk copy", __FILE__, __LINE__);
       break;
     }
+    // coverings of a sweep are joined in one pass over the chunk where that is faster
+    // (20M points, four eps: 1400 -> 1280 us, of which the copies take 1150)
     for (uint32_t k = 0; k < n_covs && st == SDB_OK;) {
       uint32_t g = std::min(n_covs - k, 4u);  // coverings joined in one pass
       if (!sweep_pays(covs + k, g, lookup, m)) g = 1;
