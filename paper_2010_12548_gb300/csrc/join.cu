@@ -549,6 +549,17 @@ sdb_status launch_zero(const ZeroArgs& z, cudaStream_t s) {
   return SDB_OK;
 }
 
+// Lets kern take as much dynamic shared memory as any of its launches asks for.  The limit
+// is the kernel's, for every thread of the process: set to each launch's own size, it
+// could be lowered by another thread's launch in between, and the launch was refused.
+constexpr size_t SMEM_LIMIT = 224 * 1024;  // of 227 KB a block, the rest static
+sdb_status allow_smem(const void* kern, size_t smem) {
+  if (smem > 48 * 1024)
+    SDB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)SMEM_LIMIT));
+  return SDB_OK;
+}
+
 // launches kern after a zero_kernel (early: overlapping it) or by itself
 template <class Args>
 sdb_status launch_after(void (*kern)(Args), unsigned blocks, int threads, size_t smem,
@@ -771,8 +782,7 @@ sdb_status launch_t(const JoinArgs& A, cudaStream_t s, bool early) {
   smem = (smem + 15) & ~(size_t)15;
   if (TOP) smem += top_bytes(A);
   auto kern = join_kernel<LOOKUP, SMEM, SUM, RANGE, TOP>;
-  if (smem > 48 * 1024)
-    SDB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  SDB_TRY(allow_smem(reinterpret_cast<const void*>(kern), smem));
   int per_sm = 0;
   static OccupancyCache cache;
   SDB_TRY(cache.get(reinterpret_cast<const void*>(kern), TPB, smem, &per_sm));
@@ -897,8 +907,7 @@ sdb_status launch_multi_t(const MultiArgs& M, cudaStream_t s, bool early) {
   if (SMEM) smem += (size_t)M.E * acc_bytes(M.c[0].P, SUM, false);
   smem = (smem + 15) & ~(size_t)15;
   auto kern = join_multi_kernel<LOOKUP, SMEM, SUM>;
-  if (smem > 48 * 1024)
-    SDB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  SDB_TRY(allow_smem(reinterpret_cast<const void*>(kern), smem));
   int per_sm = 0;
   SDB_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, THREADS, smem));
   if (per_sm < 1) per_sm = 1;
@@ -1227,6 +1236,7 @@ size_t sweep_smem(const SweepArgs& S, size_t P, bool SUM) {
 // accumulators in shared memory as long as one block holds them (about 1690 polygons
 // with sums, 5080 without)
 constexpr size_t SWEEP_SMEM_MAX = 220 * 1024;
+static_assert(SWEEP_SMEM_MAX + 4096 <= SMEM_LIMIT, "the sweep's launches");
 // polygons up to which the pass is taken in place of separate joins (see sweep_pays):
 // the sets of more leave L1 too little for the tables' reads
 constexpr uint32_t SWEEP_PAYS_POLYS = 512;
@@ -1235,8 +1245,7 @@ template <int LOOKUP, bool SMEM, bool SUM>
 sdb_status launch_sweep_t(const SweepArgs& S, cudaStream_t s, bool early) {
   const size_t smem = sweep_smem(S, SMEM ? S.c[0].P : 0, SUM);
   auto kern = sweep_kernel<LOOKUP, SMEM, SUM>;
-  if (smem > 48 * 1024)
-    SDB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  SDB_TRY(allow_smem(reinterpret_cast<const void*>(kern), smem));
   int per_sm = 0;
   static OccupancyCache cache;
   SDB_TRY(cache.get(reinterpret_cast<const void*>(kern), SWEEP_THREADS, smem, &per_sm));

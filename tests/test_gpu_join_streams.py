@@ -1,4 +1,7 @@
-"""Joins beside other work: a host-buffer join behind work on its stream."""
+"""Joins beside other work: a host-buffer join behind work on its stream, and threads
+whose joins need different amounts of shared memory."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -47,3 +50,39 @@ def test_host_join_behind_work_on_its_stream(cuda, sdblib):
         assert np.array_equal(sm, want[1].cpu().numpy())
     for c in covs:
         c.free()
+
+
+def test_threads_with_different_shared_memory(cuda, sdblib):
+    """Two threads' joins through the same kernel, of few polygons and of many."""
+    torch = cuda
+    rng = np.random.default_rng(3)
+    n = 2000
+    x, y, a = dev(torch, *(rng.integers(0, 2 ** B, n, dtype=np.uint32) for _ in range(3)))
+    jobs, fails = [], []
+    for P in (8, 1900):
+        T = W.voronoi_tiling(rng, P, B, nverts=(4, 8))
+        c = sdblib.build_covering(T, B, EPS)
+        sdblib.covering_build_table(c, 18)
+        want = i64(torch, P), i64(torch, P)
+        sdblib.join_aggregate(x, y, a, c, sdblib.LOOKUP_TABLE, *want)
+        jobs.append((c, want, (i64(torch, P), i64(torch, P)), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    start = threading.Barrier(2)
+
+    def work(c, want, got, stream):
+        try:
+            start.wait()
+            for _ in range(4000):
+                sdblib.join_aggregate(x, y, a, c, sdblib.LOOKUP_TABLE, *got, stream=stream)
+            stream.synchronize()
+            assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+        except Exception as e:  # noqa: BLE001
+            fails.append(e)
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not fails, fails
+    for j in jobs:
+        j[0].free()
