@@ -1267,10 +1267,12 @@ sdb_status launch_pick(const JoinArgs& A, int lookup, bool has_sum, cudaStream_t
     return has_sum ? launch_t<0, false, true, RANGE>(A, s, early) : launch_t<0, false, false, RANGE>(A, s, early);
   }
   // The table lookups with the top level in shared memory.  The range join's
-  // accumulators (32 bytes a polygon) leave room for two blocks per SM up to about
-  // 640 polygons; above that its 64 warps without the level are better.
-  const bool top =
-      A.top && (!RANGE || !smem || acc_bytes(A.P, has_sum, RANGE) <= (size_t)20 * 1024);
+  // accumulators (32 bytes a polygon, 8 without sums) take the room of L1 and, with many
+  // polygons, of a block; 10M points, us with the level and without: sums, 263 polygons
+  // 59 and 65, 330: 66 and 64, 400: 72 and 66, 630: 91 and 71; no sums, 263: 45 and 57,
+  // 630: 52 and 61, 800: 56 and 61, 1024: 99 and 61.  Accumulating in global memory
+  // either takes the same, and 100,000 points 18 and 15.
+  const bool top = A.top && (!RANGE || (smem && A.P <= (has_sum ? 300u : 800u)));
   {
     if (top && lookup == SDB_LOOKUP_TABLE) {
       if (smem)
