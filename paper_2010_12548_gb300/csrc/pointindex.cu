@@ -328,28 +328,30 @@ __device__ __forceinline__ void group_sums(uint32_t group, uint32_t c, uint64_t 
 // polygon add up by warp reductions and send one atomic pair.  4.2M ranges over 50M
 // points: 138 us in two kernels with a global atomic pair per range and polygon,
 // this 115 us (a hash of polygons in shared memory per 256 ranges: 231 us, its
-// 64-bit shared atomics being slow).
+// 64-bit shared atomics being slow).  Lists of many polygons take a warp a round each,
+// so where few ranges leave warps idle a warp takes fewer than 31 (`per`: 15, 7 or 3;
+// 200 overlapping stars, 4096 ranges: the call 51 -> 34 us).
 template <bool RS, bool SUM>
 __global__ __launch_bounds__(256) void point_ranges_kernel(
-    const uint64_t* __restrict__ start, uint64_t R, uint32_t sh, Spline S,
+    const uint64_t* __restrict__ start, uint64_t R, uint32_t per, uint32_t sh, Spline S,
     const uint32_t* __restrict__ pay, const uint32_t* __restrict__ list_off,
     const uint32_t* __restrict__ list_ids, const int64_t* __restrict__ prefix,
     unsigned long long* __restrict__ count, unsigned long long* __restrict__ sum) {
   const uint32_t lane = threadIdx.x & 31;
-  const uint64_t r0 = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 31;
+  const uint64_t r0 = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per;
   if (r0 >= R) return;  // whole warps
-  const uint64_t r = min(r0 + lane, R);
+  const uint64_t r = min(r0 + min(lane, per), R);
   const uint64_t q = __ldg(start + r) << sh;
-  const bool on = lane < 31 && r0 + lane < R;
+  const bool on = lane < per && r0 + lane < R;
   const uint32_t py = on ? __ldg(pay + r) : NONE;
   uint64_t p;
   if (!RS) {
     p = lower_bound_in(S.key, 0, S.n, q);
   } else {
     uint32_t a = 0;
-    if (lane == 0 || lane == 31)
+    if (lane == 0 || lane == per)
       a = q <= S.kmin ? 0u : q > S.kmax ? (uint32_t)S.ns - 1 : spline_segment(S, q);
-    const uint32_t b = __shfl_sync(FULL, a, 31);
+    const uint32_t b = __shfl_sync(FULL, a, per);
     a = __shfl_sync(FULL, a, 0);
     if (q <= S.kmin) {
       p = 0;
@@ -362,7 +364,7 @@ __global__ __launch_bounds__(256) void point_ranges_kernel(
         len -= half;
       }
       // a boundary that two warps share is counted by the one it starts
-      p = spline_position(S, a, q, r == r0 + lane && (lane < 31 || r == R));
+      p = spline_position(S, a, q, r == r0 + lane && (lane < per || r == R));
     }
   }
   const uint32_t lo = (uint32_t)p, hi = __shfl_down_sync(FULL, lo, 1);
@@ -518,8 +520,10 @@ sdb_status point_index_aggregate(const sdb_points* p, const sdb_covering* cov, i
   auto* su = reinterpret_cast<unsigned long long*>(sum);
   auto kern = rs ? (sum ? point_ranges_kernel<true, true> : point_ranges_kernel<true, false>)
                  : (sum ? point_ranges_kernel<false, true> : point_ranges_kernel<false, false>);
-  const uint64_t warps = (R + 30) / 31;
-  kern<<<grid_for(warps, 8), 256, 0, s>>>(cov->start, R, sh, S, cov->pay, cov->list_off,
+  uint32_t per = 31;  // ranges per warp, fewer while there are not 16 warps per SM
+  while (per > 3 && R < (uint64_t)per * 16 * num_sms()) per >>= 1;
+  const uint64_t warps = (R + per - 1) / per;
+  kern<<<grid_for(warps, 8), 256, 0, s>>>(cov->start, R, per, sh, S, cov->pay, cov->list_off,
                                           cov->list_ids, p->prefix, c, su);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
