@@ -101,8 +101,10 @@ __device__ __forceinline__ long long warp_max(long long v) {
 // goes to leaf lam_i; the leaves lam_{i-1} < l <= lam_i have exactly i starts
 // below their base (lam_{-1} = -1, and start_R = 4^F stands for leaf L).  A thread's
 // work is one chain of dependent reads: BELOW_ITEMS starts per thread, all read first
-// (263-zone sweep, 27M ranges: 122 us with one, 101 with four).
-constexpr int BELOW_ITEMS = 4;
+// (263-zone sweep, 27M ranges: 122 us with one, 101 with four).  One start per thread
+// where leaves outnumber ranges: the leaves between two starts are then the longer chain
+// (2^20 leaves over 4^8 ids, the whole index: 670 us with four, 440 with one).
+template <int BELOW_ITEMS>
 __global__ void leaf_below_kernel(const uint64_t* __restrict__ start, uint64_t R,
                                   const float* __restrict__ knot, uint32_t wshift, float inv_w,
                                   uint32_t L, uint32_t* __restrict__ below) {
@@ -179,44 +181,55 @@ __device__ __forceinline__ void fit_leaf(const uint64_t* __restrict__ start, uin
   *lo = warp_max(elo);
 }
 
-// one warp per leaf: centred least squares (FP32), error window
-__global__ void leaf_fit_kernel(const uint64_t* __restrict__ start, uint64_t R,
-                                const uint64_t* __restrict__ base,
-                                const uint32_t* __restrict__ below, uint32_t L,
-                                LeafRec* __restrict__ leaves) {
-  uint32_t l = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
-  if (l >= L) return;
-  const uint64_t b0 = base[l], b1 = base[l + 1];
-  // range holding b0: the last start <= b0 (b0 < 4^F = start[R] for l < L)
-  const uint32_t c0 = below[l];
-  uint64_t first = (c0 < R && start[c0] == b0) ? c0 : (uint64_t)c0 - 1;
-  first = first < R ? first : R - 1;
-  LeafRec lr;
-  lr.base = b0;
-  lr.a = 0.f;
-  lr.b = 0.f;
-  lr.errlo = 0;
-  lr.errhi = 0;
-  if (b0 >= b1) {  // no id is routed here
-    lr.first = lr.last = (uint32_t)first;
-    if (lane == 0) leaves[l] = lr;
-    return;
+// PER leaves per warp: a lane looks at each, writes it if no id is routed to it or one
+// range holds all of its ids (the constant line, without error), and the warp fits the
+// others one after the other: centred least squares (FP32), error window.  One leaf per
+// warp, or 32 where leaves outnumber ranges, few are fitted and 4096 warps are left (2^20
+// leaves over 4^8 ids, the whole index: 440 -> 290 us; 250,000 ranges: 720 -> 300).
+template <int PER>
+__global__ __launch_bounds__(256, 6) void leaf_fit_kernel(const uint64_t* __restrict__ start,
+                                                          uint64_t R,
+                                                          const uint64_t* __restrict__ base,
+                                                          const uint32_t* __restrict__ below,
+                                                          uint32_t L, LeafRec* __restrict__ leaves) {
+  const uint32_t l0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * PER;
+  const int lane = threadIdx.x & 31;
+  if (l0 >= L) return;  // whole warps (L is a multiple of PER)
+  uint64_t b0 = 0, b1 = 0, first = 0, last = 0;
+  bool fit = false;
+  if (lane < PER) {
+    const uint32_t l = l0 + lane;
+    b0 = base[l];
+    b1 = base[l + 1];
+    // range holding b0: the last start <= b0 (b0 < 4^F = start[R] for l < L)
+    const uint32_t c0 = below[l];
+    first = (c0 < R && start[c0] == b0) ? c0 : (uint64_t)c0 - 1;
+    first = first < R ? first : R - 1;
+    last = first;
+    if (b0 < b1) {
+      last = (uint64_t)below[l + 1] - 1;  // range holding b1 - 1
+      last = last < first ? first : (last < R ? last : R - 1);
+    }
+    fit = last > first;
+    if (!fit) leaves[l] = LeafRec{b0, 0.f, 0.f, (uint32_t)first, (uint32_t)last, 0, 0};
   }
-  uint64_t last = (uint64_t)below[l + 1] - 1;  // range holding b1 - 1
-  last = last < first ? first : (last < R ? last : R - 1);
-  lr.first = (uint32_t)first;
-  lr.last = (uint32_t)last;
-  const uint64_t n = last - first + 1;
-  long long ehi = 0, elo = 0;
-  if (b1 - b0 <= 0xffffffffull)
-    fit_leaf<uint32_t, int32_t>(start, first, n, b0, b1, &lr, &elo, &ehi);
-  else
-    fit_leaf<uint64_t, int64_t>(start, first, n, b0, b1, &lr, &elo, &ehi);
-  const long long CAP = 1ll << 30;
-  lr.errhi = (int32_t)(ehi > CAP ? CAP : ehi);
-  lr.errlo = (int32_t)(elo > CAP ? CAP : elo);
-  if (lane == 0) leaves[l] = lr;
+  for (uint32_t todo = __ballot_sync(0xffffffffu, fit); todo; todo &= todo - 1) {
+    const int j = __ffs(todo) - 1;
+    const uint64_t B0 = __shfl_sync(0xffffffffu, (unsigned long long)b0, j);
+    const uint64_t B1 = __shfl_sync(0xffffffffu, (unsigned long long)b1, j);
+    const uint64_t f = __shfl_sync(0xffffffffu, (unsigned long long)first, j);
+    const uint64_t n = __shfl_sync(0xffffffffu, (unsigned long long)last, j) - f + 1;
+    LeafRec lr{B0, 0.f, 0.f, (uint32_t)f, (uint32_t)(f + n - 1), 0, 0};
+    long long ehi = 0, elo = 0;
+    if (B1 - B0 <= 0xffffffffull)
+      fit_leaf<uint32_t, int32_t>(start, f, n, B0, B1, &lr, &elo, &ehi);
+    else
+      fit_leaf<uint64_t, int64_t>(start, f, n, B0, B1, &lr, &elo, &ehi);
+    const long long CAP = 1ll << 30;
+    lr.errhi = (int32_t)(ehi > CAP ? CAP : ehi);
+    lr.errlo = (int32_t)(elo > CAP ? CAP : elo);
+    if (lane == 0) leaves[l0 + j] = lr;
+  }
 }
 
 }  // namespace
@@ -264,12 +277,20 @@ sdb_status build_learned_index(sdb_covering* cov, uint32_t leaf_bits, uint32_t r
                                                                  base);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
-  leaf_below_kernel<<<grid_for((size_t)R + 1, 256 * BELOW_ITEMS), 256, 0, s>>>(cov->start, R, cov->knots, wshift,
-                                                                   inv_w, L, below);
+  if (R > L)
+    leaf_below_kernel<4><<<grid_for((size_t)R + 1, 256 * 4), 256, 0, s>>>(cov->start, R, cov->knots,
+                                                                          wshift, inv_w, L, below);
+  else
+    leaf_below_kernel<1><<<grid_for((size_t)R + 1, 256), 256, 0, s>>>(cov->start, R, cov->knots,
+                                                                      wshift, inv_w, L, below);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
-  leaf_fit_kernel<<<grid_for((size_t)L * 32, 256), 256, 0, s>>>(cov->start, R, base, below, L,
-                                                                  cov->leaves);
+  if (R > L || L < (1u << 17))
+    leaf_fit_kernel<1><<<grid_for((size_t)L * 32, 256), 256, 0, s>>>(cov->start, R, base, below, L,
+                                                                     cov->leaves);
+  else
+    leaf_fit_kernel<32><<<grid_for(L, 256), 256, 0, s>>>(cov->start, R, base, below, L,
+                                                         cov->leaves);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
   SDB_TRY_CUDA(cudaStreamSynchronize(s));

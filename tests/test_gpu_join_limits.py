@@ -24,7 +24,7 @@ def covering(sdb, T, flags=0, bits=18):
     return c
 
 
-@pytest.mark.parametrize("P", [255, 256, 300, 630, 650, 1024, 1025])
+@pytest.mark.parametrize("P", [255, 300, 301, 650, 800, 801, 1024, 1025])
 def test_range_join_by_polygon_count(cuda, sdblib, orc, P):
     torch = cuda
     T = W.voronoi_tiling(np.random.default_rng(P), P, B, nverts=(4, 12))

@@ -1,10 +1,12 @@
 """Joins beside other work: a host-buffer join behind work on its stream, and threads
 whose joins need different amounts of shared memory."""
-import threading
+import os
+import subprocess
 
 import numpy as np
 import pytest
 
+from paper_2010_12548_gb300 import build
 from paper_2010_12548_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -52,37 +54,60 @@ def test_host_join_behind_work_on_its_stream(cuda, sdblib):
         c.free()
 
 
-def test_threads_with_different_shared_memory(cuda, sdblib):
-    """Two threads' joins through the same kernel, of few polygons and of many."""
-    torch = cuda
-    rng = np.random.default_rng(3)
-    n = 2000
-    x, y, a = dev(torch, *(rng.integers(0, 2 ** B, n, dtype=np.uint32) for _ in range(3)))
-    jobs, fails = [], []
-    for P in (8, 1900):
-        T = W.voronoi_tiling(rng, P, B, nverts=(4, 8))
-        c = sdblib.build_covering(T, B, EPS)
-        sdblib.covering_build_table(c, 18)
-        want = i64(torch, P), i64(torch, P)
-        sdblib.join_aggregate(x, y, a, c, sdblib.LOOKUP_TABLE, *want)
-        jobs.append((c, want, (i64(torch, P), i64(torch, P)), torch.cuda.Stream()))
-    torch.cuda.synchronize()
-    start = threading.Barrier(2)
+THREADS = r"""
+#include <cuda_runtime.h>
+#include <atomic>
+#include <cstdio>
+#include <thread>
+#include <vector>
+#include "sdb.h"
+int main() {
+  const uint32_t n = 2000;
+  uint32_t* x;
+  if (cudaMalloc(&x, n * 4) || cudaMemset(x, 1, n * 4)) return 2;
+  sdb_covering* cov[2];
+  for (int k = 0; k < 2; ++k) {
+    const uint32_t P = k ? 1900 : 8;
+    std::vector<uint32_t> off(P + 1), vx, vy;
+    for (uint32_t j = 0; j < P; ++j) {
+      const uint32_t a = 100 + 300 * (j % 45), b = 100 + 300 * (j / 45);
+      for (uint32_t i = 0; i < 4; ++i) {
+        vx.push_back(a + (i == 1 || i == 2 ? 200 : 0));
+        vy.push_back(b + (i >= 2 ? 200 : 0));
+      }
+      off[j + 1] = 4 * (j + 1);
+    }
+    const sdb_polygons p{P, off.data(), vx.data(), vy.data()};
+    if (sdb_build_covering(&p, 18, 64, nullptr, &cov[k])) return 3;
+    if (sdb_covering_build_table(cov[k], 18, nullptr)) return 4;
+  }
+  std::atomic<int> failed{0};
+  auto work = [&](int k) {
+    cudaStream_t s;
+    uint64_t* c;
+    cudaStreamCreate(&s);
+    cudaMalloc(&c, 2 * 1900 * 8);
+    for (int i = 0; i < 30000; ++i)
+      if (sdb_join_aggregate(x, x, (int32_t*)x, n, cov[k], SDB_LOOKUP_TABLE, c, (int64_t*)c + 1900, s)
+          && !failed++)
+        printf("%s\n", sdb_last_error());
+    cudaStreamSynchronize(s);
+  };
+  std::thread a(work, 0), b(work, 1);
+  a.join();
+  b.join();
+  printf("failed: %d\n", failed.load());
+  return failed != 0;
+}
+"""
 
-    def work(c, want, got, stream):
-        try:
-            start.wait()
-            for _ in range(4000):
-                sdblib.join_aggregate(x, y, a, c, sdblib.LOOKUP_TABLE, *got, stream=stream)
-            stream.synchronize()
-            assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
-        except Exception as e:  # noqa: BLE001
-            fails.append(e)
-    threads = [threading.Thread(target=work, args=j) for j in jobs]
-    for t in threads:
-        t.start()
-    for t in threads:
-        t.join()
-    assert not fails, fails
-    for j in jobs:
-        j[0].free()
+
+def test_threads_with_different_shared_memory(cuda, sdblib, tmp_path):
+    """Two threads' joins through the same kernel, of few polygons and of many."""
+    src, exe = tmp_path / "threads.cu", str(tmp_path / "threads")
+    src.write_text(THREADS)
+    subprocess.check_call([build.nvcc(), *build.ARCH, "-std=c++17", "-I", build.INCLUDE, "-o", exe,
+                           str(src), sdblib.LIB_PATH,
+                           "-Xlinker", "-rpath=" + os.path.dirname(sdblib.LIB_PATH)])
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stdout
