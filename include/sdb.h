@@ -463,9 +463,10 @@ typedef struct sdb_batch_info {
   uint64_t max_ranges;     /* largest covering of one query */
   uint64_t n_cells;        /* raster cells emitted before merging */
   uint64_t candidates;     /* points in the viewports' candidate index ranges */
-  uint64_t n_tiles;        /* work items of the persistent launch */
-  uint32_t tile;           /* points per work item */
-  uint32_t points_per_thread;
+  uint64_t n_tiles;        /* tiles of at most `tile` points */
+  uint32_t tile;           /* points per tile, as set (the launch cuts longer ones) */
+  uint32_t points_per_thread; /* as set: a warp takes 64 times as many points at once, or
+                                 fewer in small batches */
   uint32_t lookup;         /* SDB_LOOKUP_BINARY or SDB_LOOKUP_LEARNED */
   uint32_t indexed_queries;/* queries searched through their learned index */
   uint64_t n_leaves;       /* learned leaves over all queries */
@@ -506,16 +507,17 @@ sdb_status sdb_batch_run(sdb_batch *b, int mode, uint64_t *d_count, int64_t *d_s
  * device -- a linear root over the span of its range starts picking one of up
  * to 2^16 leaves (about SDB_BATCH_RANGES_PER_LEAF ranges each), each leaf an
  * FP32 least-squares line with the largest prediction errors below and above
- * measured by the lookup's own arithmetic; a point searches its leaf's error
- * window, the result is verified and binary search over the query's ranges is
+ * measured by the lookup's own arithmetic.  The first and last of the consecutive
+ * points that a warp takes search their leaf's error window (the others lie between
+ * them), the result is verified and binary search over the query's ranges is
  * the counted fallback, so results are identical to binary search.  Smaller
  * coverings keep binary search.  Synchronises cuda_stream.  SDB_EINVAL: another
  * lookup. */
 #define SDB_BATCH_LEARNED_MIN_RANGES 64u
 #define SDB_BATCH_RANGES_PER_LEAF 8u
 sdb_status sdb_batch_set_lookup(sdb_batch *b, int lookup, void *cuda_stream);
-/* Learned searches of the most recent run that fell back to binary search.
- * Synchronises cuda_stream. */
+/* Learned searches of the most recent run that fell back to binary search (of the
+ * points that search, see above).  Synchronises cuda_stream. */
 sdb_status sdb_batch_fallbacks(const sdb_batch *b, void *cuda_stream, uint64_t *out);
 
 /* Autotuner: times the persistent launch on this batch for tiles of 1024,

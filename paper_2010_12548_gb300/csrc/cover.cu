@@ -21,8 +21,10 @@
 // rightward ray from (0,0)+.
 //
 // Where the queries' levels are deep enough the refinement stops five levels above
-// the finest one and the rest is done in bitmaps (covertiles.cu).  Otherwise, and
-// for overlapping polygons, emitted cells become (lo = h * 4^(F-L), level) records; a sweep over all
+// the finest one and the rest is done in bitmaps (covertiles.cu), for one query's
+// overlapping polygons too.  Otherwise (finest level below 8, the non-conservative
+// rule, too many polygons in a tile or over one another, overlap among a batch's
+// queries) emitted cells become (lo = h * 4^(F-L), level) records; a sweep over all
 // record endpoints (sort, unique, per-interval polygon lists, merge of equal
 // neighbours) gives the canonical ranges.
 #include "cover_internal.cuh"

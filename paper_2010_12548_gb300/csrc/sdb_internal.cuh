@@ -335,14 +335,13 @@ struct BatchQueryDev {
   uint64_t sbase;  // first entry of the query's covering slice in its chunk
   uint32_t R;      // ranges in the slice (the sentinel follows)
   uint32_t chunk;
-  uint32_t k, nsteps, st0;
+  uint32_t k;
   uint32_t x0, y0, x1, y1;
   uint32_t out_off;
   // learned index of the slice (nleaves = 0: binary search): ids below llo lie
   // in range 0, ids from lhi on in range R - 1; between them leaf
   // min(nleaves - 1, (h - llo) >> lwshift) of the batch's leaf array, from loff
   uint32_t nleaves, loff, lwshift;
-  uint32_t npoly;  // output slots of the query (its subset's size)
   uint64_t llo, lhi;
 };
 struct BatchChunkDev {
