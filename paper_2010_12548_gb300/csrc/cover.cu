@@ -1714,7 +1714,7 @@ sdb_status build_coverings(const PolyEdges& pe, const CoverSpec& spec, cudaStrea
   // A tile is kept when its cell holds points of the viewport, and then counts as a
   // whole: polygons that overlap only outside a viewport, in a tile at its edge, look
   // nested.  The refinement drops cells one by one and decides.
-  if (outcome == TileOutcome::nested && spec.Q != 1 && !clipped(spec)) {
+  if (outcome == TileOutcome::overlapping || (outcome == TileOutcome::nested && !clipped(spec))) {
     set_error("batched coverings need polygons that do not overlap within a query");
     return SDB_EINVAL;
   }

@@ -59,11 +59,13 @@ sdb_status finish_queries(const QueryFix* dq, const uint64_t* qopen, const uint3
                           uint64_t n_elements, uint64_t n_cells, const QueryOut* d_out,
                           CoverSet* out, cudaStream_t s);
 
-enum class TileOutcome { made, nested, crowded };
+enum class TileOutcome { made, nested, overlapping, crowded };
 // The covering set from the n_rec coarse records (rkey, rval) and the n_tile
-// tile items with their edge lists (covertiles.cu).  nested: cells of different
-// polygons of one of several queries overlap at different levels; crowded: a tile
-// meets too many polygons, or too many lie over one another; then nothing is made.
+// tile items with their edge lists (covertiles.cu).  overlapping: cells of different
+// polygons of one of several queries overlap at different levels inside a tile; nested:
+// the same of coarser cells and whole tiles, of which a viewport may keep no cell;
+// crowded: a tile meets too many polygons, or too many lie over one another; then
+// nothing is made.
 sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_rec, const Item* items,
                        uint64_t n_tile, const uint32_t* elist, const Edge* edges,
                        const uint32_t* pair_query, const uint32_t* pair_slot,

@@ -1434,7 +1434,9 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   SDB_TRY_CUDA(cudaMemcpyAsync(hsums.data(), front, 3 * SPREAD * 8, cudaMemcpyDeviceToHost, s));
   SDB_TRY_CUDA(cudaStreamSynchronize(s));
   if (hflag[1] || (Q > 1 && (hflag[0] || hflag[2]))) {
-    *outcome = hflag[1] ? TileOutcome::crowded : TileOutcome::nested;
+    *outcome = hflag[1]   ? TileOutcome::crowded
+               : hflag[2] ? TileOutcome::overlapping
+                          : TileOutcome::nested;
     return SDB_OK;
   }
   unsigned long long nfront = 0;
