@@ -213,16 +213,20 @@ __global__ void tile_count_kernel(const uint32_t* __restrict__ cand,
   atomicMax(all + 1, (unsigned long long)most);
 }
 
-__global__ void tile_fill_kernel(const uint32_t* __restrict__ cand,
-                                 const uint32_t* __restrict__ ncand, uint32_t Q, uint32_t T,
-                                 const uint64_t* __restrict__ toff, TileRec* __restrict__ tiles) {
-  uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= Q) return;
+// a block per query: one of many points has many tiles
+__global__ __launch_bounds__(128) void tile_fill_kernel(const uint32_t* __restrict__ cand,
+                                                        const uint32_t* __restrict__ ncand,
+                                                        uint32_t T,
+                                                        const uint64_t* __restrict__ toff,
+                                                        TileRec* __restrict__ tiles) {
+  const uint32_t q = blockIdx.x;
   uint64_t t = toff[q];
   for (uint32_t i = 0; i < ncand[q]; ++i) {
     const uint32_t a = cand[(size_t)q * MAXC * 2 + 2 * i], b = cand[(size_t)q * MAXC * 2 + 2 * i + 1];
-    for (uint64_t s = a; s < b; s += T)
-      tiles[t++] = TileRec{q, (uint32_t)s, (uint32_t)min((uint64_t)b, s + T), 0};
+    const uint64_t m = ((uint64_t)b - a + T - 1) / T;
+    for (uint64_t j = threadIdx.x; j < m; j += 128)
+      tiles[t + j] = TileRec{q, (uint32_t)(a + j * T), (uint32_t)min((uint64_t)b, a + (j + 1) * T), 0};
+    t += m;
   }
 }
 
@@ -330,7 +334,7 @@ struct SlotSum {
 // was encoded from its coordinates and looked up by itself, and a block cleared and
 // scanned 2048 slots per 4096 points or, for larger subsets, sent two global
 // atomics per point: 512 views over 50M points 298 us, this 246 with 4096-point tiles
-// and 186 with pieces of 1024.
+// and 167 with pieces of 256.
 template <int G, bool SUM>
 __global__ __launch_bounds__(THREADS) void batch_kernel(BatchArgs A, uint32_t tile_lo,
                                                         uint32_t tile_hi,
@@ -631,11 +635,11 @@ sdb_status batch_query_dev(uint32_t B, const sdb_query& Qu, uint64_t out_off, Ba
 
 // The kernel's grid takes every tile for as many units as the largest may have, and most
 // ranges of a view are short, so the kernel's tiles are pieces of at most PIECE points
-// whatever size is set: with the units past the ranges' ends of 4096-point tiles, 512 views
-// over 50M points took 245 us instead of 186, and with those of 16384-point tiles, 64 small
-// views took 65 instead of 31.  A tile of "everything" would be 2^26 units for each of a batch's thousands of ranges,
-// seconds of them.
-constexpr uint32_t PIECE = 1024;
+// whatever size is set: one unit of the longest kind.  512 views over 50M points take
+// 245 us with 4096-point tiles, 186 with pieces of 1024, 177 with 512, 167 with 256; 4,096
+// views over 200M 5.43, 5.16, 4.80 and 4.88 ms.  A tile of "everything" would be 2^26 units
+// for each of a batch's thousands of ranges, seconds of them.
+constexpr uint32_t PIECE = 256;
 sdb_status batch_core_tiles(BatchCore* c, uint32_t T, cudaStream_t s) {
   Scratch sc(s);
   uint64_t *nt, *toff, *dtot;
@@ -665,8 +669,7 @@ sdb_status batch_core_tiles(BatchCore* c, uint32_t T, cudaStream_t s) {
   if (c->tiles) dfree(c->tiles, s);
   c->tiles = nullptr;
   SDB_TRY(dalloc_n(&c->tiles, total, s));
-  tile_fill_kernel<<<grid_for(c->Q, 128), 128, 0, s>>>(c->cand, c->ncand, c->Q, piece, toff,
-                                                       c->tiles);
+  tile_fill_kernel<<<c->Q, 128, 0, s>>>(c->cand, c->ncand, piece, toff, c->tiles);
   note_launch();
   SDB_TRY_CUDA(cudaGetLastError());
   SDB_TRY_CUDA(cudaStreamSynchronize(s));
