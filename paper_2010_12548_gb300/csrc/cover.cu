@@ -1382,8 +1382,9 @@ static bool tiles_crowded(const PolyEdges& pe, const CoverSpec& spec,
   struct Count {
     uint32_t tag, n;  // a tile by 32 bits of its hash
   };
-  constexpr uint32_t BITS = 13;  // at most half full
-  std::vector<Count> table(1u << BITS, Count{0, 0});
+  uint32_t bits = 9;  // at most half full
+  while ((1ull << bits) < 2 * (pairs / step + 1)) ++bits;
+  std::vector<Count> table((size_t)1 << bits, Count{0, 0});
   uint32_t skip = 0;
   for (uint32_t i = 0; i < spec.NP; ++i) {
     const uint32_t q = spec.pair_query[i];
@@ -1395,8 +1396,8 @@ static bool tiles_crowded(const PolyEdges& pe, const CoverSpec& spec,
     const uint64_t key = ((uint64_t)(x >> sh) << 25 | (y >> sh)) ^ ((uint64_t)q << 50);
     const uint64_t hash = key * 0x9E3779B97F4A7C15ull;
     const uint32_t tag = (uint32_t)(hash >> 16);
-    uint32_t at = (uint32_t)(hash >> (64 - BITS));
-    while (table[at].n && table[at].tag != tag) at = (at + 1) & ((1u << BITS) - 1);
+    uint32_t at = (uint32_t)(hash >> (64 - bits));
+    while (table[at].n && table[at].tag != tag) at = (at + 1) & ((1u << bits) - 1);
     table[at].tag = tag;
     if (++table[at].n >= SEEN && (uint64_t)table[at].n * step > MANY) return true;
   }

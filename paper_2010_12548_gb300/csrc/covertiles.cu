@@ -42,7 +42,8 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr uint32_t NONE = 0xffffffffu;
 constexpr int TPB = 256;
 constexpr int WPB = TPB / 32;
-constexpr uint32_t SPREAD = 256;  // counters that a sum over all blocks is spread over
+// counters that a sum over all tiles, and one over all blocks, is spread over
+constexpr uint32_t FRONT_SPREAD = 256, SPREAD = 64;
 
 // element info: slot (bits 0..25), covers the group's first cell (26), with the
 // boundary flag (27), covers its last cell (28), with the flag (29), tile (30)
@@ -378,7 +379,7 @@ __global__ __launch_bounds__(TPB, 4) void tile_raster_kernel(TileArgs A) {
       A.inner[a] = ((uint64_t)ns << 32) | ent;
       A.cells[a] = ncell >> 8;
       // frontier size, as the refinement would meet it; spread over counters
-      atomicAdd(A.front + (g & (SPREAD - 1)), (unsigned long long)fr);
+      atomicAdd(A.front + (g & (FRONT_SPREAD - 1)), (unsigned long long)fr);
     }
   }
 }
@@ -429,7 +430,7 @@ __global__ __launch_bounds__(TPB) void crowd_raster_kernel(TileArgs A) {
       if (lane == 0) {
         A.inner[a] = ((uint64_t)ns << 32) | s_sum[2];
         A.cells[a] = s_sum[0] >> 8;
-        atomicAdd(A.front + (g & (SPREAD - 1)), (unsigned long long)s_sum[1]);
+        atomicAdd(A.front + (g & (FRONT_SPREAD - 1)), (unsigned long long)s_sum[1]);
       }
     }
   }
@@ -1344,13 +1345,13 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   }
   uint2* heads;
   TileRec* rec;
-  uint32_t *n_heads, *info, *cells, *bits, *bbits = nullptr, *qhead;
+  uint32_t *info, *cells, *bits, *bbits = nullptr, *qhead;
   uint8_t *level, *code;
   uint64_t *inner, *cnt, *off, *coff, *tot;
-  unsigned int* dflag;  // nested, crowded, overlapping inside tiles
+  // nested, crowded, overlapping inside tiles; then the numbers of tile groups
+  unsigned int* dflag;
   unsigned long long *front, *sums;  // the last level's frontier, GroupTotals
   SDB_TRY(sc.get(&heads, n_tile));
-  SDB_TRY(sc.get(&n_heads, 2));
   SDB_TRY(sc.get(&rec, ne));
   SDB_TRY(sc.get(&info, ne));
   SDB_TRY(sc.get(&cells, ne));
@@ -1362,15 +1363,14 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   SDB_TRY(sc.get(&coff, ne));
   SDB_TRY(sc.get(&tot, 2));
   SDB_TRY(sc.get(&qhead, Q));
-  SDB_TRY(sc.get(&dflag, 3));
-  SDB_TRY(sc.get(&front, 3 * SPREAD));
-  sums = front + SPREAD;
+  SDB_TRY(sc.get(&dflag, 5));
+  SDB_TRY(sc.get(&front, FRONT_SPREAD + 2 * SPREAD));
+  sums = front + FRONT_SPREAD;
   SDB_TRY(sc.get(&bits, n_tile * 32));
   if (spec.flags) SDB_TRY(sc.get(&bbits, n_tile * 32));
-  SDB_TRY_CUDA(cudaMemsetAsync(n_heads, 0, 8, s));
-  SDB_TRY_CUDA(cudaMemsetAsync(dflag, 0, 12, s));
+  SDB_TRY_CUDA(cudaMemsetAsync(dflag, 0, 20, s));
   SDB_TRY_CUDA(cudaMemsetAsync(tot, 0, 16, s));
-  SDB_TRY_CUDA(cudaMemsetAsync(front, 0, 3 * SPREAD * 8, s));
+  SDB_TRY_CUDA(cudaMemsetAsync(front, 0, (FRONT_SPREAD + 2 * SPREAD) * 8, s));
   SDB_TRY_CUDA(cudaMemsetAsync(qhead, 0xff, (size_t)Q * 4, s));
   TileArgs ta{};
   ta.rec = rec;
@@ -1381,7 +1381,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   ta.flags = spec.flags ? 1u : 0u;
   ta.key = sk;
   ta.ne = ne;
-  ta.heads = TileHeads{heads, n_heads, (uint32_t)n_tile};
+  ta.heads = TileHeads{heads, dflag + 3, (uint32_t)n_tile};
   ta.bits = bits;
   ta.bbits = bbits;
   ta.info = info;
@@ -1404,7 +1404,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
       TraceScope tr1("cover.raster", s);
       tile_raster_kernel<<<tile_grid, TPB, 0, s>>>(ta);
       note_launch();
-      if (n_tile > CROWD) {
+      if (n_tile > CROWD && (Q > 1 || spec.NP > CROWD)) {
         crowd_raster_kernel<<<crowd_grid, TPB, 0, s>>>(ta);
         note_launch();
       }
@@ -1426,13 +1426,13 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
   if (ne && spec.split)
     SDB_TRY_CUDA(cudaMemcpyAsync(hqoff.data(), dqoff, (size_t)Q * 8, cudaMemcpyDeviceToHost, s));
   uint64_t htot[2] = {0, 0};
-  unsigned int hflag[3] = {0, 0, 0};
+  unsigned int hflag[5] = {0, 0, 0, 0, 0};
   std::vector<uint32_t> hhead(Q);
-  std::vector<unsigned long long> hsums(3 * SPREAD);
+  std::vector<unsigned long long> hsums(FRONT_SPREAD + 2 * SPREAD);
   SDB_TRY_CUDA(cudaMemcpyAsync(htot, tot, 16, cudaMemcpyDeviceToHost, s));
-  SDB_TRY_CUDA(cudaMemcpyAsync(hflag, dflag, 12, cudaMemcpyDeviceToHost, s));
+  SDB_TRY_CUDA(cudaMemcpyAsync(hflag, dflag, 20, cudaMemcpyDeviceToHost, s));
   SDB_TRY_CUDA(cudaMemcpyAsync(hhead.data(), qhead, (size_t)Q * 4, cudaMemcpyDeviceToHost, s));
-  SDB_TRY_CUDA(cudaMemcpyAsync(hsums.data(), front, 3 * SPREAD * 8, cudaMemcpyDeviceToHost, s));
+  SDB_TRY_CUDA(cudaMemcpyAsync(hsums.data(), front, hsums.size() * 8, cudaMemcpyDeviceToHost, s));
   SDB_TRY_CUDA(cudaStreamSynchronize(s));
   if (hflag[1] || (Q > 1 && (hflag[0] || hflag[2]))) {
     *outcome = hflag[1]   ? TileOutcome::crowded
@@ -1441,8 +1441,8 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
     return SDB_OK;
   }
   unsigned long long nfront = 0;
-  for (uint32_t i = 0; i < SPREAD; ++i) nfront += hsums[i];
-  GroupTotals total = group_totals(hsums.data() + SPREAD);
+  for (uint32_t i = 0; i < FRONT_SPREAD; ++i) nfront += hsums[i];
+  GroupTotals total = group_totals(hsums.data() + FRONT_SPREAD);
   const uint64_t ncells = htot[1];
   // the limits of the refinement to the finest level
   if (4 * nfront > 0xffffffffull) {
@@ -1544,7 +1544,7 @@ sdb_status cover_tiles(const uint64_t* rkey, const uint32_t* rval, uint64_t n_re
       else
         tile_emit_kernel<false><<<tile_grid, TPB, 0, s>>>(ta, off, code, dextra, ga.lomask, tb, ro);
       note_launch();
-      if (n_tile > CROWD) {
+      if (hflag[4]) {
         if (nested)
           crowd_emit_kernel<true><<<crowd_grid, TPB, 0, s>>>(ta, off, code, dextra, ga.lomask, tb, ro);
         else
