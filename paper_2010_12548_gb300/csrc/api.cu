@@ -703,11 +703,6 @@ sdb_status sdb_join_aggregate_host(const uint32_t* h_x, const uint32_t* h_y, con
   int64_t* d_sum = nullptr;
   SDB_TRY(sc.get(&d_cnt, outn));
   if (h_sum) SDB_TRY(sc.get(&d_sum, outn));
-  SDB_TRY_CUDA(cudaMemsetAsync(d_cnt, 0, outn * 8, s));
-  if (d_sum) SDB_TRY_CUDA(cudaMemsetAsync(d_sum, 0, outn * 8, s));
-  if (lookup == SDB_LOOKUP_LEARNED || lookup == SDB_LOOKUP_TABLE_LEARNED)
-    for (uint32_t c = 0; c < n_covs; ++c)
-      SDB_TRY_CUDA(cudaMemsetAsync(covs[c]->fallbacks, 0, sizeof(unsigned long long), s));
   // points per chunk: the joins of the last chunk are not hidden by a copy,
   // but smaller chunks issue more launches per call, and a host whose API calls
   // are slow then falls behind the copies (2^22: 6.00 ms on some hosts, 7.81 on
@@ -731,9 +726,15 @@ sdb_status sdb_join_aggregate_host(const uint32_t* h_x, const uint32_t* h_y, con
   }
   sdb_status st = SDB_OK;
   // the chunks' buffers are s's own: what they held before may still be read by work
-  // enqueued on s, so the copies start after it
-  if (cudaEventRecord(done[0], s) != cudaSuccess || cudaStreamWaitEvent(cs, done[0], 0) != cudaSuccess)
-    st = cuda_status(cudaGetLastError(), "ordering the copies", __FILE__, __LINE__);
+  // enqueued on s, so the copies start after it (and beside the outputs' clearing)
+  cudaError_t e0 = cudaEventRecord(done[0], s);
+  if (e0 == cudaSuccess) e0 = cudaStreamWaitEvent(cs, done[0], 0);
+  if (e0 == cudaSuccess) e0 = cudaMemsetAsync(d_cnt, 0, outn * 8, s);
+  if (e0 == cudaSuccess && d_sum) e0 = cudaMemsetAsync(d_sum, 0, outn * 8, s);
+  if (lookup == SDB_LOOKUP_LEARNED || lookup == SDB_LOOKUP_TABLE_LEARNED)
+    for (uint32_t c = 0; c < n_covs && e0 == cudaSuccess; ++c)
+      e0 = cudaMemsetAsync(covs[c]->fallbacks, 0, sizeof(unsigned long long), s);
+  if (e0 != cudaSuccess) st = cuda_status(e0, "starting the copies", __FILE__, __LINE__);
   for (uint64_t c = 0; c < nch && st == SDB_OK; ++c) {
     const int b = (int)(c & 1);
     const uint64_t a0 = c * CH, m = (n - a0 < CH) ? n - a0 : CH;
