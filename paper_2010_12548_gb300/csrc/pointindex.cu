@@ -327,10 +327,11 @@ __device__ __forceinline__ void group_sums(uint32_t group, uint32_t c, uint64_t 
 // are not read.  The curve visits few polygons in 31 ranges: the lanes of one
 // polygon add up by warp reductions and send one atomic pair.  4.2M ranges over 50M
 // points: 138 us in two kernels with a global atomic pair per range and polygon,
-// this 115 us, 149 and 125 with the outputs' clearing (a hash of polygons in shared memory per 256 ranges: 231 us, its
-// 64-bit shared atomics being slow).  Lists of many polygons take a warp a round each,
-// so where few ranges leave warps idle a warp takes fewer than 31 (`per`: 15, 7 or 3;
-// 200 overlapping stars, 4096 ranges: the call 51 -> 34 us).
+// this 115 us, 149 and 125 with the outputs' clearing (a hash of polygons in shared
+// memory per 256 ranges: 231 us, its 64-bit shared atomics being slow).  Lists of many
+// polygons take a warp a round each, so where few ranges leave warps idle a warp takes
+// fewer than 31 (`per`: 15, 7 or 3; 200 overlapping stars, 4096 ranges: the call 51 ->
+// 34 us).
 template <bool RS, bool SUM>
 __global__ __launch_bounds__(256) void point_ranges_kernel(
     const uint64_t* __restrict__ start, uint64_t R, uint32_t per, uint32_t sh, Spline S,
