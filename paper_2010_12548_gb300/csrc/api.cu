@@ -726,9 +726,14 @@ sdb_status sdb_join_aggregate_host(const uint32_t* h_x, const uint32_t* h_y, con
   }
   sdb_status st = SDB_OK;
   // the chunks' buffers are s's own: what they held before may still be read by work
-  // enqueued on s, so the copies start after it (and beside the outputs' clearing)
-  cudaError_t e0 = cudaEventRecord(done[0], s);
-  if (e0 == cudaSuccess) e0 = cudaStreamWaitEvent(cs, done[0], 0);
+  // enqueued on s, so the copies start after it (and beside the outputs' clearing); an
+  // idle stream, the usual case, spares them the wait (8 of a small call's 80 us)
+  cudaError_t e0 = cudaStreamQuery(s);
+  if (e0 == cudaErrorNotReady) {
+    cudaGetLastError();
+    e0 = cudaEventRecord(done[0], s);
+    if (e0 == cudaSuccess) e0 = cudaStreamWaitEvent(cs, done[0], 0);
+  }
   if (e0 == cudaSuccess) e0 = cudaMemsetAsync(d_cnt, 0, outn * 8, s);
   if (e0 == cudaSuccess && d_sum) e0 = cudaMemsetAsync(d_sum, 0, outn * 8, s);
   if (lookup == SDB_LOOKUP_LEARNED || lookup == SDB_LOOKUP_TABLE_LEARNED)
